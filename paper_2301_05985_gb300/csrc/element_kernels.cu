@@ -454,14 +454,15 @@ double element_kernel_flops(int D, bool jv) {
     if (!jv) return NC * (common + 2 * (6 * D + 4 + acc) + poisson) + 8 * to_m + 3 * from_m;
     return NC * (common + 2 * val + 3 * grad + 2 * (12 * D + 8 + acc) + poisson) + 11 * to_m + 3 * from_m;
   }
-  // lane form, per lane: axis stages of the value/gradient interpolation (3 flops per
-  // interpolated track, 4 per value + new derivative from one difference), the physics
-  // at the lane's Gauss point, and the transposed stages of the three test fields
-  const double tri = D * (D - 1) / 2.0;
-  const double vg = 3 * tri + 4 * D, g = vg - 2, v = 3 * D, tt = 6 * D + 3 * tri + 1;
-  const double state = 2 * vg + 2 * v + g + D * v + 2 * D + 3 + 30;
-  const double phys = jv ? 2 * vg + g + 101 : 53;
-  return NC * (state + phys + 3 * tt);
+  // lane form (lane_ops.cuh, scaled and reflected), per lane: per axis k a value costs one
+  // fused multiply-add, a value with gradient a subtraction and 1 + k of them, a test its
+  // transpose; then the physics per species and of the Poisson row
+  const double tri = D * (D - 1.0);
+  const double v = 2 * D, vg = 3 * D + tri, g = vg - 2, tt = 4 * D + tri;
+  const double state = 2 * vg + g + 2 * v + D * v + (2 * D - 1) + D + 12 + 2 * (2 + 2 * D + 2 * D - 1 + 2);
+  const double tests = 3 * tt + 3 + D + 5;
+  if (!jv) return NC * (state + 2 * (3 + 1 + 4 * D + 1) + tests);
+  return NC * (state + 2 * vg + g + 2 * (1 + 2 * D + 4 * D - 1 + 2 + 3 + 3 + 1 + 6 * D + 1) + tests);
 }
 
 template <typename T>

@@ -4,17 +4,11 @@
 //
 // Physics per Gauss point as in Def. 3 of arXiv 2301.05985 with the fine scales
 // c^f = -tau_c R_c (Sec. 3.1; the same statement as element_kernels.cu).  Interpolation
-// is a tensor product of 1D operators on the two nodes of an axis: at the Gauss point
-// next to node b (xi = -g for b = 0, +g for b = 1, g = 1/sqrt 3)
-//     value:       a u_b + b' u_{1-b} = u_b - b' (u_b - u_{1-b}),   a = (1 + g)/2, b' = (1 - g)/2
-//     derivative:  (u_1 - u_0) / h           (constant along the axis)
-// applied axis by axis with the partner value fetched by a lane shuffle (lane ^ 2^k);
-// value and derivative share the difference u_b - u_{1-b}.  The FP32 kernels execute no
-// FP64 instruction (GB300 runs FP64 at 1/64 of the FP32 rate): powers of two come from
-// the exponent bits and the parameters arrive converted.
-// The test side (element vector r_c = w sum_q [N_c(q) S_q + grad N_c(q) . Phi_q], w =
-// (h/2)^d) is the transpose: the value operator is symmetric and the derivative's
-// transpose sends s_b (x_0 + x_1) / h to node b (s_0 = -1, s_1 = +1).
+// and the test side are the butterflies of lane_ops.cuh (a partner value per axis by lane
+// shuffle); the residual and J V use their scaled reflected form, the stored linearisation
+// and the block diagonal the plain one.  The FP32 kernels execute no FP64 instruction
+// (GB300 runs FP64 at 1/64 of the FP32 rate): powers of two come from the exponent bits
+// and the parameters arrive converted.
 #include <algorithm>
 #include <cstdint>
 #include <type_traits>
@@ -179,7 +173,14 @@ __device__ __forceinline__ void scatter4(const ElemArgs<T>& A, int32_t id, const
   }
 }
 
-// T: storage type of the vectors; C: arithmetic type (T, or double-float for FP64 data)
+// T: storage type of the vectors; C: arithmetic type (T, or double-float for FP64 data).
+// What bounds it, on the membrane-band octree (971,776 elements) with advection:
+//   double-float residual: the FP32 pipe (480 M warp instructions, packed ones twice as
+//   long); 1.47 ms before, 0.595 ms now.  Before: accurate double-float operations only
+//   (FMA pipe 57 %), 41 conversions and FP64 additions per lane (FP64 pipe 45 %), 59 KB of
+//   straight code per warp.
+//   FP64 J V: the FP64 pipe (86 %); on the uniform level-6 cube 1.03 ms before, 0.76 ms now,
+//   by the operation count (318 to 230 FP64 instructions per lane).
 template <typename T, typename C, int D, bool JV>
 __global__ void __launch_bounds__(256, lane_min_blocks<T, C>()) k_element_lanes(ElemArgs<T> A, LaneParams<C> K) {
   constexpr int NC = 1 << D;
@@ -192,16 +193,17 @@ __global__ void __launch_bounds__(256, lane_min_blocks<T, C>()) k_element_lanes(
   const int32_t id = valid ? __ldg(A.conn + e * NC + c) : 0;
   const int lev = valid ? A.level[e] : 0;
 
-  const C inv_h = pow2i(lev, C(0));
-  const C w = pow2i(-D * (lev + 1), C(0));  // (h/2)^D
-  const C nb = C(-0.5 * (1.0 - kG));
-  C sh[3];
-#pragma unroll
-  for (int k = 0; k < 3; ++k) sh[k] = ((c >> k) & 1) ? inv_h : -inv_h;
-  const C G2 = pow2i(2 * lev + 2, C(0));  // (2/h)^2
-  const C kappa = K.kappa;
-  const C tau0 = fma(K.cid * G2, G2, K.tau_t);
-  const C e2 = K.e2;
+  // scaled quantities (lane_ops.cuh; c~ = c / a^D, g~ = reflected gradient h / a^(D-1)):
+  //   V = (a^(D-1) / h) v~ reflected,  beta = a^(D-2) / h^2,  delta = a^2 h^2,  alpha = a^D
+  //   S~ = kappa c~ + h~ + V . g~c,   R~ = S~ - z beta g~phi . g~c          (times alpha)
+  //   Phi~ = g~c + z alpha (c~ - tau R~) g~phi + tau delta R~ V             (times a^(D-1) / h)
+  // and the element vector is (h/2)^D a^D beta times the test transpose of (delta S~, Phi~)
+  const C rho = C(kRho);
+  const C beta = const_pow2(ipow(kVal, D - 2), 2 * lev, C(0));
+  const C delta = const_pow2(kVal * kVal, -2 * lev, C(0));
+  constexpr double cW = ipow(kVal, 2 * D - 2);
+  const int eW = 2 * lev - D * (lev + 1);
+  const C kappa = K.kappa, e2 = K.e2;
 
   C un[3], vn[3], hn[2];
   if constexpr (sizeof(T) == 4) {
@@ -218,65 +220,95 @@ __global__ void __launch_bounds__(256, lane_min_blocks<T, C>()) k_element_lanes(
     load_node_c<T, C, 2>(A, id, valid, A.hs, 2, hn);
   }
 
-  // state at this lane's Gauss point
-  C cv[2], gc[2][3], gp[3], v[3], hq[2], tau, R[2], P[2][3];
-  lane_state<C, D>(un, vn, hn, nb, sh, kappa, tau0, G2, cv, gc, gp, v, hq, tau, R, P);
-
-  C S[3], Phi[3][3];
-  if constexpr (!JV) {
-#pragma unroll
-    for (int s = 0; s < 2; ++s) {
-      const C z = s == 0 ? C(1) : C(-1);
-      C vg = C(0);
-#pragma unroll
-      for (int k = 0; k < 3; ++k) vg = fma(v[k], gc[s][k], vg);
-      S[s] = fma(kappa, cv[s], hq[s] + vg);
-      const C tR = tau * R[s];
-      const C zc = z * cv[s];
-#pragma unroll
-      for (int k = 0; k < 3; ++k) Phi[s][k] = fma(tR, P[s][k], fma(zc, gp[k], gc[s][k]));
-    }
-    S[2] = fma(tau, R[0] - R[1], cv[1] - cv[0]);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) Phi[2][k] = e2 * gp[k];
-  } else {
-    C dn[3];
+  // state at this lane's Gauss point; the species, (v_0, v_1) and (phi, v_2) or (phi, dphi)
+  // run as pairs
+  using C2 = pair_t<C>;
+  const C2 rho2 = both<C>(rho);
+  C V[D], vd[D], gp[3], dgp[3];
+  {
+    const C2 v01 = lane_v<C2, D>(pair(vn[0], vn[1]), rho2);
+    vd[0] = first(v01);
+    vd[1] = second(v01);
+  }
+  C dn[3] = {C(0), C(0), C(0)};
+  if constexpr (JV) {
     if constexpr (sizeof(T) == 4) {
       if (A.V4) load_dir4(A, id, valid, dn);
       else load_node_c<T, C, 3>(A, id, valid, A.V, 3, dn);
     } else {
       load_node_c<T, C, 3>(A, id, valid, A.V, 3, dn);
     }
-    C dcv[2], dgc[2][3], dgp[3], dR[2];
+    if constexpr (D == 3) vd[2] = lane_v<C, D>(vn[2], rho);
+  }
+  if constexpr (JV || D == 3) {
+    C2 val, g[3];
+    lane_vg<C2, D, !JV>(pair(un[2], JV ? dn[2] : vn[2]), rho2, val, g);
 #pragma unroll
-    for (int s = 0; s < 2; ++s) interp_vg<C, D>(dn[s], nb, sh, dcv[s], dgc[s]);
-    interp_g<C, D>(dn[2], nb, sh, dgp);
-#pragma unroll
-    for (int s = 0; s < 2; ++s) {
-      const C z = s == 0 ? C(1) : C(-1);
-      C vg = C(0), pg = C(0), gcd = C(0);
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        vg = fma(v[k], dgc[s][k], vg);
-        pg = fma(P[s][k], dgc[s][k], pg);
-        gcd = fma(gc[s][k], dgp[k], gcd);
-      }
-      dR[s] = fma(kappa, dcv[s], pg - z * gcd);
-      S[s] = fma(kappa, dcv[s], vg);
-      const C tdR = tau * dR[s];
-      const C zdc = z * dcv[s];
-      const C zc_tR = z * (cv[s] - tau * R[s]);
-#pragma unroll
-      for (int k = 0; k < 3; ++k) Phi[s][k] = fma(tdR, P[s][k], fma(zc_tR, dgp[k], fma(zdc, gp[k], dgc[s][k])));
+    for (int k = 0; k < D; ++k) {
+      gp[k] = first(g[k]);
+      if (JV) dgp[k] = second(g[k]);
     }
-    S[2] = fma(tau, dR[0] - dR[1], dcv[1] - dcv[0]);
+    if constexpr (!JV) vd[2] = second(val);
+  } else {
+    C unused;
+    lane_vg<C, D, false>(un[2], rho, unused, gp);
+  }
+  C vv;
 #pragma unroll
-    for (int k = 0; k < 3; ++k) Phi[2][k] = e2 * dgp[k];
+  for (int k = 0; k < D; ++k) {
+    vv = k == 0 ? vd[k] * vd[k] : fma_q(vd[k], vd[k], vv);
+    V[k] = reflect(times_const(vd[k], ipow(kVal, D - 1), lev), reflect_mask(c, k));
+  }
+  // 4/dt^2 + C_I d (2/h)^4 + (2/h)^2 |v|^2
+  const C tau = inv_sqrt(fma_q(const_pow2(ipow(kVal, 2 * D), 2 * lev + 2, C(0)), vv,
+                             times_pow2(K.cid, 4 * lev + 4) + K.tau_t));
+  const C2 taud = both<C>(tau * delta), tau2 = both<C>(tau);
+  const C2 zb = pair(-beta, beta), kap2 = both<C>(kappa);
+  constexpr double alpha = ipow(kVal, D);
+  C2 cv, gc[3];
+  lane_vg<C2, D, true>(pair(un[0], un[1]), rho2, cv, gc);
+  C2 sv = fma_q(kap2, cv, lane_v<C2, D>(pair(hn[0], hn[1]), rho2));
+  C2 gg = both<C>(gp[0]) * gc[0];
+#pragma unroll
+  for (int k = 1; k < D; ++k) gg = fma_q(both<C>(gp[k]), gc[k], gg);
+#pragma unroll
+  for (int k = 0; k < D; ++k) sv = fma_q(both<C>(V[k]), gc[k], sv);
+  const C2 R = fma_q(zb, gg, sv);
+  C2 S, Phi[3];
+  C Sp, Pp[3];
+  if constexpr (!JV) {
+    const C2 q = times_pm(cv - tau2 * R, alpha), p = taud * R;
+#pragma unroll
+    for (int k = 0; k < D; ++k) Phi[k] = fma_q(p, both<C>(V[k]), fma_q(q, both<C>(gp[k]), gc[k]));
+    S = times_const2(sv, kVal * kVal, -2 * lev);
+    Sp = times_const(fma_q(tau, first(R) - second(R), second(cv) - first(cv)), kVal * kVal, -2 * lev);
+#pragma unroll
+    for (int k = 0; k < D; ++k) Pp[k] = e2 * gp[k];
+  } else {
+    C2 dcv, dgc[3];
+    lane_vg<C2, D, true>(pair(dn[0], dn[1]), rho2, dcv, dgc);
+    C2 dsv = kap2 * dcv, dgg = both<C>(gp[0]) * dgc[0];
+#pragma unroll
+    for (int k = 1; k < D; ++k) dgg = fma_q(both<C>(gp[k]), dgc[k], dgg);
+#pragma unroll
+    for (int k = 0; k < D; ++k) {
+      dgg = fma_q(both<C>(dgp[k]), gc[k], dgg);
+      dsv = fma_q(both<C>(V[k]), dgc[k], dsv);
+    }
+    const C2 dR = fma_q(zb, dgg, dsv);
+    const C2 q1 = times_pm(cv - tau2 * R, alpha), q2 = times_pm(dcv - tau2 * dR, alpha), p = taud * dR;
+#pragma unroll
+    for (int k = 0; k < D; ++k)
+      Phi[k] = fma_q(p, both<C>(V[k]), fma_q(q2, both<C>(gp[k]), fma_q(q1, both<C>(dgp[k]), dgc[k])));
+    S = times_const2(dsv, kVal * kVal, -2 * lev);
+    Sp = times_const(fma_q(tau, first(dR) - second(dR), second(dcv) - first(dcv)), kVal * kVal, -2 * lev);
+#pragma unroll
+    for (int k = 0; k < D; ++k) Pp[k] = e2 * dgp[k];
   }
 
-  C r[3];
-#pragma unroll
-  for (int f = 0; f < 3; ++f) r[f] = w * test_t<C, D>(S[f], Phi[f], nb, sh);
+  const C2 rs = lane_test<C2, D>(S, Phi, rho2);
+  const T r[3] = {times_const(to_storage<T>(first(rs)), cW, eW), times_const(to_storage<T>(second(rs)), cW, eW),
+                  times_const(to_storage<T>(lane_test<C, D>(Sp, Pp, rho)), cW, eW)};
   if (!valid) return;
   if constexpr (sizeof(T) == 4) {
     if (A.out4) {
@@ -284,12 +316,9 @@ __global__ void __launch_bounds__(256, lane_min_blocks<T, C>()) k_element_lanes(
       return;
     }
   }
-  T ro[3];
-#pragma unroll
-  for (int f = 0; f < 3; ++f) ro[f] = to_storage<T>(r[f]);
   if (id >= 0) {
 #pragma unroll
-    for (int f = 0; f < 3; ++f) atomicAdd(A.out + 3 * (int64_t)id + f, ro[f]);
+    for (int f = 0; f < 3; ++f) atomicAdd(A.out + 3 * (int64_t)id + f, r[f]);
   } else {
     const int32_t hh = -id - 1;
     const int np = A.hang_np[hh];
@@ -297,7 +326,7 @@ __global__ void __launch_bounds__(256, lane_min_blocks<T, C>()) k_element_lanes(
     for (int p = 0; p < np; ++p) {
       const int32_t pid = A.hang_par[4 * hh + p];
 #pragma unroll
-      for (int f = 0; f < 3; ++f) atomicAdd(A.out + 3 * (int64_t)pid + f, wgt * ro[f]);
+      for (int f = 0; f < 3; ++f) atomicAdd(A.out + 3 * (int64_t)pid + f, wgt * r[f]);
     }
   }
 }

@@ -79,10 +79,9 @@ bool element_kernel_is_lanes();
 // true when the FP64 residual runs in double-float arithmetic (lane-group kernel, unless
 // PNP_RESIDUAL_ARITH=f64 selects FP64 arithmetic)
 bool residual_double_float();
-// FP32 operations per FP64 operation of the double-float arithmetic: a sum costs 20, a
-// product 10, a fused multiply-add (2 FP64 flops) 30, so 15 per flop for the FMA-dominated
-// element formulation
-constexpr double kDfFlopsPerFlop = 15.0;
+// FP32 operations per FP64 operation of the double-float arithmetic: a quick fused
+// multiply-add (2 FP64 flops) costs 18, a quick sum 11, the accurate sums 20, a product 10
+constexpr double kDfFlopsPerFlop = 10.0;
 // FP32 J V from a stored linearisation (element_lanes.cu): launch_lane_state computes, per
 // element lane, the state's Gauss-point quantities J V needs (qp: rows * 2^dim * n_elem
 // float4, A.rec set; rows = 4, or 3 when the advection field is zero); launch_jv_from_state

@@ -138,15 +138,23 @@ __device__ __forceinline__ void scatter_rows(const NsArgs<T>& A, int32_t id, con
 // physical constants in the kernel's arithmetic type
 template <typename C>
 struct NsK {
-  C isc, kap, tau_t, cid, fb;  // 1/Sc, beta0/dt, 4/dt^2, C_I Sc^2 d, kappa / (2 Lambda^2)
+  C isc, kis, tau_t, cid, fb;  // 1/Sc, beta0/(Sc dt), 4/dt^2, C_I Sc^2 d, kappa / (2 Lambda^2)
 };
 
 // One lane per (element, corner): the lane's Gauss point is the one next to its corner.
 // DATA adds the history and body-force terms (the residual F = A X - b); without them
 // the kernel applies the matrix.  T: storage type of the vectors; C: arithmetic type (T,
-// or double-float for FP64 data: GB300 runs FP64 at 1/64 of the FP32 rate).
+// or double-float for FP64 data: GB300 runs FP64 at 1/64 of the FP32 rate).  The
+// double-float matrix action is bound by the FP32 pipe: 1.41 ms before, 0.594 ms now per
+// launch on the membrane-band octree (971,776 elements), by the scaled operators, quick
+// sums and integer conversions of lane_ops.cuh and df32.cuh.
+// blocks per SM the register cap is set for (FP32: 40 registers without spills)
+template <typename T>
+constexpr int ns_min_blocks() {
+  return sizeof(T) == 4 ? 6 : 2;
+}
 template <typename T, typename C, int D, bool DATA>
-__global__ void __launch_bounds__(kNsThreads) k_ns_lanes(NsArgs<T> A, NsK<C> K) {
+__global__ void __launch_bounds__(kNsThreads, ns_min_blocks<T>()) k_ns_lanes(NsArgs<T> A, NsK<C> K) {
   constexpr int NC = 1 << D;
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if ((t & ~int64_t(31)) / NC >= A.n_elem) return;  // shuffles need the whole warp
@@ -155,49 +163,62 @@ __global__ void __launch_bounds__(kNsThreads) k_ns_lanes(NsArgs<T> A, NsK<C> K) 
   const bool valid = e < A.n_elem;
   const int32_t id = valid ? __ldg(A.conn + e * NC + c) : 0;
   const int lev = valid ? A.level[e] : 0;
-  const C inv_h = pow2i(lev, C(0));
-  const C w = pow2i(-D * (lev + 1), C(0));  // (h/2)^D
-  const C nb = C(-0.5 * (1.0 - kG));
-  C sh[3];
+  // scaled quantities (lane_ops.cuh; v~ = v / a^D, g~ = reflected gradient h / a^(D-1)):
+  //   V = (1/Sc) (a^(D-1) / h) v^ reflected (v^ the advection),  delta = a^2 h^2
+  //   R~_i = (1/Sc) (kappa v~_i + h~_i) + V . g~v_i + s_i g~p_i / (a h)     (times a^D)
+  //   momentum row i: test transpose of (delta R~_i, g~v_i + tau delta R~_i V + e_i s_i tau_sol d~),
+  //   d~ = sum_i s_i g~v_ii, times (h/2)^D a^D beta, beta = a^(D-2) / h^2;
+  //   solenoidality row: of (delta d~, s_j tau delta R~_j), times (h/2)^D a^(2D-3) / h^3
+  const C rho = C(kRho);
+  uint32_t sg[3];
 #pragma unroll
-  for (int k = 0; k < 3; ++k) sh[k] = ((c >> k) & 1) ? inv_h : -inv_h;
-  const C G2 = pow2i(2 * lev + 2, C(0));        // (2/h)^2
-  const C iG2d = pow2i(-2 * lev - 2, C(0)) * C(1.0 / D);  // 1 / (d (2/h)^2)
+  for (int k = 0; k < 3; ++k) sg[k] = reflect_mask(c, k);
 
   T xs[4], as[4];
   load4(A.hang_par, A.hang_np, A.X, id, valid, xs);
   load4(A.hang_par, A.hang_np, A.adv, id, valid, as);
-  C xn[4], an[4];
-#pragma unroll
-  for (int f = 0; f < 4; ++f) {
-    xn[f] = to_compute<C>(xs[f]);
-    an[f] = to_compute<C>(as[f]);
+  // (v_x, v_y) and (v_z, p) run as pairs, as do the test rows (0, 1) and (2, 3)
+  using C2 = pair_t<C>;
+  const C2 rho2 = both<C>(rho);
+  C V[D], va[D], vv;
+  {
+    const C2 v01 = lane_v<C2, D>(pair(to_compute<C>(as[0]), to_compute<C>(as[1])), rho2);
+    va[0] = first(v01);
+    va[1] = second(v01);
+    if constexpr (D == 3) va[2] = lane_v<C, D>(to_compute<C>(as[2]), rho);
   }
-  C v[3] = {C(0), C(0), C(0)}, gv[3][3], gp[3], va[3] = {C(0), C(0), C(0)};
-#pragma unroll
-  for (int i = 0; i < D; ++i) interp_vg<C, D>(xn[i], nb, sh, v[i], gv[i]);
-#pragma unroll
-  for (int i = D; i < 3; ++i) gv[i][0] = gv[i][1] = gv[i][2] = C(0);
-  interp_g<C, D>(xn[3], nb, sh, gp);
-  C vv = C(0);
 #pragma unroll
   for (int i = 0; i < D; ++i) {
-    va[i] = interp_v<C, D>(an[i], nb);
-    vv = fma(va[i], va[i], vv);
+    vv = i == 0 ? va[0] * va[0] : fma_q(va[i], va[i], vv);
+    V[i] = reflect(times_const(K.isc * va[i], ipow(kVal, D - 1), lev), sg[i]);
   }
-  const C arg = fma(K.cid * G2, G2, fma(G2, vv, K.tau_t));
+  const C arg = fma_q(const_pow2(ipow(kVal, 2 * D), 2 * lev + 2, C(0)), vv, times_pow2(K.cid, 4 * lev + 4) + K.tau_t);
   const C tau_m = inv_sqrt(arg);
-  const C tau_s = (arg * tau_m) * iG2d;  // 1 / (tr(G) tau_m) = sqrt(arg) / (d (2/h)^2)
-  C div = C(0);
+  // 1 / (tr(G) tau_m) = sqrt(arg) / (d (2/h)^2)
+  const C tau_s = (arg * tau_m) * const_pow2(1.0 / D, -2 * lev - 2, C(0));
+  C2 v01, g01[3], v2p, g2p[3];
+  C gp[3];
+  lane_vg<C2, D, true>(pair(to_compute<C>(xs[0]), to_compute<C>(xs[1])), rho2, v01, g01);
+  if constexpr (D == 3) {
+    lane_vg<C2, D, true>(pair(to_compute<C>(xs[2]), to_compute<C>(xs[3])), rho2, v2p, g2p);
 #pragma unroll
-  for (int i = 0; i < D; ++i) div += gv[i][i];
-  C Rm[3] = {C(0), C(0), C(0)};
+    for (int k = 0; k < D; ++k) gp[k] = second(g2p[k]);
+  } else {
+    C unused;
+    lane_vg<C, D, false>(to_compute<C>(xs[3]), rho, unused, gp);
+  }
+  C div = reflect(first(g01[0]), sg[0]) + reflect(second(g01[1]), sg[1]);
+  if constexpr (D == 3) div = div + reflect(first(g2p[2]), sg[2]);
 #pragma unroll
-  for (int i = 0; i < D; ++i) {
-    C a = K.kap * v[i];
+  for (int k = 0; k < D; ++k) gp[k] = reflect(times_const(gp[k], 1.0 / kVal, lev), sg[k]);
+  C2 R01 = fma_q(both<C>(K.kis), v01, pair(gp[0], gp[1]));
 #pragma unroll
-    for (int j = 0; j < D; ++j) a = fma(va[j], gv[i][j], a);
-    Rm[i] = fma(K.isc, a, gp[i]);
+  for (int j = 0; j < D; ++j) R01 = fma_q(both<C>(V[j]), g01[j], R01);
+  C R2 = C(0);
+  if constexpr (D == 3) {
+    R2 = fma_q(K.kis, first(v2p), gp[2]);
+#pragma unroll
+    for (int j = 0; j < D; ++j) R2 = fma_q(V[j], first(g2p[j]), R2);
   }
   if constexpr (DATA) {
     // history h_i and the body force kappa/(2 Lambda^2) (c+ - c-) grad phi of the PNP state
@@ -218,41 +239,48 @@ __global__ void __launch_bounds__(kNsThreads) k_ns_lanes(NsArgs<T> A, NsK<C> K) 
         }
       }
     }
-    const C rho = interp_v<C, D>(to_compute<C>(u3[0] - u3[1]), nb);
+    // f rho grad phi / a^D = (f a^(D-1) / h) rho~ s_i g~phi_i
+    C2 val, g[3];
+    lane_vg<C2, D, true>(pair(to_compute<C>(u3[2]), to_compute<C>(u3[0] - u3[1])), rho2, val, g);
+    const C frho = const_pow2(ipow(kVal, D - 1), lev, C(0)) * (K.fb * second(val));
     C gphi[3];
-    interp_g<C, D>(to_compute<C>(u3[2]), nb, sh, gphi);
-    const C frho = K.fb * rho;
 #pragma unroll
-    for (int i = 0; i < D; ++i) {
-      const C hq = interp_v<C, D>(to_compute<C>(hs[i]), nb);
-      Rm[i] += fma(K.isc, hq, frho * gphi[i]);
-    }
+    for (int k = 0; k < D; ++k) gphi[k] = first(g[k]);
+    R01 = R01 + fma_q(both<C>(K.isc), lane_v<C2, D>(pair(to_compute<C>(hs[0]), to_compute<C>(hs[1])), rho2),
+                    pair(reflect(frho * gphi[0], sg[0]), reflect(frho * gphi[1], sg[1])));
+    if constexpr (D == 3) R2 = R2 + fma_q(K.isc, lane_v<C, D>(to_compute<C>(hs[2]), rho), reflect(frho * gphi[2], sg[2]));
   }
-  C r[4];
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    if (i < D) {
-      C Phi[3];
-      const C su = K.isc * tau_m * Rm[i];
-#pragma unroll
-      for (int j = 0; j < 3; ++j) Phi[j] = fma(su, va[j], gv[i][j]);
-      Phi[i] = fma(tau_s, div, Phi[i]);
-      r[i] = w * test_t<C, D>(Rm[i], Phi, nb, sh);
-    } else {
-      r[i] = C(0);
-    }
-  }
+  constexpr double cW = ipow(kVal, 2 * D - 2), cWp = ipow(kVal, 2 * D - 3), cd = kVal * kVal;
+  const int eW = 2 * lev - D * (lev + 1), eWp = eW + lev, ed = -2 * lev;
+  const C tsd = tau_s * div;
+  T r[4];
+  const C2 rd01 = times_const2(R01, cd, ed), su01 = both<C>(tau_m) * rd01;
+  const C rd2 = times_const(R2, cd, ed), su2 = tau_m * rd2;
   {
-    C Phi[3];
+    C2 Phi[3];
 #pragma unroll
-    for (int j = 0; j < 3; ++j) Phi[j] = tau_m * Rm[j];
-    r[3] = w * test_t<C, D>(div, Phi, nb, sh);
+    for (int j = 0; j < D; ++j) Phi[j] = fma_q(su01, both<C>(V[j]), g01[j]);
+    Phi[0] = pair(first(Phi[0]) + reflect(tsd, sg[0]), second(Phi[0]));
+    Phi[1] = pair(first(Phi[1]), second(Phi[1]) + reflect(tsd, sg[1]));
+    const C2 t = lane_test<C2, D>(rd01, Phi, rho2);
+    r[0] = times_const(to_storage<T>(first(t)), cW, eW);
+    r[1] = times_const(to_storage<T>(second(t)), cW, eW);
+  }
+  C Pq[3] = {reflect(first(su01), sg[0]), reflect(second(su01), sg[1]), reflect(su2, sg[2])};
+  if constexpr (D == 3) {
+    C2 Phi[3];
+#pragma unroll
+    for (int j = 0; j < D; ++j) Phi[j] = pair(fma_q(su2, V[j], first(g2p[j])), Pq[j]);
+    Phi[2] = pair(first(Phi[2]) + reflect(tsd, sg[2]), second(Phi[2]));
+    const C2 t = lane_test<C2, D>(pair(rd2, times_const(div, cd, ed)), Phi, rho2);
+    r[2] = times_const(to_storage<T>(first(t)), cW, eW);
+    r[3] = times_const(to_storage<T>(second(t)), cWp, eWp);
+  } else {
+    r[2] = T(0);
+    r[3] = times_const(to_storage<T>(lane_test<C, D>(times_const(div, cd, ed), Pq, rho)), cWp, eWp);
   }
   if (!valid) return;
-  T ro[4];
-#pragma unroll
-  for (int f = 0; f < 4; ++f) ro[f] = to_storage<T>(r[f]);
-  scatter_rows(A, id, ro);
+  scatter_rows(A, id, r);
 }
 
 // Dirichlet / pin rows (mode 0: X - g, the residual; 1: X, the matrix) of free nodes.
@@ -835,7 +863,7 @@ static NsArgs<T> ns_args(const pnp_ctx* c, const T* X, const T* adv, T* out) {
 
 template <typename C, typename T>
 static NsK<C> ns_k(const NsArgs<T>& A) {
-  return NsK<C>{C(A.isc), C(A.kap), C(A.tau_t), C(A.cid), C(A.fb)};
+  return NsK<C>{C(A.isc), C(A.isc * A.kap), C(A.tau_t), C(A.cid), C(A.fb)};
 }
 
 // the FP64 rows in double-float arithmetic (default) or FP64 arithmetic
@@ -847,10 +875,10 @@ static void launch_ns64(const NsArgs<double>& A, int blocks, cudaStream_t s) {
 
 // element-kernel flops per lane (FP counts of the code above, fma = 2)
 static double ns_lane_flops(int D, bool data) {
-  const double tri = D * (D - 1) / 2.0;
-  const double vg = 3 * tri + 4 * D, v = 3 * D, g = vg - 2, tt = 6 * D + 3 * tri + 1;
-  double f = D * vg + g + D * v + 2 * D + 12 + D * (2 + 2 * D + 2) + (D + 1) * (3 + 2 * D + tt) + 8;
-  if (data) f += 4 * v + g + 8 * D;
+  const double tri = D * (D - 1.0);
+  const double v = 2 * D, vg = 3 * D + tri, g = vg - 2, tt = 4 * D + tri;
+  double f = D * vg + g + D * v + (2 * D - 1) + D + 14 + D + D * (2 + 2 * D) + D * (2 + 2 * D + 1) + (D + 1) * (tt + 1) + 2;
+  if (data) f += D * v + v + g + D + 2 + 3 * D;
   return f;
 }
 
@@ -890,9 +918,9 @@ int ctx_ns_apply64(pnp_ctx* c, const double* X, const double* Ubody, double* F, 
   A.U = Ubody;
   const int64_t lanes = c->n_elem << c->dim;
   {
-    // flops: the FP64 formulation's, times 15 FP32 operations per double-float operation
+    // flops: the FP64 formulation's, times the FP32 operations of a double-float operation
     ProfScope ps(c, PNP_PROF_NS, 72.0 * N + (data ? 56.0 * N : 0.0) + 32.0 * N + c->conn_bytes(),
-                 ns_lane_flops(c->dim, data) * lanes * (residual_double_float() ? 15.0 : 1.0));
+                 ns_lane_flops(c->dim, data) * lanes * (residual_double_float() ? kDfFlopsPerFlop : 1.0));
     if (c->n_elem) {
       const int blocks = nblk(lanes, kNsThreads);
       if (c->dim == 2) {
