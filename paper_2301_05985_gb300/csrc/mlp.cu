@@ -1,6 +1,6 @@
-// mlp.cu -- learned Newton start: stencil features, a BF16 tensor-core MLP (forward and
-// backward through mma.sync m16n8k16, FP32 accumulation), Adam, training on solver
-// trajectories, and the judged start of a time step.
+// mlp.cu -- learned Newton start: stencil features, the network's state (inference in
+// mlp_tc.cu, training gradient in mlp_train.cu), Adam, training on solver trajectories, and
+// the judged start of a time step.
 //
 // The paper has no learned component; this follows the library's own design: a per-node
 // network maps the 3x3x3 stencil of (c+, c-, phi, u_z) at t^k and t^{k-1} to the
@@ -18,6 +18,7 @@
 
 #include "ctx.h"
 #include "mlp_tc.h"
+#include "mlp_train.h"
 
 #define CK(call)                                 \
   do {                                           \
@@ -150,7 +151,7 @@ __global__ void k_f32_rows(int64_t rows, int cols, int ldin, int ldout, const fl
 }
 
 // ------------------------------------------------------------------ GEMM (mma.sync bf16)
-enum { EPI_F32 = 0, EPI_FWD_GELU = 1, EPI_BWD_GELU = 2 };
+enum { EPI_F32 = 0, EPI_FWD_GELU = 1 };
 
 struct GemmArgs {
   int M, N, K;
@@ -163,17 +164,11 @@ struct GemmArgs {
   int64_t ldc;
   bf16* Cb;
   int64_t ldcb;
-  const float* Zs;   // saved pre-activation (backward)
-  int64_t ldz;
 };
 
 constexpr int BM = 64, BN = 64, BK = 32, SPAD = 8;
 
 __device__ __forceinline__ float gelu_f(float z) { return 0.5f * z * (1.f + erff(z * 0.70710678118654752f)); }
-__device__ __forceinline__ float gelu_prime_f(float z) {
-  return 0.5f * (1.f + erff(z * 0.70710678118654752f)) + z * expf(-0.5f * z * z) * 0.39894228040143268f;
-}
-
 __device__ __forceinline__ uint32_t ld_b32(const bf16* p) { return *reinterpret_cast<const uint32_t*>(p); }
 
 __device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], const uint32_t (&b)[2]) {
@@ -252,14 +247,8 @@ __global__ void __launch_bounds__(128) k_gemm(GemmArgs g) {
         const float v = acc[i][j][q];
         if (EPI == EPI_F32) {
           g.Cf[(int64_t)m * g.ldc + n] = v + (g.bias ? g.bias[n] : 0.f);
-        } else if (EPI == EPI_FWD_GELU) {
-          const float z = v + g.bias[n];
-          if (g.Cf) g.Cf[(int64_t)m * g.ldc + n] = z;
-          g.Cb[(int64_t)m * g.ldcb + n] = __float2bfloat16(gelu_f(z));
         } else {
-          const float dz = v * gelu_prime_f(g.Zs[(int64_t)m * g.ldz + n]);
-          g.Cf[(int64_t)m * g.ldc + n] = dz;
-          g.Cb[(int64_t)m * g.ldcb + n] = __float2bfloat16(dz);
+          g.Cb[(int64_t)m * g.ldcb + n] = __float2bfloat16(gelu_f(v + g.bias[n]));
         }
       }
 }
@@ -270,48 +259,6 @@ cudaError_t gemm(const GemmArgs& g, cudaStream_t s) {
   k_gemm<EPI><<<grid, 128, 0, s>>>(g);
   note_launch();
   return cudaGetLastError();
-}
-
-// loss = mean (out - y)^2 over rows x 3; dOut = 2 (out - y) / (3 rows)
-__global__ void k_loss_grad(int64_t rows, const float* __restrict__ out, const float* __restrict__ Y,
-                            bf16* __restrict__ dOb, float* __restrict__ dOf, double* __restrict__ part) {
-  __shared__ double sh[256];
-  double s = 0;
-  const double scale = 2.0 / (3.0 * (double)rows);
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < rows * NOP;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int col = (int)(t % NOP);
-    float d = 0.f;
-    if (col < NO) {
-      const double e = (double)out[t] - (double)Y[t];
-      s += e * e;
-      d = (float)(scale * e);
-    }
-    dOb[t] = __float2bfloat16(d);
-    dOf[t] = d;
-  }
-  sh[threadIdx.x] = s;
-  __syncthreads();
-  for (int k = blockDim.x / 2; k > 0; k >>= 1) {
-    if (threadIdx.x < k) sh[threadIdx.x] += sh[threadIdx.x + k];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
-}
-
-// db[n] = sum_r dZ[r][n]  (one block per column, fixed order)
-__global__ void k_colsum(int64_t rows, int ld, const float* __restrict__ dZ, float* __restrict__ db) {
-  __shared__ float sh[256];
-  const int n = blockIdx.x;
-  float s = 0.f;
-  for (int64_t r = threadIdx.x; r < rows; r += blockDim.x) s += dZ[r * ld + n];
-  sh[threadIdx.x] = s;
-  __syncthreads();
-  for (int k = blockDim.x / 2; k > 0; k >>= 1) {
-    if (threadIdx.x < k) sh[threadIdx.x] += sh[threadIdx.x + k];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) db[n] = sh[0];
 }
 
 __global__ void k_adam(int64_t n, float* __restrict__ P, const float* __restrict__ G, float* __restrict__ m,
@@ -414,9 +361,11 @@ struct Mlp {
   int32_t *free_nodes = nullptr, *st_ptr = nullptr, *st_idx = nullptr;
   double* st_w = nullptr;
   // workspace (kMaxRows rows)
-  bf16 *X = nullptr, *A1 = nullptr, *A2 = nullptr, *A3 = nullptr, *dZa = nullptr, *dZb = nullptr, *dOb = nullptr;
-  float *Z1 = nullptr, *Z2 = nullptr, *Z3 = nullptr, *out = nullptr, *Y = nullptr, *dZf = nullptr, *dOf = nullptr;
+  bf16 *X = nullptr, *A1 = nullptr, *A2 = nullptr, *A3 = nullptr, *dZ1 = nullptr, *dZ2 = nullptr, *dZ3 = nullptr,
+       *dO = nullptr;
+  float *out = nullptr, *Y = nullptr, *gpart = nullptr;  // gpart: partial gradients (mlp_train.cu)
   double* part = nullptr;
+  double* loss = nullptr;  // [1 + mlp_grad_max_ctas()]: the loss and its partials
   int32_t* d_rows = nullptr;
   int64_t* d_state = nullptr;
   // training data
@@ -433,8 +382,8 @@ namespace {
 
 void mlp_free(Mlp* m) {
   void* ptrs[] = {m->P,  m->G,  m->Am, m->Av, m->W1, m->W2, m->W3, m->W4, m->b1,     m->b2,      m->b3,
-                  m->b4, m->X,  m->A1, m->A2, m->A3, m->dZa, m->dZb, m->dOb, m->Z1,   m->Z2,      m->Z3,
-                  m->out, m->Y, m->dZf, m->dOf, m->part, m->d_rows, m->d_state, m->free_nodes, m->st_ptr,
+                  m->b4, m->X,  m->A1, m->A2, m->A3, m->dZ1, m->dZ2, m->dZ3, m->dO,   m->gpart,   m->loss,
+                  m->out, m->Y, m->part, m->d_rows, m->d_state, m->free_nodes, m->st_ptr,
                   m->st_idx, m->st_w, m->states, m->uz};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -571,25 +520,6 @@ GemmArgs gargs(int M, int N, int K, const bf16* A, int64_t sam, int64_t sak, con
   return g;
 }
 
-// forward of `rows` standardised rows in m->X; output in m->out [rows][8]
-int mlp_forward_rows(pnp_ctx* c, Mlp* m, int64_t rows) {
-  cudaStream_t s = c->stream;
-  const int R = (int)rows;
-  GemmArgs g = gargs(R, HID, K0P, m->X, K0P, 1, m->W1, HID, 1);
-  g.bias = m->b1; g.Cf = m->Z1; g.ldc = HID; g.Cb = m->A1; g.ldcb = HID;
-  CK(gemm<EPI_FWD_GELU>(g, s));
-  g = gargs(R, HID, HID, m->A1, HID, 1, m->W2, HID, 1);
-  g.bias = m->b2; g.Cf = m->Z2; g.ldc = HID; g.Cb = m->A2; g.ldcb = HID;
-  CK(gemm<EPI_FWD_GELU>(g, s));
-  g = gargs(R, HID, HID, m->A2, HID, 1, m->W3, HID, 1);
-  g.bias = m->b3; g.Cf = m->Z3; g.ldc = HID; g.Cb = m->A3; g.ldcb = HID;
-  CK(gemm<EPI_FWD_GELU>(g, s));
-  g = gargs(R, NO, HID, m->A3, HID, 1, m->W4, NOP, 1);
-  g.bias = m->b4; g.Cf = m->out; g.ldc = NOP;
-  CK(gemm<EPI_F32>(g, s));
-  return PNP_OK;
-}
-
 // inference of `rows` standardised rows in m->X on the tensor cores (tcgen05, all layers
 // in one kernel, no saved activations); output in m->out [rows][8]
 int mlp_infer_rows(pnp_ctx* c, Mlp* m, int64_t rows) {
@@ -619,54 +549,29 @@ int mlp_check_infer(pnp_ctx* c) {
   return PNP_OK;
 }
 
-// loss and packed gradient for `rows` rows (X, Y in the workspace); loss on the host
-int mlp_backward_rows(pnp_ctx* c, Mlp* m, int64_t rows, double* loss) {
-  cudaStream_t s = c->stream;
-  const int R = (int)rows;
-  const int nb = 256;
-  k_loss_grad<<<nb, 256, 0, s>>>(rows, m->out, m->Y, m->dOb, m->dOf, m->part);
-  note_launch();
-  // layer 4
-  GemmArgs g = gargs(HID, NO, R, m->A3, 1, HID, m->dOb, NOP, 1);
-  g.Cf = m->G + oW4; g.ldc = NO;
-  CK(gemm<EPI_F32>(g, s));
-  k_colsum<<<NO, 256, 0, s>>>(rows, NOP, m->dOf, m->G + ob4);
-  note_launch();
-  g = gargs(R, HID, NO, m->dOb, NOP, 1, m->W4, 1, NOP);
-  g.Zs = m->Z3; g.ldz = HID; g.Cf = m->dZf; g.ldc = HID; g.Cb = m->dZa; g.ldcb = HID;
-  CK(gemm<EPI_BWD_GELU>(g, s));
-  // layer 3
-  g = gargs(HID, HID, R, m->A2, 1, HID, m->dZa, HID, 1);
-  g.Cf = m->G + oW3; g.ldc = HID;
-  CK(gemm<EPI_F32>(g, s));
-  k_colsum<<<HID, 256, 0, s>>>(rows, HID, m->dZf, m->G + ob3);
-  note_launch();
-  g = gargs(R, HID, HID, m->dZa, HID, 1, m->W3, 1, HID);
-  g.Zs = m->Z2; g.ldz = HID; g.Cf = m->dZf; g.ldc = HID; g.Cb = m->dZb; g.ldcb = HID;
-  CK(gemm<EPI_BWD_GELU>(g, s));
-  // layer 2
-  g = gargs(HID, HID, R, m->A1, 1, HID, m->dZb, HID, 1);
-  g.Cf = m->G + oW2; g.ldc = HID;
-  CK(gemm<EPI_F32>(g, s));
-  k_colsum<<<HID, 256, 0, s>>>(rows, HID, m->dZf, m->G + ob2);
-  note_launch();
-  g = gargs(R, HID, HID, m->dZb, HID, 1, m->W2, 1, HID);
-  g.Zs = m->Z1; g.ldz = HID; g.Cf = m->dZf; g.ldc = HID; g.Cb = m->dZa; g.ldcb = HID;
-  CK(gemm<EPI_BWD_GELU>(g, s));
-  // layer 1
-  g = gargs(K0, HID, R, m->X, 1, K0P, m->dZa, HID, 1);
-  g.Cf = m->G + oW1; g.ldc = HID;
-  CK(gemm<EPI_F32>(g, s));
-  k_colsum<<<HID, 256, 0, s>>>(rows, HID, m->dZf, m->G + ob1);
-  note_launch();
-  CK(cudaGetLastError());
+// loss and packed gradient (device) of `rows` rows: inputs Xf [rows][216] (or, when null, the
+// BF16 rows in m->X), targets Y [rows][ldy]; the loss to the host when wanted
+int mlp_gradient(pnp_ctx* c, Mlp* m, int64_t rows, const float* Xf, const float* Y, int ldy, float* grad,
+                 double* loss) {
+  MlpGradArgs a;
+  a.rows = rows;
+  a.Xf = Xf;
+  a.Xb = m->X;
+  a.Y = Y;
+  a.ldy = ldy;
+  a.W1 = m->W1; a.W2 = m->W2; a.W3 = m->W3; a.W4 = m->W4;
+  a.b1 = m->b1; a.b2 = m->b2; a.b3 = m->b3; a.b4 = m->b4;
+  a.A[0] = m->A1; a.A[1] = m->A2; a.A[2] = m->A3;
+  a.dZ[0] = m->dZ1; a.dZ[1] = m->dZ2; a.dZ[2] = m->dZ3;
+  a.dO = m->dO;
+  a.part = m->gpart;
+  a.loss_part = m->loss + 1;
+  a.grad = grad;
+  a.loss = m->loss;
+  CK(launch_mlp_grad(a, c->stream));
   if (loss) {
-    std::vector<double> hp(nb);
-    CK(cudaMemcpyAsync(hp.data(), m->part, sizeof(double) * nb, cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
-    double t = 0;
-    for (double v : hp) t += v;
-    *loss = t / (3.0 * (double)rows);
+    CK(cudaMemcpyAsync(loss, m->loss, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+    CK(cudaStreamSynchronize(c->stream));
   }
   return PNP_OK;
 }
@@ -737,16 +642,14 @@ int pnp_mlp_init(pnp_ctx* c, uint64_t seed) {
   A((void**)&m->A1, 2 * R * HID);
   A((void**)&m->A2, 2 * R * HID);
   A((void**)&m->A3, 2 * R * HID);
-  A((void**)&m->dZa, 2 * R * HID);
-  A((void**)&m->dZb, 2 * R * HID);
-  A((void**)&m->dOb, 2 * R * NOP);
-  A((void**)&m->Z1, 4 * R * HID);
-  A((void**)&m->Z2, 4 * R * HID);
-  A((void**)&m->Z3, 4 * R * HID);
+  A((void**)&m->dZ1, 2 * R * HID);
+  A((void**)&m->dZ2, 2 * R * HID);
+  A((void**)&m->dZ3, 2 * R * HID);
+  A((void**)&m->dO, 2 * R * NOP);
+  A((void**)&m->gpart, sizeof(float) * mlp_grad_part_floats());
+  A((void**)&m->loss, sizeof(double) * (1 + mlp_grad_max_ctas()));
   A((void**)&m->out, 4 * R * NOP);
   A((void**)&m->Y, 4 * R * NOP);
-  A((void**)&m->dZf, 4 * R * HID);
-  A((void**)&m->dOf, 4 * R * NOP);
   A((void**)&m->part, 8 * 256 * 16);
   A((void**)&m->d_rows, 4 * R);
   A((void**)&m->d_state, 8 * R);
@@ -905,15 +808,8 @@ int pnp_mlp_loss_grad(pnp_ctx* c, const float* X, const float* Yt, int64_t B, fl
   MLP_GUARD(c);
   if (!X || !Yt || !grad || B <= 0 || B > kMaxRows) PNP_FAIL(PNP_ERR_ARG, "pnp_mlp_loss_grad: bad arguments");
   Mlp* m = c->mlp;
-  k_f32_to_bf16_rows<<<nblk(B * K0P, 256), 256, 0, c->stream>>>(B, K0, K0, K0P, X, m->X);
-  note_launch();
-  k_f32_rows<<<nblk(B * NOP, 256), 256, 0, c->stream>>>(B, NO, NO, NOP, Yt, m->Y);
-  note_launch();
-  RC(mlp_forward_rows(c, m, B));
   double l = 0;
-  RC(mlp_backward_rows(c, m, B, &l));
-  CK(cudaMemcpyAsync(grad, m->G, 4 * (size_t)PNP_MLP_PARAMS, cudaMemcpyDeviceToDevice, c->stream));
-  CK(cudaStreamSynchronize(c->stream));
+  RC(mlp_gradient(c, m, B, X, Yt, NO, grad, &l));
   if (loss) *loss = l;
   return PNP_OK;
 }
@@ -998,10 +894,9 @@ int pnp_mlp_train(pnp_ctx* c, const pnp_train_cfg* cfg, pnp_train_stats* st) {
                                             m->out_mu[1], m->out_mu[2], m->out_sd[0], m->out_sd[1], m->out_sd[2],
                                             m->Y);
     note_launch();
-    if ((rc = mlp_forward_rows(c, m, B))) break;
     double l = 0;
     const bool want = it == 0 || it + 1 == cfg->steps;
-    if ((rc = mlp_backward_rows(c, m, B, want ? &l : nullptr))) break;
+    if ((rc = mlp_gradient(c, m, B, nullptr, m->Y, NOP, m->G, want ? &l : nullptr))) break;
     if (it == 0) l_first = l;
     if (it + 1 == cfg->steps) l_last = l;
     if ((rc = mlp_adam(c, m, m->G, cfg))) break;
