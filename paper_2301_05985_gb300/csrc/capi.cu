@@ -249,7 +249,7 @@ static void free_ctx_memory(pnp_ctx* c) {
   void* ptrs[] = {c->d_conn, c->d_anchor, c->d_level, c->d_faces, c->d_hnode, c->d_hpar, c->d_hnp, c->U, c->Uk, c->Ukm1,
                   c->adv, c->vel, c->vel_prev, c->hs, c->U32, c->adv32, c->hs32, c->V32, c->JV32, c->F,
                   c->dU, c->Ut, c->Ft, c->rhs, c->Dinv, c->D32, c->basis, c->w, c->z, c->r, c->part, c->dsc,
-                  c->dflag, c->Zb, c->Qin, c->Dinv32, c->isc, c->iinv, c->rec32, c->V4, c->JV4, c->qp32,
+                  c->dflag, c->ticket, c->Zb, c->Qin, c->Dinv32, c->isc, c->iinv, c->rec32, c->V4, c->JV4, c->qp32,
                   c->Z64, c->Qin64, c->zin64, c->isc64};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -322,6 +322,7 @@ int pnp_ctx_create(const pnp_mesh* m, const pnp_params* p, void* stream, pnp_ctx
   ALLOC(c->z, v3);
   ALLOC(c->r, v3);
   ALLOC(c->dflag, sizeof(int) * 4);
+  ALLOC(c->ticket, sizeof(unsigned));
 #undef ALLOC
   std::vector<uint8_t> faces(m->node_faces);
   for (int64_t i = 0; i < N; ++i)
@@ -332,6 +333,7 @@ int pnp_ctx_create(const pnp_mesh* m, const pnp_params* p, void* stream, pnp_ctx
     if (bytes && e == cudaSuccess) e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, s);
   };
   if (e == cudaSuccess) e = cudaMemsetAsync(c->dflag, 0, sizeof(int) * 4, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(c->ticket, 0, sizeof(unsigned), s);
   up(c->d_conn, m->el_conn.data(), sizeof(int32_t) * m->el_conn.size());
   up(c->d_level, m->el_level.data(), m->el_level.size());
   up(c->d_faces, faces.data(), faces.size());
@@ -418,7 +420,7 @@ int ctx_alloc_krylov(pnp_ctx* c, int m) {
       std::max<size_t>(std::max<size_t>((size_t)kRedBlocks, (size_t)kInnerBlocks), (size_t)multi_dot_blocks(c->n3()));
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->part, sizeof(double) * part_rows * (m + 2));
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->dsc, sizeof(double) * (4 * (m + 2) + 16));
-  if (e == cudaSuccess) e = cudaMallocHost((void**)&c->hpin, sizeof(double) * (4 * (m + 2) + 16));
+  if (e == cudaSuccess) e = cudaMallocHost((void**)&c->hpin, sizeof(double) * (6 * (m + 2) + 16));
   if (e != cudaSuccess) {
     pnp_set_error("Krylov scratch allocation (%zu bytes) failed: %s", bb, cudaGetErrorString(e));
     return e == cudaErrorMemoryAllocation ? PNP_ERR_NOMEM : PNP_ERR_CUDA;
@@ -500,6 +502,8 @@ void pnp_ctx_destroy(pnp_ctx* c) {
     cudaEventDestroy(pe.second.second);
   }
   for (cudaEvent_t e : c->ev_pool) cudaEventDestroy(e);
+  for (cudaEvent_t e : c->step_done)
+    if (e) cudaEventDestroy(e);
   if (c->inner_exec) cudaGraphExecDestroy(c->inner_exec);
   if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
   free_ctx_memory(c);
@@ -733,8 +737,7 @@ int pnp_norm2(pnp_ctx* c, const double* x, int64_t n, double* result) {
     return PNP_OK;
   }
   double* slot = c->dsc + 4 * (c->m_alloc + 2) + 9;
-  CK(launch_norm2(n, x, c->part, slot, c->stream));
-  CK(cudaMemcpyAsync(c->hpin + 1, slot, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+  CK(launch_norm2(n, x, c->part, c->ticket, slot, c->hpin + 1, c->stream));
   CK(cudaStreamSynchronize(c->stream));
   *result = c->hpin[1];
   return PNP_OK;

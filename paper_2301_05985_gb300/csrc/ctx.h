@@ -61,11 +61,13 @@ struct pnp_ctx {
   float* D32 = nullptr;    // [N][9] FP32 block diagonal (mixed-precision preconditioner)
   double* basis = nullptr; // [(m+1)][3N]
   double *w = nullptr, *z = nullptr, *r = nullptr;
-  double* part = nullptr;  // reduction partials [kRedBlocks][m+2]
+  double* part = nullptr;  // reduction partials, (m + 2) vectors' worth
   double* dsc = nullptr;   // small device scalars [2*(m+2) + 8]
   double* hpin = nullptr;  // pinned host mirror of dsc
   int* dflag = nullptr;
+  unsigned* ticket = nullptr;  // counter of the reductions' last block (this stream's launches)
   int m_alloc = 0;
+  cudaEvent_t step_done[2] = {nullptr, nullptr};  // GMRES iterations queued ahead of the host
   // flexible outer GMRES with an inner FP32 GMRES(d) preconditioner
   float* Zb = nullptr;      // [m][3N] preconditioned Krylov vectors
   float* Qin = nullptr;     // [(d+1)][ldq] inner basis (unnormalised), rows padded with zeros
@@ -204,9 +206,10 @@ struct ProfScope {
 int ctx_check(pnp_ctx* c, cudaError_t e, const char* what);
 int ctx_prepare_history(pnp_ctx* c);
 int ctx_residual(pnp_ctx* c, const double* U, double* F);
-int ctx_jv64(pnp_ctx* c, const double* U, const double* V, double* JV);
+// cleared: JV is zero already (the block-Jacobi apply before it cleared it)
+int ctx_jv64(pnp_ctx* c, const double* U, const double* V, double* JV, bool cleared = false);
 int ctx_prepare_f32(pnp_ctx* c, const double* U);
-int ctx_jv32(pnp_ctx* c, const float* V32, float* JV32);
+int ctx_jv32(pnp_ctx* c, const float* V32, float* JV32, bool cleared = false);
 // PNP_ERR_DEVICE_FLAG once a wait of the staged J V has given up (the flag is latched)
 int ctx_check_staged_waits(pnp_ctx* c);
 int ctx_block_diag(pnp_ctx* c, const double* U, double* D);

@@ -365,29 +365,28 @@ __global__ void k_patch_finalize(PatchArgs<T> A, bool jv) {
 }
 
 // ------------------------------------------------------------------ row fix-ups
-// mode 0: F = U - g on Dirichlet rows;  mode 1: out = V on Dirichlet rows.
+// Dirichlet rows (mode 0: out = in - g, the residual; 1: out = in, J V) for threads i < N;
+// threads N + h write the constraint row of hanging node h: out_h = in_h - sum_p w_p in_p.
+// One launch: on small meshes the operator's time is its launches.
 template <typename T>
-__global__ void k_dirichlet_rows(int64_t N, const uint8_t* __restrict__ faces, BcTable bc, const T* __restrict__ in,
-                                 T* __restrict__ out, int mode) {
+__global__ void k_rows(int64_t N, int64_t H, const uint8_t* __restrict__ faces, BcTable bc,
+                       const int32_t* __restrict__ hnode, const int32_t* __restrict__ hpar,
+                       const uint8_t* __restrict__ hnp, const T* __restrict__ in, T* __restrict__ out, int mode) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= N) return;
-  const uint8_t fm = faces[i];
-  if (fm & 0x80) return;  // hanging: constraint row written separately
+  if (i < N) {
+    const uint8_t fm = faces[i];
+    if (!fm || (fm & 0x80)) return;  // interior, or hanging: written by a thread past N
 #pragma unroll
-  for (int f = 0; f < 3; ++f) {
-    const unsigned msk = fm & bc.dir_faces[f] & 0x3F;
-    if (msk) {
-      const int face = 31 - __clz(msk);
-      out[3 * i + f] = mode == 0 ? T(double(in[3 * i + f]) - bc.val[face][f]) : in[3 * i + f];
+    for (int f = 0; f < 3; ++f) {
+      const unsigned msk = fm & bc.dir_faces[f] & 0x3F;
+      if (msk) {
+        const int face = 31 - __clz(msk);
+        out[3 * i + f] = mode == 0 ? T(double(in[3 * i + f]) - bc.val[face][f]) : in[3 * i + f];
+      }
     }
+    return;
   }
-}
-
-// out_h = in_h - sum_p w_p in_p  (constraint rows of hanging nodes)
-template <typename T>
-__global__ void k_hanging_rows(int64_t H, const int32_t* __restrict__ hnode, const int32_t* __restrict__ hpar,
-                               const uint8_t* __restrict__ hnp, const T* __restrict__ in, T* __restrict__ out) {
-  const int64_t h = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t h = i - N;
   if (h >= H) return;
   const int np = hnp[h];
   const T wgt = np == 2 ? T(0.5) : T(0.25);
@@ -502,9 +501,12 @@ template cudaError_t launch_patch<float>(int, bool, const PatchArgs<float>&, cud
 
 template <typename T>
 cudaError_t launch_row_fixups(const RowArgs& R, const T* in, T* out, int mode, cudaStream_t s) {
-  const int t = 256;
-  if (R.n_nodes) { k_dirichlet_rows<T><<<nblk(R.n_nodes, t), t, 0, s>>>(R.n_nodes, R.faces, R.bc, in, out, mode); note_launch(); }
-  if (R.n_hanging) { k_hanging_rows<T><<<nblk(R.n_hanging, t), t, 0, s>>>(R.n_hanging, R.hnode, R.hpar, R.hnp, in, out); note_launch(); }
+  if (R.n_nodes + R.n_hanging) {
+    const int t = block_threads(R.n_nodes + R.n_hanging);
+    k_rows<T><<<block_count(R.n_nodes + R.n_hanging, t), t, 0, s>>>(R.n_nodes, R.n_hanging, R.faces, R.bc, R.hnode, R.hpar,
+                                                                  R.hnp, in, out, mode);
+    note_launch();
+  }
   return cudaGetLastError();
 }
 template cudaError_t launch_row_fixups<double>(const RowArgs&, const double*, double*, int, cudaStream_t);

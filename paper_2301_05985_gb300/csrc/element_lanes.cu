@@ -791,9 +791,8 @@ __global__ void __launch_bounds__(256) k_block_diag_lanes(ElemArgs<T> A, LanePar
 template <typename T>
 cudaError_t launch_element_lanes(int dim, bool jv, const ElemArgs<T>& A, cudaStream_t s) {
   if (A.n_elem == 0) return cudaSuccess;
-  const int t = 256;
-  const int64_t threads = A.n_elem << dim;
-  const unsigned blocks = (unsigned)((threads + t - 1) / t);
+  const int t = block_threads(A.n_elem << dim);
+  const unsigned blocks = block_count(A.n_elem << dim, t);
   const LaneParams<T> K{T(A.P.kappa), T(A.P.tau_t), T(A.P.C_I * dim), T(A.P.eps2x2)};
   if (dim == 2) {
     if (jv) k_element_lanes<T, T, 2, true><<<blocks, t, 0, s>>>(A, K);
@@ -811,8 +810,8 @@ template cudaError_t launch_element_lanes<float>(int, bool, const ElemArgs<float
 // FP64 residual with double-float arithmetic (FP32 pipe), FP64 data in and out
 cudaError_t launch_residual_df(int dim, const ElemArgs<double>& A, cudaStream_t s) {
   if (A.n_elem == 0) return cudaSuccess;
-  const int t = 256;
-  const unsigned blocks = (unsigned)(((A.n_elem << dim) + t - 1) / t);
+  const int t = block_threads(A.n_elem << dim);
+  const unsigned blocks = block_count(A.n_elem << dim, t);
   const LaneParams<df> K{df(A.P.kappa), df(A.P.tau_t), df(A.P.C_I * dim), df(A.P.eps2x2)};
   if (dim == 2) k_element_lanes<double, df, 2, false><<<blocks, t, 0, s>>>(A, K);
   else k_element_lanes<double, df, 3, false><<<blocks, t, 0, s>>>(A, K);
@@ -891,8 +890,8 @@ double jv_from_state_flops(int D) {
 template <typename T>
 cudaError_t launch_block_diag_lanes(int dim, const ElemArgs<T>& A, T* Dout, cudaStream_t s) {
   if (A.n_elem == 0) return cudaSuccess;
-  const int t = 256;
-  const unsigned blocks = (unsigned)(((A.n_elem << dim) + t - 1) / t);
+  const int t = block_threads(A.n_elem << dim);
+  const unsigned blocks = block_count(A.n_elem << dim, t);
   const LaneParams<T> K{T(A.P.kappa), T(A.P.tau_t), T(A.P.C_I * dim), T(A.P.eps2x2)};
   if (dim == 2) k_block_diag_lanes<T, 2><<<blocks, t, 0, s>>>(A, K, Dout);
   else k_block_diag_lanes<T, 3><<<blocks, t, 0, s>>>(A, K, Dout);

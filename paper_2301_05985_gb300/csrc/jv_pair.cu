@@ -312,14 +312,15 @@ cudaError_t launch_jv_pair(const ElemArgs<float>& A, bool advection, cudaStream_
   if (!A.rec || !A.conn) return cudaErrorInvalidValue;
   const bool pad = A.V4 && A.out4;
   if (!pad && (!A.V || !A.out)) return cudaErrorInvalidValue;
-  const unsigned blocks = (unsigned)((2 * A.n_elem + kPairThreads - 1) / kPairThreads);
+  const int t = block_threads(2 * A.n_elem);
+  const unsigned blocks = block_count(2 * A.n_elem, t);
   const float kappa = (float)A.P.kappa, tau_t = (float)A.P.tau_t, cid = (float)(A.P.C_I * 3), e2 = (float)A.P.eps2x2;
   if (advection) {
-    if (pad) k_jv_pair<true, true><<<blocks, kPairThreads, 0, s>>>(A, kappa, tau_t, cid, e2);
-    else k_jv_pair<true, false><<<blocks, kPairThreads, 0, s>>>(A, kappa, tau_t, cid, e2);
+    if (pad) k_jv_pair<true, true><<<blocks, t, 0, s>>>(A, kappa, tau_t, cid, e2);
+    else k_jv_pair<true, false><<<blocks, t, 0, s>>>(A, kappa, tau_t, cid, e2);
   } else {
-    if (pad) k_jv_pair<false, true><<<blocks, kPairThreads, 0, s>>>(A, kappa, tau_t, cid, e2);
-    else k_jv_pair<false, false><<<blocks, kPairThreads, 0, s>>>(A, kappa, tau_t, cid, e2);
+    if (pad) k_jv_pair<false, true><<<blocks, t, 0, s>>>(A, kappa, tau_t, cid, e2);
+    else k_jv_pair<false, false><<<blocks, t, 0, s>>>(A, kappa, tau_t, cid, e2);
   }
   note_launch();
   return cudaGetLastError();

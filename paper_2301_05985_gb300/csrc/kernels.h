@@ -45,6 +45,17 @@ int64_t launch_count();
 // counts a capture of the inner solve (read by pnp_graph_captures)
 void note_capture();
 
+// Threads per block for n independent threads: 256, and fewer (down to a warp) while that
+// leaves less than two blocks per SM.  A small mesh's kernels otherwise sit on a few SMs: the
+// FP64 J V of 1,024 quadrilaterals as 16 blocks of 8 warps shared 16 FP64 pipes (16 clocks
+// per warp instruction) and took 14 us, as 128 blocks of one warp 5 us.
+inline int block_threads(int64_t n) {
+  int t = 256;
+  while (t > 32 && (n + t - 1) / t < 304) t /= 2;
+  return t;
+}
+inline unsigned block_count(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
+
 // Arguments of the shared-memory patch kernels (residual / Jv over Morton patches).
 template <typename T>
 struct PatchArgs {
@@ -128,23 +139,41 @@ cudaError_t launch_to_f64(int64_t n, const float* x, double* y, cudaStream_t s);
 cudaError_t launch_axpby(int64_t n, double a, const double* x, double b, double* y, cudaStream_t s);
 // z = a x + b y
 cudaError_t launch_axpbyz(int64_t n, double a, const double* x, double b, const double* y, double* z, cudaStream_t s);
-// partial sums of x.y into part[kRedBlocks], then result[0] = sum (device)
-cudaError_t launch_dot(int64_t n, const double* x, const double* y, double* part, double* result, cudaStream_t s);
-cudaError_t launch_norm2(int64_t n, const double* x, double* part, double* result, cudaStream_t s);
-// w -= sum_i h[i] Vb[i*ld + .], i < k ; optionally hacc[i] += h[i]
+// result[0] = x . y or ||x||_2 on the device, and in mapped pinned memory at host (may be
+// null); part: kRedBlocks doubles; ticket: a zeroed counter of the stream
+cudaError_t launch_dot(int64_t n, const double* x, const double* y, double* part, unsigned* ticket, double* result,
+                       double* host, cudaStream_t s);
+cudaError_t launch_norm2(int64_t n, const double* x, double* part, unsigned* ticket, double* result, double* host,
+                         cudaStream_t s);
+// w -= sum_i h[i] Vb[i*ld + .], i < k
 cudaError_t launch_multi_axpy(int64_t n, int k, const double* Vb, int64_t ld, const double* h, double* w,
-                              double* hacc, cudaStream_t s);
-// z_i = Dinv_i v_i per node (3x3 blocks); optionally also a float copy z32 (may be null)
-cudaError_t launch_block_apply(int64_t N, const double* Dinv, const double* v, double scale, double* z, float* z32,
-                               cudaStream_t s);
-// blocks (= partial rows) of the multi-dot for vectors of n entries
+                              cudaStream_t s);
+// z_i = Dinv_i v_i per node (3x3 blocks); optionally also a float copy z32, and zeros into
+// clear / clear32 [N][3] (the accumulator of the J V that follows); each may be null
+// The factor of v is `scale`, or *scale_dev when that is given.
+cudaError_t launch_block_apply(int64_t N, const double* Dinv, const double* v, double scale, const double* scale_dev,
+                               double* z, float* z32, double* clear, float* clear32, cudaStream_t s);
+// blocks (= partials per vector) of the multi-dot for vectors of n entries
 int multi_dot_blocks(int64_t n);
-// d[i] = V_i . w for i < k, plus d[k] = w . w when with_self (part: [multi_dot_blocks(n)][k+1])
-cudaError_t launch_multi_dot_ext(int64_t n, int k, bool with_self, const double* Vb, int64_t ld, const double* w,
-                                 double* part, double* d, cudaStream_t s);
-// w -= sum_i d[i] dinv[i] V_i (i < k);  nrm2[0] = w . w afterwards
+// d[i] = V_i . w for i < k (part: [k][multi_dot_blocks(n)])
+cudaError_t launch_multi_dot(int64_t n, int k, const double* Vb, int64_t ld, const double* w, double* part,
+                             unsigned* ticket, double* d, cudaStream_t s);
+// What ends a Gram-Schmidt pass: w . w (nrm2) and, where given, its reciprocal (dinv_next)
+// and that of its root (inv_s_next) on the device; to mapped pinned memory w . w (host_nrm2) and the k projections of one or
+// two passes (host0 <- d0, host1 <- d1).  Null: not written.
+struct GsFinish {
+  double* nrm2;
+  double* dinv_next = nullptr;
+  double* inv_s_next = nullptr;
+  double* host_nrm2 = nullptr;
+  const double* d0 = nullptr;
+  double* host0 = nullptr;
+  const double* d1 = nullptr;
+  double* host1 = nullptr;
+};
+// w -= sum_i d[i] dinv[i] V_i (i < k), then what `f` says
 cudaError_t launch_multi_axpy_norm(int64_t n, int k, const double* Vb, int64_t ld, const double* d, const double* dinv,
-                                   double* w, double* part, double* nrm2, cudaStream_t s);
+                                   double* w, double* part, unsigned* ticket, const GsFinish& f, cudaStream_t s);
 // Dinv = inverse of the 3x3 blocks of D (Gauss-Jordan with partial pivoting, FP64);
 // flag[0] |= 1 on a singular or non-finite block.  D may alias Dinv when T = double.
 template <typename T>
@@ -153,6 +182,8 @@ cudaError_t launch_block_invert(int64_t N, const T* D, double* Dinv, int* flag, 
 cudaError_t launch_make_consistent(const RowArgs& R, double* U, cudaStream_t s);
 // out[j] = sum_b part[b*k + j] for j < k (one block per output, fixed order)
 cudaError_t launch_reduce_parts(int nparts, int k, const double* part, double* out, cudaStream_t s);
+// out[j] = sum_b part[j*nparts + b]
+cudaError_t launch_reduce_cols(int nparts, int k, const double* part, double* out, cudaStream_t s);
 
 // ---------------------------------------------- inner FP32 GMRES (inner_krylov.cu)
 int inner_dot_blocks(int64_t n);

@@ -792,8 +792,9 @@ int ctx_ns_alloc(pnp_ctx* c) {
             get((void**)&S->rh, f4) && get((void**)&S->p, f4) && get((void**)&S->v, f4) && get((void**)&S->t, f4) &&
             get((void**)&S->ph, f4) && get((void**)&S->sh, f4) && get((void**)&S->x, f4) &&
             get((void**)&S->part, sizeof(double) * 2 * kRedBlocks) && get((void**)&S->sc, sizeof(double) * kScalars);
-  // pinned host scalars: the BiCGStab scalars, or FGMRES projections (m <= 200)
-  if (ok) ok = cudaMallocHost((void**)&S->hsc, sizeof(double) * 256) == cudaSuccess;
+  // pinned host scalars: the BiCGStab scalars, or both passes' FGMRES projections and the
+  // norm (2 m + 3 doubles, m <= 200; written by the device)
+  if (ok) ok = cudaMallocHost((void**)&S->hsc, sizeof(double) * 512) == cudaSuccess;
   if (!ok) {
     cudaGetLastError();
     ctx_ns_release(c);
@@ -868,9 +869,11 @@ static NsK<C> ns_k(const NsArgs<T>& A) {
 
 // the FP64 rows in double-float arithmetic (default) or FP64 arithmetic
 template <int D, bool DATA>
-static void launch_ns64(const NsArgs<double>& A, int blocks, cudaStream_t s) {
-  if (residual_double_float()) k_ns_lanes<double, df, D, DATA><<<blocks, kNsThreads, 0, s>>>(A, ns_k<df>(A));
-  else k_ns_lanes<double, double, D, DATA><<<blocks, kNsThreads, 0, s>>>(A, ns_k<double>(A));
+static void launch_ns64(const NsArgs<double>& A, cudaStream_t s) {
+  const int t = block_threads(A.n_elem << D);
+  const unsigned blocks = block_count(A.n_elem << D, t);
+  if (residual_double_float()) k_ns_lanes<double, df, D, DATA><<<blocks, t, 0, s>>>(A, ns_k<df>(A));
+  else k_ns_lanes<double, double, D, DATA><<<blocks, t, 0, s>>>(A, ns_k<double>(A));
 }
 
 // element-kernel flops per lane (FP counts of the code above, fma = 2)
@@ -885,8 +888,7 @@ static double ns_lane_flops(int D, bool data) {
 // ||x||_2 of a [N][4] FP64 vector
 static int ctx_norm4(pnp_ctx* c, const double* x, double* out) {
   double* slot = c->dsc + 4 * (c->m_alloc + 2) + 8;
-  CK(launch_norm2(4 * c->n_nodes, x, c->part, slot, c->stream));
-  CK(cudaMemcpyAsync(c->hpin, slot, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+  CK(launch_norm2(4 * c->n_nodes, x, c->part, c->ticket, slot, c->hpin, c->stream));
   CK(cudaStreamSynchronize(c->stream));
   *out = c->hpin[0];
   return PNP_OK;
@@ -922,13 +924,12 @@ int ctx_ns_apply64(pnp_ctx* c, const double* X, const double* Ubody, double* F, 
     ProfScope ps(c, PNP_PROF_NS, 72.0 * N + (data ? 56.0 * N : 0.0) + 32.0 * N + c->conn_bytes(),
                  ns_lane_flops(c->dim, data) * lanes * (residual_double_float() ? kDfFlopsPerFlop : 1.0));
     if (c->n_elem) {
-      const int blocks = nblk(lanes, kNsThreads);
       if (c->dim == 2) {
-        if (data) launch_ns64<2, true>(A, blocks, s);
-        else launch_ns64<2, false>(A, blocks, s);
+        if (data) launch_ns64<2, true>(A, s);
+        else launch_ns64<2, false>(A, s);
       } else {
-        if (data) launch_ns64<3, true>(A, blocks, s);
-        else launch_ns64<3, false>(A, blocks, s);
+        if (data) launch_ns64<3, true>(A, s);
+        else launch_ns64<3, false>(A, s);
       }
       note_launch();
     }
@@ -957,9 +958,10 @@ int ctx_ns_apply32(pnp_ctx* c, const float4* x, float4* y) {
   {
     ProfScope ps(c, PNP_PROF_NS32, 48.0 * N + c->conn_bytes(), ns_lane_flops(c->dim, false) * lanes);
     if (c->n_elem) {
-      const int blocks = nblk(lanes, kNsThreads);
-      if (c->dim == 2) k_ns_lanes<float, float, 2, false><<<blocks, kNsThreads, 0, s>>>(A, ns_k<float>(A));
-      else k_ns_lanes<float, float, 3, false><<<blocks, kNsThreads, 0, s>>>(A, ns_k<float>(A));
+      const int t = block_threads(lanes);
+      const unsigned blocks = block_count(lanes, t);
+      if (c->dim == 2) k_ns_lanes<float, float, 2, false><<<blocks, t, 0, s>>>(A, ns_k<float>(A));
+      else k_ns_lanes<float, float, 3, false><<<blocks, t, 0, s>>>(A, ns_k<float>(A));
       note_launch();
     }
   }
@@ -987,8 +989,10 @@ int ctx_ns_block_diag(pnp_ctx* c, double* Dg) {
   const int64_t lanes = c->n_elem << c->dim;
   ProfScope ps(c, PNP_PROF_NS, 32.0 * N + 128.0 * N + c->conn_bytes());
   if (c->n_elem) {
-    if (c->dim == 2) k_ns_diag<2><<<nblk(lanes, kNsThreads), kNsThreads, 0, s>>>(A, Dg);
-    else k_ns_diag<3><<<nblk(lanes, kNsThreads), kNsThreads, 0, s>>>(A, Dg);
+    const int t = block_threads(lanes);
+    const unsigned blocks = block_count(lanes, t);
+    if (c->dim == 2) k_ns_diag<2><<<blocks, t, 0, s>>>(A, Dg);
+    else k_ns_diag<3><<<blocks, t, 0, s>>>(A, Dg);
     note_launch();
   }
   CK(cudaGetLastError());
@@ -1286,24 +1290,24 @@ static int ns_fgmres(pnp_ctx* c, const double* Ubody, double target, double& f, 
         // orders of magnitude: one pass loses orthogonality and the Arnoldi estimate with it)
         const double nj = (double)n * (j + 1);
         ProfScope ps(c, PNP_PROF_NS_KRYLOV, 16.0 * (2.0 * nj + 3.0 * n), 8.0 * nj);
-        CK(launch_multi_dot_ext(n, j + 1, false, S->Q, n, w, S->fpart, dd, s));
-        CK(launch_multi_axpy_norm(n, j + 1, S->Q, n, dd, dinv, w, S->fpart, dnrm, s));
-        CK(launch_multi_dot_ext(n, j + 1, false, S->Q, n, w, S->fpart, dd2, s));
-        CK(launch_multi_axpy_norm(n, j + 1, S->Q, n, dd2, dinv, w, S->fpart, dnrm, s));
+        CK(launch_multi_dot(n, j + 1, S->Q, n, w, S->fpart, c->ticket, dd, s));
+        CK(launch_multi_axpy_norm(n, j + 1, S->Q, n, dd, dinv, w, S->fpart, c->ticket, GsFinish{dnrm}, s));
+        CK(launch_multi_dot(n, j + 1, S->Q, n, w, S->fpart, c->ticket, dd2, s));
+        GsFinish f{dnrm};
+        f.dinv_next = dinv + j + 1;
+        f.host_nrm2 = S->hsc + (m + 1);
+        f.d0 = dd;
+        f.host0 = S->hsc;
+        f.d1 = dd2;
+        f.host1 = S->hsc + (m + 2);
+        CK(launch_multi_axpy_norm(n, j + 1, S->Q, n, dd2, dinv, w, S->fpart, c->ticket, f, s));
       }
-      CK(cudaMemcpyAsync(S->hsc, dd, sizeof(double) * (j + 1), cudaMemcpyDeviceToHost, s));
-      CK(cudaMemcpyAsync(S->hsc + (m + 2), dd2, sizeof(double) * (j + 1), cudaMemcpyDeviceToHost, s));
-      CK(cudaMemcpyAsync(S->hsc + (m + 1), dnrm, sizeof(double), cudaMemcpyDeviceToHost, s));
       CK(cudaStreamSynchronize(s));
       for (int i = 0; i <= j; ++i) Hij(i, j) = (S->hsc[i] + S->hsc[m + 2 + i]) / sv[i];
       const double nrm = std::sqrt(S->hsc[m + 1]);
       if (!std::isfinite(nrm)) PNP_FAIL(PNP_ERR_NAN, "ns: FGMRES vector norm is not finite");
       sv[j + 1] = nrm;
       Hij(j + 1, j) = nrm;
-      if (nrm > 0) {
-        hp[j + 1] = 1.0 / (nrm * nrm);
-        CK(cudaMemcpyAsync(dinv + j + 1, hp.data() + j + 1, sizeof(double), cudaMemcpyHostToDevice, s));
-      }
       for (int i = 0; i < j; ++i) {
         const double t = cs[i] * Hij(i, j) + sn[i] * Hij(i + 1, j);
         Hij(i + 1, j) = -sn[i] * Hij(i, j) + cs[i] * Hij(i + 1, j);

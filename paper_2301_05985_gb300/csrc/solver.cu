@@ -110,7 +110,7 @@ int ctx_residual(pnp_ctx* c, const double* U, double* F) {
   return PNP_OK;
 }
 
-int ctx_jv64(pnp_ctx* c, const double* U, const double* V, double* JV) {
+int ctx_jv64(pnp_ctx* c, const double* U, const double* V, double* JV, bool cleared) {
   if (c->use_patches) {
     {
       ProfScope ps(c, PNP_PROF_JV64, 112.0 * c->n_nodes + c->conn_bytes(), element_kernel_flops(c->dim, true) * c->n_elem);
@@ -118,7 +118,7 @@ int ctx_jv64(pnp_ctx* c, const double* U, const double* V, double* JV) {
     }
     RC(hanging_rows<double>(c, V, JV));
   } else {
-    CK(cudaMemsetAsync(JV, 0, sizeof(double) * c->n3(), c->stream));
+    if (!cleared) CK(cudaMemsetAsync(JV, 0, sizeof(double) * c->n3(), c->stream));
     {
       ProfScope ps(c, PNP_PROF_JV64, 112.0 * c->n_nodes + c->conn_bytes(), element_kernel_flops(c->dim, true) * c->n_elem);
       CK(launch_element<double>(c->dim, true, elem_args<double>(c, U, V, c->hs, c->adv, JV), c->stream));
@@ -145,7 +145,7 @@ int ctx_prepare_f32(pnp_ctx* c, const double* U) {
   return PNP_OK;
 }
 
-int ctx_jv32(pnp_ctx* c, const float* V32, float* JV32) {
+int ctx_jv32(pnp_ctx* c, const float* V32, float* JV32, bool cleared) {
   if (c->use_patches) {
     {
       ProfScope ps(c, PNP_PROF_JV32, 56.0 * c->n_nodes + c->conn_bytes(), element_kernel_flops(c->dim, true) * c->n_elem);
@@ -154,7 +154,7 @@ int ctx_jv32(pnp_ctx* c, const float* V32, float* JV32) {
     }
     RC(hanging_rows<float>(c, V32, JV32));
   } else {
-    CK(cudaMemsetAsync(JV32, 0, sizeof(float) * c->n3(), c->stream));
+    if (!cleared) CK(cudaMemsetAsync(JV32, 0, sizeof(float) * c->n3(), c->stream));
     ElemArgs<float> A = elem_args<float>(c, c->U32, V32, c->hs32, c->adv32, JV32);
     A.rec = c->rec32;
     if (use_jv_pair(c)) {
@@ -196,8 +196,7 @@ int ctx_block_diag32(pnp_ctx* c, float* D) {
 
 int ctx_norm(pnp_ctx* c, const double* x, double* out) {
   double* slot = c->dsc + 4 * (c->m_alloc + 2) + 8;
-  CK(launch_norm2(c->n3(), x, c->part, slot, c->stream));
-  CK(cudaMemcpyAsync(c->hpin, slot, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+  CK(launch_norm2(c->n3(), x, c->part, c->ticket, slot, c->hpin, c->stream));
   CK(cudaStreamSynchronize(c->stream));
   *out = c->hpin[0];
   return PNP_OK;
@@ -205,8 +204,7 @@ int ctx_norm(pnp_ctx* c, const double* x, double* out) {
 
 int ctx_dot(pnp_ctx* c, const double* x, const double* y, double* out) {
   double* slot = c->dsc + 4 * (c->m_alloc + 2) + 10;
-  CK(launch_dot(c->n3(), x, y, c->part, slot, c->stream));
-  CK(cudaMemcpyAsync(c->hpin, slot, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+  CK(launch_dot(c->n3(), x, y, c->part, c->ticket, slot, c->hpin, c->stream));
   CK(cudaStreamSynchronize(c->stream));
   *out = c->hpin[0];
   return PNP_OK;
@@ -519,17 +517,19 @@ static int inner_gmres64(pnp_ctx* c, const double* U, const double* u, double* z
     double* w = Q + (size_t)(j + 1) * n;
     {
       ProfScope ps(c, PNP_PROF_PRECOND, 120.0 * N, 18.0 * N);
-      CK(launch_block_apply(N, c->Dinv, Q + (size_t)j * n, 1.0 / sv[j], c->zin64, nullptr, s));
+      CK(launch_block_apply(N, c->Dinv, Q + (size_t)j * n, 1.0 / sv[j], nullptr, c->zin64, nullptr, w, nullptr, s));
     }
-    RC(ctx_jv64(c, U, c->zin64, w));
+    RC(ctx_jv64(c, U, c->zin64, w, true));
     const double nj = (double)n * (j + 1);
     {
       ProfScope ps(c, PNP_PROF_ORTHO, 8.0 * (nj + n), 2.0 * nj);
-      CK(launch_multi_dot_ext(n, j + 1, false, Q, n, w, c->part, dd, s));
+      CK(launch_multi_dot(n, j + 1, Q, n, w, c->part, c->ticket, dd, s));
     }
     {
       ProfScope ps(c, PNP_PROF_ORTHO_UPDATE, 8.0 * (nj + 2.0 * n), 2.0 * (nj + n));
-      CK(launch_multi_axpy_norm(n, j + 1, Q, n, dd, dinv, w, c->part, dnrm, s));
+      GsFinish f{dnrm};
+      f.dinv_next = dinv + j + 1;
+      CK(launch_multi_axpy_norm(n, j + 1, Q, n, dd, dinv, w, c->part, c->ticket, f, s));
     }
     CK(cudaMemcpyAsync(hp.data(), dd, sizeof(double) * (j + 1), cudaMemcpyDeviceToHost, s));
     CK(cudaMemcpyAsync(hp.data() + (d + 1), dnrm, sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -539,10 +539,6 @@ static int inner_gmres64(pnp_ctx* c, const double* U, const double* u, double* z
     if (!std::isfinite(nrm)) PNP_FAIL(PNP_ERR_NAN, "inner gmres: Krylov vector norm is not finite");
     sv[j + 1] = nrm;
     Hij(j + 1, j) = nrm;
-    if (nrm > 0) {
-      up[j + 1] = 1.0 / (nrm * nrm);
-      CK(cudaMemcpyAsync(dinv + j + 1, up.data() + j + 1, sizeof(double), cudaMemcpyHostToDevice, s));
-    }
     for (int i = 0; i < j; ++i) {
       const double t = cs[i] * Hij(i, j) + sn[i] * Hij(i + 1, j);
       Hij(i + 1, j) = -sn[i] * Hij(i, j) + cs[i] * Hij(i + 1, j);
@@ -568,9 +564,9 @@ static int inner_gmres64(pnp_ctx* c, const double* U, const double* u, double* z
   for (int i = 0; i < k; ++i) up[i] = -y[i] / sv[i];
   CK(cudaMemcpyAsync(coef, up.data(), sizeof(double) * k, cudaMemcpyHostToDevice, s));
   CK(cudaMemsetAsync(c->zin64, 0, sizeof(double) * n, s));
-  CK(launch_multi_axpy(n, k, Q, n, coef, c->zin64, nullptr, s));
+  CK(launch_multi_axpy(n, k, Q, n, coef, c->zin64, s));
   ProfScope ps(c, PNP_PROF_PRECOND, 120.0 * N, 18.0 * N);
-  CK(launch_block_apply(N, c->Dinv, c->zin64, 1.0, z, nullptr, s));
+  CK(launch_block_apply(N, c->Dinv, c->zin64, 1.0, nullptr, z, nullptr, nullptr, nullptr, s));
   CK(cudaStreamSynchronize(s));  // the host vectors above go out of scope
   return PNP_OK;
 }
@@ -622,10 +618,22 @@ int ctx_gmres(pnp_ctx* c, const double* U, const double* b, double* x, double rt
   double* dnrm = c->dsc + 2 * (m + 2);    // [1]  w . w after a pass
   double* dcoef = c->dsc + 2 * (m + 2) + 2;  // [m+1] solution-update coefficients
   double* dd2 = c->dsc + 3 * (m + 2) + 2;    // [m+2] projections of the second pass
-  double* hp = c->hpin;                     // [0, m+2): D2H scratch
-  double* hup = c->hpin + (m + 2);          // [m+2]: H2D slots for 1/s_i^2
-  double* hco = c->hpin + 2 * (m + 2) + 2;  // [m+1]: H2D slots for the update coefficients
-  double* hp2 = c->hpin + 3 * (m + 2) + 2;  // [m+2]: D2H of the second pass
+  double* inv_s = c->dsc + 2 * (m + 2) + 1;  // [1]  1 / s_(j+1)
+  // pinned: the numbers of an iteration (projections [m+2], of the second pass [m+2]) for
+  // even and odd iterations, and upload slots
+  double* hp[2] = {c->hpin, c->hpin + 4 * (m + 2) + 16};
+  double* hup = c->hpin + (m + 2);          // 1/s_0^2
+  double* hco = c->hpin + 2 * (m + 2) + 2;  // [m+1]: the update coefficients
+  double* hp2[2] = {c->hpin + 3 * (m + 2) + 2, c->hpin + 5 * (m + 2) + 16};
+  const bool two = c->prm.gmres_cgs2 != 0;
+  // Small systems: an iteration is five launches of a few microseconds, as long as the host's
+  // wait for it and the launches of the next.  The host then queues one iteration ahead (a
+  // discarded one per solve at most).  2^18 unknowns: there an FP64 iteration takes 1 ms and
+  // the wait is 1 %.  3,267 unknowns: 47 us per iteration without, 36 us with it.
+  const bool ahead = !flex && !flex64 && n <= (int64_t(1) << 18);
+  if (ahead)
+    for (cudaEvent_t& e : c->step_done)
+      if (!e) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
   *its_out = 0;
   double bn;
   RC(ctx_norm(c, b, &bn));
@@ -663,7 +671,9 @@ int ctx_gmres(pnp_ctx* c, const double* U, const double* b, double* x, double rt
     double res = beta;
     bool breakdown = false;
     bool mg_slow = false;  // the multigrid cycle is not converging: give up on it early
-    for (int j = 0; j < m && total < max_it; ++j) {
+    // One iteration's launches.  The step's numbers go to the pinned slots of its parity with
+    // the last launch (no copies), the scale of the next basis vector stays on the device.
+    auto enqueue = [&](int j) -> int {
       const double* uj = V + (size_t)j * n;
       double* w = V + (size_t)(j + 1) * n;
       // z = M^-1 (u_j / s_j) ; w = J z   (flexible: z_j = P(u_j) / s_j kept in Zb)
@@ -685,49 +695,70 @@ int ctx_gmres(pnp_ctx* c, const double* U, const double* b, double* x, double rt
       } else if (prec == PNP_F64) {
         {
           ProfScope ps(c, PNP_PROF_PRECOND, 120.0 * c->n_nodes, 18.0 * c->n_nodes);
-          CK(launch_block_apply(c->n_nodes, c->Dinv, uj, 1.0 / sv[j], c->z, nullptr, s));
+          CK(launch_block_apply(c->n_nodes, c->Dinv, uj, 1.0 / sv[0], j > 0 ? inv_s : nullptr, c->z, nullptr, w,
+                                nullptr, s));
         }
-        RC(ctx_jv64(c, U, c->z, w));
+        RC(ctx_jv64(c, U, c->z, w, true));
       } else {
         {
           ProfScope ps(c, PNP_PROF_PRECOND, 108.0 * c->n_nodes, 18.0 * c->n_nodes);
-          CK(launch_block_apply(c->n_nodes, c->Dinv, uj, 1.0 / sv[j], nullptr, c->V32, s));
+          CK(launch_block_apply(c->n_nodes, c->Dinv, uj, 1.0 / sv[0], j > 0 ? inv_s : nullptr, nullptr, c->V32, nullptr,
+                                c->JV32, s));
         }
-        RC(ctx_jv32(c, c->V32, c->JV32));
+        RC(ctx_jv32(c, c->V32, c->JV32, true));
         ProfScope ps(c, PNP_PROF_PRECOND, 36.0 * c->n_nodes);
         CK(launch_to_f64(n, c->JV32, w, s));
       }
-      double w1sq;
-      {
-        // classical Gram-Schmidt (a second pass when gmres_cgs2), one host round trip
-        // per iteration; the projections of the two passes go to separate device slots
-        const bool two = c->prm.gmres_cgs2 != 0;
-        const double nj = (double)n * (j + 1);
-        for (int pass = 0; pass < (two ? 2 : 1); ++pass) {
-          double* dp = pass == 0 ? dd : dd2;
-          {
-            ProfScope ps(c, PNP_PROF_ORTHO, 8.0 * (nj + n), 2.0 * nj);
-            CK(launch_multi_dot_ext(n, j + 1, false, V, n, w, c->part, dp, s));
-          }
-          ProfScope ps(c, PNP_PROF_ORTHO_UPDATE, 8.0 * (nj + 2.0 * n), 2.0 * (nj + n));
-          CK(launch_multi_axpy_norm(n, j + 1, V, n, dp, dinv, w, c->part, dnrm, s));
+      // classical Gram-Schmidt (a second pass when gmres_cgs2); the projections of the two
+      // passes go to separate device slots
+      const double nj = (double)n * (j + 1);
+      for (int pass = 0; pass < (two ? 2 : 1); ++pass) {
+        double* dp = pass == 0 ? dd : dd2;
+        {
+          ProfScope ps(c, PNP_PROF_ORTHO, 8.0 * (nj + n), 2.0 * nj);
+          CK(launch_multi_dot(n, j + 1, V, n, w, c->part, c->ticket, dp, s));
         }
-        if (two) CK(cudaMemcpyAsync(hp2, dd2, sizeof(double) * (j + 1), cudaMemcpyDeviceToHost, s));
-        CK(cudaMemcpyAsync(hp, dd, sizeof(double) * (j + 1), cudaMemcpyDeviceToHost, s));
-        CK(cudaMemcpyAsync(hp + (m + 1), dnrm, sizeof(double), cudaMemcpyDeviceToHost, s));
-        CK(cudaStreamSynchronize(s));
-        if (!two)
-          for (int i = 0; i <= j; ++i) hp2[i] = 0.0;
+        GsFinish f{dnrm};
+        if (pass == (two ? 1 : 0)) {
+          double* hj = hp[j & 1];
+          f.dinv_next = dinv + j + 1;
+          f.inv_s_next = inv_s;
+          f.host_nrm2 = hj + (m + 1);
+          f.d0 = dd;
+          f.host0 = hj;
+          if (two) {
+            f.d1 = dd2;
+            f.host1 = hp2[j & 1];
+          }
+        }
+        ProfScope ps(c, PNP_PROF_ORTHO_UPDATE, 8.0 * (nj + 2.0 * n), 2.0 * (nj + n));
+        CK(launch_multi_axpy_norm(n, j + 1, V, n, dp, dinv, w, c->part, c->ticket, f, s));
       }
-      for (int i = 0; i <= j; ++i) h[i] = (hp[i] + hp2[i]) / sv[i];
-      w1sq = hp[m + 1];
+      if (ahead) CK(cudaEventRecord(c->step_done[j & 1], s));
+      return PNP_OK;
+    };
+    bool queued = false;  // iteration j is already on the stream
+    for (int j = 0; j < m && total < max_it; ++j) {
+      if (!queued) RC(enqueue(j));
+      queued = false;
+      if (ahead) {
+        // the next iteration follows without waiting for the host, unless this one may end
+        // the solve (the last known residual near the tolerance)
+        if (j + 1 < m && total + 1 < max_it && res > 4.0 * tol) {
+          RC(enqueue(j + 1));
+          queued = true;
+        }
+        CK(cudaEventSynchronize(c->step_done[j & 1]));
+      } else {
+        CK(cudaStreamSynchronize(s));
+      }
+      const double *hj = hp[j & 1], *hj2 = hp2[j & 1];
+      double w1sq;
+      for (int i = 0; i <= j; ++i) h[i] = (two ? hj[i] + hj2[i] : hj[i]) / sv[i];
+      w1sq = hj[m + 1];
       const double nrm = std::sqrt(w1sq);
       if (!std::isfinite(nrm)) PNP_FAIL(PNP_ERR_NAN, "gmres: Krylov vector norm is not finite");
       sv[j + 1] = nrm;
-      if (nrm > 0) {
-        hup[j + 1] = 1.0 / w1sq;
-        CK(cudaMemcpyAsync(dinv + j + 1, hup + j + 1, sizeof(double), cudaMemcpyHostToDevice, s));
-      }
       for (int i = 0; i <= j; ++i) Hij(i, j) = h[i];
       Hij(j + 1, j) = nrm;
       for (int i = 0; i < j; ++i) {
@@ -756,6 +787,8 @@ int ctx_gmres(pnp_ctx* c, const double* U, const double* b, double* x, double rt
         break;
       }
     }
+    // an iteration queued behind the one that ended the cycle is not part of the solve
+    if (queued) c->jv_count--;
     // y = H^-1 g ; x += M^-1 (sum_i y_i u_i / s_i)
     for (int i = k - 1; i >= 0; --i) {
       double t = g[i];
@@ -770,13 +803,13 @@ int ctx_gmres(pnp_ctx* c, const double* U, const double* b, double* x, double rt
     } else if (flex64) {
       for (int i = 0; i < k; ++i) hco[i] = -y[i] / sv[i];
       CK(cudaMemcpyAsync(dcoef, hco, sizeof(double) * k, cudaMemcpyHostToDevice, s));
-      CK(launch_multi_axpy(n, k, c->Z64, n, dcoef, x, nullptr, s));
+      CK(launch_multi_axpy(n, k, c->Z64, n, dcoef, x, s));
     } else {
       for (int i = 0; i < k; ++i) hco[i] = -y[i] / sv[i];
       CK(cudaMemcpyAsync(dcoef, hco, sizeof(double) * k, cudaMemcpyHostToDevice, s));
       CK(cudaMemsetAsync(c->w, 0, sizeof(double) * n, s));
-      CK(launch_multi_axpy(n, k, V, n, dcoef, c->w, nullptr, s));
-      CK(launch_block_apply(c->n_nodes, c->Dinv, c->w, 1.0, c->z, nullptr, s));
+      CK(launch_multi_axpy(n, k, V, n, dcoef, c->w, s));
+      CK(launch_block_apply(c->n_nodes, c->Dinv, c->w, 1.0, nullptr, c->z, nullptr, nullptr, nullptr, s));
       CK(launch_axpby(n, 1.0, c->z, 1.0, x, s));
     }
     // true residual (restart vector); when the Arnoldi estimate claims convergence it is

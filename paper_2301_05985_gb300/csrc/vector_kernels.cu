@@ -5,6 +5,7 @@
 #include <atomic>
 
 #include "kernels.h"
+#include "last_block.cuh"
 
 static std::atomic<int64_t> g_launches{0};
 void note_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
@@ -62,25 +63,40 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
   return r;
 }
 
-__global__ void __launch_bounds__(kRedThreads) k_dot_part(int64_t n, const double* __restrict__ x,
-                                                          const double* __restrict__ y, double* __restrict__ part) {
+// partial sums of x . y per block; the last block adds them (fixed order) and writes the sum,
+// or its square root, to the device and (host, may be null) to mapped pinned memory: one
+// launch where the partials, their sum and a copy to the host were three operations
+__global__ void __launch_bounds__(kRedThreads) k_dot(int64_t n, const double* __restrict__ x,
+                                                     const double* __restrict__ y, double* part, unsigned* ticket,
+                                                     int take_sqrt, double* __restrict__ out,
+                                                     double* __restrict__ host) {
   __shared__ double sh[kRedThreads];
   double s = 0;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     s += x[i] * y[i];
   s = block_sum(s, sh);
   if (threadIdx.x == 0) part[blockIdx.x] = s;
+  if (!last_block(ticket, gridDim.x)) return;
+  s = 0;
+  for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) s += __ldcg(part + b);
+  s = block_sum(s, sh);
+  if (threadIdx.x == 0) {
+    const double r = take_sqrt ? sqrt(s) : s;
+    out[0] = r;
+    if (host) host[0] = r;
+  }
 }
 
-// one block per output: out[j] = sum_b part[b*k + j]  (optionally sqrt)
-__global__ void __launch_bounds__(kRedThreads) k_reduce_parts(int nparts, int k, const double* __restrict__ part,
-                                                              double* __restrict__ out, int take_sqrt) {
+// one block per output: out[j] = sum_b part[b * sb + j * sj]
+__global__ void __launch_bounds__(kRedThreads) k_reduce_parts(int nparts, int64_t sb, int64_t sj,
+                                                              const double* __restrict__ part,
+                                                              double* __restrict__ out) {
   __shared__ double sh[kRedThreads];
   const int j = blockIdx.x;
   double s = 0;
-  for (int b = threadIdx.x; b < nparts; b += blockDim.x) s += part[(int64_t)b * k + j];
+  for (int b = threadIdx.x; b < nparts; b += blockDim.x) s += part[b * sb + j * sj];
   s = block_sum(s, sh);
-  if (threadIdx.x == 0) out[j] = take_sqrt ? sqrt(s) : s;
+  if (threadIdx.x == 0) out[j] = s;
 }
 
 // Sum over the warp of four per-lane values at once (reduce-scatter: 6 adds per lane
@@ -96,71 +112,83 @@ __device__ __forceinline__ double warp_sum4(const double (&s)[4], int lane) {
   return b;
 }
 
-// d_i = V_i . w (i < k; and w . w as entry k when kk > k).  Each block owns a contiguous
-// chunk of kMdRows x 256 rows: w's rows stay in registers while the block sweeps the basis
-// four vectors at a time (4 x kMdRows independent loads per thread, one reduce-scatter
-// over the warp, fixed order).  The FP64 pipe bounds the kernel on GB300, so the rows per
-// thread are many enough that the reduction adds stay small next to the FMAs.  Per-block
-// partials part[block][kk].
-constexpr int kMdRows = 16;
-__global__ void __launch_bounds__(256, 4) k_multi_dot2(int64_t n, int k, int kk, const double* __restrict__ Vb,
-                                                    int64_t ld, const double* __restrict__ w,
-                                                    double* __restrict__ part) {
-  __shared__ double sh[64][8];
+// d_i = V_i . w (i < k).  A block owns 256 R rows: w's rows stay in registers while the block
+// sweeps its share of the basis four vectors at a time (4 R independent loads per thread,
+// one reduce-scatter over the warp, fixed order).  The partials go to part[i][block]; with
+// `ticket`, the last block adds them (a warp per vector).
+// Rows and split by size (multi_dot_shape): for long vectors the FP64 pipe bounds the kernel
+// (78 % of its peak) and R = 16 rows per thread keep the reduction adds small next to the
+// FMAs; for short ones it is latency, and with R = 16 a 3,267-entry vector was one block
+// that swept the whole basis alone (28 us at up to 30 vectors).  Short vectors take one row
+// per thread and a block per four vectors.
+template <int R>
+__global__ void __launch_bounds__(256, 4) k_multi_dot(int64_t n, int k, const double* __restrict__ Vb, int64_t ld,
+                                                      const double* __restrict__ w, double* part, unsigned* ticket,
+                                                      double* __restrict__ d) {
+  __shared__ double sh[4][8];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int64_t base = (int64_t)blockIdx.x * (256 * kMdRows) + threadIdx.x;
-  double wv[kMdRows];
+  const int64_t base = (int64_t)blockIdx.x * (256 * R) + threadIdx.x;
+  const int nb = gridDim.x;
+  const int per = ((k + 3) / 4 + gridDim.y - 1) / gridDim.y * 4;  // vectors of this block
+  const int jb = blockIdx.y * per, je = min(k, jb + per);
+  double wv[R];
 #pragma unroll
-  for (int r = 0; r < kMdRows; ++r) {
+  for (int r = 0; r < R; ++r) {
     const int64_t t = base + r * 256;
     wv[r] = t < n ? w[t] : 0.0;
   }
-  for (int i0 = 0; i0 < kk; i0 += 64) {
-    const int cnt = min(64, kk - i0);
-    // four basis vectors per pass: 4 x kMdRows independent loads, four interleaved shuffle trees
-    for (int j0 = 0; j0 < cnt; j0 += 4) {
-      double s[4] = {0.0, 0.0, 0.0, 0.0};
+  for (int j0 = jb; j0 < je; j0 += 4) {
+    double s[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int i = i0 + j0 + q;
-        if (j0 + q < cnt) {
-          const double* vi = i < k ? Vb + (int64_t)i * ld : w;
+    for (int q = 0; q < 4; ++q) {
+      if (j0 + q < je) {
+        const double* vi = Vb + (int64_t)(j0 + q) * ld;
 #pragma unroll
-          for (int r = 0; r < kMdRows; ++r) {
-            const int64_t t = base + r * 256;
-            if (t < n) s[q] = fma(__ldg(vi + t), wv[r], s[q]);
-          }
+        for (int r = 0; r < R; ++r) {
+          const int64_t t = base + r * 256;
+          if (t < n) s[q] = fma(__ldg(vi + t), wv[r], s[q]);
         }
       }
-      const double tot = warp_sum4(s, lane);
-      const int q = (lane >> 3) & 3;
-      if ((lane & 7) == 0 && j0 + q < cnt) sh[j0 + q][wid] = tot;
     }
+    const double tot = warp_sum4(s, lane);
+    if ((lane & 7) == 0) sh[(lane >> 3) & 3][wid] = tot;
     __syncthreads();
-    for (int j = threadIdx.x; j < cnt; j += blockDim.x) {
-      double s = 0.0;
+    if (threadIdx.x < 4 && j0 + (int)threadIdx.x < je) {
+      double t = 0.0;
 #pragma unroll
-      for (int q = 0; q < 8; ++q) s += sh[j][q];
-      part[(int64_t)blockIdx.x * kk + i0 + j] = s;
+      for (int q = 0; q < 8; ++q) t += sh[threadIdx.x][q];
+      part[(int64_t)(j0 + threadIdx.x) * nb + blockIdx.x] = t;
     }
     __syncthreads();
   }
+  if (!ticket || !last_block(ticket, gridDim.x * gridDim.y)) return;
+  for (int j = wid; j < k; j += 8) {
+    double t = 0.0;
+    for (int b = lane; b < nb; b += 32) t += __ldcg(part + (int64_t)j * nb + b);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (lane == 0) d[j] = t;
+  }
 }
 
-// w -= sum_i (d_i * dinv_i) V_i  and per-block partial sums of the updated w . w
+// w -= sum_i (d_i * dinv_i) V_i and w . w of the updated w; the last block adds the partials
+// and finishes the Krylov step: w . w and its reciprocal for the next vector on the device,
+// and what the host needs of the step into mapped pinned memory (GsFinish)
 __global__ void __launch_bounds__(kRedThreads) k_multi_axpy_norm(int64_t n, int k, const double* __restrict__ Vb,
                                                                  int64_t ld, const double* __restrict__ d,
                                                                  const double* __restrict__ dinv,
-                                                                 double* __restrict__ w, double* __restrict__ part) {
+                                                                 double* __restrict__ w, double* part,
+                                                                 unsigned* ticket, GsFinish f) {
   extern __shared__ double cf[];
   __shared__ double sh[kRedThreads];
   for (int i = threadIdx.x; i < k; i += blockDim.x) cf[i] = d[i] * dinv[i];
   __syncthreads();
   double ss = 0.0;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
-    // two independent chains (the loads are independent anyway); one add to join them
+    // two independent chains; eight loads in flight
     double v0 = w[t], v1 = 0.0;
     int i = 0;
+#pragma unroll 4
     for (; i + 2 <= k; i += 2) {
       v0 -= cf[i] * Vb[(int64_t)i * ld + t];
       v1 -= cf[i + 1] * Vb[(int64_t)(i + 1) * ld + t];
@@ -172,16 +200,27 @@ __global__ void __launch_bounds__(kRedThreads) k_multi_axpy_norm(int64_t n, int 
   }
   ss = block_sum(ss, sh);
   if (threadIdx.x == 0) part[blockIdx.x] = ss;
+  if (!last_block(ticket, gridDim.x)) return;
+  ss = 0.0;
+  for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) ss += __ldcg(part + b);
+  ss = block_sum(ss, sh);
+  if (threadIdx.x == 0) {
+    f.nrm2[0] = ss;
+    if (f.dinv_next) f.dinv_next[0] = ss > 0.0 ? 1.0 / ss : 0.0;
+    if (f.inv_s_next) f.inv_s_next[0] = ss > 0.0 ? 1.0 / sqrt(ss) : 0.0;
+    if (f.host_nrm2) f.host_nrm2[0] = ss;
+  }
+  if (f.host0)
+    for (int i = threadIdx.x; i < k; i += blockDim.x) f.host0[i] = f.d0[i];
+  if (f.host1)
+    for (int i = threadIdx.x; i < k; i += blockDim.x) f.host1[i] = f.d1[i];
 }
 
 __global__ void __launch_bounds__(256) k_multi_axpy(int64_t n, int k, const double* __restrict__ Vb, int64_t ld,
-                                                    const double* __restrict__ h, double* __restrict__ w,
-                                                    double* __restrict__ hacc) {
+                                                    const double* __restrict__ h, double* __restrict__ w) {
   extern __shared__ double hs[];
   for (int i = threadIdx.x; i < k; i += blockDim.x) hs[i] = h[i];
   __syncthreads();
-  if (hacc && blockIdx.x == 0)
-    for (int i = threadIdx.x; i < k; i += blockDim.x) hacc[i] += hs[i];
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
     double v = w[t];
     for (int i = 0; i < k; ++i) v -= hs[i] * Vb[(int64_t)i * ld + t];
@@ -190,9 +229,13 @@ __global__ void __launch_bounds__(256) k_multi_axpy(int64_t n, int k, const doub
 }
 
 __global__ void k_block_apply(int64_t N, const double* __restrict__ Dinv, const double* __restrict__ v, double scale,
-                              double* __restrict__ z, float* __restrict__ z32) {
+                              const double* __restrict__ scale_dev, double* __restrict__ z, float* __restrict__ z32, double* __restrict__ clear,
+                              float* __restrict__ clear32) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= N) return;
+  if (clear) clear[3 * i] = clear[3 * i + 1] = clear[3 * i + 2] = 0.0;
+  if (clear32) clear32[3 * i] = clear32[3 * i + 1] = clear32[3 * i + 2] = 0.f;
+  if (scale_dev) scale = *scale_dev;
   const double* B = Dinv + 9 * i;
   const double a = scale * v[3 * i], b = scale * v[3 * i + 1], c = scale * v[3 * i + 2];
   const double r0 = B[0] * a + B[1] * b + B[2] * c;
@@ -304,20 +347,30 @@ cudaError_t launch_axpbyz(int64_t n, double a, const double* x, double b, const 
   if (n) { k_axpbyz<<<gs_blocks(n, 256), 256, 0, s>>>(n, a, x, b, y, z); note_launch(); }
   return cudaGetLastError();
 }
-cudaError_t launch_dot(int64_t n, const double* x, const double* y, double* part, double* result, cudaStream_t s) {
-  k_dot_part<<<kRedBlocks, kRedThreads, 0, s>>>(n, x, y, part); note_launch();
-  k_reduce_parts<<<1, kRedThreads, 0, s>>>(kRedBlocks, 1, part, result, 0); note_launch();
+// threads and blocks of a reduction over n entries: at most kRedBlocks blocks of 256, for
+// short vectors (fewer than 64 kRedBlocks entries) blocks of 64
+static int red_threads(int64_t n) { return n < int64_t(64) * kRedBlocks ? 64 : kRedThreads; }
+static int red_blocks(int64_t n) {
+  const int t = red_threads(n);
+  return (int)std::min<int64_t>(kRedBlocks, std::max<int64_t>(1, (n + t - 1) / t));
+}
+
+cudaError_t launch_dot(int64_t n, const double* x, const double* y, double* part, unsigned* ticket, double* result,
+                       double* host, cudaStream_t s) {
+  k_dot<<<red_blocks(n), red_threads(n), 0, s>>>(n, x, y, part, ticket, 0, result, host);
+  note_launch();
   return cudaGetLastError();
 }
-cudaError_t launch_norm2(int64_t n, const double* x, double* part, double* result, cudaStream_t s) {
-  k_dot_part<<<kRedBlocks, kRedThreads, 0, s>>>(n, x, x, part); note_launch();
-  k_reduce_parts<<<1, kRedThreads, 0, s>>>(kRedBlocks, 1, part, result, 1); note_launch();
+cudaError_t launch_norm2(int64_t n, const double* x, double* part, unsigned* ticket, double* result, double* host,
+                         cudaStream_t s) {
+  k_dot<<<red_blocks(n), red_threads(n), 0, s>>>(n, x, x, part, ticket, 1, result, host);
+  note_launch();
   return cudaGetLastError();
 }
 cudaError_t launch_multi_axpy(int64_t n, int k, const double* Vb, int64_t ld, const double* h, double* w,
-                              double* hacc, cudaStream_t s) {
+                              cudaStream_t s) {
   if (k <= 0) return cudaSuccess;
-  k_multi_axpy<<<gs_blocks(n, 256), 256, k * sizeof(double), s>>>(n, k, Vb, ld, h, w, hacc); note_launch();
+  k_multi_axpy<<<gs_blocks(n, 256), 256, k * sizeof(double), s>>>(n, k, Vb, ld, h, w); note_launch();
   return cudaGetLastError();
 }
 __global__ void k_node_records(int64_t N, const double* __restrict__ U, const double* __restrict__ hs,
@@ -339,32 +392,55 @@ cudaError_t launch_node_records(int64_t N, const double* U, const double* hs, co
 
 cudaError_t launch_reduce_parts(int nparts, int k, const double* part, double* out, cudaStream_t s) {
   if (k <= 0) return cudaSuccess;
-  k_reduce_parts<<<k, kRedThreads, 0, s>>>(nparts, k, part, out, 0);
+  k_reduce_parts<<<k, kRedThreads, 0, s>>>(nparts, k, 1, part, out);
+  note_launch();
+  return cudaGetLastError();
+}
+cudaError_t launch_reduce_cols(int nparts, int k, const double* part, double* out, cudaStream_t s) {
+  if (k <= 0) return cudaSuccess;
+  k_reduce_parts<<<k, kRedThreads, 0, s>>>(nparts, 1, nparts, part, out);
   note_launch();
   return cudaGetLastError();
 }
 
-int multi_dot_blocks(int64_t n) { return (int)std::max<int64_t>(1, (n + 256 * kMdRows - 1) / (256 * kMdRows)); }
+// rows per thread: 16 while that leaves two blocks per SM (vectors of 1.2 M entries and
+// more), 4 down to 155 k entries, 1 below
+static int multi_dot_rows(int64_t n) { return n >= int64_t(304) * 4096 ? 16 : n >= int64_t(152) * 1024 ? 4 : 1; }
+int multi_dot_blocks(int64_t n) {
+  const int64_t rows = 256 * multi_dot_rows(n);
+  return (int)std::max<int64_t>(1, (n + rows - 1) / rows);
+}
 
-cudaError_t launch_multi_dot_ext(int64_t n, int k, bool with_self, const double* Vb, int64_t ld, const double* w,
-                                 double* part, double* d, cudaStream_t s) {
-  const int kk = k + (with_self ? 1 : 0);
-  if (kk <= 0) return cudaSuccess;
-  const int nb = multi_dot_blocks(n);
-  k_multi_dot2<<<nb, 256, 0, s>>>(n, k, kk, Vb, ld, w, part); note_launch();
-  k_reduce_parts<<<kk, kRedThreads, 0, s>>>(nb, kk, part, d, 0); note_launch();
-  return cudaGetLastError();
+cudaError_t launch_multi_dot(int64_t n, int k, const double* Vb, int64_t ld, const double* w, double* part,
+                             unsigned* ticket, double* d, cudaStream_t s) {
+  if (k <= 0) return cudaSuccess;
+  const int nb = multi_dot_blocks(n), rows = multi_dot_rows(n), groups = (k + 3) / 4;
+  // short vectors: a block per four vectors until the chip has eight blocks per SM
+  const int gy = rows == 16 ? 1 : (int)std::min<int64_t>(groups, std::max<int64_t>(1, 1216 / nb));
+  // the last block adds up to 16 k partials (about 4 us); beyond that a block per vector does
+  const bool fused = (int64_t)nb * k <= 16384;
+  unsigned* tk = fused ? ticket : nullptr;
+  const dim3 grid(nb, gy);
+  if (rows == 16) k_multi_dot<16><<<grid, 256, 0, s>>>(n, k, Vb, ld, w, part, tk, d);
+  else if (rows == 4) k_multi_dot<4><<<grid, 256, 0, s>>>(n, k, Vb, ld, w, part, tk, d);
+  else k_multi_dot<1><<<grid, 256, 0, s>>>(n, k, Vb, ld, w, part, tk, d);
+  note_launch();
+  return fused ? cudaGetLastError() : launch_reduce_cols(nb, k, part, d, s);
 }
 cudaError_t launch_multi_axpy_norm(int64_t n, int k, const double* Vb, int64_t ld, const double* d, const double* dinv,
-                                   double* w, double* part, double* nrm2, cudaStream_t s) {
-  k_multi_axpy_norm<<<kRedBlocks, kRedThreads, (k > 0 ? k : 1) * sizeof(double), s>>>(n, k, Vb, ld, d, dinv, w, part);
+                                   double* w, double* part, unsigned* ticket, const GsFinish& f, cudaStream_t s) {
+  k_multi_axpy_norm<<<red_blocks(n), red_threads(n), (k > 0 ? k : 1) * sizeof(double), s>>>(n, k, Vb, ld, d, dinv, w,
+                                                                                           part, ticket, f);
   note_launch();
-  k_reduce_parts<<<1, kRedThreads, 0, s>>>(kRedBlocks, 1, part, nrm2, 0); note_launch();
   return cudaGetLastError();
 }
-cudaError_t launch_block_apply(int64_t N, const double* Dinv, const double* v, double scale, double* z, float* z32,
-                               cudaStream_t s) {
-  if (N) { k_block_apply<<<nblk(N, 256), 256, 0, s>>>(N, Dinv, v, scale, z, z32); note_launch(); }
+cudaError_t launch_block_apply(int64_t N, const double* Dinv, const double* v, double scale, const double* scale_dev,
+                               double* z, float* z32, double* clear, float* clear32, cudaStream_t s) {
+  if (N) {
+    const int t = block_threads(N);
+    k_block_apply<<<block_count(N, t), t, 0, s>>>(N, Dinv, v, scale, scale_dev, z, z32, clear, clear32);
+    note_launch();
+  }
   return cudaGetLastError();
 }
 template <typename T>
