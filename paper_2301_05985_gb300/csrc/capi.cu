@@ -310,7 +310,7 @@ int pnp_ctx_create(const pnp_mesh* m, const pnp_params* p, void* stream, pnp_ctx
   ALLOC(c->hs32, sizeof(float) * 2 * N);
   ALLOC(c->rec32, sizeof(float4) * 2 * N);
   ALLOC(c->V32, sizeof(float) * 3 * N);
-  ALLOC(c->JV32, sizeof(float) * 3 * N);
+  ALLOC(c->JV32, sizeof(float) * (3 * N + 4));  // the inner solve writes whole float4
   ALLOC(c->F, v3);
   ALLOC(c->dU, v3);
   ALLOC(c->Ut, v3);

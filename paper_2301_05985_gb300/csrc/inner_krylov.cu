@@ -7,6 +7,7 @@
 #include <cstdint>
 
 #include "kernels.h"
+#include "last_block.cuh"
 
 namespace {
 
@@ -38,23 +39,28 @@ __device__ __forceinline__ double block_sum_d(double v, double* sh) {
 // The inner basis has rows padded to a multiple of four floats (zeros beyond the
 // vector's length), so both Gram-Schmidt kernels move float4: four entries per load.
 
-// d_i = U_i . w (i < k) for FP32 vectors of n4 float4.  Persistent grid (kInnerBlocks, 8
-// per SM): each block strides over chunks of 256 x kRows float4; for every group of four
-// basis vectors a thread accumulates its rows of all chunks (w re-read from L2 per
-// group), then one warp reduce-scatter and a fixed-order block sum give the block's
-// partials part[block][k].
+// d_i = U_i . w (i < k) for FP32 vectors of n4 float4.  At most kInnerBlocks blocks (8 per
+// SM) stride over chunks of 256 x kRows float4; for every group of four basis vectors a
+// thread accumulates its rows of all chunks (w re-read from L2 per group), then one warp
+// reduce-scatter and a fixed-order block sum give the block's partials part[i][block].
+// Long vectors stream at HBM rate (89 %).  Short ones (a 163 k-node mesh: 240 chunks, the
+// basis in L2) are latency: there blockIdx.y takes a share of the groups, and the last block
+// adds the partials (`ticket` given) instead of a second launch.
 constexpr int kRows = 2;
 __device__ __forceinline__ float dot4(float4 a, float4 b, float s) {
   return fmaf(a.x, b.x, fmaf(a.y, b.y, fmaf(a.z, b.z, fmaf(a.w, b.w, s))));
 }
 __global__ void __launch_bounds__(256, 8) k_multi_dot_f32(int64_t n4, int k, const float4* __restrict__ Ub,
-                                                          int64_t ld4, const float4* __restrict__ w,
-                                                          double* __restrict__ part) {
+                                                          int64_t ld4, const float4* __restrict__ w, double* part,
+                                                          unsigned* ticket, double* __restrict__ d) {
   __shared__ float sh[4][8];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int64_t chunk = 256 * kRows;
-  for (int j0 = 0; j0 < k; j0 += 4) {
-    const int cnt = min(4, k - j0);
+  const int nb = gridDim.x;
+  const int per = ((k + 3) / 4 + gridDim.y - 1) / gridDim.y * 4;  // vectors of this block
+  const int je = min(k, ((int)blockIdx.y + 1) * per);
+  for (int j0 = blockIdx.y * per; j0 < je; j0 += 4) {
+    const int cnt = min(4, je - j0);
     float s[4] = {0.0f, 0.0f, 0.0f, 0.0f};
     for (int64_t c0 = (int64_t)blockIdx.x * chunk; c0 < n4; c0 += (int64_t)gridDim.x * chunk) {
       float4 wv[kRows];
@@ -76,33 +82,56 @@ __global__ void __launch_bounds__(256, 8) k_multi_dot_f32(int64_t n4, int k, con
       }
     }
     const float tot = warp_sum4f(s, lane);
-    const int q = (lane >> 3) & 3;
-    if ((lane & 7) == 0) sh[q][wid] = tot;
+    if ((lane & 7) == 0) sh[(lane >> 3) & 3][wid] = tot;
     __syncthreads();
     if (threadIdx.x < cnt) {
       double t = 0.0;
 #pragma unroll
       for (int v = 0; v < 8; ++v) t += (double)sh[threadIdx.x][v];
-      part[(int64_t)blockIdx.x * k + j0 + threadIdx.x] = t;
+      part[(int64_t)(j0 + threadIdx.x) * nb + blockIdx.x] = t;
     }
     __syncthreads();
   }
+  if (!ticket || !last_block(ticket, gridDim.x * gridDim.y)) return;
+  for (int j = wid; j < k; j += 8) {
+    double t = 0.0;
+#pragma unroll 4
+    for (int b = lane; b < nb; b += 32) t += __ldcg(part + (int64_t)j * nb + b);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (lane == 0) d[j] = t;
+  }
 }
 
-// w -= sum_i (d_i dinv_i) U_i (i < k) in FP32 on n4 float4, then per-block partials of
-// w . w.  Persistent grid of 6 blocks per SM.
+// Arnoldi bookkeeping of the inner process.  Basis vectors u_i are kept unnormalised
+// with norms s_i (q_i = u_i / s_i).  The steps only store the Hessenberg columns
+// h_i = d_i / s_i, h_(j+1) = s_(j+1); the Givens rotations wait for the least-squares
+// kernel at the end, where the columns rotate in parallel.  (Rotating column j as it
+// arrived kept one thread busy with up to 2 d dependent FP64 operations between two steps:
+// 11 us per step at d = 24, as a launch of its own.)
+// Scalar layout: H [(d+1) x d] row-major.
+struct InnerStep {
+  int j, d;            // column j of d; j < 0: the start vector
+  const double* dd;    // projections of the step
+  double *sv, *dinv;   // norms s_i and 1 / s_i^2
+  float* inv_s;        // 1 / s_i
+  double* H;
+};
+
+// w -= sum_i (d_i dinv_i) U_i (i < k) in FP32 on n4 float4, and w . w: at most kUpdBlocks
+// blocks (6 per SM); the last one adds the partials and ends the Arnoldi step.
 constexpr int kUpdBlocks = 6 * 152;
 __global__ void __launch_bounds__(256, 6) k_multi_axpy_norm_f32(int64_t n4, int k, const float4* __restrict__ Ub,
-                                                             int64_t ld4, const double* __restrict__ d,
-                                                             const double* __restrict__ dinv, float4* __restrict__ w,
-                                                             double* __restrict__ part) {
+                                                             int64_t ld4, float4* __restrict__ w, double* part,
+                                                             unsigned* ticket, InnerStep S) {
   extern __shared__ float cf[];
   __shared__ double sh[256];
-  for (int i = threadIdx.x; i < k; i += blockDim.x) cf[i] = (float)(d[i] * dinv[i]);
+  for (int i = threadIdx.x; i < k; i += blockDim.x) cf[i] = (float)(S.dd[i] * S.dinv[i]);
   __syncthreads();
   float ss = 0.0f;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n4; t += (int64_t)gridDim.x * blockDim.x) {
     float4 a = w[t];
+#pragma unroll 4
     for (int i = 0; i < k; ++i) {
       const float4 u = Ub[(int64_t)i * ld4 + t];
       const float c = -cf[i];
@@ -114,8 +143,22 @@ __global__ void __launch_bounds__(256, 6) k_multi_axpy_norm_f32(int64_t n4, int 
     if (k > 0) w[t] = a;
     ss = fmaf(a.x, a.x, fmaf(a.y, a.y, fmaf(a.z, a.z, fmaf(a.w, a.w, ss))));
   }
-  const double tot = block_sum_d((double)ss, sh);
+  double tot = block_sum_d((double)ss, sh);
   if (threadIdx.x == 0) part[blockIdx.x] = tot;
+  if (!last_block(ticket, gridDim.x)) return;
+  tot = 0.0;
+#pragma unroll 4
+  for (int b = threadIdx.x; b < (int)gridDim.x; b += 256) tot += __ldcg(part + b);
+  tot = block_sum_d(tot, sh);
+  const int i = threadIdx.x;
+  if (i == 0) {
+    const double s = sqrt(tot);
+    S.sv[S.j + 1] = s;
+    S.dinv[S.j + 1] = s > 0 ? 1.0 / (s * s) : 0.0;
+    S.inv_s[S.j + 1] = s > 0 ? (float)(1.0 / s) : 0.0f;
+    if (S.j >= 0) S.H[(int64_t)(S.j + 1) * S.d + S.j] = s;
+  }
+  if (i <= S.j) S.H[(int64_t)i * S.d + S.j] = S.sv[i] > 0 ? S.dd[i] / S.sv[i] : 0.0;
 }
 
 // y_i = Dinv_i (inv_s[0] u_i) per node, FP32 3x3 blocks
@@ -132,9 +175,11 @@ __global__ void k_block_apply32(int64_t N, const float* __restrict__ Dinv, const
 }
 
 __global__ void k_block_apply32_pad(int64_t N, const float* __restrict__ Dinv, const float* __restrict__ u,
-                                    const float* __restrict__ inv_s, float4* __restrict__ y) {
+                                    const float* __restrict__ inv_s, float4* __restrict__ y,
+                                    float4* __restrict__ clear) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= N) return;
+  clear[i] = make_float4(0.f, 0.f, 0.f, 0.f);
   const float sc = inv_s ? inv_s[0] : 1.0f;
   const float* B = Dinv + 9 * i;
   const float a = sc * u[3 * i], b = sc * u[3 * i + 1], c = sc * u[3 * i + 2];
@@ -186,148 +231,71 @@ __global__ void k_pack_jv4(int64_t N, int64_t H, const uint8_t* __restrict__ fac
   out[3 * id + 2] = sv.z;
 }
 
-// Arnoldi bookkeeping of the inner process.  Basis vectors u_i are kept unnormalised
-// with norms s_i (q_i = u_i / s_i); the Hessenberg columns are reduced by Givens rotations
-// as they arrive, so the least-squares solve at the end is a back-substitution.
-// Scalar layout: R [(d+1) x d] row-major, cs[d], sn[d], g[d+1], kv[1] (the number of
-// columns before the first breakdown, as a double).
-struct InnerScalars {
-  double *R, *cs, *sn, *g, *kv;
-};
-__device__ __forceinline__ InnerScalars inner_scalars(double* base, int d) {
-  InnerScalars S;
-  S.R = base;
-  S.cs = S.R + (size_t)(d + 1) * d;
-  S.sn = S.cs + d;
-  S.g = S.sn + d;
-  S.kv = S.g + (d + 1);
-  return S;
-}
-
-// sum of the norm partials of k_multi_axpy_norm_f32 in a fixed order (one block of 64)
-// sum of the norm partials by one block of kBookThreads threads: every thread issues its
-// loads at once (at most four), then a fixed-order tree
-constexpr int kBookThreads = 256;
-__device__ __forceinline__ double sum_parts(const double* __restrict__ part, int nparts, double* sh) {
-  double t0 = 0.0, t1 = 0.0, t2 = 0.0, t3 = 0.0;
-  int b = threadIdx.x;
-  for (; b + 3 * kBookThreads < nparts; b += 4 * kBookThreads) {
-    t0 += part[b];
-    t1 += part[b + kBookThreads];
-    t2 += part[b + 2 * kBookThreads];
-    t3 += part[b + 3 * kBookThreads];
-  }
-  for (; b < nparts; b += kBookThreads) t0 += part[b];
-  sh[threadIdx.x] = (t0 + t1) + (t2 + t3);
-  __syncthreads();
-  for (int o = kBookThreads / 2; o > 0; o >>= 1) {
-    if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-    __syncthreads();
-  }
-  return sh[0];
-}
-
-__global__ void __launch_bounds__(kBookThreads) k_inner_start(int d, const double* __restrict__ part, int nparts,
-                                                              double* sv, double* dinv, float* inv_s, double* sc) {
-  __shared__ double sh[kBookThreads];
-  const InnerScalars S = inner_scalars(sc, d);
-  for (int i = threadIdx.x; i <= d; i += blockDim.x) S.g[i] = 0.0;
-  const double nrm2 = sum_parts(part, nparts, sh);
-  if (threadIdx.x == 0) {
-    const double s = sqrt(nrm2);
-    sv[0] = s;
-    dinv[0] = s > 0 ? 1.0 / (s * s) : 0.0;
-    inv_s[0] = s > 0 ? (float)(1.0 / s) : 0.0f;
-    S.g[0] = s;
-    S.kv[0] = 0.0;
-  }
-}
-
-// column j: h_i = d_i / s_i (i <= j), h_{j+1} = ||u_{j+1}||; apply the earlier rotations,
-// make rotation j, update g.  One block of kBookThreads threads (the first kMaxInner hold
-// the column).
+// Least squares of the inner process and coef_i = y_i / s_i, so that sum_i y_i q_i = sum_i
+// coef_i u_i.  Thread l holds column l: step j makes rotation j from column j and applies it
+// to the columns after it; then a column-oriented back-substitution over the columns before
+// the first breakdown (a zero rotated column).
 constexpr int kMaxInner = 64;
-static_assert(kBookThreads >= kMaxInner, "one thread per column entry");
-__global__ void __launch_bounds__(kBookThreads) k_inner_col(int j, int d, const double* __restrict__ dd,
-                                                            const double* __restrict__ part, int nparts, double* sv,
-                                                            double* dinv, float* inv_s, double* sc) {
-  __shared__ double h[kMaxInner + 1];
-  __shared__ double sh[kBookThreads];
-  __shared__ double cs[kMaxInner], sn[kMaxInner];
-  const InnerScalars S = inner_scalars(sc, d);
-  const int i = threadIdx.x;
-  if (i <= j) h[i] = sv[i] > 0 ? dd[i] / sv[i] : 0.0;
-  if (i < j) {
-    cs[i] = S.cs[i];
-    sn[i] = S.sn[i];
+__global__ void __launch_bounds__(kMaxInner) k_inner_lsq(int d, const double* __restrict__ sv,
+                                                         const double* __restrict__ Hg, double* __restrict__ coef) {
+  __shared__ double H[kMaxInner + 1][kMaxInner + 1], g[kMaxInner + 1], cs[kMaxInner], sn[kMaxInner], y[kMaxInner];
+  __shared__ int kv;
+  const int l = threadIdx.x;
+  for (int t = l; t < (d + 1) * d; t += kMaxInner) {
+    const int r = t / d, c = t - r * d;
+    H[r][c] = r <= c + 1 ? Hg[t] : 0.0;
   }
-  const double nrm2 = sum_parts(part, nparts, sh);
-  if (i == 0) {
-    const double s = sqrt(nrm2);
-    h[j + 1] = s;
-    sv[j + 1] = s;
-    dinv[j + 1] = s > 0 ? 1.0 / (s * s) : 0.0;
-    inv_s[j + 1] = s > 0 ? (float)(1.0 / s) : 0.0f;
-  }
+  for (int t = l; t <= d; t += kMaxInner) g[t] = t == 0 ? sv[0] : 0.0;
+  if (l == 0) kv = 0;
   __syncthreads();
-  if (i != 0) return;
-  for (int l = 0; l < j; ++l) {
-    const double t = cs[l] * h[l] + sn[l] * h[l + 1];
-    h[l + 1] = -sn[l] * h[l] + cs[l] * h[l + 1];
-    h[l] = t;
-  }
-  const double rr = hypot(h[j], h[j + 1]);
-  if (rr > 0) {
-    S.cs[j] = h[j] / rr;
-    S.sn[j] = h[j + 1] / rr;
-    h[j] = rr;
-    S.g[j + 1] = -S.sn[j] * S.g[j];
-    S.g[j] = S.cs[j] * S.g[j];
-    if (S.kv[0] == (double)j) S.kv[0] = j + 1;
-  } else {
-    S.cs[j] = 1.0;
-    S.sn[j] = 0.0;
-  }
-  for (int l = 0; l <= j; ++l) S.R[l * d + j] = h[l];
-}
-
-// y = R^-1 g over the columns before the first breakdown; coef_i = y_i / s_i, so that
-// sum_i y_i q_i = sum_i coef_i u_i.  The block stages R, g and s in shared memory, then
-// one thread back-substitutes.
-__global__ void __launch_bounds__(kMaxInner) k_inner_lsq(int d, const double* __restrict__ sv, double* sc,
-                                                         double* __restrict__ coef) {
-  __shared__ double R[kMaxInner * kMaxInner], g[kMaxInner], y[kMaxInner];
-  const InnerScalars S = inner_scalars(sc, d);
-  const int k = (int)S.kv[0];
-  for (int t = threadIdx.x; t < k * d; t += blockDim.x) R[t] = S.R[t];
-  for (int t = threadIdx.x; t < k; t += blockDim.x) g[t] = S.g[t];
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int i = k - 1; i >= 0; --i) {
-      double t = g[i];
-      for (int l = i + 1; l < k; ++l) t -= R[i * d + l] * y[l];
-      y[i] = t / R[i * d + i];
+  for (int j = 0; j < d; ++j) {
+    if (l == j) {
+      const double rr = hypot(H[j][j], H[j + 1][j]);
+      cs[j] = 1.0;
+      sn[j] = 0.0;
+      if (rr > 0) {
+        cs[j] = H[j][j] / rr;
+        sn[j] = H[j + 1][j] / rr;
+        H[j][j] = rr;
+        g[j + 1] = -sn[j] * g[j];
+        g[j] = cs[j] * g[j];
+        if (kv == j) kv = j + 1;
+      }
+    }
+    __syncthreads();
+    if (l > j && l < d) {
+      const double t = cs[j] * H[j][l] + sn[j] * H[j + 1][l];
+      H[j + 1][l] = -sn[j] * H[j][l] + cs[j] * H[j + 1][l];
+      H[j][l] = t;
     }
   }
-  __syncthreads();
-  for (int t = threadIdx.x; t < d; t += blockDim.x) coef[t] = t < k ? y[t] / sv[t] : 0.0;
+  const int k = kv;
+  for (int i = k - 1; i >= 0; --i) {
+    if (l == i) y[i] = g[i] / H[i][i];
+    __syncthreads();
+    if (l < i) g[l] -= H[l][i] * y[i];
+  }
+  if (l < d) coef[l] = l < k ? y[l] / sv[l] : 0.0;
 }
 
-// out = sum_i coef_i U_i (FP32 vectors, coefficients on the device)
-__global__ void k_combine_f32(int64_t n, int k, const float* __restrict__ Ub, int64_t ld,
-                              const double* __restrict__ coef, float* __restrict__ out) {
+// out = sum_i coef_i U_i (FP32 vectors of n4 float4, coefficients on the device)
+__global__ void k_combine_f32(int64_t n4, int k, const float4* __restrict__ Ub, int64_t ld4,
+                              const double* __restrict__ coef, float4* __restrict__ out) {
   extern __shared__ float cf[];
   for (int i = threadIdx.x; i < k; i += blockDim.x) cf[i] = (float)coef[i];
   __syncthreads();
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
-    float v0 = 0.0f, v1 = 0.0f;
-    int i = 0;
-    for (; i + 2 <= k; i += 2) {
-      v0 = fmaf(cf[i], Ub[(int64_t)i * ld + t], v0);
-      v1 = fmaf(cf[i + 1], Ub[(int64_t)(i + 1) * ld + t], v1);
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n4; t += (int64_t)gridDim.x * blockDim.x) {
+    float4 v[2] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
+#pragma unroll 4
+    for (int i = 0; i < k; ++i) {
+      const float4 u = Ub[(int64_t)i * ld4 + t];
+      float4& a = v[i & 1];
+      a.x = fmaf(cf[i], u.x, a.x);
+      a.y = fmaf(cf[i], u.y, a.y);
+      a.z = fmaf(cf[i], u.z, a.z);
+      a.w = fmaf(cf[i], u.w, a.w);
     }
-    if (i < k) v0 = fmaf(cf[i], Ub[(int64_t)i * ld + t], v0);
-    out[t] = v0 + v1;
+    out[t] = make_float4(v[0].x + v[1].x, v[0].y + v[1].y, v[0].z + v[1].z, v[0].w + v[1].w);
   }
 }
 
@@ -357,27 +325,43 @@ __global__ void k_to_f64_scaled(int64_t n, const float* __restrict__ x, double s
 
 }  // namespace
 
-int inner_dot_blocks(int64_t) { return kInnerBlocks; }
+int inner_dot_blocks(int64_t n) {
+  const int64_t chunk = 4 * 256 * kRows;
+  return (int)std::min<int64_t>(kInnerBlocks, std::max<int64_t>(1, (n + chunk - 1) / chunk));
+}
 int inner_max_depth() { return kMaxInner; }
 
-cudaError_t launch_multi_dot_f32(int64_t n, int k, const float* Ub, int64_t ld, const float* w, double* part, double* d,
-                                 cudaStream_t s) {
+cudaError_t launch_multi_dot_f32(int64_t n, int k, const float* Ub, int64_t ld, const float* w, double* part,
+                                 unsigned* ticket, double* d, cudaStream_t s) {
   if (k <= 0) return cudaSuccess;
   if ((n | ld) & 3) return cudaErrorInvalidValue;  // rows padded to float4
-  const int nb = inner_dot_blocks(n);
-  k_multi_dot_f32<<<nb, 256, 0, s>>>(n / 4, k, (const float4*)Ub, ld / 4, (const float4*)w, part);
+  const int nb = inner_dot_blocks(n), groups = (k + 3) / 4;
+  const int gy = std::min(groups, std::max(1, kInnerBlocks / nb));
+  // the last block adds up to 16 k partials; beyond that a block per vector does
+  const bool fused = (int64_t)nb * k <= 16384;
+  k_multi_dot_f32<<<dim3(nb, gy), 256, 0, s>>>(n / 4, k, (const float4*)Ub, ld / 4, (const float4*)w, part,
+                                               fused ? ticket : nullptr, d);
   note_launch();
-  launch_reduce_parts(nb, k, part, d, s);
-  return cudaGetLastError();
+  return fused ? cudaGetLastError() : launch_reduce_cols(nb, k, part, d, s);
 }
 
-cudaError_t launch_multi_axpy_norm_f32(int64_t n, int k, const float* Ub, int64_t ld, const double* d,
-                                       const double* dinv, float* w, double* part, cudaStream_t s) {
+static cudaError_t launch_update(int64_t n, int k, const float* Ub, int64_t ld, float* w, double* part,
+                                 unsigned* ticket, const InnerStep& S, cudaStream_t s) {
   if ((n | ld) & 3) return cudaErrorInvalidValue;  // rows padded to float4
-  k_multi_axpy_norm_f32<<<kUpdBlocks, 256, (k > 0 ? k : 1) * sizeof(float), s>>>(n / 4, k, (const float4*)Ub, ld / 4,
-                                                                                 d, dinv, (float4*)w, part);
+  const int nb = (int)std::min<int64_t>(kUpdBlocks, std::max<int64_t>(1, (n / 4 + 255) / 256));
+  k_multi_axpy_norm_f32<<<nb, 256, (k > 0 ? k : 1) * sizeof(float), s>>>(n / 4, k, (const float4*)Ub, ld / 4, (float4*)w,
+                                                                        part, ticket, S);
   note_launch();
   return cudaGetLastError();
+}
+cudaError_t launch_inner_start(int64_t n, int d, float* u0, double* part, unsigned* ticket, double* sv, double* dinv,
+                               float* inv_s, cudaStream_t s) {
+  return launch_update(n, 0, u0, n, u0, part, ticket, InnerStep{-1, d, nullptr, sv, dinv, inv_s, nullptr}, s);
+}
+cudaError_t launch_inner_update(int64_t n, int j, int d, const float* Ub, int64_t ld, const double* dd, float* w,
+                                double* part, unsigned* ticket, double* sv, double* dinv, float* inv_s, double* H,
+                                cudaStream_t s) {
+  return launch_update(n, j + 1, Ub, ld, w, part, ticket, InnerStep{j, d, dd, sv, dinv, inv_s, H}, s);
 }
 
 cudaError_t launch_block_apply32(int64_t N, const float* Dinv32, const float* u, const float* inv_s, float* y,
@@ -390,9 +374,10 @@ cudaError_t launch_block_apply32(int64_t N, const float* Dinv32, const float* u,
 }
 
 cudaError_t launch_block_apply32_pad(int64_t N, const float* Dinv32, const float* u, const float* inv_s, float4* y4,
-                                     cudaStream_t s) {
+                                     float4* clear, cudaStream_t s) {
   if (N) {
-    k_block_apply32_pad<<<nblk(N, 256), 256, 0, s>>>(N, Dinv32, u, inv_s, y4);
+    const int t = block_threads(N);
+    k_block_apply32_pad<<<block_count(N, t), t, 0, s>>>(N, Dinv32, u, inv_s, y4, clear);
     note_launch();
   }
   return cudaGetLastError();
@@ -408,36 +393,25 @@ cudaError_t launch_pad4(int64_t N, const float* x, float4* y4, cudaStream_t s) {
 
 cudaError_t launch_pack_jv4(const RowArgs& R, const float4* V4, const float4* acc4, float* out, cudaStream_t s) {
   if (R.n_nodes + R.n_hanging) {
-    k_pack_jv4<<<nblk(R.n_nodes + R.n_hanging, 256), 256, 0, s>>>(R.n_nodes, R.n_hanging, R.faces, R.bc, R.hnode,
+    const int t = block_threads(R.n_nodes + R.n_hanging);
+    k_pack_jv4<<<block_count(R.n_nodes + R.n_hanging, t), t, 0, s>>>(R.n_nodes, R.n_hanging, R.faces, R.bc, R.hnode,
                                                                   R.hpar, R.hnp, V4, acc4, out);
     note_launch();
   }
   return cudaGetLastError();
 }
 
-cudaError_t launch_inner_start(int d, const double* part, double* sv, double* dinv, float* inv_s, double* sc,
-                               cudaStream_t s) {
-  k_inner_start<<<1, kBookThreads, 0, s>>>(d, part, kUpdBlocks, sv, dinv, inv_s, sc);
-  note_launch();
-  return cudaGetLastError();
-}
-
-cudaError_t launch_inner_col(int j, int d, const double* dd, const double* part, double* sv, double* dinv, float* inv_s,
-                             double* sc, cudaStream_t s) {
-  k_inner_col<<<1, kBookThreads, 0, s>>>(j, d, dd, part, kUpdBlocks, sv, dinv, inv_s, sc);
-  note_launch();
-  return cudaGetLastError();
-}
-
-cudaError_t launch_inner_lsq(int d, const double* sv, double* sc, double* coef, cudaStream_t s) {
-  k_inner_lsq<<<1, kMaxInner, 0, s>>>(d, sv, sc, coef);
+cudaError_t launch_inner_lsq(int d, const double* sv, const double* H, double* coef, cudaStream_t s) {
+  k_inner_lsq<<<1, kMaxInner, 0, s>>>(d, sv, H, coef);
   note_launch();
   return cudaGetLastError();
 }
 
 cudaError_t launch_combine_f32(int64_t n, int k, const float* Ub, int64_t ld, const double* coef, float* out,
                                cudaStream_t s) {
-  k_combine_f32<<<kRedBlocks, 256, (k > 0 ? k : 1) * sizeof(float), s>>>(n, k, Ub, ld, coef, out);
+  if ((n | ld) & 3) return cudaErrorInvalidValue;  // rows padded to float4
+  const unsigned nb = (unsigned)std::min<int64_t>(2 * kRedBlocks, std::max<int64_t>(1, (n / 4 + 255) / 256));
+  k_combine_f32<<<nb, 256, (k > 0 ? k : 1) * sizeof(float), s>>>(n / 4, k, (const float4*)Ub, ld / 4, coef, (float4*)out);
   note_launch();
   return cudaGetLastError();
 }

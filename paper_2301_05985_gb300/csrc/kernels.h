@@ -186,35 +186,38 @@ cudaError_t launch_reduce_parts(int nparts, int k, const double* part, double* o
 cudaError_t launch_reduce_cols(int nparts, int k, const double* part, double* out, cudaStream_t s);
 
 // ---------------------------------------------- inner FP32 GMRES (inner_krylov.cu)
+// All on FP32 vectors of n entries, n and ld multiples of 4, 16-byte aligned (rows padded
+// with zeros); ticket: a zeroed counter of the stream; part: inner_dot_blocks(n) doubles per
+// vector, at least kInnerBlocks.
 int inner_dot_blocks(int64_t n);
 int inner_max_depth();
-// d_i = U_i . w (FP32 vectors, i < k); part: [inner_dot_blocks(n)][k].  n and ld are
-// multiples of 4 and the vectors 16-byte aligned (rows padded with zeros)
-cudaError_t launch_multi_dot_f32(int64_t n, int k, const float* Ub, int64_t ld, const float* w, double* part, double* d,
-                                 cudaStream_t s);
-// w -= sum_i d_i dinv_i U_i (i < k, FP32) and the per-block partials of w . w in part
-// (summed by launch_inner_start / launch_inner_col); n, ld multiples of 4 as above
-cudaError_t launch_multi_axpy_norm_f32(int64_t n, int k, const float* Ub, int64_t ld, const double* d,
-                                       const double* dinv, float* w, double* part, cudaStream_t s);
-// y = Dinv32 (inv_s[0] u) per node (inv_s may be null: scale 1); y4: the same, padded
+// d_i = U_i . w (i < k)
+cudaError_t launch_multi_dot_f32(int64_t n, int k, const float* Ub, int64_t ld, const float* w, double* part,
+                                 unsigned* ticket, double* d, cudaStream_t s);
+// The Arnoldi bookkeeping stays on the device: norms s_i (sv), 1 / s_i^2 (dinv), 1 / s_i
+// (inv_s) and the Hessenberg matrix H [(d+1) x d].  start: s_0 = ||u0||; update: step j,
+// w -= sum_{i <= j} dd_i dinv_i U_i, s_(j+1) = ||w|| and column j of H; lsq: the least
+// squares, coef_i = y_i / s_i.
+cudaError_t launch_inner_start(int64_t n, int d, float* u0, double* part, unsigned* ticket, double* sv, double* dinv,
+                               float* inv_s, cudaStream_t s);
+cudaError_t launch_inner_update(int64_t n, int j, int d, const float* Ub, int64_t ld, const double* dd, float* w,
+                                double* part, unsigned* ticket, double* sv, double* dinv, float* inv_s, double* H,
+                                cudaStream_t s);
+inline size_t inner_scalar_doubles(int d) { return (size_t)(d + 1) * d; }
+cudaError_t launch_inner_lsq(int d, const double* sv, const double* H, double* coef, cudaStream_t s);
+// y = Dinv32 (inv_s[0] u) per node (inv_s may be null: scale 1); y4: the same, padded, and
+// zeros into clear [N] (the accumulator of the J V that follows)
 cudaError_t launch_block_apply32(int64_t N, const float* Dinv32, const float* u, const float* inv_s, float* y,
                                  cudaStream_t s);
 cudaError_t launch_block_apply32_pad(int64_t N, const float* Dinv32, const float* u, const float* inv_s, float4* y4,
-                                     cudaStream_t s);
+                                     float4* clear, cudaStream_t s);
 // out [N][3] <- acc4 with the Dirichlet rows set to V4 and the hanging rows to
 // V4_h - sum_p w_p V4_p (the J V row fix-ups of the padded FP32 path)
 cudaError_t launch_pack_jv4(const RowArgs& R, const float4* V4, const float4* acc4, float* out, cudaStream_t s);
 // y4[i] = (x[3i], x[3i+1], x[3i+2], 0)
 cudaError_t launch_pad4(int64_t N, const float* x, float4* y4, cudaStream_t s);
-// inner Arnoldi bookkeeping; sc holds the rotated Hessenberg, the rotations, g and the
-// number of columns before a breakdown: inner_scalar_doubles(d) doubles
-inline size_t inner_scalar_doubles(int d) { return (size_t)(d + 1) * d + 2 * (size_t)d + (size_t)(d + 1) + 1; }
-cudaError_t launch_inner_start(int d, const double* part, double* sv, double* dinv, float* inv_s, double* sc,
-                               cudaStream_t s);
-cudaError_t launch_inner_col(int j, int d, const double* dd, const double* part, double* sv, double* dinv, float* inv_s,
-                             double* sc, cudaStream_t s);
-cudaError_t launch_inner_lsq(int d, const double* sv, double* sc, double* coef, cudaStream_t s);
-// out = sum_i coef_i U_i (FP32); x += sum_i coef_i Z_i (FP32 vectors into FP64)
+// out = sum_i coef_i U_i (FP32, n and ld multiples of 4); x += sum_i coef_i Z_i (FP32 vectors
+// into FP64)
 cudaError_t launch_combine_f32(int64_t n, int k, const float* Ub, int64_t ld, const double* coef, float* out,
                                cudaStream_t s);
 cudaError_t launch_combine_f32_add_f64(int64_t n, int k, const float* Zb, int64_t ld, const double* coef, double* x,

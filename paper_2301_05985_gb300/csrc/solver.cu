@@ -255,10 +255,11 @@ int ctx_check_staged_waits(pnp_ctx* c) {
 // Dirichlet and hanging rows of J V.  Lane-group kernel only.
 // With from_state, the state's Gauss-point quantities come from the linearisation stored
 // by launch_lane_state for the current Krylov solve.
-static int ctx_jv32_pad(pnp_ctx* c, const float4* V4, float* out, bool from_state) {
-  // a memset: clearing the accumulator inside the pack, right after the vector atomics
-  // that filled it, measured several times slower on GB300
-  CK(cudaMemsetAsync(c->JV4, 0, sizeof(float4) * c->n_nodes, c->stream));
+// cleared: JV4 is zero already, from the block-Jacobi apply that made V4 (clearing it
+// inside the pack, right after the vector atomics that filled it, measured several times
+// slower than a memset on GB300).
+static int ctx_jv32_pad(pnp_ctx* c, const float4* V4, float* out, bool from_state, bool cleared = false) {
+  if (!cleared) CK(cudaMemsetAsync(c->JV4, 0, sizeof(float4) * c->n_nodes, c->stream));
   {
     ElemArgs<float> A = elem_args<float>(c, c->U32, nullptr, c->hs32, c->adv32, nullptr);
     A.rec = c->rec32;
@@ -327,26 +328,25 @@ static int inner_gmres32_body(pnp_ctx* c, bool from_state) {
   const int64_t n = c->n3(), N = c->n_nodes, ldq = c->ldq;
   cudaStream_t s = c->stream;
   float* Q = c->Qin;  // rows of ldq floats, the entries past n stay zero
-  double* sc = c->isc;                           // rotated Hessenberg, rotations, g, count
-  double* sv = sc + inner_scalar_doubles(d);     // [d+1] norms s_i of the basis vectors
+  double* H = c->isc;                            // Hessenberg matrix
+  double* sv = H + inner_scalar_doubles(d);      // [d+1] norms s_i of the basis vectors
   double* dinv = sv + (d + 2);                   // [d+1] 1 / s_i^2
   double* dd = dinv + (d + 2);                   // [d+1] projections
   double* coef = dd + (d + 2);                   // [d] combination coefficients
   float* inv_s = c->iinv;
   {
     ProfScope ps(c, PNP_PROF_INNER, 4.0 * n, 2.0 * n);
-    CK(launch_multi_axpy_norm_f32(ldq, 0, Q, ldq, dd, dinv, Q, c->part, s));
+    CK(launch_inner_start(ldq, d, Q, c->part, c->ticket, sv, dinv, inv_s, s));
   }
-  CK(launch_inner_start(d, c->part, sv, dinv, inv_s, sc, s));
   const bool pad = !c->use_patches && element_kernel_is_lanes();
   for (int j = 0; j < d; ++j) {
     float* w = Q + (size_t)(j + 1) * ldq;
     if (pad) {
       {
         ProfScope ps(c, PNP_PROF_PRECOND, 60.0 * N, 18.0 * N);
-        CK(launch_block_apply32_pad(N, c->Dinv32, Q + (size_t)j * ldq, inv_s + j, c->V4, s));
+        CK(launch_block_apply32_pad(N, c->Dinv32, Q + (size_t)j * ldq, inv_s + j, c->V4, c->JV4, s));
       }
-      RC(ctx_jv32_pad(c, c->V4, w, from_state));
+      RC(ctx_jv32_pad(c, c->V4, w, from_state, true));
     } else {
       {
         ProfScope ps(c, PNP_PROF_PRECOND, 60.0 * N, 18.0 * N);
@@ -357,13 +357,12 @@ static int inner_gmres32_body(pnp_ctx* c, bool from_state) {
     {
       const double nj = (double)n * (j + 1);
       ProfScope ps(c, PNP_PROF_INNER, 4.0 * (nj + n) + 4.0 * (nj + 2.0 * n), 4.0 * nj + 2.0 * n);
-      CK(launch_multi_dot_f32(ldq, j + 1, Q, ldq, w, c->part, dd, s));
-      CK(launch_multi_axpy_norm_f32(ldq, j + 1, Q, ldq, dd, dinv, w, c->part, s));
+      CK(launch_multi_dot_f32(ldq, j + 1, Q, ldq, w, c->part, c->ticket, dd, s));
+      CK(launch_inner_update(ldq, j, d, Q, ldq, dd, w, c->part, c->ticket, sv, dinv, inv_s, H, s));
     }
-    CK(launch_inner_col(j, d, dd, c->part, sv, dinv, inv_s, sc, s));
   }
-  CK(launch_inner_lsq(d, sv, sc, coef, s));
-  CK(launch_combine_f32(n, d, Q, ldq, coef, c->JV32, s));
+  CK(launch_inner_lsq(d, sv, H, coef, s));
+  CK(launch_combine_f32(ldq, d, Q, ldq, coef, c->JV32, s));
   return PNP_OK;
 }
 
