@@ -465,7 +465,7 @@ def kernel_table(prof, peaks, total_ms, N, E):
 def load_traffic(workload, coupled=True):
     """Per-class DRAM traffic from the committed ncu summary, for kernels whose source is
     unchanged since the capture and whose variant the step runs (the coupled step's PNP
-    solve has an advection field: four stored rows per lane; the PNP step alone three)."""
+    solve has an advection field, the PNP step alone none)."""
     import hashlib
     try:
         tj = json.load(open(os.path.join(ROOT, "profiles", "traffic.json")))

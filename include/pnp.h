@@ -304,17 +304,14 @@ int pnp_residual(pnp_ctx* c, const double* U, double* F);
 int pnp_jv(pnp_ctx* c, const double* U, const void* V, void* JV, int precision);
 /* FP32 J V through a stored linearisation, for many directions at one state (the
  * inner Krylov solve of the flexible GMRES uses the same kernels).  pnp_linearize
- * evaluates at U (device FP64 [n][3]), with the context's history, advection, parameters
- * and boundary conditions at this call, the state's quantities at every element's
- * Gauss points that J V needs (Def. 3 linearised: v, grad phi, grad c+-, tau_c and
- * z (c - tau_c R) per Gauss point, FP32, 64 B each, held by the context; 48 B when the
- * advection field is zero: v and tau_c are then not stored, tau_c follows from the level).
+ * takes down the state J V depends on, in FP32: 32 bytes per node (U (device FP64
+ * [n][3]), history and advection at this call, held by the context) and the
+ * parameters; whether the advection field is zero is decided here.
  * pnp_jv_linearized then returns JV = J V for FP32 device vectors V, JV [n][3], equal to
  * pnp_jv(..., PNP_F32) at that U up to FP32 summation order.  A later solver call
  * (pnp_gmres, pnp_newton_solve, pnp_time_step) replaces the stored linearisation;
  * pnp_jv_linearized then returns PNP_ERR_STATE until pnp_linearize is called again.
- * The J V kernel streams the stored quantities through shared memory with bulk copies;
- * if one of its bounded waits on them gives up, the block waits (with a longer bound) for
+ * The J V kernel streams its mesh tables through shared memory with bulk copies; if one of its bounded waits on them gives up, the block waits (with a longer bound) for
  * the copies it issued, exits, and the call raises PNP_ERR_DEVICE_FLAG (here, and from the
  * solver calls that use it).  The flag stays set until the next linearisation (a
  * pnp_linearize, or the start of the next flexible Krylov solve). */

@@ -249,7 +249,7 @@ static void free_ctx_memory(pnp_ctx* c) {
   void* ptrs[] = {c->d_conn, c->d_anchor, c->d_level, c->d_faces, c->d_hnode, c->d_hpar, c->d_hnp, c->U, c->Uk, c->Ukm1,
                   c->adv, c->vel, c->vel_prev, c->hs, c->U32, c->adv32, c->hs32, c->V32, c->JV32, c->F,
                   c->dU, c->Ut, c->Ft, c->rhs, c->Dinv, c->D32, c->basis, c->w, c->z, c->r, c->part, c->dsc,
-                  c->dflag, c->ticket, c->Zb, c->Qin, c->Dinv32, c->isc, c->iinv, c->rec32, c->V4, c->JV4, c->qp32,
+                  c->dflag, c->ticket, c->Zb, c->Qin, c->Dinv32, c->isc, c->iinv, c->rec32, c->rec_lin, c->d_tiles,
                   c->Z64, c->Qin64, c->zin64, c->isc64};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -258,6 +258,7 @@ static void free_ctx_memory(pnp_ctx* c) {
   if (c->part64) cudaFree(c->part64);
   if (c->part32) cudaFree(c->part32);
   if (c->hpin) cudaFreeHost(c->hpin);
+  if (c->hflag) cudaFreeHost(c->hflag);
 }
 
 int pnp_ctx_create(const pnp_mesh* m, const pnp_params* p, void* stream, pnp_ctx** out) {
@@ -321,9 +322,17 @@ int pnp_ctx_create(const pnp_mesh* m, const pnp_params* p, void* stream, pnp_ctx
   ALLOC(c->w, v3);
   ALLOC(c->z, v3);
   ALLOC(c->r, v3);
-  ALLOC(c->dflag, sizeof(int) * 4);
+  ALLOC(c->dflag, sizeof(int) * 8);
   ALLOC(c->ticket, sizeof(unsigned));
 #undef ALLOC
+  if (cudaMallocHost((void**)&c->hflag, sizeof(int) * 2) != cudaSuccess) {
+    cudaGetLastError();
+    c->hflag = nullptr;
+    pnp_set_error("pnp_ctx_create: out of pinned memory");
+    return fail(PNP_ERR_NOMEM);
+  }
+  c->hflag[0] = c->hflag[1] = 0;
+  c->wait_flag = c->hflag;
   std::vector<uint8_t> faces(m->node_faces);
   for (int64_t i = 0; i < N; ++i)
     if (m->node_hang[i] >= 0) faces[i] |= 0x80;
@@ -332,7 +341,7 @@ int pnp_ctx_create(const pnp_mesh* m, const pnp_params* p, void* stream, pnp_ctx
   auto up = [&](void* dst, const void* src, size_t bytes) {
     if (bytes && e == cudaSuccess) e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, s);
   };
-  if (e == cudaSuccess) e = cudaMemsetAsync(c->dflag, 0, sizeof(int) * 4, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(c->dflag, 0, sizeof(int) * 8, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->ticket, 0, sizeof(unsigned), s);
   up(c->d_conn, m->el_conn.data(), sizeof(int32_t) * m->el_conn.size());
   up(c->d_level, m->el_level.data(), m->el_level.size());
@@ -436,12 +445,11 @@ int ctx_alloc_inner(pnp_ctx* c, int m, int d) {
   m = std::max(m, c->inner_m);
   d = std::max(d, c->inner_d);
   if (int rc = ctx_alloc_krylov(c, std::max(c->m_alloc, d))) return rc;  // partials for d projections
-  void* old[] = {c->Zb, c->Qin, c->Dinv32, c->isc, c->iinv, c->V4, c->JV4, c->qp32};
+  void* old[] = {c->Zb, c->Qin, c->Dinv32, c->isc, c->iinv};
   for (void* q : old)
     if (q) cudaFree(q);
   c->Zb = c->Qin = c->Dinv32 = c->iinv = nullptr;
   c->isc = nullptr;
-  c->V4 = c->JV4 = c->qp32 = nullptr;
   c->inner_m = c->inner_d = 0;
   const size_t n = (size_t)c->n3();
   cudaError_t e = cudaMalloc((void**)&c->Zb, sizeof(float) * (size_t)m * n);
@@ -451,10 +459,6 @@ int ctx_alloc_inner(pnp_ctx* c, int m, int d) {
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->Dinv32, sizeof(float) * 9 * (size_t)c->n_nodes);
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->isc, sizeof(double) * (inner_scalar_doubles(d) + 5 * (size_t)(d + 2)));
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->iinv, sizeof(float) * (size_t)(d + 2));
-  if (e == cudaSuccess) e = cudaMalloc((void**)&c->V4, sizeof(float4) * (size_t)c->n_nodes);
-  if (e == cudaSuccess) e = cudaMalloc((void**)&c->JV4, sizeof(float4) * (size_t)c->n_nodes);
-  if (e == cudaSuccess) e = cudaMemset(c->JV4, 0, sizeof(float4) * (size_t)c->n_nodes);
-  // the stored linearisation (qp32) is allocated by its first use (ctx_linearize32)
   if (e != cudaSuccess) {
     pnp_set_error("inner Krylov scratch allocation failed: %s", cudaGetErrorString(e));
     return e == cudaErrorMemoryAllocation ? PNP_ERR_NOMEM : PNP_ERR_CUDA;
@@ -622,8 +626,7 @@ int pnp_make_consistent(pnp_ctx* c) {
 int pnp_residual(pnp_ctx* c, const double* U, double* F) {
   CTX_GUARD(c);
   if (!U || !F) PNP_FAIL(PNP_ERR_ARG, "pnp_residual: null pointer");
-  if (int rc = ctx_prepare_history(c)) return rc;
-  if (int rc = ctx_residual(c, U, F)) return rc;
+  if (int rc = ctx_history_residual(c, U, F)) return rc;
   CK(cudaStreamSynchronize(c->stream));
   return PNP_OK;
 }
@@ -635,8 +638,22 @@ int pnp_jv(pnp_ctx* c, const double* U, const void* V, void* JV, int precision) 
   if (precision == PNP_F64) {
     if (int rc = ctx_jv64(c, U, (const double*)V, (double*)JV)) return rc;
   } else if (precision == PNP_F32) {
-    if (int rc = ctx_prepare_f32(c, U)) return rc;
-    if (int rc = ctx_jv32(c, (const float*)V, (float*)JV)) return rc;
+    if (int rc = ctx_prepare_f32(c, U, false)) return rc;
+    // this call's own wait limit (the default) and flag
+    const int polls = c->wait_polls;
+    int* flag = c->wait_flag;
+    c->wait_polls = -1;
+    c->wait_flag = c->hflag + 1;
+    const int rc = ctx_jv32(c, (const float*)V, (float*)JV);
+    c->wait_polls = polls;
+    c->wait_flag = flag;
+    if (rc) return rc;
+    CK(cudaStreamSynchronize(c->stream));
+    if (c->hflag[1]) {
+      c->hflag[1] = 0;
+      PNP_FAIL(PNP_ERR_DEVICE_FLAG, "J V: a staged copy of the mesh tables did not complete");
+    }
+    return PNP_OK;
   } else {
     PNP_FAIL(PNP_ERR_ARG, "pnp_jv: bad precision %d", precision);
   }
@@ -647,10 +664,8 @@ int pnp_jv(pnp_ctx* c, const double* U, const void* V, void* JV, int precision) 
 int pnp_linearize(pnp_ctx* c, const double* U) {
   CTX_GUARD(c);
   if (!U) PNP_FAIL(PNP_ERR_ARG, "pnp_linearize: null pointer");
-  if (int rc = ctx_alloc_inner(c, c->prm.gmres_restart, std::max(1, c->prm.gmres_inner))) return rc;
   if (int rc = ctx_prepare_history(c)) return rc;
-  if (int rc = ctx_prepare_f32(c, U)) return rc;
-  if (int rc = ctx_linearize32(c)) return rc;
+  if (int rc = ctx_linearize(c, U)) return rc;
   c->lin_user = true;
   CK(cudaStreamSynchronize(c->stream));
   return PNP_OK;
@@ -677,7 +692,7 @@ int pnp_block_diag_f32(pnp_ctx* c, const double* U, float* D) {
   CTX_GUARD(c);
   if (!U || !D) PNP_FAIL(PNP_ERR_ARG, "pnp_block_diag_f32: null pointer");
   if (int rc = ctx_prepare_history(c)) return rc;
-  if (int rc = ctx_prepare_f32(c, U)) return rc;
+  if (int rc = ctx_prepare_f32(c, U, false)) return rc;
   if (int rc = ctx_block_diag32(c, D)) return rc;
   CK(cudaStreamSynchronize(c->stream));
   return PNP_OK;

@@ -39,6 +39,8 @@ struct pnp_ctx {
   int32_t* d_hnode = nullptr;
   int32_t* d_hpar = nullptr;
   uint8_t* d_hnp = nullptr;
+  TileTab tab;              // node tables of the FP32 J V's tiles (first use: solver.cu)
+  uint8_t* d_tiles = nullptr;
 
   // Morton patches for the shared-memory element kernels (device), their partial buffers
   bool use_patches = true;
@@ -65,6 +67,10 @@ struct pnp_ctx {
   double* dsc = nullptr;   // small device scalars [2*(m+2) + 8]
   double* hpin = nullptr;  // pinned host mirror of dsc
   int* dflag = nullptr;
+  // pinned, set by a tile J V whose bounded wait gave up: [0] of solves and the stored
+  // linearisation, [1] of pnp_jv.  wait_flag: [0], or on a multigrid level the owner's [0]
+  int* hflag = nullptr;
+  int* wait_flag = nullptr;
   unsigned* ticket = nullptr;  // counter of the reductions' last block (this stream's launches)
   int m_alloc = 0;
   cudaEvent_t step_done[2] = {nullptr, nullptr};  // GMRES iterations queued ahead of the host
@@ -83,12 +89,12 @@ struct pnp_ctx {
   double* isc64 = nullptr;  // [3 (d+2) + 2] inner projections, 1 / s_i^2, norm, combination
   int inner64_m = 0, inner64_d = 0;
   float4* rec32 = nullptr;  // [N][2] FP32 node records of the state for the FP32 J V
-  float4* V4 = nullptr;     // [N] padded FP32 direction of the inner solve's J V
-  float4* JV4 = nullptr;    // [N] padded FP32 J V accumulator
-  float4* qp32 = nullptr;   // [4][2^dim E] stored Gauss-point linearisation of the FP32 J V
-  bool lin_user = false;    // qp32 holds the linearisation of the last pnp_linearize
-  int lin_rows = 4;         // float4 rows per lane in qp32 (3 without advection)
-  bool adv_zero = false;    // the advection field was zero at the last ctx_prepare_f32
+  // the linearisation of pnp_linearize: node records as rec32, and its parameters
+  float4* rec_lin = nullptr;
+  PhysParams lin_phys{};
+  bool lin_adv = true;      // its advection field was not zero
+  bool lin_user = false;    // rec_lin holds the linearisation of the last pnp_linearize
+  bool adv_zero = false;    // the advection field was found zero at the last ctx_prepare_f32
   int wait_polls = -1;      // poll limit of the staged J V's waits (< 0: the kernel's default)
   // the inner FP32 GMRES captured as a CUDA graph (replayed while profiling is off): the
   // launches depend only on the key below, captured on a stream of the context's own
@@ -157,6 +163,13 @@ struct pnp_ctx {
     R.bc = bc_table();
     return R;
   }
+  TileMesh tile_mesh() const {
+    TileMesh M;
+    M.tab = tab;
+    const BcTable t = bc_table();
+    M.dir = (uint32_t)t.dir_faces[0] | (uint32_t)t.dir_faces[1] << 8 | (uint32_t)t.dir_faces[2] << 16;
+    return M;
+  }
   BcTable bc_table() const {
     BcTable t{};
     for (int f = 0; f < 3; ++f) {
@@ -206,10 +219,13 @@ struct ProfScope {
 int ctx_check(pnp_ctx* c, cudaError_t e, const char* what);
 int ctx_prepare_history(pnp_ctx* c);
 int ctx_residual(pnp_ctx* c, const double* U, double* F);
-// cleared: JV is zero already (the block-Jacobi apply before it cleared it)
-int ctx_jv64(pnp_ctx* c, const double* U, const double* V, double* JV, bool cleared = false);
-int ctx_prepare_f32(pnp_ctx* c, const double* U);
-int ctx_jv32(pnp_ctx* c, const float* V32, float* JV32, bool cleared = false);
+// the history (ctx_prepare_history) and the residual
+int ctx_history_residual(pnp_ctx* c, const double* U, double* F);
+// rows_done: the rows of JV are initialised (the block-Jacobi apply before it did)
+int ctx_jv64(pnp_ctx* c, const double* U, const double* V, double* JV, bool rows_done = false);
+// check_adv: also finds out whether the advection field is zero (one norm and a wait)
+int ctx_prepare_f32(pnp_ctx* c, const double* U, bool check_adv);
+int ctx_jv32(pnp_ctx* c, const float* V32, float* JV32);
 // PNP_ERR_DEVICE_FLAG once a wait of the staged J V has given up (the flag is latched)
 int ctx_check_staged_waits(pnp_ctx* c);
 int ctx_block_diag(pnp_ctx* c, const double* U, double* D);
@@ -222,7 +238,7 @@ int ctx_gmres(pnp_ctx* c, const double* U, const double* b, double* x, double rt
 int ctx_newton(pnp_ctx* c, pnp_solve_stats* st, const double* ref_state = nullptr);
 int ctx_alloc_inner(pnp_ctx* c, int m, int d);
 int ctx_alloc_inner64(pnp_ctx* c, int m, int d);
-int ctx_linearize32(pnp_ctx* c);
+int ctx_linearize(pnp_ctx* c, const double* U);
 int ctx_jv32_linearized(pnp_ctx* c, const float* V, float* JV);
 int ctx_time_step(pnp_ctx* c, pnp_solve_stats* st);
 int ctx_alloc_krylov(pnp_ctx* c, int m);

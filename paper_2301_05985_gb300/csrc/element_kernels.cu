@@ -420,7 +420,7 @@ inline int nblk(int64_t n, int t) { return (int)((n + t - 1) / t); }
 }  // namespace
 
 // ------------------------------------------------------------------ launchers
-// Element kernel of launch_element: one lane group per element unless
+// Element kernels: one lane group per element, or node tiles, unless
 // PNP_ELEMENT_KERNEL=thread selects one thread per element (modal sum factorisation).
 static bool per_thread_elements() {
   static const bool v = [] {
@@ -464,12 +464,10 @@ double element_kernel_flops(int D, bool jv) {
   return NC * (state + 2 * vg + g + 2 * (1 + 2 * D + 4 * D - 1 + 2 + 3 + 3 + 1 + 6 * D + 1) + tests);
 }
 
+// one thread per element (modal sum factorisation); PNP_ELEMENT_KERNEL=thread selects it
 template <typename T>
 cudaError_t launch_element(int dim, bool jv, const ElemArgs<T>& A, cudaStream_t s) {
   if (A.n_elem == 0) return cudaSuccess;
-  // default: one lane group per element; PNP_ELEMENT_KERNEL=thread selects one thread
-  // per element (modal sum factorisation in registers)
-  if (!per_thread_elements()) return launch_element_lanes<T>(dim, jv, A, s);
   const int t = 128;
   if (dim == 2) {
     if (jv) { k_element<T, 2, true><<<nblk(A.n_elem, t), t, 0, s>>>(A); note_launch(); }

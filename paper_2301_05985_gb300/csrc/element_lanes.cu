@@ -1,38 +1,16 @@
-// element_lanes.cu -- the VMS PNP residual and its Jacobian action with one lane group
-// per element: 2^d lanes of a warp share an element, lane c holds corner c and the
-// Gauss point next to it.
-//
-// Physics per Gauss point as in Def. 3 of arXiv 2301.05985 with the fine scales
-// c^f = -tau_c R_c (Sec. 3.1; the same statement as element_kernels.cu).  Interpolation
-// and the test side are the butterflies of lane_ops.cuh (a partner value per axis by lane
-// shuffle); the residual and J V use their scaled reflected form, the stored linearisation
-// and the block diagonal the plain one.  The FP32 kernels execute no FP64 instruction
-// (GB300 runs FP64 at 1/64 of the FP32 rate): powers of two come from the exponent bits
-// and the parameters arrive converted.
-#include <algorithm>
+// element_lanes.cu -- element kernels of the VMS PNP block with one lane group per element
+// (2^d lanes of a warp share an element, lane c holds corner c and the Gauss point next to
+// it) that gather and scatter lane by lane: the residual and the J V of FP64 vectors
+// (pnp_lane.cuh) and the block diagonal of the Jacobian.  The FP32 J V runs on node tiles
+// (element_tiles.cu).  The FP32 kernels execute no FP64
+// instruction (GB300 runs FP64 at 1/64 of the FP32 rate): powers of two come from the
+// exponent bits and the parameters arrive converted.
 #include <cstdint>
 #include <type_traits>
 
-#include "df32.cuh"
-#include "kernels.h"
-#include "lane_ops.cuh"
+#include "pnp_lane.cuh"
 
 namespace {
-
-// blocks per SM the lane kernel's register cap is set for
-template <typename T, typename C>
-constexpr int lane_min_blocks() {
-  return sizeof(T) == 4 ? 5 : (std::is_same<C, df>::value ? 4 : 3);
-}
-
-// physical parameters in the kernel's arithmetic type
-template <typename T>
-struct LaneParams {
-  T kappa;   // beta0 / dt
-  T tau_t;   // 4 / dt^2
-  T cid;     // C_I d
-  T e2;      // 2 Lambda^2
-};
 
 // nodal values of NF interleaved fields at node id (hanging: the parents' mean)
 template <typename T, int NF>
@@ -52,28 +30,6 @@ __device__ __forceinline__ void load_node(const ElemArgs<T>& A, int32_t id, bool
       const int32_t pid = A.hang_par[4 * h + p];
 #pragma unroll
       for (int f = 0; f < NF; ++f) dst[f] += wgt * __ldg(src + (int64_t)stride * pid + f);
-    }
-  }
-}
-
-// the same in arithmetic type C from storage type T
-template <typename T, typename C, int NF>
-__device__ __forceinline__ void load_node_c(const ElemArgs<T>& A, int32_t id, bool valid, const T* __restrict__ src,
-                                            int stride, C (&dst)[NF]) {
-#pragma unroll
-  for (int f = 0; f < NF; ++f) dst[f] = C(0);
-  if (!valid) return;
-  if (id >= 0) {
-#pragma unroll
-    for (int f = 0; f < NF; ++f) dst[f] = to_compute<C>(__ldg(src + (int64_t)stride * id + f));
-  } else {
-    const int32_t h = -id - 1;
-    const int np = A.hang_np[h];
-    const C wgt = np == 2 ? C(0.5) : C(0.25);
-    for (int p = 0; p < np; ++p) {
-      const int32_t pid = A.hang_par[4 * h + p];
-#pragma unroll
-      for (int f = 0; f < NF; ++f) dst[f] += wgt * to_compute<C>(__ldg(src + (int64_t)stride * pid + f));
     }
   }
 }
@@ -139,50 +95,29 @@ __device__ __forceinline__ void lane_state(const T (&un)[3], const T (&vn)[3], c
   }
 }
 
-// the padded FP32 direction at node id (hanging: the parents' mean)
-template <typename T>
-__device__ __forceinline__ void load_dir4(const ElemArgs<T>& A, int32_t id, bool valid, float (&dn)[3]) {
-  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (valid) {
-    if (id >= 0) {
-      v = __ldg(A.V4 + id);
-    } else {
-      const int32_t h = -id - 1;
-      const int np = A.hang_np[h];
-      const float wgt = np == 2 ? 0.5f : 0.25f;
-      for (int p = 0; p < np; ++p) {
-        const float4 a = __ldg(A.V4 + A.hang_par[4 * h + p]);
-        v.x += wgt * a.x; v.y += wgt * a.y; v.z += wgt * a.z;
-      }
-    }
-  }
-  dn[0] = v.x; dn[1] = v.y; dn[2] = v.z;
+// loaded nodal values in the arithmetic type C
+template <typename C, int NF>
+__device__ __forceinline__ void load_node_c(const ElemArgs<double>& A, int32_t id, bool valid,
+                                            const double* __restrict__ src, int stride, C (&dst)[NF]) {
+  double x[NF];
+  load_node<double, NF>(A, id, valid, src, stride, x);
+#pragma unroll
+  for (int f = 0; f < NF; ++f) dst[f] = to_compute<C>(x[f]);
 }
 
-// one vector atomic per target node (hanging: weighted to its parents)
-template <typename T>
-__device__ __forceinline__ void scatter4(const ElemArgs<T>& A, int32_t id, const float (&r)[3]) {
-  if (id >= 0) {
-    atomicAdd(A.out4 + id, make_float4(r[0], r[1], r[2], 0.f));
-  } else {
-    const int32_t h = -id - 1;
-    const int np = A.hang_np[h];
-    const float wgt = np == 2 ? 0.5f : 0.25f;
-    for (int p = 0; p < np; ++p)
-      atomicAdd(A.out4 + A.hang_par[4 * h + p], make_float4(wgt * r[0], wgt * r[1], wgt * r[2], 0.f));
-  }
-}
-
-// T: storage type of the vectors; C: arithmetic type (T, or double-float for FP64 data).
+// The operators on FP64 vectors, arithmetic C (double, or double-float).  They add to the
+// weak-form rows only (Dirichlet and hanging rows were written by the row initialisation).
 // What bounds it, on the membrane-band octree (971,776 elements) with advection:
 //   double-float residual: the FP32 pipe (480 M warp instructions, packed ones twice as
 //   long); 1.47 ms before, 0.595 ms now.  Before: accurate double-float operations only
 //   (FMA pipe 57 %), 41 conversions and FP64 additions per lane (FP64 pipe 45 %), 59 KB of
-//   straight code per warp.
+//   straight code per warp.  (On node tiles as the FP32 J V: 0.591 ms, no gain: the barriers
+//   between its phases cost what the fewer loads and atomics save.)
 //   FP64 J V: the FP64 pipe (86 %); on the uniform level-6 cube 1.03 ms before, 0.76 ms now,
 //   by the operation count (318 to 230 FP64 instructions per lane).
-template <typename T, typename C, int D, bool JV>
-__global__ void __launch_bounds__(256, lane_min_blocks<T, C>()) k_element_lanes(ElemArgs<T> A, LaneParams<C> K) {
+template <typename C, int D, bool JV>
+__global__ void __launch_bounds__(256, sizeof(C) == 8 && !std::is_same<C, double>::value ? 4 : 3)
+    k_element_lanes(ElemArgs<double> A, LaneParams<C> K) {
   constexpr int NC = 1 << D;
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   // warps whose first element is past the end leave together (shuffles need the warp)
@@ -192,400 +127,35 @@ __global__ void __launch_bounds__(256, lane_min_blocks<T, C>()) k_element_lanes(
   const bool valid = e < A.n_elem;
   const int32_t id = valid ? __ldg(A.conn + e * NC + c) : 0;
   const int lev = valid ? A.level[e] : 0;
-
-  // scaled quantities (lane_ops.cuh; c~ = c / a^D, g~ = reflected gradient h / a^(D-1)):
-  //   V = (a^(D-1) / h) v~ reflected,  beta = a^(D-2) / h^2,  delta = a^2 h^2,  alpha = a^D
-  //   S~ = kappa c~ + h~ + V . g~c,   R~ = S~ - z beta g~phi . g~c          (times alpha)
-  //   Phi~ = g~c + z alpha (c~ - tau R~) g~phi + tau delta R~ V             (times a^(D-1) / h)
-  // and the element vector is (h/2)^D a^D beta times the test transpose of (delta S~, Phi~)
-  const C rho = C(kRho);
-  const C beta = const_pow2(ipow(kVal, D - 2), 2 * lev, C(0));
-  const C delta = const_pow2(kVal * kVal, -2 * lev, C(0));
-  constexpr double cW = ipow(kVal, 2 * D - 2);
-  const int eW = 2 * lev - D * (lev + 1);
-  const C kappa = K.kappa, e2 = K.e2;
-
-  C un[3], vn[3], hn[2];
-  if constexpr (sizeof(T) == 4) {
-    if (A.rec) {
-      load_record(A, id, valid, un, hn, vn);
-    } else {
-      load_node_c<T, C, 3>(A, id, valid, A.U, 3, un);
-      load_node_c<T, C, 3>(A, id, valid, A.adv, 3, vn);
-      load_node_c<T, C, 2>(A, id, valid, A.hs, 2, hn);
-    }
-  } else {
-    load_node_c<T, C, 3>(A, id, valid, A.U, 3, un);
-    load_node_c<T, C, 3>(A, id, valid, A.adv, 3, vn);
-    load_node_c<T, C, 2>(A, id, valid, A.hs, 2, hn);
-  }
-
-  // state at this lane's Gauss point; the species, (v_0, v_1) and (phi, v_2) or (phi, dphi)
-  // run as pairs
-  using C2 = pair_t<C>;
-  const C2 rho2 = both<C>(rho);
-  C V[D], vd[D], gp[3], dgp[3];
-  {
-    const C2 v01 = lane_v<C2, D>(pair(vn[0], vn[1]), rho2);
-    vd[0] = first(v01);
-    vd[1] = second(v01);
-  }
-  C dn[3] = {C(0), C(0), C(0)};
-  if constexpr (JV) {
-    if constexpr (sizeof(T) == 4) {
-      if (A.V4) load_dir4(A, id, valid, dn);
-      else load_node_c<T, C, 3>(A, id, valid, A.V, 3, dn);
-    } else {
-      load_node_c<T, C, 3>(A, id, valid, A.V, 3, dn);
-    }
-    if constexpr (D == 3) vd[2] = lane_v<C, D>(vn[2], rho);
-  }
-  if constexpr (JV || D == 3) {
-    C2 val, g[3];
-    lane_vg<C2, D, !JV>(pair(un[2], JV ? dn[2] : vn[2]), rho2, val, g);
-#pragma unroll
-    for (int k = 0; k < D; ++k) {
-      gp[k] = first(g[k]);
-      if (JV) dgp[k] = second(g[k]);
-    }
-    if constexpr (!JV) vd[2] = second(val);
-  } else {
-    C unused;
-    lane_vg<C, D, false>(un[2], rho, unused, gp);
-  }
-  C vv;
-#pragma unroll
-  for (int k = 0; k < D; ++k) {
-    vv = k == 0 ? vd[k] * vd[k] : fma_q(vd[k], vd[k], vv);
-    V[k] = reflect(times_const(vd[k], ipow(kVal, D - 1), lev), reflect_mask(c, k));
-  }
-  // 4/dt^2 + C_I d (2/h)^4 + (2/h)^2 |v|^2
-  const C tau = inv_sqrt(fma_q(const_pow2(ipow(kVal, 2 * D), 2 * lev + 2, C(0)), vv,
-                             times_pow2(K.cid, 4 * lev + 4) + K.tau_t));
-  const C2 taud = both<C>(tau * delta), tau2 = both<C>(tau);
-  const C2 zb = pair(-beta, beta), kap2 = both<C>(kappa);
-  constexpr double alpha = ipow(kVal, D);
-  C2 cv, gc[3];
-  lane_vg<C2, D, true>(pair(un[0], un[1]), rho2, cv, gc);
-  C2 sv = fma_q(kap2, cv, lane_v<C2, D>(pair(hn[0], hn[1]), rho2));
-  C2 gg = both<C>(gp[0]) * gc[0];
-#pragma unroll
-  for (int k = 1; k < D; ++k) gg = fma_q(both<C>(gp[k]), gc[k], gg);
-#pragma unroll
-  for (int k = 0; k < D; ++k) sv = fma_q(both<C>(V[k]), gc[k], sv);
-  const C2 R = fma_q(zb, gg, sv);
-  C2 S, Phi[3];
-  C Sp, Pp[3];
-  if constexpr (!JV) {
-    const C2 q = times_pm(cv - tau2 * R, alpha), p = taud * R;
-#pragma unroll
-    for (int k = 0; k < D; ++k) Phi[k] = fma_q(p, both<C>(V[k]), fma_q(q, both<C>(gp[k]), gc[k]));
-    S = times_const2(sv, kVal * kVal, -2 * lev);
-    Sp = times_const(fma_q(tau, first(R) - second(R), second(cv) - first(cv)), kVal * kVal, -2 * lev);
-#pragma unroll
-    for (int k = 0; k < D; ++k) Pp[k] = e2 * gp[k];
-  } else {
-    C2 dcv, dgc[3];
-    lane_vg<C2, D, true>(pair(dn[0], dn[1]), rho2, dcv, dgc);
-    C2 dsv = kap2 * dcv, dgg = both<C>(gp[0]) * dgc[0];
-#pragma unroll
-    for (int k = 1; k < D; ++k) dgg = fma_q(both<C>(gp[k]), dgc[k], dgg);
-#pragma unroll
-    for (int k = 0; k < D; ++k) {
-      dgg = fma_q(both<C>(dgp[k]), gc[k], dgg);
-      dsv = fma_q(both<C>(V[k]), dgc[k], dsv);
-    }
-    const C2 dR = fma_q(zb, dgg, dsv);
-    const C2 q1 = times_pm(cv - tau2 * R, alpha), q2 = times_pm(dcv - tau2 * dR, alpha), p = taud * dR;
-#pragma unroll
-    for (int k = 0; k < D; ++k)
-      Phi[k] = fma_q(p, both<C>(V[k]), fma_q(q2, both<C>(gp[k]), fma_q(q1, both<C>(dgp[k]), dgc[k])));
-    S = times_const2(dsv, kVal * kVal, -2 * lev);
-    Sp = times_const(fma_q(tau, first(dR) - second(dR), second(dcv) - first(dcv)), kVal * kVal, -2 * lev);
-#pragma unroll
-    for (int k = 0; k < D; ++k) Pp[k] = e2 * dgp[k];
-  }
-
-  const C2 rs = lane_test<C2, D>(S, Phi, rho2);
-  const T r[3] = {times_const(to_storage<T>(first(rs)), cW, eW), times_const(to_storage<T>(second(rs)), cW, eW),
-                  times_const(to_storage<T>(lane_test<C, D>(Sp, Pp, rho)), cW, eW)};
+  C un[3], vn[3], hn[2], dn[3];
+  load_node_c<C, 3>(A, id, valid, A.U, 3, un);
+  load_node_c<C, 3>(A, id, valid, A.adv, 3, vn);
+  load_node_c<C, 2>(A, id, valid, A.hs, 2, hn);
+  if constexpr (JV) load_node_c<C, 3>(A, id, valid, A.V, 3, dn);
+  pair_t<C> rs;
+  C rp;
+  lane_pnp<C, D, JV, true>(un, hn, vn, dn, c, lev, K, rs, rp);
   if (!valid) return;
-  if constexpr (sizeof(T) == 4) {
-    if (A.out4) {
-      scatter4(A, id, r);
-      return;
-    }
-  }
+  const double w = const_pow2(lane_weight_c(D), lane_weight_e(D, lev), 0.0);
+  const double r[3] = {w * to_storage<double>(first(rs)), w * to_storage<double>(second(rs)), w * to_storage<double>(rp)};
   if (id >= 0) {
+    const uint32_t fm = A.faces[id] & 0x3Fu;
 #pragma unroll
-    for (int f = 0; f < 3; ++f) atomicAdd(A.out + 3 * (int64_t)id + f, r[f]);
+    for (int f = 0; f < 3; ++f)
+      if (!(fm & (A.dir >> (8 * f)))) atomicAdd(A.out + 3 * (int64_t)id + f, r[f]);
   } else {
     const int32_t hh = -id - 1;
     const int np = A.hang_np[hh];
-    const T wgt = np == 2 ? T(0.5) : T(0.25);
+    const double wgt = np == 2 ? 0.5 : 0.25;
     for (int p = 0; p < np; ++p) {
       const int32_t pid = A.hang_par[4 * hh + p];
+      const uint32_t fm = A.faces[pid] & 0x3Fu;
 #pragma unroll
-      for (int f = 0; f < 3; ++f) atomicAdd(A.out + 3 * (int64_t)pid + f, wgt * r[f]);
+      for (int f = 0; f < 3; ++f)
+        if (!(fm & (A.dir >> (8 * f)))) atomicAdd(A.out + 3 * (int64_t)pid + f, wgt * r[f]);
     }
   }
 }
-
-// ---- FP32 J V from a stored linearisation ---------------------------------------
-// Inside one Krylov solve the state (U, h, v) is fixed, so the Gauss-point quantities J V
-// needs from it are computed once per solve and stored per lane, NR float4 in lane-major
-// order (qp[j * L + t], L = 2^d E).  With advection (NR = 4): (v0 v1 v2 gp0)
-// (gp1 gp2 gc+0 gc+1) (gc+2 gc-0 gc-1 gc-2) (tau, z+(c+ - tau R+), z-(c- - tau R-), level).
-// Without (the advection field is zero, NR = 3): (gp0 gp1 gp2 gc+0) (gc+1 gc+2 gc-0 gc-1)
-// (gc-2, z+(c+ - tau R+), z-(c- - tau R-), level), and tau = (4/dt^2 + C_I d (2/h)^4)^(-1/2)
-// is recomputed from the level (the same FP32 value: |v|^2 = 0).  The level is stored as
-// integer bits.  Each J V then reads 16 NR bytes per lane, coalesced, instead of gathering
-// and interpolating the state.
-constexpr int kLaneThreads = 256;
-
-template <int D, int NR>
-__global__ void __launch_bounds__(kLaneThreads, 5) k_lane_state(ElemArgs<float> A, LaneParams<float> K, float4* qp) {
-  constexpr int NC = 1 << D;
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if ((t & ~int64_t(31)) / NC >= A.n_elem) return;
-  const int64_t e = t / NC;
-  const int c = (int)(t & (NC - 1));
-  const bool valid = e < A.n_elem;
-  const int32_t id = valid ? __ldg(A.conn + e * NC + c) : 0;
-  const int lev = valid ? A.level[e] : 0;
-  const float inv_h = pow2i(lev, 0.0f);
-  const float nb = float(-0.5 * (1.0 - kG));
-  float sh[3];
-#pragma unroll
-  for (int k = 0; k < 3; ++k) sh[k] = ((c >> k) & 1) ? inv_h : -inv_h;
-  const float G2 = pow2i(2 * lev + 2, 0.0f);
-  const float tau0 = fmaf(K.cid * G2, G2, K.tau_t);
-  float un[3], vn[3], hn[2];
-  load_record(A, id, valid, un, hn, vn);
-  float cv[2], gc[2][3], gp[3], v[3], hq[2], tau, R[2], P[2][3];
-  lane_state<float, D>(un, vn, hn, nb, sh, K.kappa, tau0, G2, cv, gc, gp, v, hq, tau, R, P);
-  if (!valid) return;
-  const int64_t L = A.n_elem * NC;
-  const float zc0 = cv[0] - tau * R[0], zc1 = -(cv[1] - tau * R[1]);
-  if constexpr (NR == 4) {
-    qp[t] = make_float4(v[0], v[1], v[2], gp[0]);
-    qp[L + t] = make_float4(gp[1], gp[2], gc[0][0], gc[0][1]);
-    qp[2 * L + t] = make_float4(gc[0][2], gc[1][0], gc[1][1], gc[1][2]);
-    qp[3 * L + t] = make_float4(tau, zc0, zc1, __int_as_float(lev));
-  } else {
-    qp[t] = make_float4(gp[0], gp[1], gp[2], gc[0][0]);
-    qp[L + t] = make_float4(gc[0][1], gc[0][2], gc[1][0], gc[1][1]);
-    qp[2 * L + t] = make_float4(gc[1][2], zc0, zc1, __int_as_float(lev));
-  }
-}
-
-// The J V kernel streams the stored state through shared memory: a persistent grid
-// walks tiles of kLaneThreads lanes, and per tile one thread issues bulk copies (TMA,
-// cp.async.bulk) of the four state rows and the tile's connectivity into a stage of
-// shared memory, completing on the stage's mbarrier.  kStages tiles are in flight per
-// block, so the state's HBM stream does not wait on the per-lane arithmetic and
-// atomics of the tile before.  Two stages with five blocks per SM measured fastest: three
-// (four blocks per SM) and four (three) were 6% and 16% slower per launch.
-constexpr int kStages = 2;
-constexpr size_t jv_stage_bytes(int S, int NR) {
-  return (size_t)S * ((size_t)NR * kLaneThreads * 16 + kLaneThreads * 4 + 8);
-}
-// try_wait polls before a wait on a stage gives up (about a second by default; a launch
-// argument), and the longer limit of the drain that follows a give-up: the block waits
-// for the copies it issued before it exits
-constexpr int kWaitPolls = 1 << 22;
-constexpr int kDrainPolls = 1 << 24;
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
-// bounded wait for the phase of the given parity to complete; false when it did not
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int polls = kWaitPolls) {
-  const uint32_t a = smem_u32(bar);
-  for (int i = 0; i < polls; ++i) {
-    uint32_t done;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-        : "=r"(done)
-        : "r"(a), "r"(parity)
-        : "memory");
-    if (done) return true;
-  }
-  return false;
-}
-// global -> shared bulk copy of `bytes` (multiple of 16, both addresses 16-byte aligned)
-__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                   smem_u32(dst)),
-               "l"(src), "r"(bytes), "r"(smem_u32(bar))
-               : "memory");
-}
-
-template <int D, int NS, int NR>
-__global__ void __launch_bounds__(kLaneThreads, 5) k_jv_from_state(ElemArgs<float> A, LaneParams<float> K,
-                                                                 const float4* __restrict__ qp, int* err,
-                                                                 int polls) {
-  constexpr int NC = 1 << D;
-  extern __shared__ __align__(128) uint8_t jv_smem[];
-  // NS stages of {NR state rows, connectivity} and NS mbarriers (jv_stage_bytes(NS, NR))
-  auto sq = reinterpret_cast<float4(*)[NR][kLaneThreads]>(jv_smem);
-  auto sconn = reinterpret_cast<int32_t(*)[kLaneThreads]>(jv_smem + NS * NR * kLaneThreads * sizeof(float4));
-  uint64_t* bar = reinterpret_cast<uint64_t*>(jv_smem + NS * (NR * kLaneThreads * sizeof(float4) + kLaneThreads * 4));
-  const int tid = threadIdx.x;
-  const int64_t L = A.n_elem * NC;
-  const int64_t n_tiles = (L + kLaneThreads - 1) / kLaneThreads;
-  const int64_t G = gridDim.x;
-  // thread 0: copy tile `tl` into stage `st` (sizes are multiples of 16 bytes: L and the
-  // tile start are multiples of 2^d lanes, 4 B of connectivity per lane)
-  auto issue = [&](int64_t tl, int st) {
-    const int64_t t0 = tl * kLaneThreads;
-    const uint32_t n = (uint32_t)(L - t0 < kLaneThreads ? L - t0 : kLaneThreads);
-    mbar_expect_tx(&bar[st], (uint32_t)NR * 16u * n + 4u * n);
-#pragma unroll
-    for (int j = 0; j < NR; ++j) bulk_g2s(&sq[st][j][0], qp + j * L + t0, 16u * n, &bar[st]);
-    bulk_g2s(&sconn[st][0], A.conn + t0, 4u * n, &bar[st]);
-  };
-  if (tid == 0) {
-#pragma unroll
-    for (int st = 0; st < NS; ++st) mbar_init(&bar[st], 1);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  __syncthreads();
-  uint32_t pending = 0;  // thread 0: stages with a copy in flight
-  if (tid == 0) {
-#pragma unroll
-    for (int st = 0; st < NS; ++st)
-      if (blockIdx.x + st * G < n_tiles) {
-        issue(blockIdx.x + st * G, st);
-        pending |= 1u << st;
-      }
-  }
-
-  const float nb = float(-0.5 * (1.0 - kG));
-  const float kappa = K.kappa, e2 = K.e2;
-  for (int k = 0;; ++k) {
-    const int64_t tl = blockIdx.x + (int64_t)k * G;
-    if (tl >= n_tiles) break;
-    const int st = k % NS;
-    const uint32_t parity = (uint32_t)(k / NS) & 1u;
-    const bool ok = mbar_wait(&bar[st], parity, polls);
-    if (__syncthreads_or(!ok)) {
-      // a copy did not complete: flag it, let the copies still in flight land, return
-      if (tid == 0) {
-        atomicOr(err, 1);
-        for (int j = 0; j < NS; ++j) {
-          const int kk = k + ((j - st + NS) % NS);
-          if (pending >> j & 1u) mbar_wait(&bar[j], (uint32_t)(kk / NS) & 1u, kDrainPolls);
-        }
-      }
-      return;
-    }
-    const int64_t t = tl * kLaneThreads + tid;
-    const bool valid = t < L;
-    float4 q0 = make_float4(0.f, 0.f, 0.f, 0.f), q1 = q0, q2 = q0, q3 = q0;
-    int32_t id = 0;
-    if (valid) {
-      q0 = sq[st][0][tid];
-      q1 = sq[st][1][tid];
-      q2 = sq[st][2][tid];
-      if constexpr (NR == 4) q3 = sq[st][NR - 1][tid];
-      id = sconn[st][tid];
-    }
-    __syncthreads();  // stage st is read: refill it with the tile NS ahead
-    if (tid == 0) {
-      pending &= ~(1u << st);
-      if (tl + NS * G < n_tiles) {
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        issue(tl + NS * G, st);
-        pending |= 1u << st;
-      }
-    }
-
-    const int c = (int)(t & (NC - 1));
-    float v[3], gp[3], gc[2][3], tau, zc_tR[2];
-    int lev;
-    if constexpr (NR == 4) {
-      lev = __float_as_int(q3.w);  // 0 for lanes past the end
-      v[0] = q0.x; v[1] = q0.y; v[2] = q0.z;
-      gp[0] = q0.w; gp[1] = q1.x; gp[2] = q1.y;
-      gc[0][0] = q1.z; gc[0][1] = q1.w; gc[0][2] = q2.x;
-      gc[1][0] = q2.y; gc[1][1] = q2.z; gc[1][2] = q2.w;
-      tau = q3.x;
-      zc_tR[0] = q3.y; zc_tR[1] = q3.z;
-    } else {
-      lev = __float_as_int(q2.w);
-      v[0] = v[1] = v[2] = 0.0f;
-      gp[0] = q0.x; gp[1] = q0.y; gp[2] = q0.z;
-      gc[0][0] = q0.w; gc[0][1] = q1.x; gc[0][2] = q1.y;
-      gc[1][0] = q1.z; gc[1][1] = q1.w; gc[1][2] = q2.x;
-      zc_tR[0] = q2.y; zc_tR[1] = q2.z;
-      const float G2 = pow2i(2 * lev + 2, 0.0f);
-      tau = rsqrtf(fmaf(K.cid * G2, G2, K.tau_t));
-    }
-    const float inv_h = pow2i(lev, 0.0f);
-    const float w = pow2i(-D * (lev + 1), 0.0f);
-    float sh[3];
-#pragma unroll
-    for (int kk = 0; kk < 3; ++kk) sh[kk] = ((c >> kk) & 1) ? inv_h : -inv_h;
-    float dn[3];
-    if (A.V4) load_dir4(A, id, valid, dn);
-    else load_node<float, 3>(A, id, valid, A.V, 3, dn);
-    float dcv[2], dgc[2][3], dgp[3], dR[2], S[3], Phi[3][3];
-#pragma unroll
-    for (int s = 0; s < 2; ++s) interp_vg<float, D>(dn[s], nb, sh, dcv[s], dgc[s]);
-    interp_g<float, D>(dn[2], nb, sh, dgp);
-#pragma unroll
-    for (int s = 0; s < 2; ++s) {
-      const float z = s == 0 ? 1.0f : -1.0f;
-      float P[3], vg = 0.0f, pg = 0.0f, gcd = 0.0f;
-#pragma unroll
-      for (int kk = 0; kk < 3; ++kk) {
-        P[kk] = v[kk] - z * gp[kk];
-        vg = fmaf(v[kk], dgc[s][kk], vg);
-        pg = fmaf(P[kk], dgc[s][kk], pg);
-        gcd = fmaf(gc[s][kk], dgp[kk], gcd);
-      }
-      dR[s] = fmaf(kappa, dcv[s], pg - z * gcd);
-      S[s] = fmaf(kappa, dcv[s], vg);
-      const float tdR = tau * dR[s];
-      const float zdc = z * dcv[s];
-#pragma unroll
-      for (int kk = 0; kk < 3; ++kk)
-        Phi[s][kk] = fmaf(tdR, P[kk], fmaf(zc_tR[s], dgp[kk], fmaf(zdc, gp[kk], dgc[s][kk])));
-    }
-    S[2] = fmaf(tau, dR[0] - dR[1], dcv[1] - dcv[0]);
-#pragma unroll
-    for (int kk = 0; kk < 3; ++kk) Phi[2][kk] = e2 * dgp[kk];
-    float r[3];
-#pragma unroll
-    for (int f = 0; f < 3; ++f) r[f] = w * test_t<float, D>(S[f], Phi[f], nb, sh);
-    if (!valid) continue;
-    if (A.out4) {
-      scatter4(A, id, r);
-      continue;
-    }
-    if (id >= 0) {
-#pragma unroll
-      for (int f = 0; f < 3; ++f) atomicAdd(A.out + 3 * (int64_t)id + f, r[f]);
-    } else {
-      const int32_t hh = -id - 1;
-      const int np = A.hang_np[hh];
-      const float wgt = np == 2 ? 0.5f : 0.25f;
-      for (int p = 0; p < np; ++p) {
-        const int32_t pid = A.hang_par[4 * hh + p];
-#pragma unroll
-        for (int f = 0; f < 3; ++f) atomicAdd(A.out + 3 * (int64_t)pid + f, wgt * r[f]);
-      }
-    }
-  }
-}
-
 
 // ---- block diagonal of the Jacobian (block-Jacobi preconditioner) ----------------
 // D_n = sum over elements, Gauss points and local pairs (i, j) whose constraint targets
@@ -788,103 +358,22 @@ __global__ void __launch_bounds__(256) k_block_diag_lanes(ElemArgs<T> A, LanePar
 
 }  // namespace
 
-template <typename T>
-cudaError_t launch_element_lanes(int dim, bool jv, const ElemArgs<T>& A, cudaStream_t s) {
+template <typename C, bool JV>
+static cudaError_t launch_lanes(int dim, const ElemArgs<double>& A, cudaStream_t s) {
   if (A.n_elem == 0) return cudaSuccess;
   const int t = block_threads(A.n_elem << dim);
   const unsigned blocks = block_count(A.n_elem << dim, t);
-  const LaneParams<T> K{T(A.P.kappa), T(A.P.tau_t), T(A.P.C_I * dim), T(A.P.eps2x2)};
-  if (dim == 2) {
-    if (jv) k_element_lanes<T, T, 2, true><<<blocks, t, 0, s>>>(A, K);
-    else k_element_lanes<T, T, 2, false><<<blocks, t, 0, s>>>(A, K);
-  } else {
-    if (jv) k_element_lanes<T, T, 3, true><<<blocks, t, 0, s>>>(A, K);
-    else k_element_lanes<T, T, 3, false><<<blocks, t, 0, s>>>(A, K);
-  }
+  const LaneParams<C> K = lane_params<C>(A.P, dim);
+  if (dim == 2) k_element_lanes<C, 2, JV><<<blocks, t, 0, s>>>(A, K);
+  else k_element_lanes<C, 3, JV><<<blocks, t, 0, s>>>(A, K);
   note_launch();
   return cudaGetLastError();
 }
-template cudaError_t launch_element_lanes<double>(int, bool, const ElemArgs<double>&, cudaStream_t);
-template cudaError_t launch_element_lanes<float>(int, bool, const ElemArgs<float>&, cudaStream_t);
-
-// FP64 residual with double-float arithmetic (FP32 pipe), FP64 data in and out
-cudaError_t launch_residual_df(int dim, const ElemArgs<double>& A, cudaStream_t s) {
-  if (A.n_elem == 0) return cudaSuccess;
-  const int t = block_threads(A.n_elem << dim);
-  const unsigned blocks = block_count(A.n_elem << dim, t);
-  const LaneParams<df> K{df(A.P.kappa), df(A.P.tau_t), df(A.P.C_I * dim), df(A.P.eps2x2)};
-  if (dim == 2) k_element_lanes<double, df, 2, false><<<blocks, t, 0, s>>>(A, K);
-  else k_element_lanes<double, df, 3, false><<<blocks, t, 0, s>>>(A, K);
-  note_launch();
-  return cudaGetLastError();
+cudaError_t launch_residual_lanes(int dim, bool double_float, const ElemArgs<double>& A, cudaStream_t s) {
+  return double_float ? launch_lanes<df, false>(dim, A, s) : launch_lanes<double, false>(dim, A, s);
 }
-
-// the stored linearisation of the FP32 J V (qp: 4 * 2^dim * n_elem float4; A.rec set)
-cudaError_t launch_lane_state(int dim, const ElemArgs<float>& A, float4* qp, int rows, cudaStream_t s) {
-  if (A.n_elem == 0) return cudaSuccess;
-  if (rows != 3 && rows != 4) return cudaErrorInvalidValue;
-  const LaneParams<float> K{float(A.P.kappa), float(A.P.tau_t), float(A.P.C_I * dim), float(A.P.eps2x2)};
-  const unsigned blocks = (unsigned)(((A.n_elem << dim) + kLaneThreads - 1) / kLaneThreads);
-  if (dim == 2) {
-    if (rows == 4) k_lane_state<2, 4><<<blocks, kLaneThreads, 0, s>>>(A, K, qp);
-    else k_lane_state<2, 3><<<blocks, kLaneThreads, 0, s>>>(A, K, qp);
-  } else {
-    if (rows == 4) k_lane_state<3, 4><<<blocks, kLaneThreads, 0, s>>>(A, K, qp);
-    else k_lane_state<3, 3><<<blocks, kLaneThreads, 0, s>>>(A, K, qp);
-  }
-  note_launch();
-  return cudaGetLastError();
-}
-
-template <int S, int NR>
-static cudaError_t launch_jv_stages(int dim, const ElemArgs<float>& A, const LaneParams<float>& K, const float4* qp,
-                                    int* err, int polls, cudaStream_t s) {
-  // persistent grid: the resident blocks of every SM, no more than there are tiles
-  static int per_sm[2] = {0, 0}, n_sm = 0;
-  const size_t smem = jv_stage_bytes(S, NR);
-  if (n_sm == 0) {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_jv_from_state<2, S, NR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_jv_from_state<3, S, NR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess)
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[0], k_jv_from_state<2, S, NR>, kLaneThreads, smem);
-    if (e == cudaSuccess)
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[1], k_jv_from_state<3, S, NR>, kLaneThreads, smem);
-    if (e != cudaSuccess) {
-      n_sm = 0;
-      return e;
-    }
-  }
-  const int64_t tiles = ((A.n_elem << dim) + kLaneThreads - 1) / kLaneThreads;
-  const unsigned blocks = (unsigned)std::min<int64_t>(tiles, (int64_t)n_sm * std::max(1, per_sm[dim - 2]));
-  if (dim == 2) k_jv_from_state<2, S, NR><<<blocks, kLaneThreads, smem, s>>>(A, K, qp, err, polls);
-  else k_jv_from_state<3, S, NR><<<blocks, kLaneThreads, smem, s>>>(A, K, qp, err, polls);
-  return cudaSuccess;
-}
-
-cudaError_t launch_jv_from_state(int dim, const ElemArgs<float>& A, const float4* qp, int rows, int* err,
-                                 int polls, cudaStream_t s) {
-  if (polls < 0) polls = kWaitPolls;
-  if (A.n_elem == 0) return cudaSuccess;
-  if (rows != 3 && rows != 4) return cudaErrorInvalidValue;
-  const LaneParams<float> K{float(A.P.kappa), float(A.P.tau_t), float(A.P.C_I * dim), float(A.P.eps2x2)};
-  const cudaError_t e = rows == 4 ? launch_jv_stages<kStages, 4>(dim, A, K, qp, err, polls, s)
-                                  : launch_jv_stages<kStages, 3>(dim, A, K, qp, err, polls, s);
-  if (e != cudaSuccess) return e;
-  note_launch();
-  return cudaGetLastError();
-}
-
-// per lane of the stored-linearisation J V: direction values and gradients, the J V
-// physics (incl. P_s), three transposes; the state part is read, not computed
-double jv_from_state_flops(int D) {
-  const double tri = D * (D - 1) / 2.0;
-  const double vg = 3 * tri + 4 * D, g = vg - 2, tt = 6 * D + 3 * tri + 1;
-  return (double)(1 << D) * (2 * vg + g + 101 + 12 + 3 * tt);
+cudaError_t launch_jv64_lanes(int dim, const ElemArgs<double>& A, cudaStream_t s) {
+  return launch_lanes<double, true>(dim, A, s);
 }
 
 template <typename T>
@@ -892,7 +381,7 @@ cudaError_t launch_block_diag_lanes(int dim, const ElemArgs<T>& A, T* Dout, cuda
   if (A.n_elem == 0) return cudaSuccess;
   const int t = block_threads(A.n_elem << dim);
   const unsigned blocks = block_count(A.n_elem << dim, t);
-  const LaneParams<T> K{T(A.P.kappa), T(A.P.tau_t), T(A.P.C_I * dim), T(A.P.eps2x2)};
+  const LaneParams<T> K = lane_params<T>(A.P, dim);
   if (dim == 2) k_block_diag_lanes<T, 2><<<blocks, t, 0, s>>>(A, K, Dout);
   else k_block_diag_lanes<T, 3><<<blocks, t, 0, s>>>(A, K, Dout);
   note_launch();

@@ -174,63 +174,6 @@ __global__ void k_block_apply32(int64_t N, const float* __restrict__ Dinv, const
   y[3 * i + 2] = fmaf(B[6], a, fmaf(B[7], b, B[8] * c));
 }
 
-__global__ void k_block_apply32_pad(int64_t N, const float* __restrict__ Dinv, const float* __restrict__ u,
-                                    const float* __restrict__ inv_s, float4* __restrict__ y,
-                                    float4* __restrict__ clear) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= N) return;
-  clear[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-  const float sc = inv_s ? inv_s[0] : 1.0f;
-  const float* B = Dinv + 9 * i;
-  const float a = sc * u[3 * i], b = sc * u[3 * i + 1], c = sc * u[3 * i + 2];
-  y[i] = make_float4(fmaf(B[0], a, fmaf(B[1], b, B[2] * c)), fmaf(B[3], a, fmaf(B[4], b, B[5] * c)),
-                     fmaf(B[6], a, fmaf(B[7], b, B[8] * c)), 0.0f);
-}
-
-__global__ void k_pad4(int64_t N, const float* __restrict__ x, float4* __restrict__ y) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i < N) y[i] = make_float4(x[3 * i], x[3 * i + 1], x[3 * i + 2], 0.0f);
-}
-
-// out <- acc with the Dirichlet rows of J V (= V) for threads i < N; threads N + h write
-// the constraint row of hanging node h: out_h = V_h - sum_p w_p V_p (V padded)
-__global__ void k_pack_jv4(int64_t N, int64_t H, const uint8_t* __restrict__ faces, BcTable bc,
-                           const int32_t* __restrict__ hnode, const int32_t* __restrict__ hpar,
-                           const uint8_t* __restrict__ hnp, const float4* __restrict__ V4,
-                           const float4* __restrict__ acc, float* __restrict__ out) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i < N) {
-    const uint8_t fm = faces[i];
-    if (fm & 0x80) return;
-    const float4 a = acc[i];
-    float r[3] = {a.x, a.y, a.z};
-    if (fm & 0x3F) {
-      const float4 v = V4[i];
-      const float vv[3] = {v.x, v.y, v.z};
-#pragma unroll
-      for (int f = 0; f < 3; ++f)
-        if (fm & bc.dir_faces[f] & 0x3F) r[f] = vv[f];
-    }
-    out[3 * i] = r[0];
-    out[3 * i + 1] = r[1];
-    out[3 * i + 2] = r[2];
-    return;
-  }
-  const int64_t h = i - N;
-  if (h >= H) return;
-  const int np = hnp[h];
-  const float wgt = np == 2 ? 0.5f : 0.25f;
-  const int64_t id = hnode[h];
-  float4 sv = V4[id];
-  for (int p = 0; p < np; ++p) {
-    const float4 a = V4[hpar[4 * h + p]];
-    sv.x -= wgt * a.x; sv.y -= wgt * a.y; sv.z -= wgt * a.z;
-  }
-  out[3 * id] = sv.x;
-  out[3 * id + 1] = sv.y;
-  out[3 * id + 2] = sv.z;
-}
-
 // Least squares of the inner process and coef_i = y_i / s_i, so that sum_i y_i q_i = sum_i
 // coef_i u_i.  Thread l holds column l: step j makes rotation j from column j and applies it
 // to the columns after it; then a column-oriented back-substitution over the columns before
@@ -368,34 +311,6 @@ cudaError_t launch_block_apply32(int64_t N, const float* Dinv32, const float* u,
                                  cudaStream_t s) {
   if (N) {
     k_block_apply32<<<nblk(N, 256), 256, 0, s>>>(N, Dinv32, u, inv_s, y);
-    note_launch();
-  }
-  return cudaGetLastError();
-}
-
-cudaError_t launch_block_apply32_pad(int64_t N, const float* Dinv32, const float* u, const float* inv_s, float4* y4,
-                                     float4* clear, cudaStream_t s) {
-  if (N) {
-    const int t = block_threads(N);
-    k_block_apply32_pad<<<block_count(N, t), t, 0, s>>>(N, Dinv32, u, inv_s, y4, clear);
-    note_launch();
-  }
-  return cudaGetLastError();
-}
-
-cudaError_t launch_pad4(int64_t N, const float* x, float4* y4, cudaStream_t s) {
-  if (N) {
-    k_pad4<<<nblk(N, 256), 256, 0, s>>>(N, x, y4);
-    note_launch();
-  }
-  return cudaGetLastError();
-}
-
-cudaError_t launch_pack_jv4(const RowArgs& R, const float4* V4, const float4* acc4, float* out, cudaStream_t s) {
-  if (R.n_nodes + R.n_hanging) {
-    const int t = block_threads(R.n_nodes + R.n_hanging);
-    k_pack_jv4<<<block_count(R.n_nodes + R.n_hanging, t), t, 0, s>>>(R.n_nodes, R.n_hanging, R.faces, R.bc, R.hnode,
-                                                                  R.hpar, R.hnp, V4, acc4, out);
     note_launch();
   }
   return cudaGetLastError();

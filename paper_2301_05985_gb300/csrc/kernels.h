@@ -3,6 +3,7 @@
 
 #include "patches.h"
 #include "pnp_internal.h"
+#include "tiles.h"
 
 // Arguments of the fused element kernels (residual / Jv / block diagonal).
 template <typename T>
@@ -18,13 +19,20 @@ struct ElemArgs {
   const T* adv;            // [N][3] advection velocity
   T* out;                  // [N][3] accumulated (must be zeroed first)
   PhysParams P;
-  // FP32 lane kernel only (may be null): per node {c+, c-, phi, h+, h-, v0, v1, v2}, 32 B
+  // lane kernels on FP64 vectors: the nodes' boundary faces, and the Dirichlet faces of field
+  // f in byte f (those rows are not added to)
+  const uint8_t* faces = nullptr;
+  uint32_t dir = 0;
+  // FP32 block diagonal only (may be null): per node {c+, c-, phi, h+, h-, v0, v1, v2}, 32 B
   // aligned, the same values as U, hs and adv in one sector
   const float4* rec = nullptr;
-  // FP32 J V only (may be null): direction and accumulated output padded to [N] float4,
-  // read with one 16-byte load and added with one vector atomic per node
-  const float4* V4 = nullptr;
-  float4* out4 = nullptr;
+};
+
+// What the tile kernel (element_tiles.cu) needs of the mesh: the node tables and which rows
+// are Dirichlet rows.
+struct TileMesh {
+  TileTab tab;
+  uint32_t dir;  // byte f: the faces on which field f is Dirichlet (bit per face)
 };
 
 // Arguments of the Dirichlet / hanging row kernels.
@@ -74,17 +82,41 @@ struct PatchArgs {
 template <typename T>
 cudaError_t launch_patch(int dim, bool jv, const PatchArgs<T>& A, cudaStream_t s);
 
+// one thread per element; out zeroed first, Dirichlet and hanging rows left to
+// launch_row_fixups
 template <typename T>
 cudaError_t launch_element(int dim, bool jv, const ElemArgs<T>& A, cudaStream_t s);
-// the same operator with 2^dim lanes per element (element_lanes.cu)
-template <typename T>
-cudaError_t launch_element_lanes(int dim, bool jv, const ElemArgs<T>& A, cudaStream_t s);
-// floating-point operations per element (an FMA counts 2) of the element kernel that
-// launch_element runs, counted from the formulation it evaluates
+// ---- kernels that add to the weak-form rows of `out` only: the rows are initialised first
+// (launch_init_rows or a kernel that does the same).
+// The residual of FP64 vectors with 2^dim lanes per element (element_lanes.cu), in
+// double-float arithmetic (pairs of floats, about 48 bits, on the FP32 pipe) or in FP64
+cudaError_t launch_residual_lanes(int dim, bool double_float, const ElemArgs<double>& A, cudaStream_t s);
+// J V in FP64, the same lanes
+cudaError_t launch_jv64_lanes(int dim, const ElemArgs<double>& A, cudaStream_t s);
+// floating-point operations per element (an FMA counts 2) of the residual or J V, counted
+// from the formulation that runs (lanes, or one thread per element)
 double element_kernel_flops(int dim, bool jv);
-// the FP64 residual of the lane-group kernel evaluated in double-float arithmetic (pairs
-// of floats, about 48 bits, on the FP32 pipe); FP64 inputs and output as launch_element
-cudaError_t launch_residual_df(int dim, const ElemArgs<double>& A, cudaStream_t s);
+// FP32 J V [N][3] on node tiles (element_tiles.cu) at the state of the node records
+// (launch_node_records); `advection` false when the advection field is zero.  err[0] = 1
+// (mapped pinned memory) when a wait on a staged table gave up after `polls` polls (< 0: the
+// default, about a second).  plan_jv_tiles: the grids for a table (t.blocks), once.
+cudaError_t plan_jv_tiles(int dim, TileTab& t);
+cudaError_t launch_jv_tiles(int dim, const TileMesh& M, const float4* rec, bool advection, const float* V,
+                            const PhysParams& P, float* out, int* err, int polls, cudaStream_t s);
+double jv_tiles_flops(int dim, bool advection);
+// out = 0 on weak-form rows, in - g (mode 0) or in (mode 1) on Dirichlet rows, the
+// constraint of in on hanging rows
+template <typename T>
+cudaError_t launch_init_rows(const RowArgs& R, const T* in, T* out, int mode, cudaStream_t s);
+// the rows of the residual F at U (mode 0) and the history hs = (b1 c^k + b2 c^{k-1}) / dt
+// (Uk null: zero)
+cudaError_t launch_init_residual(const RowArgs& R, const double* U, double* F, const double* Uk, const double* Ukm1,
+                                 double b1, double b2, double inv_dt, double* hs, cudaStream_t s);
+// y = Dinv (scale u) per node, scale = scale_dev[0] when given, and the rows of J V of y
+// (mode 1) into out
+template <typename T>
+cudaError_t launch_block_apply_rows(const RowArgs& R, const T* Dinv, const T* u, T scale, const T* scale_dev, T* y,
+                                    T* out, cudaStream_t s);
 // true when launch_element runs the lane-group kernel (not PNP_ELEMENT_KERNEL=thread)
 bool element_kernel_is_lanes();
 // true when the FP64 residual runs in double-float arithmetic (lane-group kernel, unless
@@ -93,21 +125,6 @@ bool residual_double_float();
 // FP32 operations per FP64 operation of the double-float arithmetic: a quick fused
 // multiply-add (2 FP64 flops) costs 18, a quick sum 11, the accurate sums 20, a product 10
 constexpr double kDfFlopsPerFlop = 10.0;
-// FP32 J V from a stored linearisation (element_lanes.cu): launch_lane_state computes, per
-// element lane, the state's Gauss-point quantities J V needs (qp: rows * 2^dim * n_elem
-// float4, A.rec set; rows = 4, or 3 when the advection field is zero); launch_jv_from_state
-// applies J V with them (A.V or A.V4, A.out or A.out4; qp and A.conn 16-byte aligned).
-// err[0] |= 1 when a staged copy's wait gave up.
-cudaError_t launch_lane_state(int dim, const ElemArgs<float>& A, float4* qp, int rows, cudaStream_t s);
-// polls: the limit of each bounded wait on a stage (< 0: the default, about a second)
-cudaError_t launch_jv_from_state(int dim, const ElemArgs<float>& A, const float4* qp, int rows, int* err,
-                                 int polls, cudaStream_t s);
-double jv_from_state_flops(int dim);
-// FP32 J V on hexahedra with two lanes per element (jv_pair.cu): the state from the node
-// records (A.rec), the direction A.V4 (with A.out4) or A.V (with A.out); `advection`
-// false when the advection field is zero (tau_c then depends on the level only)
-cudaError_t launch_jv_pair(const ElemArgs<float>& A, bool advection, cudaStream_t s);
-double jv_pair_flops(bool advection);
 // Dout [N][9] += the 3x3 diagonal blocks of the Jacobian (lane-group kernel; Dout zeroed
 // first, Dirichlet and hanging rows left to launch_diag_rows)
 template <typename T>
@@ -148,11 +165,10 @@ cudaError_t launch_norm2(int64_t n, const double* x, double* part, unsigned* tic
 // w -= sum_i h[i] Vb[i*ld + .], i < k
 cudaError_t launch_multi_axpy(int64_t n, int k, const double* Vb, int64_t ld, const double* h, double* w,
                               cudaStream_t s);
-// z_i = Dinv_i v_i per node (3x3 blocks); optionally also a float copy z32, and zeros into
-// clear / clear32 [N][3] (the accumulator of the J V that follows); each may be null
+// z_i = Dinv_i v_i per node (3x3 blocks) in FP64 and / or as floats z32 (either may be null).
 // The factor of v is `scale`, or *scale_dev when that is given.
 cudaError_t launch_block_apply(int64_t N, const double* Dinv, const double* v, double scale, const double* scale_dev,
-                               double* z, float* z32, double* clear, float* clear32, cudaStream_t s);
+                               double* z, float* z32, cudaStream_t s);
 // blocks (= partials per vector) of the multi-dot for vectors of n entries
 int multi_dot_blocks(int64_t n);
 // d[i] = V_i . w for i < k (part: [k][multi_dot_blocks(n)])
@@ -205,17 +221,9 @@ cudaError_t launch_inner_update(int64_t n, int j, int d, const float* Ub, int64_
                                 cudaStream_t s);
 inline size_t inner_scalar_doubles(int d) { return (size_t)(d + 1) * d; }
 cudaError_t launch_inner_lsq(int d, const double* sv, const double* H, double* coef, cudaStream_t s);
-// y = Dinv32 (inv_s[0] u) per node (inv_s may be null: scale 1); y4: the same, padded, and
-// zeros into clear [N] (the accumulator of the J V that follows)
+// y = Dinv32 (inv_s[0] u) per node (inv_s may be null: scale 1)
 cudaError_t launch_block_apply32(int64_t N, const float* Dinv32, const float* u, const float* inv_s, float* y,
                                  cudaStream_t s);
-cudaError_t launch_block_apply32_pad(int64_t N, const float* Dinv32, const float* u, const float* inv_s, float4* y4,
-                                     float4* clear, cudaStream_t s);
-// out [N][3] <- acc4 with the Dirichlet rows set to V4 and the hanging rows to
-// V4_h - sum_p w_p V4_p (the J V row fix-ups of the padded FP32 path)
-cudaError_t launch_pack_jv4(const RowArgs& R, const float4* V4, const float4* acc4, float* out, cudaStream_t s);
-// y4[i] = (x[3i], x[3i+1], x[3i+2], 0)
-cudaError_t launch_pad4(int64_t N, const float* x, float4* y4, cudaStream_t s);
 // out = sum_i coef_i U_i (FP32, n and ld multiples of 4); x += sum_i coef_i Z_i (FP32 vectors
 // into FP64)
 cudaError_t launch_combine_f32(int64_t n, int k, const float* Ub, int64_t ld, const double* coef, float* out,

@@ -169,6 +169,7 @@ int ctx_mg_setup(pnp_ctx* c, int levels) {
     }
     std::memcpy(L.sub->bc_type, c->bc_type, sizeof(c->bc_type));
     std::memcpy(L.sub->bc_val, c->bc_val, sizeof(c->bc_val));
+    L.sub->wait_flag = c->wait_flag;
     const int64_t Nc = cm.n_nodes;
     A((void**)&L.p_ptr, sizeof(int64_t) * T.p_ptr.size());
     A((void**)&L.p_col, sizeof(int32_t) * T.p_col.size());
@@ -205,7 +206,7 @@ int ctx_mg_setup(pnp_ctx* c, int levels) {
 }
 
 static int mg_blocks(pnp_ctx* c, const double* U, float* Dinv32) {
-  RC(ctx_prepare_f32(c, U));
+  RC(ctx_prepare_f32(c, U, false));
   RC(ctx_block_diag32(c, c->D32));
   CK(launch_block_invert<float>(c->n_nodes, c->D32, c->Dinv, c->dflag, c->stream));
   CK(launch_to_f32(9 * c->n_nodes, c->Dinv, Dinv32, c->stream));
@@ -243,6 +244,7 @@ int ctx_mg_prepare(pnp_ctx* c, const double* U) {
     RC(ctx_prepare_history(sc));
     CK(cudaMemsetAsync(sc->dflag, 0, sizeof(int), s));
     RC(mg_blocks(sc, sc->U, lv[l].Dinv32));
+    sc->adv_zero = c->adv_zero;  // zero on the finest level: zero at its nodes here
     int flag = 0;
     CK(cudaMemcpyAsync(&flag, sc->dflag, sizeof(int), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));

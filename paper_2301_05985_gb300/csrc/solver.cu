@@ -83,6 +83,26 @@ static int hanging_rows(pnp_ctx* c, const T* in, T* out) {
   return ctx_check(c, launch_row_fixups<T>(R, in, out, 0, c->stream), "hanging rows");
 }
 
+// the operators add to initialised rows, unless an environment variable selects the patch
+// or the one-thread-per-element kernels
+static bool on_lanes(const pnp_ctx* c) { return !c->use_patches && element_kernel_is_lanes(); }
+static ElemArgs<double> lane_args(const pnp_ctx* c, const double* U, const double* V, double* out) {
+  ElemArgs<double> A = elem_args<double>(c, U, V, c->hs, c->adv, out);
+  A.faces = c->d_faces;
+  A.dir = c->tile_mesh().dir;
+  return A;
+}
+
+// adds the residual to the initialised rows of F
+static int residual_lanes(pnp_ctx* c, const double* U, double* F) {
+  // of the double-float formulation: FP32-pipe operations
+  const bool dfl = residual_double_float();
+  ProfScope ps(c, PNP_PROF_RESIDUAL, 88.0 * c->n_nodes + c->conn_bytes(),
+               (dfl ? kDfFlopsPerFlop : 1.0) * element_kernel_flops(c->dim, false) * c->n_elem);
+  CK(launch_residual_lanes(c->dim, dfl, lane_args(c, U, nullptr, F), c->stream));
+  return PNP_OK;
+}
+
 int ctx_residual(pnp_ctx* c, const double* U, double* F) {
   if (c->use_patches) {
     {
@@ -92,14 +112,12 @@ int ctx_residual(pnp_ctx* c, const double* U, double* F) {
                               c->stream));
     }
     RC(hanging_rows<double>(c, U, F));
+  } else if (on_lanes(c)) {
+    CK(launch_init_rows<double>(c->rows(), U, F, 0, c->stream));
+    RC(residual_lanes(c, U, F));
   } else {
     CK(cudaMemsetAsync(F, 0, sizeof(double) * c->n3(), c->stream));
-    if (residual_double_float()) {
-      // FP32-pipe operations of the double-float formulation
-      ProfScope ps(c, PNP_PROF_RESIDUAL, 88.0 * c->n_nodes + c->conn_bytes(),
-                   kDfFlopsPerFlop * element_kernel_flops(c->dim, false) * c->n_elem);
-      CK(launch_residual_df(c->dim, elem_args<double>(c, U, nullptr, c->hs, c->adv, F), c->stream));
-    } else {
+    {
       ProfScope ps(c, PNP_PROF_RESIDUAL, 88.0 * c->n_nodes + c->conn_bytes(),
                    element_kernel_flops(c->dim, false) * c->n_elem);
       CK(launch_element<double>(c->dim, false, elem_args<double>(c, U, nullptr, c->hs, c->adv, F), c->stream));
@@ -110,17 +128,35 @@ int ctx_residual(pnp_ctx* c, const double* U, double* F) {
   return PNP_OK;
 }
 
-int ctx_jv64(pnp_ctx* c, const double* U, const double* V, double* JV, bool cleared) {
+int ctx_history_residual(pnp_ctx* c, const double* U, double* F) {
+  if (!on_lanes(c)) {
+    RC(ctx_prepare_history(c));
+    return ctx_residual(c, U, F);
+  }
+  const pnp_params& p = c->prm;
+  CK(launch_init_residual(c->rows(), U, F, p.steady ? nullptr : c->Uk, c->Ukm1, p.beta1, p.beta2,
+                          p.steady ? 0.0 : 1.0 / p.dt, c->hs, c->stream));
+  RC(residual_lanes(c, U, F));
+  c->res_count++;
+  return PNP_OK;
+}
+
+int ctx_jv64(pnp_ctx* c, const double* U, const double* V, double* JV, bool rows_done) {
+  const double bytes = 112.0 * c->n_nodes + c->conn_bytes(), flops = element_kernel_flops(c->dim, true) * c->n_elem;
   if (c->use_patches) {
     {
-      ProfScope ps(c, PNP_PROF_JV64, 112.0 * c->n_nodes + c->conn_bytes(), element_kernel_flops(c->dim, true) * c->n_elem);
+      ProfScope ps(c, PNP_PROF_JV64, bytes, flops);
       CK(launch_patch<double>(c->dim, true, patch_args<double>(c, U, V, c->hs, c->adv, JV, c->part64), c->stream));
     }
     RC(hanging_rows<double>(c, V, JV));
+  } else if (on_lanes(c)) {
+    if (!rows_done) CK(launch_init_rows<double>(c->rows(), V, JV, 1, c->stream));
+    ProfScope ps(c, PNP_PROF_JV64, bytes, flops);
+    CK(launch_jv64_lanes(c->dim, lane_args(c, U, V, JV), c->stream));
   } else {
-    if (!cleared) CK(cudaMemsetAsync(JV, 0, sizeof(double) * c->n3(), c->stream));
+    CK(cudaMemsetAsync(JV, 0, sizeof(double) * c->n3(), c->stream));
     {
-      ProfScope ps(c, PNP_PROF_JV64, 112.0 * c->n_nodes + c->conn_bytes(), element_kernel_flops(c->dim, true) * c->n_elem);
+      ProfScope ps(c, PNP_PROF_JV64, bytes, flops);
       CK(launch_element<double>(c->dim, true, elem_args<double>(c, U, V, c->hs, c->adv, JV), c->stream));
     }
     CK(launch_row_fixups<double>(c->rows(), V, JV, 1, c->stream));
@@ -129,23 +165,85 @@ int ctx_jv64(pnp_ctx* c, const double* U, const double* V, double* JV, bool clea
   return PNP_OK;
 }
 
-// the FP32 J V of hexahedral meshes runs the two-lanes-per-element kernel (jv_pair.cu)
-static bool use_jv_pair(const pnp_ctx* c) { return c->dim == 3 && !c->use_patches && element_kernel_is_lanes(); }
+// z = M^-1 (scale u) in FP64 with the inverted blocks, then w = J z
+static int precond_jv64(pnp_ctx* c, const double* U, const double* u, double scale, const double* scale_dev, double* z,
+                        double* w) {
+  const bool rows = on_lanes(c);
+  {
+    ProfScope ps(c, PNP_PROF_PRECOND, 120.0 * c->n_nodes, 18.0 * c->n_nodes);
+    if (rows) CK(launch_block_apply_rows<double>(c->rows(), c->Dinv, u, scale, scale_dev, z, w, c->stream));
+    else CK(launch_block_apply(c->n_nodes, c->Dinv, u, scale, scale_dev, z, nullptr, c->stream));
+  }
+  return ctx_jv64(c, U, z, w, rows);
+}
 
-int ctx_prepare_f32(pnp_ctx* c, const double* U) {
-  if (use_jv_pair(c)) {
+// The FP32 J V runs on node tiles and node records (on_lanes); the patch and the
+// one-thread-per-element kernels read FP32 copies of the fields.
+
+// the node tables of the tiles, built with their first use
+static int ctx_tiles(pnp_ctx* c) {
+  if (c->tab.rec || c->n_elem == 0) return PNP_OK;
+  const int nc = 1 << c->dim;
+  TileTab t;
+  // two threads per hexahedron, four per quadrilateral
+  t.threads = block_threads(c->n_elem * (c->dim == 3 ? 2 : 4));
+  if (c->dim == 3 && t.threads > 128) t.threads = 128;
+  t.corners = c->dim == 3 ? 4 * t.threads : t.threads;
+  t.n = (c->n_elem * nc + t.corners - 1) / t.corners;
+  const TileMeshTables M{c->n_elem, c->n_nodes, c->n_hanging, c->d_conn, c->d_hpar, c->d_level, c->d_faces, c->d_hnp};
+  CK(cudaMemsetAsync(c->dflag + 4, 0, 3 * sizeof(int), c->stream));
+  CK(launch_build_tiles(c->dim, M, t.corners, 0, 0, nullptr, c->dflag + 4, c->stream));
+  int most[3] = {0, 0, 0};
+  CK(cudaMemcpyAsync(most, c->dflag + 4, sizeof(most), cudaMemcpyDeviceToHost, c->stream));
+  CK(cudaStreamSynchronize(c->stream));
+  t.cap = (most[0] + 15) / 16 * 16;
+  t.slots = most[1];
+  t.hcap = (most[2] + 3) / 4 * 4;
+  t.bytes = tile_bytes(t.corners, nc, t.cap, t.hcap);
+  CK(plan_jv_tiles(c->dim, t));
+  const cudaError_t e = cudaMalloc((void**)&c->d_tiles, (size_t)t.bytes * (size_t)t.n);
+  if (e != cudaSuccess) {
+    c->d_tiles = nullptr;
+    PNP_FAIL(e == cudaErrorMemoryAllocation ? PNP_ERR_NOMEM : PNP_ERR_CUDA, "node tables: allocation failed: %s",
+             cudaGetErrorString(e));
+  }
+  CK(launch_build_tiles(c->dim, M, t.corners, t.cap, t.hcap, c->d_tiles, nullptr, c->stream));
+  t.rec = c->d_tiles;
+  c->tab = t;
+  return PNP_OK;
+}
+
+int ctx_prepare_f32(pnp_ctx* c, const double* U, bool check_adv) {
+  c->adv_zero = false;
+  if (check_adv && on_lanes(c)) {
+    RC(ctx_tiles(c));  // here, not under a stream capture
     double vn = 0.0;
     RC(ctx_norm(c, c->adv, &vn));
     c->adv_zero = vn == 0.0;
   }
-  CK(launch_to_f32(c->n3(), U, c->U32, c->stream));
-  CK(launch_to_f32(2 * c->n_nodes, c->hs, c->hs32, c->stream));
-  CK(launch_to_f32(c->n3(), c->adv, c->adv32, c->stream));
+  if (!on_lanes(c)) {
+    CK(launch_to_f32(c->n3(), U, c->U32, c->stream));
+    CK(launch_to_f32(2 * c->n_nodes, c->hs, c->hs32, c->stream));
+    CK(launch_to_f32(c->n3(), c->adv, c->adv32, c->stream));
+  }
   CK(launch_node_records(c->n_nodes, U, c->hs, c->adv, c->rec32, c->stream));
   return PNP_OK;
 }
 
-int ctx_jv32(pnp_ctx* c, const float* V32, float* JV32, bool cleared) {
+// adds J V to the initialised rows of JV32, at the node records `rec`
+static int jv_tiles(pnp_ctx* c, const float4* rec, const PhysParams& P, bool adv, const float* V32, float* JV32) {
+  RC(ctx_tiles(c));
+  ProfScope ps(c, PNP_PROF_JV32, 56.0 * c->n_nodes + c->conn_bytes(), jv_tiles_flops(c->dim, adv) * c->n_elem);
+  CK(launch_jv_tiles(c->dim, c->tile_mesh(), rec, adv, V32, P, JV32, c->wait_flag, c->wait_polls, c->stream));
+  c->jv_count++;
+  return PNP_OK;
+}
+
+int ctx_jv32(pnp_ctx* c, const float* V32, float* JV32) {
+  if (on_lanes(c)) {
+    CK(launch_init_rows<float>(c->rows(), V32, JV32, 1, c->stream));
+    return jv_tiles(c, c->rec32, c->phys(), !c->adv_zero, V32, JV32);
+  }
   if (c->use_patches) {
     {
       ProfScope ps(c, PNP_PROF_JV32, 56.0 * c->n_nodes + c->conn_bytes(), element_kernel_flops(c->dim, true) * c->n_elem);
@@ -154,15 +252,10 @@ int ctx_jv32(pnp_ctx* c, const float* V32, float* JV32, bool cleared) {
     }
     RC(hanging_rows<float>(c, V32, JV32));
   } else {
-    if (!cleared) CK(cudaMemsetAsync(JV32, 0, sizeof(float) * c->n3(), c->stream));
-    ElemArgs<float> A = elem_args<float>(c, c->U32, V32, c->hs32, c->adv32, JV32);
-    A.rec = c->rec32;
-    if (use_jv_pair(c)) {
-      ProfScope ps(c, PNP_PROF_JV32, 56.0 * c->n_nodes + c->conn_bytes(), jv_pair_flops(!c->adv_zero) * c->n_elem);
-      CK(launch_jv_pair(A, !c->adv_zero, c->stream));
-    } else {
+    CK(cudaMemsetAsync(JV32, 0, sizeof(float) * c->n3(), c->stream));
+    {
       ProfScope ps(c, PNP_PROF_JV32, 56.0 * c->n_nodes + c->conn_bytes(), element_kernel_flops(c->dim, true) * c->n_elem);
-      CK(launch_element<float>(c->dim, true, A, c->stream));
+      CK(launch_element<float>(c->dim, true, elem_args<float>(c, c->U32, V32, c->hs32, c->adv32, JV32), c->stream));
     }
     CK(launch_row_fixups<float>(c->rows(), V32, JV32, 1, c->stream));
   }
@@ -214,7 +307,7 @@ int ctx_dot(pnp_ctx* c, const double* x, const double* y, double* out) {
 static int build_preconditioner(pnp_ctx* c, const double* U, int prec) {
   CK(cudaMemsetAsync(c->dflag, 0, sizeof(int), c->stream));
   if (prec == PNP_F32) {
-    RC(ctx_prepare_f32(c, U));
+    RC(ctx_prepare_f32(c, U, true));
     RC(ctx_block_diag32(c, c->D32));
     CK(launch_block_invert<float>(c->n_nodes, c->D32, c->Dinv, c->dflag, c->stream));
     if (c->prm.gmres_inner > 0) {
@@ -243,77 +336,38 @@ static int apply_op(pnp_ctx* c, const double* U, const double* x, double* w, int
 
 // PNP_ERR_DEVICE_FLAG when a wait of the staged J V gave up (its copies never landed)
 int ctx_check_staged_waits(pnp_ctx* c) {
-  int flag = 0;
-  CK(cudaMemcpyAsync(&flag, c->dflag + 1, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
   CK(cudaStreamSynchronize(c->stream));
-  if (flag) PNP_FAIL(PNP_ERR_DEVICE_FLAG, "J V: a staged copy of the stored linearisation did not complete");
+  if (c->hflag[0]) PNP_FAIL(PNP_ERR_DEVICE_FLAG, "J V: a staged copy of the mesh tables did not complete");
   return PNP_OK;
 }
 
-// FP32 J V of the inner solve: the direction padded to 16 bytes per node (one load), the
-// output accumulated with one vector atomic per node, then packed to [N][3] with the
-// Dirichlet and hanging rows of J V.  Lane-group kernel only.
-// With from_state, the state's Gauss-point quantities come from the linearisation stored
-// by launch_lane_state for the current Krylov solve.
-// cleared: JV4 is zero already, from the block-Jacobi apply that made V4 (clearing it
-// inside the pack, right after the vector atomics that filled it, measured several times
-// slower than a memset on GB300).
-static int ctx_jv32_pad(pnp_ctx* c, const float4* V4, float* out, bool from_state, bool cleared = false) {
-  if (!cleared) CK(cudaMemsetAsync(c->JV4, 0, sizeof(float4) * c->n_nodes, c->stream));
-  {
-    ElemArgs<float> A = elem_args<float>(c, c->U32, nullptr, c->hs32, c->adv32, nullptr);
-    A.rec = c->rec32;
-    A.V4 = V4;
-    A.out4 = c->JV4;
-    if (from_state) {
-      // direction in, result out (12 B per node each), the stored state (64 B per lane)
-      ProfScope ps(c, PNP_PROF_JV32,
-                   24.0 * c->n_nodes + 16.0 * c->lin_rows * (double)(c->n_elem << c->dim) + c->conn_bytes(),
-                   jv_from_state_flops(c->dim) * c->n_elem);
-      CK(launch_jv_from_state(c->dim, A, c->qp32, c->lin_rows, c->dflag + 1, c->wait_polls, c->stream));
-    } else if (use_jv_pair(c)) {
-      ProfScope ps(c, PNP_PROF_JV32, 56.0 * c->n_nodes + c->conn_bytes(), jv_pair_flops(!c->adv_zero) * c->n_elem);
-      CK(launch_jv_pair(A, !c->adv_zero, c->stream));
-    } else {
-      ProfScope ps(c, PNP_PROF_JV32, 56.0 * c->n_nodes + c->conn_bytes(),
-                   element_kernel_flops(c->dim, true) * c->n_elem);
-      CK(launch_element_lanes<float>(c->dim, true, A, c->stream));
-    }
-  }
-  CK(launch_pack_jv4(c->rows(), V4, c->JV4, out, c->stream));
-  c->jv_count++;
-  return PNP_OK;
-}
-
-// Gauss-point linearisation of the FP32 J V at the prepared FP32 state (ctx_prepare_f32)
-int ctx_linearize32(pnp_ctx* c) {
-  if (!c->qp32) {
-    const cudaError_t e = cudaMalloc((void**)&c->qp32, sizeof(float4) * 4 * ((size_t)c->n_elem << c->dim));
+// The linearisation of pnp_linearize at U: the node records of the state, kept apart from
+// the solver's, with this call's parameters.
+int ctx_linearize(pnp_ctx* c, const double* U) {
+  RC(ctx_tiles(c));
+  if (!c->rec_lin) {
+    const cudaError_t e = cudaMalloc((void**)&c->rec_lin, sizeof(float4) * 2 * (size_t)c->n_nodes);
     if (e != cudaSuccess) {
-      c->qp32 = nullptr;
+      c->rec_lin = nullptr;
       PNP_FAIL(e == cudaErrorMemoryAllocation ? PNP_ERR_NOMEM : PNP_ERR_CUDA,
                "stored linearisation: allocation failed: %s", cudaGetErrorString(e));
     }
   }
   // a new linearisation clears the give-up flag of the staged J V's waits
-  CK(cudaMemsetAsync(c->dflag + 1, 0, sizeof(int), c->stream));
-  // a zero advection field (pure PNP) leaves v out of the stored state: three rows
+  CK(cudaStreamSynchronize(c->stream));
+  c->hflag[0] = 0;
   double vn = 0.0;
   RC(ctx_norm(c, c->adv, &vn));
-  c->lin_rows = vn == 0.0 ? 3 : 4;
-  ElemArgs<float> A = elem_args<float>(c, c->U32, nullptr, c->hs32, c->adv32, nullptr);
-  A.rec = c->rec32;
-  ProfScope ps(c, PNP_PROF_PRECOND,
-               32.0 * c->n_nodes + 16.0 * c->lin_rows * (double)(c->n_elem << c->dim) + c->conn_bytes());
-  CK(launch_lane_state(c->dim, A, c->qp32, c->lin_rows, c->stream));
-  c->lin_user = false;
+  c->lin_adv = vn != 0.0;
+  c->lin_phys = c->phys();
+  CK(launch_node_records(c->n_nodes, U, c->hs, c->adv, c->rec_lin, c->stream));
   return PNP_OK;
 }
 
 // JV = J V (FP32 [n][3]) from the stored linearisation
 int ctx_jv32_linearized(pnp_ctx* c, const float* V, float* JV) {
-  CK(launch_pad4(c->n_nodes, V, c->V4, c->stream));
-  return ctx_jv32_pad(c, c->V4, JV, true);
+  CK(launch_init_rows<float>(c->rows(), V, JV, 1, c->stream));
+  return jv_tiles(c, c->rec_lin, c->lin_phys, c->lin_adv, V, JV);
 }
 
 // z = P(u): d steps of right-preconditioned FP32 GMRES on (J M^-1) t = u from t = 0, then
@@ -323,7 +377,7 @@ int ctx_jv32_linearized(pnp_ctx* c, const float* V, float* JV) {
 // Arnoldi with the device-side bookkeeping, and t = sum_i y_i q_i into c->JV32.  Every
 // launch depends only on the context's buffers, sizes and parameters (no host round
 // trip), so the sequence can be captured as a graph.
-static int inner_gmres32_body(pnp_ctx* c, bool from_state) {
+static int inner_gmres32_body(pnp_ctx* c) {
   const int d = c->prm.gmres_inner;
   const int64_t n = c->n3(), N = c->n_nodes, ldq = c->ldq;
   cudaStream_t s = c->stream;
@@ -338,22 +392,17 @@ static int inner_gmres32_body(pnp_ctx* c, bool from_state) {
     ProfScope ps(c, PNP_PROF_INNER, 4.0 * n, 2.0 * n);
     CK(launch_inner_start(ldq, d, Q, c->part, c->ticket, sv, dinv, inv_s, s));
   }
-  const bool pad = !c->use_patches && element_kernel_is_lanes();
+  const bool tiles = on_lanes(c);
   for (int j = 0; j < d; ++j) {
     float* w = Q + (size_t)(j + 1) * ldq;
-    if (pad) {
-      {
-        ProfScope ps(c, PNP_PROF_PRECOND, 60.0 * N, 18.0 * N);
-        CK(launch_block_apply32_pad(N, c->Dinv32, Q + (size_t)j * ldq, inv_s + j, c->V4, c->JV4, s));
-      }
-      RC(ctx_jv32_pad(c, c->V4, w, from_state, true));
-    } else {
-      {
-        ProfScope ps(c, PNP_PROF_PRECOND, 60.0 * N, 18.0 * N);
-        CK(launch_block_apply32(N, c->Dinv32, Q + (size_t)j * ldq, inv_s + j, c->V32, s));
-      }
-      RC(ctx_jv32(c, c->V32, w));
+    {
+      ProfScope ps(c, PNP_PROF_PRECOND, 60.0 * N, 18.0 * N);
+      if (tiles)
+        CK(launch_block_apply_rows<float>(c->rows(), c->Dinv32, Q + (size_t)j * ldq, 1.0f, inv_s + j, c->V32, w, s));
+      else CK(launch_block_apply32(N, c->Dinv32, Q + (size_t)j * ldq, inv_s + j, c->V32, s));
     }
+    if (tiles) RC(jv_tiles(c, c->rec32, c->phys(), !c->adv_zero, c->V32, w));
+    else RC(ctx_jv32(c, c->V32, w));
     {
       const double nj = (double)n * (j + 1);
       ProfScope ps(c, PNP_PROF_INNER, 4.0 * (nj + n) + 4.0 * (nj + 2.0 * n), 4.0 * nj + 2.0 * n);
@@ -367,11 +416,11 @@ static int inner_gmres32_body(pnp_ctx* c, bool from_state) {
 }
 
 // what the captured inner solve depends on: sizes, buffers, parameters, boundary table
-static std::vector<unsigned char> inner_graph_key(const pnp_ctx* c, bool from_state) {
+static std::vector<unsigned char> inner_graph_key(const pnp_ctx* c) {
   struct Key {
-    int d, dim, from_state, pad, use_patches, steady, lin_rows, adv_zero;
+    int d, dim, tiles, steady, adv_zero, wait_polls;
     int64_t n_nodes, n_elem, ldq;
-    const void* bufs[14];
+    const void* bufs[11];
     double phys[4];
     double bc_val[6][3];
     uint8_t dir_faces[4];
@@ -379,15 +428,13 @@ static std::vector<unsigned char> inner_graph_key(const pnp_ctx* c, bool from_st
   std::memset(&k, 0, sizeof(k));
   k.d = c->prm.gmres_inner;
   k.dim = c->dim;
-  k.from_state = from_state;
-  k.pad = element_kernel_is_lanes();
-  k.use_patches = c->use_patches;
-  k.lin_rows = c->lin_rows;
+  k.tiles = on_lanes(c);
+  k.wait_polls = c->wait_polls;
   k.adv_zero = c->adv_zero;
   k.n_nodes = c->n_nodes;
   k.n_elem = c->n_elem;
   k.ldq = c->ldq;
-  const void* b[14] = {c->Qin, c->isc, c->iinv, c->Dinv32, c->V4, c->JV4, c->qp32, c->part, c->JV32,
+  const void* b[11] = {c->Qin, c->isc, c->iinv, c->Dinv32, c->part, c->JV32,
                        c->V32, c->U32, c->hs32, c->adv32, c->rec32};
   std::memcpy(k.bufs, b, sizeof(b));
   const PhysParams P = c->phys();
@@ -417,7 +464,7 @@ static bool inner_graph_enabled(const pnp_ctx* c) {
 
 // true when the graph was captured; on false the caller runs the solve eagerly (a capture
 // that the runtime refuses turns the graph off for the context, with no error latched)
-static bool inner_graph_capture(pnp_ctx* c, bool from_state) {
+static bool inner_graph_capture(pnp_ctx* c) {
   if (c->inner_exec) {
     cudaGraphExecDestroy(c->inner_exec);
     c->inner_exec = nullptr;
@@ -434,7 +481,7 @@ static bool inner_graph_capture(pnp_ctx* c, bool from_state) {
   const int64_t l0 = launch_count();
   const int jv0 = c->jv_count;
   cudaError_t e = cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal);
-  int rc = e == cudaSuccess ? inner_gmres32_body(c, from_state) : PNP_OK;
+  int rc = e == cudaSuccess ? inner_gmres32_body(c) : PNP_OK;
   cudaGraph_t g = nullptr;
   if (e == cudaSuccess) {
     const cudaError_t e2 = cudaStreamEndCapture(c->cap_stream, &g);
@@ -456,7 +503,7 @@ static bool inner_graph_capture(pnp_ctx* c, bool from_state) {
     c->latched = latched0;  // a refused capture is not a device error
     return false;
   }
-  c->inner_key = inner_graph_key(c, from_state);
+  c->inner_key = inner_graph_key(c);
   note_capture();
   return true;
 }
@@ -464,19 +511,19 @@ static bool inner_graph_capture(pnp_ctx* c, bool from_state) {
 // z = P(u): d steps of right-preconditioned FP32 GMRES on (J M^-1) t = u from t = 0, then
 // z = M^-1 t (M: the block diagonal).  A fixed number of steps with the Hessenberg
 // bookkeeping on the device: no host round trip.  P is homogeneous, P(a u) = a P(u).
-static int inner_gmres32(pnp_ctx* c, const double* u, float* z32, bool from_state) {
+static int inner_gmres32(pnp_ctx* c, const double* u, float* z32) {
   const int64_t n = c->n3(), N = c->n_nodes;
   cudaStream_t s = c->stream;
   CK(launch_to_f32(n, u, c->Qin, s));
   bool replay = inner_graph_enabled(c);
-  if (replay && (!c->inner_exec || c->inner_key != inner_graph_key(c, from_state)))
-    replay = inner_graph_capture(c, from_state);
+  if (replay && (!c->inner_exec || c->inner_key != inner_graph_key(c)))
+    replay = inner_graph_capture(c);
   if (replay) {
     CK(cudaGraphLaunch(c->inner_exec, s));
     note_launches(c->inner_graph_launches);
     c->jv_count += c->inner_graph_jv;
   } else {
-    RC(inner_gmres32_body(c, from_state));
+    RC(inner_gmres32_body(c));
     c->inner_eager_done = true;
   }
   ProfScope ps(c, PNP_PROF_PRECOND, 60.0 * N, 18.0 * N);
@@ -514,11 +561,7 @@ static int inner_gmres64(pnp_ctx* c, const double* U, const double* u, double* z
   int k = 0;
   for (int j = 0; j < d; ++j) {
     double* w = Q + (size_t)(j + 1) * n;
-    {
-      ProfScope ps(c, PNP_PROF_PRECOND, 120.0 * N, 18.0 * N);
-      CK(launch_block_apply(N, c->Dinv, Q + (size_t)j * n, 1.0 / sv[j], nullptr, c->zin64, nullptr, w, nullptr, s));
-    }
-    RC(ctx_jv64(c, U, c->zin64, w, true));
+    RC(precond_jv64(c, U, Q + (size_t)j * n, 1.0 / sv[j], nullptr, c->zin64, w));
     const double nj = (double)n * (j + 1);
     {
       ProfScope ps(c, PNP_PROF_ORTHO, 8.0 * (nj + n), 2.0 * nj);
@@ -565,7 +608,7 @@ static int inner_gmres64(pnp_ctx* c, const double* U, const double* u, double* z
   CK(cudaMemsetAsync(c->zin64, 0, sizeof(double) * n, s));
   CK(launch_multi_axpy(n, k, Q, n, coef, c->zin64, s));
   ProfScope ps(c, PNP_PROF_PRECOND, 120.0 * N, 18.0 * N);
-  CK(launch_block_apply(N, c->Dinv, c->zin64, 1.0, nullptr, z, nullptr, nullptr, nullptr, s));
+  CK(launch_block_apply(N, c->Dinv, c->zin64, 1.0, nullptr, z, nullptr, s));
   CK(cudaStreamSynchronize(s));  // the host vectors above go out of scope
   return PNP_OK;
 }
@@ -584,8 +627,8 @@ int ctx_gmres(pnp_ctx* c, const double* U, const double* b, double* x, double rt
   RC(ctx_alloc_krylov(c, m));
   const int64_t n = c->n3();
   cudaStream_t s = c->stream;
+  // (in FP32 also the node records of U, for J V)
   if (!have_precond) RC(build_preconditioner(c, U, prec));
-  if (prec == PNP_F32) RC(ctx_prepare_f32(c, U));
   // multigrid preconditioner (FP32 V-cycle) of a flexible outer solve; a solve in which
   // it stagnates continues with the inner FP32 GMRES (block Jacobi) preconditioner
   const bool use_mg = prec == PNP_F32 && c->prm.mg_levels > 0;
@@ -607,10 +650,13 @@ int ctx_gmres(pnp_ctx* c, const double* U, const double* b, double* x, double rt
   // the same flexible scheme entirely in FP64 (inner FP64 GMRES, FP64 J V)
   const bool flex64 = prec == PNP_F64 && c->prm.gmres_inner > 0;
   if (flex64) RC(ctx_alloc_inner64(c, m, c->prm.gmres_inner));
-  // the inner J V reads the state's Gauss-point quantities stored once for this solve
-  const bool from_state = flex && !use_mg && !c->use_patches && element_kernel_is_lanes();
+  // the bounded waits of the tile J V raise a flag that is read at the end of the solve
+  const bool staged = prec == PNP_F32 && on_lanes(c);
   c->lin_user = false;  // a solve replaces any linearisation stored by pnp_linearize
-  if (from_state) RC(ctx_linearize32(c));
+  if (staged) {
+    CK(cudaStreamSynchronize(s));
+    c->hflag[0] = 0;
+  }
   double* V = c->basis;
   double* dd = c->dsc;                    // [m+2] dot products of one pass
   double* dinv = c->dsc + (m + 2);        // [m+2] 1 / s_i^2
@@ -679,10 +725,8 @@ int ctx_gmres(pnp_ctx* c, const double* U, const double* b, double* x, double rt
       if (flex) {
         float* zj = c->Zb + (size_t)j * n;
         if (mg_on) RC(ctx_mg_apply(c, uj, zj));
-        else RC(inner_gmres32(c, uj, zj, from_state));
-        // the outer J V applies the same linearisation as the inner one
-        if (from_state) RC(ctx_jv32_linearized(c, zj, c->JV32));
-        else RC(ctx_jv32(c, zj, c->JV32));
+        else RC(inner_gmres32(c, uj, zj));
+        RC(ctx_jv32(c, zj, c->JV32));
         ProfScope ps(c, PNP_PROF_PRECOND, 20.0 * (double)n);
         CK(launch_to_f64_scaled(n, c->JV32, 1.0 / sv[j], w, s));
       } else if (flex64) {
@@ -692,19 +736,14 @@ int ctx_gmres(pnp_ctx* c, const double* U, const double* b, double* x, double rt
         RC(ctx_jv64(c, U, zj, c->w));
         CK(launch_axpbyz(n, 1.0 / sv[j], c->w, 0.0, c->w, w, s));
       } else if (prec == PNP_F64) {
-        {
-          ProfScope ps(c, PNP_PROF_PRECOND, 120.0 * c->n_nodes, 18.0 * c->n_nodes);
-          CK(launch_block_apply(c->n_nodes, c->Dinv, uj, 1.0 / sv[0], j > 0 ? inv_s : nullptr, c->z, nullptr, w,
-                                nullptr, s));
-        }
-        RC(ctx_jv64(c, U, c->z, w, true));
+        RC(precond_jv64(c, U, uj, 1.0 / sv[0], j > 0 ? inv_s : nullptr, c->z, w));
       } else {
         {
           ProfScope ps(c, PNP_PROF_PRECOND, 108.0 * c->n_nodes, 18.0 * c->n_nodes);
-          CK(launch_block_apply(c->n_nodes, c->Dinv, uj, 1.0 / sv[0], j > 0 ? inv_s : nullptr, nullptr, c->V32, nullptr,
-                                c->JV32, s));
+          CK(launch_block_apply(c->n_nodes, c->Dinv, uj, 1.0 / sv[0], j > 0 ? inv_s : nullptr, nullptr, c->V32,
+                                s));
         }
-        RC(ctx_jv32(c, c->V32, c->JV32, true));
+        RC(ctx_jv32(c, c->V32, c->JV32));
         ProfScope ps(c, PNP_PROF_PRECOND, 36.0 * c->n_nodes);
         CK(launch_to_f64(n, c->JV32, w, s));
       }
@@ -808,7 +847,7 @@ int ctx_gmres(pnp_ctx* c, const double* U, const double* b, double* x, double rt
       CK(cudaMemcpyAsync(dcoef, hco, sizeof(double) * k, cudaMemcpyHostToDevice, s));
       CK(cudaMemsetAsync(c->w, 0, sizeof(double) * n, s));
       CK(launch_multi_axpy(n, k, V, n, dcoef, c->w, s));
-      CK(launch_block_apply(c->n_nodes, c->Dinv, c->w, 1.0, nullptr, c->z, nullptr, nullptr, nullptr, s));
+      CK(launch_block_apply(c->n_nodes, c->Dinv, c->w, 1.0, nullptr, c->z, nullptr, s));
       CK(launch_axpby(n, 1.0, c->z, 1.0, x, s));
     }
     // true residual (restart vector); when the Arnoldi estimate claims convergence it is
@@ -834,7 +873,7 @@ int ctx_gmres(pnp_ctx* c, const double* U, const double* b, double* x, double rt
     }
     if (std::isfinite(beta) && beta > 0.95 * beta_cycle) {
       CK(cudaStreamSynchronize(s));
-      if (from_state) RC(ctx_check_staged_waits(c));
+      if (staged) RC(ctx_check_staged_waits(c));
       *its_out = total;
       *rel_out = beta / bn;
       PNP_FAIL(PNP_ERR_KRYLOV_MAXIT, "gmres: stagnated after %d iterations at relative residual %.3e > %.3e", total,
@@ -845,7 +884,7 @@ int ctx_gmres(pnp_ctx* c, const double* U, const double* b, double* x, double rt
   CK(cudaStreamSynchronize(s));
   *its_out = total;
   *rel_out = beta / bn;
-  if (from_state) RC(ctx_check_staged_waits(c));
+  if (staged) RC(ctx_check_staged_waits(c));
   return PNP_OK;
 }
 

@@ -229,12 +229,9 @@ __global__ void __launch_bounds__(256) k_multi_axpy(int64_t n, int k, const doub
 }
 
 __global__ void k_block_apply(int64_t N, const double* __restrict__ Dinv, const double* __restrict__ v, double scale,
-                              const double* __restrict__ scale_dev, double* __restrict__ z, float* __restrict__ z32, double* __restrict__ clear,
-                              float* __restrict__ clear32) {
+                              const double* __restrict__ scale_dev, double* __restrict__ z, float* __restrict__ z32) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= N) return;
-  if (clear) clear[3 * i] = clear[3 * i + 1] = clear[3 * i + 2] = 0.0;
-  if (clear32) clear32[3 * i] = clear32[3 * i + 1] = clear32[3 * i + 2] = 0.f;
   if (scale_dev) scale = *scale_dev;
   const double* B = Dinv + 9 * i;
   const double a = scale * v[3 * i], b = scale * v[3 * i + 1], c = scale * v[3 * i + 2];
@@ -435,10 +432,10 @@ cudaError_t launch_multi_axpy_norm(int64_t n, int k, const double* Vb, int64_t l
   return cudaGetLastError();
 }
 cudaError_t launch_block_apply(int64_t N, const double* Dinv, const double* v, double scale, const double* scale_dev,
-                               double* z, float* z32, double* clear, float* clear32, cudaStream_t s) {
+                               double* z, float* z32, cudaStream_t s) {
   if (N) {
     const int t = block_threads(N);
-    k_block_apply<<<block_count(N, t), t, 0, s>>>(N, Dinv, v, scale, scale_dev, z, z32, clear, clear32);
+    k_block_apply<<<block_count(N, t), t, 0, s>>>(N, Dinv, v, scale, scale_dev, z, z32);
     note_launch();
   }
   return cudaGetLastError();
