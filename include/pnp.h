@@ -542,9 +542,8 @@ int pnp_mlp_get_adam_state(pnp_ctx* c, float* m, float* v, int64_t* t);
  * device memory: for callers that cannot call cudaMalloc -- e.g. a host application
  * that reserves its whole device-memory budget up front and forbids later allocations,
  * or code that must not introduce allocation (and its implicit synchronisation) into
- * a latency-critical stream.  The BF16 weights, activations and output rows live in one
- * fixed file-scope device array (about 5 MB) that every GPU loading the library keeps
- * until the process exits.
+ * a latency-critical stream.  The BF16 weights live in one fixed file-scope device array
+ * (about 0.13 MB) that every GPU loading the library keeps until the process exits.
  *   params: device FP32 [PNP_MLP_PARAMS] packed parameters (layout above);
  *   X: device FP32 [B][216] standardised inputs; Y: device FP32 [B][3] outputs;
  *   B <= PNP_NOALLOC_MAX_ROWS (larger B: PNP_ERR_ARG, split the call);
@@ -552,7 +551,7 @@ int pnp_mlp_get_adam_state(pnp_ctx* c, float* m, float* v, int64_t* t);
  * The array is part of the library's device code: CUDA commits it on a device when it
  * loads that code there, which under lazy module loading (CUDA's default) can be the
  * first call of this or another network entry point on that device -- a caller with a
- * fixed device budget should count these 5 MB in it.  Later calls allocate nothing.
+ * fixed device budget should count it.  Later calls allocate nothing.
  * The first call on a device looks up the array's device address (cudaGetSymbolAddress)
  * for that device; make that first call before any stream capture.  All calls share the
  * array, so calls that overlap on the GPU (other streams, other host threads) race and

@@ -325,13 +325,13 @@ int pnp_ctx_create(const pnp_mesh* m, const pnp_params* p, void* stream, pnp_ctx
   ALLOC(c->dflag, sizeof(int) * 8);
   ALLOC(c->ticket, sizeof(unsigned));
 #undef ALLOC
-  if (cudaMallocHost((void**)&c->hflag, sizeof(int) * 2) != cudaSuccess) {
+  if (cudaMallocHost((void**)&c->hflag, sizeof(int) * 4) != cudaSuccess) {
     cudaGetLastError();
     c->hflag = nullptr;
     pnp_set_error("pnp_ctx_create: out of pinned memory");
     return fail(PNP_ERR_NOMEM);
   }
-  c->hflag[0] = c->hflag[1] = 0;
+  c->hflag[0] = c->hflag[1] = c->hflag[2] = 0;
   c->wait_flag = c->hflag;
   std::vector<uint8_t> faces(m->node_faces);
   for (int64_t i = 0; i < N; ++i)

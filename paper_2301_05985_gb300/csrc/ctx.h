@@ -67,8 +67,8 @@ struct pnp_ctx {
   double* dsc = nullptr;   // small device scalars [2*(m+2) + 8]
   double* hpin = nullptr;  // pinned host mirror of dsc
   int* dflag = nullptr;
-  // pinned, set by a tile J V whose bounded wait gave up: [0] of solves and the stored
-  // linearisation, [1] of pnp_jv.  wait_flag: [0], or on a multigrid level the owner's [0]
+  // pinned, set by a kernel whose bounded wait gave up: the J V's [0] of solves and the
+  // stored linearisation, [1] of pnp_jv; [2] the network inference.  wait_flag: [0], or on a multigrid level the owner's [0]
   int* hflag = nullptr;
   int* wait_flag = nullptr;
   unsigned* ticket = nullptr;  // counter of the reductions' last block (this stream's launches)

@@ -132,135 +132,6 @@ __global__ void k_targets(int64_t rows, int64_t N, const int32_t* __restrict__ r
   for (int f = 3; f < NOP; ++f) Y[r * NOP + f] = 0.f;
 }
 
-__global__ void k_f32_to_bf16_rows(int64_t rows, int cols, int ldin, int ldout, const float* __restrict__ in,
-                                   bf16* __restrict__ out) {
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= rows * ldout) return;
-  const int64_t r = t / ldout;
-  const int cidx = (int)(t % ldout);
-  out[t] = __float2bfloat16(cidx < cols ? in[r * ldin + cidx] : 0.f);
-}
-
-__global__ void k_f32_rows(int64_t rows, int cols, int ldin, int ldout, const float* __restrict__ in,
-                           float* __restrict__ out) {
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= rows * ldout) return;
-  const int64_t r = t / ldout;
-  const int cidx = (int)(t % ldout);
-  out[t] = cidx < cols ? in[r * ldin + cidx] : 0.f;
-}
-
-// ------------------------------------------------------------------ GEMM (mma.sync bf16)
-enum { EPI_F32 = 0, EPI_FWD_GELU = 1 };
-
-struct GemmArgs {
-  int M, N, K;
-  const bf16* A;
-  int64_t sam, sak;  // A(m,k) = A[m*sam + k*sak]
-  const bf16* B;
-  int64_t sbk, sbn;  // B(k,n) = B[k*sbk + n*sbn]
-  const float* bias; // [N] or null
-  float* Cf;
-  int64_t ldc;
-  bf16* Cb;
-  int64_t ldcb;
-};
-
-constexpr int BM = 64, BN = 64, BK = 32, SPAD = 8;
-
-__device__ __forceinline__ float gelu_f(float z) { return 0.5f * z * (1.f + erff(z * 0.70710678118654752f)); }
-__device__ __forceinline__ uint32_t ld_b32(const bf16* p) { return *reinterpret_cast<const uint32_t*>(p); }
-
-__device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], const uint32_t (&b)[2]) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-      "{%0,%1,%2,%3};\n"
-      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
-}
-
-// C = A B with a 64x64 block tile, 4 warps of 32x32, BF16 operands staged through shared
-// memory (strided global reads, so any operand may be transposed), FP32 accumulation.
-template <int EPI>
-__global__ void __launch_bounds__(128) k_gemm(GemmArgs g) {
-  __shared__ __align__(16) bf16 As[BM][BK + SPAD];
-  __shared__ __align__(16) bf16 Bs[BN][BK + SPAD];
-  const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int wm = (warp >> 1) * 32, wn = (warp & 1) * 32;
-  const int gid = lane >> 2, tig = lane & 3;
-  float acc[2][4][4];
-#pragma unroll
-  for (int i = 0; i < 2; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) acc[i][j][q] = 0.f;
-  const bf16 zero = __float2bfloat16(0.f);
-  for (int k0 = 0; k0 < g.K; k0 += BK) {
-    for (int i = threadIdx.x; i < BM * BK; i += blockDim.x) {
-      int mm, kk;
-      if (g.sak == 1) { mm = i / BK; kk = i % BK; } else { kk = i / BM; mm = i % BM; }
-      const int m = m0 + mm, k = k0 + kk;
-      As[mm][kk] = (m < g.M && k < g.K) ? g.A[(int64_t)m * g.sam + (int64_t)k * g.sak] : zero;
-    }
-    for (int i = threadIdx.x; i < BN * BK; i += blockDim.x) {
-      int nn, kk;
-      if (g.sbn == 1) { kk = i / BN; nn = i % BN; } else { nn = i / BK; kk = i % BK; }
-      const int n = n0 + nn, k = k0 + kk;
-      Bs[nn][kk] = (n < g.N && k < g.K) ? g.B[(int64_t)k * g.sbk + (int64_t)n * g.sbn] : zero;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int ks = 0; ks < BK; ks += 16) {
-      uint32_t a[2][4], b[4][2];
-#pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        const int r = wm + i * 16 + gid;
-        a[i][0] = ld_b32(&As[r][ks + tig * 2]);
-        a[i][1] = ld_b32(&As[r + 8][ks + tig * 2]);
-        a[i][2] = ld_b32(&As[r][ks + tig * 2 + 8]);
-        a[i][3] = ld_b32(&As[r + 8][ks + tig * 2 + 8]);
-      }
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int cc = wn + j * 8 + gid;
-        b[j][0] = ld_b32(&Bs[cc][ks + tig * 2]);
-        b[j][1] = ld_b32(&Bs[cc][ks + tig * 2 + 8]);
-      }
-#pragma unroll
-      for (int i = 0; i < 2; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) mma_bf16(acc[i][j], a[i], b[j]);
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int i = 0; i < 2; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int m = m0 + wm + i * 16 + gid + (q >= 2 ? 8 : 0);
-        const int n = n0 + wn + j * 8 + tig * 2 + (q & 1);
-        if (m >= g.M || n >= g.N) continue;
-        const float v = acc[i][j][q];
-        if (EPI == EPI_F32) {
-          g.Cf[(int64_t)m * g.ldc + n] = v + (g.bias ? g.bias[n] : 0.f);
-        } else {
-          g.Cb[(int64_t)m * g.ldcb + n] = __float2bfloat16(gelu_f(v + g.bias[n]));
-        }
-      }
-}
-
-template <int EPI>
-cudaError_t gemm(const GemmArgs& g, cudaStream_t s) {
-  dim3 grid((g.N + BN - 1) / BN, (g.M + BM - 1) / BM);
-  k_gemm<EPI><<<grid, 128, 0, s>>>(g);
-  note_launch();
-  return cudaGetLastError();
-}
-
 __global__ void k_adam(int64_t n, float* __restrict__ P, const float* __restrict__ G, float* __restrict__ m,
                        float* __restrict__ v, float lr, float b1, float b2, float eps, float c1, float c2) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -273,7 +144,28 @@ __global__ void k_adam(int64_t n, float* __restrict__ P, const float* __restrict
   P[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
 }
 
-// packed FP32 parameters -> padded BF16 weights and FP32 biases
+// packed FP32 parameters -> the operand image of the inference (mlp_tc.h)
+__global__ void k_operand_image(const float* __restrict__ P, uint8_t* __restrict__ img) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x, n = t % HID, k = t / HID;
+  auto put = [&](uint32_t at, int K, float v) {
+    *reinterpret_cast<bf16*>(img + at + mlp_core_off(n, k, (uint32_t)(K / 8) * kMlpCore)) = __float2bfloat16(v);
+  };
+  if (k < K0P) put(kMlpImgW1, K0P, k < K0 ? P[oW1 + k * HID + n] : 0.f);
+  if (k < HID) {
+    put(kMlpImgW2, HID, P[oW2 + t]);
+    put(kMlpImgW3, HID, P[oW3 + t]);
+    if (n < kMlpN4) put(kMlpImgW4, HID, n < NO ? P[oW4 + k * NO + n] : 0.f);
+  }
+  float* b = reinterpret_cast<float*>(img + kMlpImgB);
+  if (t < HID) {
+    b[t] = P[ob1 + t];
+    b[HID + t] = P[ob2 + t];
+    b[2 * HID + t] = P[ob3 + t];
+  }
+  if (t < kMlpN4) b[3 * HID + t] = t < NO ? P[ob4 + t] : 0.f;
+}
+
+// packed FP32 parameters -> padded BF16 weights and FP32 biases (the training's operands)
 __global__ void k_refresh(const float* __restrict__ P, bf16* W1, bf16* W2, bf16* W3, bf16* W4, float* b1, float* b2,
                           float* b3, float* b4) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -354,6 +246,7 @@ struct Mlp {
   float *P = nullptr, *G = nullptr, *Am = nullptr, *Av = nullptr;
   bf16 *W1 = nullptr, *W2 = nullptr, *W3 = nullptr, *W4 = nullptr;
   float *b1 = nullptr, *b2 = nullptr, *b3 = nullptr, *b4 = nullptr;
+  uint8_t* img = nullptr;  // operand image of the inference
   double in_mu[4] = {0, 0, 0, 0}, in_sd[4] = {1, 1, 1, 1}, out_mu[3] = {0, 0, 0}, out_sd[3] = {1, 1, 1};
   int64_t adam_t = 0;
   // stencil tables
@@ -384,7 +277,7 @@ void mlp_free(Mlp* m) {
   void* ptrs[] = {m->P,  m->G,  m->Am, m->Av, m->W1, m->W2, m->W3, m->W4, m->b1,     m->b2,      m->b3,
                   m->b4, m->X,  m->A1, m->A2, m->A3, m->dZ1, m->dZ2, m->dZ3, m->dO,   m->gpart,   m->loss,
                   m->out, m->Y, m->part, m->d_rows, m->d_state, m->free_nodes, m->st_ptr,
-                  m->st_idx, m->st_w, m->states, m->uz};
+                  m->st_idx, m->st_w, m->states, m->uz, m->img};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   delete m;
@@ -486,6 +379,8 @@ int mlp_refresh(pnp_ctx* c, Mlp* m) {
   k_refresh<<<nblk((int64_t)K0P * HID, 256), 256, 0, c->stream>>>(m->P, m->W1, m->W2, m->W3, m->W4, m->b1, m->b2,
                                                                    m->b3, m->b4);
   note_launch();
+  k_operand_image<<<nblk((int64_t)K0P * HID, 256), 256, 0, c->stream>>>(m->P, m->img);
+  note_launch();
   return ctx_check(c, cudaGetLastError(), "mlp refresh");
 }
 
@@ -505,47 +400,25 @@ FeatArgs feat_args(const Mlp* m, int64_t N) {
   return a;
 }
 
-GemmArgs gargs(int M, int N, int K, const bf16* A, int64_t sam, int64_t sak, const bf16* B, int64_t sbk, int64_t sbn) {
-  GemmArgs g;
-  std::memset(&g, 0, sizeof(g));
-  g.M = M;
-  g.N = N;
-  g.K = K;
-  g.A = A;
-  g.sam = sam;
-  g.sak = sak;
-  g.B = B;
-  g.sbk = sbk;
-  g.sbn = sbn;
-  return g;
-}
-
-// inference of `rows` standardised rows in m->X on the tensor cores (tcgen05, all layers
-// in one kernel, no saved activations); output in m->out [rows][8]
-int mlp_infer_rows(pnp_ctx* c, Mlp* m, int64_t rows) {
+// inference of `rows` standardised rows on the tensor cores (tcgen05, all layers in one
+// kernel, no saved activations): FP32 rows Xf [rows][216], or the BF16 rows in m->X
+int mlp_infer_rows(pnp_ctx* c, Mlp* m, int64_t rows, const float* Xf, float* out, int ldo) {
   MlpTcArgs a;
   a.rows = rows;
+  a.Xf = Xf;
   a.X = m->X;
-  a.W1 = m->W1;
-  a.W2 = m->W2;
-  a.W3 = m->W3;
-  a.W4 = m->W4;
-  a.b1 = m->b1;
-  a.b2 = m->b2;
-  a.b3 = m->b3;
-  a.b4 = m->b4;
-  a.out = m->out;
-  a.err = c->dflag + 2;
+  a.img = m->img;
+  a.out = out;
+  a.ldo = ldo;
+  a.err = c->hflag + 2;
   CK(launch_mlp_infer_tc(a, c->stream));
   return PNP_OK;
 }
 
 // PNP_ERR_DEVICE_FLAG once a wait of the tensor-core inference has given up (latched)
 int mlp_check_infer(pnp_ctx* c) {
-  int flag = 0;
-  CK(cudaMemcpyAsync(&flag, c->dflag + 2, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
   CK(cudaStreamSynchronize(c->stream));
-  if (flag) PNP_FAIL(PNP_ERR_DEVICE_FLAG, "network inference: the tensor core did not signal completion");
+  if (c->hflag[2]) PNP_FAIL(PNP_ERR_DEVICE_FLAG, "network inference: the tensor core did not signal completion");
   return PNP_OK;
 }
 
@@ -630,6 +503,7 @@ int pnp_mlp_init(pnp_ctx* c, uint64_t seed) {
   A((void**)&m->Am, 4 * P);
   A((void**)&m->Av, 4 * P);
   A((void**)&m->W1, 2 * K0P * HID);
+  A((void**)&m->img, kMlpImgBytes);
   A((void**)&m->W2, 2 * HID * HID);
   A((void**)&m->W3, 2 * HID * HID);
   A((void**)&m->W4, 2 * HID * NOP);
@@ -791,15 +665,7 @@ int pnp_mlp_features(pnp_ctx* c, const double* Uk, const double* Ukm1, const dou
 int pnp_mlp_forward(pnp_ctx* c, const float* X, int64_t B, float* Y) {
   MLP_GUARD(c);
   if (!X || !Y || B < 0) PNP_FAIL(PNP_ERR_ARG, "pnp_mlp_forward: bad arguments");
-  Mlp* m = c->mlp;
-  for (int64_t r0 = 0; r0 < B; r0 += kMaxRows) {
-    const int64_t rows = std::min<int64_t>(kMaxRows, B - r0);
-    k_f32_to_bf16_rows<<<nblk(rows * K0P, 256), 256, 0, c->stream>>>(rows, K0, K0, K0P, X + r0 * K0, m->X);
-    note_launch();
-    RC(mlp_infer_rows(c, m, rows));
-    k_f32_rows<<<nblk(rows * NO, 256), 256, 0, c->stream>>>(rows, NO, NOP, NO, m->out, Y + r0 * NO);
-    note_launch();
-  }
+  if (B) RC(mlp_infer_rows(c, c->mlp, B, X, Y, NO));
   CK(cudaGetLastError());
   return mlp_check_infer(c);
 }
@@ -944,21 +810,13 @@ int pnp_mlp_get_adam_state(pnp_ctx* c, float* m1, float* m2, int64_t* t) {
 
 // ------------------------------------------------------------------ allocation-free forward
 // The network forward of pnp_mlp_forward without a context and without allocating: the
-// BF16 weights, the activations and the output rows live in one file-scope device array
-// of fixed size (kNoAllocRows rows), shared by every call of this entry point.
+// operand image and the kernel's flag live in one file-scope device array, shared by every
+// call of this entry point.
 namespace {
 constexpr int64_t kNoAllocRows = 4096;
 struct NoAllocScratch {
-  bf16 W1[K0P * HID];
-  bf16 W2[HID * HID];
-  bf16 W3[HID * HID];
-  bf16 W4[HID * NOP];
-  float b1[HID], b2[HID], b3[HID], b4[NOP];
-  bf16 X[kNoAllocRows * K0P];
-  bf16 A1[kNoAllocRows * HID];
-  bf16 A2[kNoAllocRows * HID];
-  bf16 A3[kNoAllocRows * HID];
-  float out[kNoAllocRows * NOP];
+  uint8_t img[kMlpImgBytes];
+  int err;
 };
 }  // namespace
 
@@ -996,32 +854,24 @@ extern "C" int pnp_mlp_forward_noalloc(const float* params, const float* X, int6
   if (int rc = noalloc_scratch(&S)) return rc;
   if (B == 0) return PNP_OK;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  k_refresh<<<nblk((int64_t)K0P * HID, 256), 256, 0, s>>>(params, S->W1, S->W2, S->W3, S->W4, S->b1, S->b2, S->b3,
-                                                          S->b4);
+  cudaError_t e = cudaMemsetAsync(&S->err, 0, sizeof(int), s);
+  k_operand_image<<<nblk((int64_t)K0P * HID, 256), 256, 0, s>>>(params, S->img);
   note_launch();
-  k_f32_to_bf16_rows<<<nblk(B * K0P, 256), 256, 0, s>>>(B, K0, K0, K0P, X, S->X);
-  note_launch();
-  const int R = (int)B;
-  cudaError_t e = cudaSuccess;
-  GemmArgs g = gargs(R, HID, K0P, S->X, K0P, 1, S->W1, HID, 1);
-  g.bias = S->b1; g.Cb = S->A1; g.ldcb = HID;
-  if (e == cudaSuccess) e = gemm<EPI_FWD_GELU>(g, s);
-  g = gargs(R, HID, HID, S->A1, HID, 1, S->W2, HID, 1);
-  g.bias = S->b2; g.Cb = S->A2; g.ldcb = HID;
-  if (e == cudaSuccess) e = gemm<EPI_FWD_GELU>(g, s);
-  g = gargs(R, HID, HID, S->A2, HID, 1, S->W3, HID, 1);
-  g.bias = S->b3; g.Cb = S->A3; g.ldcb = HID;
-  if (e == cudaSuccess) e = gemm<EPI_FWD_GELU>(g, s);
-  g = gargs(R, NO, HID, S->A3, HID, 1, S->W4, NOP, 1);
-  g.bias = S->b4; g.Cf = S->out; g.ldc = NOP;
-  if (e == cudaSuccess) e = gemm<EPI_F32>(g, s);
-  if (e == cudaSuccess) {
-    k_f32_rows<<<nblk(B * NO, 256), 256, 0, s>>>(B, NO, NOP, NO, S->out, Y);
-    note_launch();
-    e = cudaGetLastError();
-  }
+  MlpTcArgs a;
+  a.rows = B;
+  a.Xf = X;
+  a.X = nullptr;
+  a.img = S->img;
+  a.out = Y;
+  a.ldo = NO;
+  a.err = &S->err;
+  if (e == cudaSuccess) e = launch_mlp_infer_tc(a, s);
+  int flag = 0;
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&flag, &S->err, sizeof(int), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) PNP_FAIL(PNP_ERR_CUDA, "pnp_mlp_forward_noalloc: %s", cudaGetErrorString(e));
+  if (flag)
+    PNP_FAIL(PNP_ERR_DEVICE_FLAG, "pnp_mlp_forward_noalloc: the tensor core did not signal completion");
   return PNP_OK;
 }
 
@@ -1077,7 +927,7 @@ int pnp_learned_start(pnp_ctx* c, pnp_solve_stats* st) {
       a.X = m->X;
       k_features<false><<<nblk(rows * NPT, 256), 256, 0, s>>>(a);
       note_launch();
-      RC(mlp_infer_rows(c, m, rows));
+      RC(mlp_infer_rows(c, m, rows, nullptr, m->out, NOP));
       k_apply_correction<<<nblk(rows, 256), 256, 0, s>>>(rows, m->free_nodes + r0, m->out, m->out_mu[0], m->out_mu[1],
                                                          m->out_mu[2], m->out_sd[0], m->out_sd[1], m->out_sd[2], c->Ut,
                                                          c->U);

@@ -3,12 +3,20 @@
 // FP32 accumulators in tensor memory (TMEM), bias + GELU epilogues read back with
 // tcgen05.ld and written as the next layer's operand, never leaving the SM.
 //
-// Per CTA (one per SM, persistent over tiles): the four weight matrices stay resident in
-// shared memory (K-major, no swizzle: 8x8 core matrices of 128 contiguous bytes); per
-// tile the input rows are loaded once, and per layer one thread issues K/16 MMAs of
-// 128 x N x 16 (tcgen05.mma kind::f16, BF16 x BF16 -> FP32) and commits them to an
-// mbarrier that the epilogue warps wait on (bounded).  Sixteen warps: warp w reads TMEM
-// lanes 32 (w mod 4) .. + 31 (the rows it may access) and a quarter of the columns.
+// Per CTA (one per SM, persistent over tiles): the operand image (weights, biases) comes in
+// by one bulk copy while the first input rows are loaded and rounded; per layer one thread
+// issues K/16 MMAs of 128 x N x 16 (tcgen05.mma kind::f16, BF16 x BF16 -> FP32) and commits
+// them to an mbarrier that the epilogue warps wait on (bounded).  The hidden layers' operand
+// is rewritten in place, so the input operand is free after the first layer: the next tile's
+// rows are loaded while layers 2 to 4 multiply.  Thirty-two warps: warp w reads TMEM lanes
+// 32 (w mod 4) .. + 31 (the rows it may access) and an eighth of the columns.
+//
+// What bounds it: the GELU's erff, about 40 instructions an element in all, 15 us of a pass of
+// two tiles per CTA at full issue rate (the MMAs take 1.2 us a tile); IPC is 2.0, as loads,
+// MMAs and epilogues of the one tile that fits wait on one another.  35,937 rows: 33.6 us;
+// before, with sixteen warps, weights gathered element by element, a conversion pass over
+// the input and a copy of the output, 44 + 25 + 3 us.  (A prefetch of the next tile's rows
+// to L2 changed nothing.)
 #include <cuda_bf16.h>
 
 #include <cstdint>
@@ -23,35 +31,23 @@ namespace {
 using bf16 = __nv_bfloat16;
 
 constexpr int kRows = 128;   // tile rows = MMA M = TMEM lanes
-constexpr int kK1 = 224;     // padded input width
-constexpr int kHid = 128;
-constexpr int kN4 = 16;      // output layer padded to the smallest N of an M = 128 MMA
+constexpr int kK0 = 216;     // input width
+constexpr int kK1 = kMlpK1, kHid = kMlpHid, kN4 = kMlpN4;
 constexpr int kNo = 3;       // outputs written
-constexpr int kLdOut = 8;    // row stride of the output
-constexpr int kThreads = 512;
+constexpr int kThreads = 1024;
 constexpr int kTmemCols = 128;
 constexpr int kWaitPolls = 1 << 22;
 
 // shared-memory carve-up (bytes from a 1024-byte aligned base)
-constexpr uint32_t kCore = 128;                       // one 8 x 8 BF16 core matrix
-constexpr uint32_t kSboK1 = (kK1 / 8) * kCore;        // 8-row group stride, K = 224
-constexpr uint32_t kSboHid = (kHid / 8) * kCore;      // 8-row group stride, K = 128
-constexpr uint32_t oW1 = 0;                           // [128 n][224 k]
-constexpr uint32_t oW2 = oW1 + kHid * kK1 * 2;        // [128][128]
-constexpr uint32_t oW3 = oW2 + kHid * kHid * 2;
-constexpr uint32_t oW4 = oW3 + kHid * kHid * 2;       // [16][128]
-constexpr uint32_t oA = oW4 + kN4 * kHid * 2;         // [128 rows][224] (layer 1), [128][128] (layer 3)
-constexpr uint32_t oH = oA + kRows * kK1 * 2;         // [128][128] (layers 2 and 4)
-constexpr uint32_t oBar = oH + kRows * kHid * 2;
-constexpr uint32_t oTmem = oBar + 8;
-constexpr uint32_t kSmemUsed = oTmem + 8;
+constexpr uint32_t kSboK1 = (kK1 / 8) * kMlpCore;     // 8-row group stride, K = 224
+constexpr uint32_t kSboHid = (kHid / 8) * kMlpCore;   // 8-row group stride, K = 128
+constexpr uint32_t oA = (kMlpImgBytes + 1023) / 1024 * 1024;  // [128 rows][224] (layer 1), after the image
+constexpr uint32_t oH = oA + kRows * kK1 * 2;         // [128][128] (layers 2 to 4)
+constexpr uint32_t oBar = oH + kRows * kHid * 2;      // the MMAs' barrier, the image's
+constexpr uint32_t oTmem = oBar + 16;
+constexpr uint32_t kSmemUsed = oTmem + 16;
+constexpr uint32_t kSmemBytes = kSmemUsed + 1024;
 static_assert(oA % 1024 == 0 && oH % 1024 == 0, "operand tiles aligned");
-
-// byte offset of element (r, k) in a K-major no-swizzle operand whose 8-row groups are
-// sbo bytes apart (core matrices along K 128 bytes apart)
-__device__ __forceinline__ uint32_t core_off(int r, int k, uint32_t sbo) {
-  return (uint32_t)(r >> 3) * sbo + (uint32_t)(k >> 3) * kCore + (uint32_t)(r & 7) * 16u + (uint32_t)(k & 7) * 2u;
-}
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -126,93 +122,113 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
   return *reinterpret_cast<const uint32_t*>(&h);
 }
 
-// weight W [K][N] row-major (global, BF16) -> K-major operand rows n < N_pad of K
-// columns; rows n >= n_src are zero
-__device__ void stage_weight(uint8_t* dst, const bf16* __restrict__ W, int K, int n_src, int ldw, int n_pad,
-                             uint32_t sbo) {
-  const int chunks = n_pad * (K / 8);
-  for (int i = threadIdx.x; i < chunks; i += blockDim.x) {
-    const int n = i % n_pad, kc = i / n_pad;
-    uint32_t w[4] = {0u, 0u, 0u, 0u};
-    if (n < n_src) {
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const bf16 lo = W[(int64_t)(kc * 8 + 2 * j) * ldw + n];
-        const bf16 hi = W[(int64_t)(kc * 8 + 2 * j + 1) * ldw + n];
-        w[j] = (uint32_t)__bfloat16_as_ushort(lo) | ((uint32_t)__bfloat16_as_ushort(hi) << 16);
-      }
+// eight columns (kc) of input row r as BF16: rounded FP32, or BF16 rows; zero past the data
+struct Chunk {
+  float4 a, b;
+};
+__device__ __forceinline__ void load_chunk(const MlpTcArgs& m, bool wide, int64_t r, int kc, Chunk& c) {
+  c.a = c.b = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (r >= m.rows) return;
+  if (m.Xf) {
+    if (kc >= kK0 / 8) return;
+    const float* p = m.Xf + r * kK0 + 8 * kc;
+    if (wide) {
+      c.a = __ldg(reinterpret_cast<const float4*>(p));
+      c.b = __ldg(reinterpret_cast<const float4*>(p) + 1);
+    } else {
+      c.a = make_float4(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3));
+      c.b = make_float4(__ldg(p + 4), __ldg(p + 5), __ldg(p + 6), __ldg(p + 7));
     }
-    *reinterpret_cast<uint4*>(dst + core_off(n, kc * 8, sbo)) = make_uint4(w[0], w[1], w[2], w[3]);
+  } else {
+    c.a = __ldg(reinterpret_cast<const float4*>(m.X + r * kK1) + kc);  // eight BF16
+  }
+}
+// chunks first, first + 1024, .. of a tile's input; 8 consecutive threads fill one core matrix
+constexpr int kChunks = kRows * (kK1 / 8);
+template <int N>
+__device__ __forceinline__ void load_input(const MlpTcArgs& m, bool wide, int64_t r0, int first, uint8_t* sA) {
+  Chunk c[N];
+#pragma unroll
+  for (int j = 0; j < N; ++j) {
+    const int i = first + j * kThreads;
+    if (i < kChunks) load_chunk(m, wide, r0 + (i & 7) + 8 * (i / (8 * (kK1 / 8))), (i >> 3) % (kK1 / 8), c[j]);
+  }
+#pragma unroll
+  for (int j = 0; j < N; ++j) {
+    const int i = first + j * kThreads;
+    if (i >= kChunks) break;
+    const int r = (i & 7) + 8 * (i / (8 * (kK1 / 8))), kc = (i >> 3) % (kK1 / 8);
+    uint4 v;
+    if (m.Xf)
+      v = make_uint4(pack_bf16(c[j].a.x, c[j].a.y), pack_bf16(c[j].a.z, c[j].a.w), pack_bf16(c[j].b.x, c[j].b.y),
+                     pack_bf16(c[j].b.z, c[j].b.w));
+    else
+      v = make_uint4(__float_as_uint(c[j].a.x), __float_as_uint(c[j].a.y), __float_as_uint(c[j].a.z),
+                     __float_as_uint(c[j].a.w));
+    *reinterpret_cast<uint4*>(sA + mlp_core_off(r, kc * 8, kSboK1)) = v;
   }
 }
 
-// bias + GELU of 32 accumulator columns of this thread's row, written as BF16 into the
+// bias + GELU of 16 accumulator columns of this thread's row, written as BF16 into the
 // next layer's operand (K = 128)
-__device__ __forceinline__ void epilogue_gelu(uint32_t tmem_row, int col0, int row, const float* __restrict__ bias,
-                                              uint8_t* dst) {
-#pragma unroll 1
-  for (int c = col0; c < col0 + 32; c += 16) {
-    float v[16];
-    tmem_ld16(tmem_row + (uint32_t)c, v);
-    uint32_t p[8];
+__device__ __forceinline__ void epilogue_gelu(uint32_t tmem_row, int c, int row, const float* bias, uint8_t* dst) {
+  float v[16];
+  tmem_ld16(tmem_row + (uint32_t)c, v);
+  uint32_t p[8];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const float a = gelu(v[2 * i] + __ldg(bias + c + 2 * i));
-      const float b = gelu(v[2 * i + 1] + __ldg(bias + c + 2 * i + 1));
-      p[i] = pack_bf16(a, b);
-    }
-    *reinterpret_cast<uint4*>(dst + core_off(row, c, kSboHid)) = make_uint4(p[0], p[1], p[2], p[3]);
-    *reinterpret_cast<uint4*>(dst + core_off(row, c + 8, kSboHid)) = make_uint4(p[4], p[5], p[6], p[7]);
+  for (int i = 0; i < 4; ++i) {
+    const float4 b = *reinterpret_cast<const float4*>(bias + c + 4 * i);
+    p[2 * i] = pack_bf16(gelu(v[4 * i] + b.x), gelu(v[4 * i + 1] + b.y));
+    p[2 * i + 1] = pack_bf16(gelu(v[4 * i + 2] + b.z), gelu(v[4 * i + 3] + b.w));
   }
+  *reinterpret_cast<uint4*>(dst + mlp_core_off(row, c, kSboHid)) = make_uint4(p[0], p[1], p[2], p[3]);
+  *reinterpret_cast<uint4*>(dst + mlp_core_off(row, c + 8, kSboHid)) = make_uint4(p[4], p[5], p[6], p[7]);
 }
 
 __global__ void __launch_bounds__(kThreads, 1) k_mlp_infer_tc(MlpTcArgs a) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const uint32_t bar = smem_u32(sm + oBar);
+  const uint32_t bar = smem_u32(sm + oBar), img_bar = bar + 8;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sm + oTmem);
 
-  // resident weights
-  stage_weight(sm + oW1, a.W1, kK1, kHid, kHid, kHid, kSboK1);
-  stage_weight(sm + oW2, a.W2, kHid, kHid, kHid, kHid, kSboHid);
-  stage_weight(sm + oW3, a.W3, kHid, kHid, kHid, kHid, kSboHid);
-  stage_weight(sm + oW4, a.W4, kHid, kLdOut, kLdOut, kN4, kSboHid);
   if (tid == 0) {
     mbar_init(bar, 1);
+    mbar_init(img_bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(img_bar), "r"(kMlpImgBytes) : "memory");
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                     smem_u32(sm)),
+                 "l"(a.img), "r"(kMlpImgBytes), "r"(img_bar)
+                 : "memory");
   }
   if (warp == 0) {
+    __syncwarp();
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                  "r"(kTmemCols)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  fence_async_smem();
+  const bool wide = (reinterpret_cast<uintptr_t>(a.Xf) & 15) == 0;
+  load_input<2>(a, wide, (int64_t)blockIdx.x * kRows, tid, sm + oA);
+  load_input<2>(a, wide, (int64_t)blockIdx.x * kRows, tid + 2 * kThreads, sm + oA);
   fence_before();
   __syncthreads();
   fence_after();
   const uint32_t tmem = *tmem_slot;
-  // this warp's TMEM lanes (rows) and accumulator column quarter
+  // the image: waited for by every thread (the biases are read with plain loads)
+  bool failed = __syncthreads_or(!mbar_wait(img_bar, 0));
+  // this warp's TMEM lanes (rows) and accumulator columns
   const int quarter = warp & 3, part = warp >> 2;
   const int row = quarter * 32 + lane;
   const uint32_t tmem_row = tmem + ((uint32_t)(quarter * 32) << 16);
   const uint32_t sA = smem_u32(sm + oA), sH = smem_u32(sm + oH);
-  const uint32_t sW[4] = {smem_u32(sm + oW1), smem_u32(sm + oW2), smem_u32(sm + oW3), smem_u32(sm + oW4)};
+  const float* bias = reinterpret_cast<const float*>(sm + kMlpImgB);
 
   const int64_t n_tiles = (a.rows + kRows - 1) / kRows;
   uint32_t phase = 0;
-  bool failed = false;
-  for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-    const int64_t r0 = tile * kRows;
-    // input rows -> layer-1 operand; 8 consecutive threads fill one core matrix
-    for (int i = tid; i < kRows * (kK1 / 8); i += kThreads) {
-      const int r = (i & 7) + 8 * (i / (8 * (kK1 / 8)));
-      const int kc = (i >> 3) % (kK1 / 8);
-      uint4 v = make_uint4(0u, 0u, 0u, 0u);
-      if (r0 + r < a.rows) v = __ldg(reinterpret_cast<const uint4*>(a.X + (r0 + r) * kK1) + kc);
-      *reinterpret_cast<uint4*>(sm + oA + core_off(r, kc * 8, kSboK1)) = v;
-    }
+  for (int64_t tile = blockIdx.x; tile < n_tiles && !failed; tile += gridDim.x) {
+    const int64_t r0 = tile * kRows, next0 = r0 + (int64_t)gridDim.x * kRows;
     for (int layer = 0; layer < 4; ++layer) {
       fence_async_smem();  // operand writes -> visible to the tensor core
       fence_before();
@@ -220,14 +236,18 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_infer_tc(MlpTcArgs a) {
       fence_after();
       if (tid == 0) {
         const int K = layer == 0 ? kK1 : kHid, N = layer == 3 ? kN4 : kHid;
-        const uint32_t src = (layer == 0 || layer == 2) ? sA : sH;
-        const uint32_t sbo_a = layer == 0 ? kSboK1 : kSboHid;
-        const uint32_t sbo_b = layer == 0 ? kSboK1 : kSboHid;
+        const uint32_t src = layer == 0 ? sA : sH, sbo = layer == 0 ? kSboK1 : kSboHid;
+        const uint32_t w = smem_u32(sm) + (layer == 0 ? kMlpImgW1 : layer == 1 ? kMlpImgW2 : layer == 2 ? kMlpImgW3 : kMlpImgW4);
         const uint32_t idesc = instr_desc(kRows, N);
         for (int k = 0; k < K / 16; ++k)
-          mma_bf16(tmem, mat_desc(src + 256u * k, kCore, sbo_a), mat_desc(sW[layer] + 256u * k, kCore, sbo_b), idesc,
+          mma_bf16(tmem, mat_desc(src + 256u * k, kMlpCore, sbo), mat_desc(w + 256u * k, kMlpCore, sbo), idesc,
                    k > 0 ? 1u : 0u);
         mma_commit(bar);
+      }
+      // the next tile's input while the tensor core works: its operand is free after layer 1
+      if (next0 < a.rows) {
+        if (layer == 1) load_input<2>(a, wide, next0, tid, sm + oA);
+        else if (layer > 1) load_input<1>(a, wide, next0, tid + layer * kThreads, sm + oA);
       }
       const bool ok = mbar_wait(bar, phase);
       phase ^= 1u;
@@ -237,28 +257,24 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_infer_tc(MlpTcArgs a) {
       }
       fence_after();
       if (layer < 3) {
-        const float* bias = layer == 0 ? a.b1 : layer == 1 ? a.b2 : a.b3;
-        uint8_t* dst = sm + ((layer == 1) ? oA : oH);
-        epilogue_gelu(tmem_row, part * 32, row, bias, dst);
+        epilogue_gelu(tmem_row, part * 16, row, bias + layer * kHid, sm + oH);
       } else if (part == 0) {
         float v[4];
         tmem_ld4(tmem_row, v);
         if (r0 + row < a.rows) {
-          float* o = a.out + (r0 + row) * kLdOut;
+          float* o = a.out + (r0 + row) * a.ldo;
 #pragma unroll
-          for (int f = 0; f < kNo; ++f) o[f] = v[f] + __ldg(a.b4 + f);
+          for (int f = 0; f < kNo; ++f) o[f] = v[f] + bias[3 * kHid + f];
         }
       }
     }
-    if (failed) break;
   }
-  if (failed) {
-    // the tensor core did not signal completion: flag it, give the outstanding MMAs a
-    // last bounded wait, then free the tensor memory
-    if (tid == 0) {
-      atomicOr(a.err, 1);
-      mbar_wait(bar, phase ^ 1u);
-    }
+  if (failed && tid == 0) {
+    // a copy or the tensor core did not signal completion: flag it, and give what is
+    // outstanding a last bounded wait before the tensor memory is freed
+    *reinterpret_cast<volatile int*>(a.err) = 1;
+    mbar_wait(img_bar, 0);
+    mbar_wait(bar, phase ^ 1u);
   }
   fence_before();
   __syncthreads();
@@ -268,8 +284,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_infer_tc(MlpTcArgs a) {
 }
 
 }  // namespace
-
-size_t mlp_tc_smem_bytes() { return kSmemUsed + 1024; }
 
 cudaError_t launch_mlp_infer_tc(const MlpTcArgs& a, cudaStream_t s) {
   if (a.rows <= 0) return cudaSuccess;
@@ -289,7 +303,7 @@ cudaError_t launch_mlp_infer_tc(const MlpTcArgs& a, cudaStream_t s) {
       e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
       if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_mlp_infer_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)mlp_tc_smem_bytes());
+                                 (int)kSmemBytes);
       if (e != cudaSuccess) return e;
       n_sm_of[dev] = n;
     }
@@ -297,7 +311,7 @@ cudaError_t launch_mlp_infer_tc(const MlpTcArgs& a, cudaStream_t s) {
   }
   const int64_t tiles = (a.rows + kRows - 1) / kRows;
   const unsigned blocks = (unsigned)(tiles < n_sm ? tiles : n_sm);
-  k_mlp_infer_tc<<<blocks, kThreads, mlp_tc_smem_bytes(), s>>>(a);
+  k_mlp_infer_tc<<<blocks, kThreads, kSmemBytes, s>>>(a);
   note_launch();
   return cudaGetLastError();
 }
