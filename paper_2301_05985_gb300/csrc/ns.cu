@@ -59,6 +59,7 @@ struct NsArgs {
   const uint8_t* level;
   const int32_t* hang_par;
   const uint8_t* hang_np;
+  const uint8_t* faces;
   const T* X;          // [N][4] unknown / direction
   const T* adv;        // [N][4] v~ (slot 3 unused)
   const double* hv;    // [N][4] history (beta1 v^k + beta2 v^{k-1}) / dt (data kernel only)
@@ -115,24 +116,21 @@ __device__ __forceinline__ void load4(const int32_t* __restrict__ hpar, const ui
   d[0] = v.x; d[1] = v.y; d[2] = v.z; d[3] = v.w;
 }
 
-__device__ __forceinline__ void add4(double* out, int64_t id, const double (&r)[4], double wgt) {
-#pragma unroll
-  for (int f = 0; f < 4; ++f) atomicAdd(out + 4 * id + f, wgt * r[f]);
-}
-__device__ __forceinline__ void add4(float* out, int64_t id, const float (&r)[4], float wgt) {
-  atomicAdd(reinterpret_cast<float4*>(out) + id, make_float4(wgt * r[0], wgt * r[1], wgt * r[2], wgt * r[3]));
-}
-
-template <typename T>
-__device__ __forceinline__ void scatter_rows(const NsArgs<T>& A, int32_t id, const T (&r)[4]) {
-  if (id >= 0) {
-    add4(A.out, id, r, T(1));
-  } else {
+// the same from shared memory
+__device__ __forceinline__ void gather4(const int32_t* __restrict__ hpar, const uint8_t* __restrict__ hnp,
+                                        const float4* src, int32_t id, bool valid, float (&d)[4]) {
+  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (valid && id >= 0) v = src[id];
+  if (valid && id < 0) {
     const int32_t h = -id - 1;
-    const int np = A.hang_np[h];
-    const T wgt = np == 2 ? T(0.5) : T(0.25);
-    for (int p = 0; p < np; ++p) add4(A.out, A.hang_par[4 * h + p], r, wgt);
+    const int np = hnp[h];
+    const float w = np == 2 ? 0.5f : 0.25f;
+    for (int p = 0; p < np; ++p) {
+      const float4 a = src[hpar[4 * h + p]];
+      v.x += w * a.x; v.y += w * a.y; v.z += w * a.z; v.w += w * a.w;
+    }
   }
+  d[0] = v.x; d[1] = v.y; d[2] = v.z; d[3] = v.w;
 }
 
 // physical constants in the kernel's arithmetic type
@@ -141,28 +139,20 @@ struct NsK {
   C isc, kis, tau_t, cid, fb;  // 1/Sc, beta0/(Sc dt), 4/dt^2, C_I Sc^2 d, kappa / (2 Lambda^2)
 };
 
-// One lane per (element, corner): the lane's Gauss point is the one next to its corner.
-// DATA adds the history and body-force terms (the residual F = A X - b); without them
-// the kernel applies the matrix.  T: storage type of the vectors; C: arithmetic type (T,
-// or double-float for FP64 data: GB300 runs FP64 at 1/64 of the FP32 rate).  The
-// double-float matrix action is bound by the FP32 pipe: 1.41 ms before, 0.594 ms now per
-// launch on the membrane-band octree (971,776 elements), by the scaled operators, quick
-// sums and integer conversions of lane_ops.cuh and df32.cuh.
-// blocks per SM the register cap is set for (FP32: 40 registers without spills)
-template <typename T>
-constexpr int ns_min_blocks() {
-  return sizeof(T) == 4 ? 6 : 2;
+// Dirichlet / pin / inactive row of slot f at a free node (hanging nodes: faces bit 7)
+__device__ __forceinline__ bool ns_dir(const NsBc& bc, uint8_t fm, int64_t i, int f) {
+  if (f == 2 && bc.dim == 2) return true;
+  const bool d = (fm & bc.dir[f] & 0x3F) != 0;
+  return d || (f == 3 && i == bc.pin);
 }
-template <typename T, typename C, int D, bool DATA>
-__global__ void __launch_bounds__(kNsThreads, ns_min_blocks<T>()) k_ns_lanes(NsArgs<T> A, NsK<C> K) {
-  constexpr int NC = 1 << D;
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if ((t & ~int64_t(31)) / NC >= A.n_elem) return;  // shuffles need the whole warp
-  const int64_t e = t / NC;
-  const int c = (int)(t & (NC - 1));
-  const bool valid = e < A.n_elem;
-  const int32_t id = valid ? __ldg(A.conn + e * NC + c) : 0;
-  const int lev = valid ? A.level[e] : 0;
+
+// The NS rows at one lane (element, corner), whose Gauss point is the one next to its
+// corner, from the nodal values of the corner: x (v, p), as (advection), and with DATA hs
+// (history) and body (c+ - c-, phi).  r: the element vector's entries of the corner without
+// the factors (h/2)^D a^D beta (momentum) and (h/2)^D a^(2D-3) / h^3 (solenoidality).
+template <typename C, int D, bool DATA>
+__device__ __forceinline__ void lane_ns(const C (&xs)[4], const C (&as)[3], const C (&hs)[3], const C (&body)[2], int c,
+                                        int lev, const NsK<C>& K, C (&r)[4]) {
   // scaled quantities (lane_ops.cuh; v~ = v / a^D, g~ = reflected gradient h / a^(D-1)):
   //   V = (1/Sc) (a^(D-1) / h) v^ reflected (v^ the advection),  delta = a^2 h^2
   //   R~_i = (1/Sc) (kappa v~_i + h~_i) + V . g~v_i + s_i g~p_i / (a h)     (times a^D)
@@ -174,18 +164,15 @@ __global__ void __launch_bounds__(kNsThreads, ns_min_blocks<T>()) k_ns_lanes(NsA
 #pragma unroll
   for (int k = 0; k < 3; ++k) sg[k] = reflect_mask(c, k);
 
-  T xs[4], as[4];
-  load4(A.hang_par, A.hang_np, A.X, id, valid, xs);
-  load4(A.hang_par, A.hang_np, A.adv, id, valid, as);
   // (v_x, v_y) and (v_z, p) run as pairs, as do the test rows (0, 1) and (2, 3)
   using C2 = pair_t<C>;
   const C2 rho2 = both<C>(rho);
   C V[D], va[D], vv;
   {
-    const C2 v01 = lane_v<C2, D>(pair(to_compute<C>(as[0]), to_compute<C>(as[1])), rho2);
+    const C2 v01 = lane_v<C2, D>(pair(as[0], as[1]), rho2);
     va[0] = first(v01);
     va[1] = second(v01);
-    if constexpr (D == 3) va[2] = lane_v<C, D>(to_compute<C>(as[2]), rho);
+    if constexpr (D == 3) va[2] = lane_v<C, D>(as[2], rho);
   }
 #pragma unroll
   for (int i = 0; i < D; ++i) {
@@ -198,14 +185,14 @@ __global__ void __launch_bounds__(kNsThreads, ns_min_blocks<T>()) k_ns_lanes(NsA
   const C tau_s = (arg * tau_m) * const_pow2(1.0 / D, -2 * lev - 2, C(0));
   C2 v01, g01[3], v2p, g2p[3];
   C gp[3];
-  lane_vg<C2, D, true>(pair(to_compute<C>(xs[0]), to_compute<C>(xs[1])), rho2, v01, g01);
+  lane_vg<C2, D, true>(pair(xs[0], xs[1]), rho2, v01, g01);
   if constexpr (D == 3) {
-    lane_vg<C2, D, true>(pair(to_compute<C>(xs[2]), to_compute<C>(xs[3])), rho2, v2p, g2p);
+    lane_vg<C2, D, true>(pair(xs[2], xs[3]), rho2, v2p, g2p);
 #pragma unroll
     for (int k = 0; k < D; ++k) gp[k] = second(g2p[k]);
   } else {
     C unused;
-    lane_vg<C, D, false>(to_compute<C>(xs[3]), rho, unused, gp);
+    lane_vg<C, D, false>(xs[3], rho, unused, gp);
   }
   C div = reflect(first(g01[0]), sg[0]) + reflect(second(g01[1]), sg[1]);
   if constexpr (D == 3) div = div + reflect(first(g2p[2]), sg[2]);
@@ -222,8 +209,102 @@ __global__ void __launch_bounds__(kNsThreads, ns_min_blocks<T>()) k_ns_lanes(NsA
   }
   if constexpr (DATA) {
     // history h_i and the body force kappa/(2 Lambda^2) (c+ - c-) grad phi of the PNP state
-    double hs[4], u3[3] = {0.0, 0.0, 0.0};
-    load4(A.hang_par, A.hang_np, A.hv, id, valid, hs);
+    // f rho grad phi / a^D = (f a^(D-1) / h) rho~ s_i g~phi_i
+    C2 val, g[3];
+    lane_vg<C2, D, true>(pair(body[1], body[0]), rho2, val, g);
+    const C frho = const_pow2(ipow(kVal, D - 1), lev, C(0)) * (K.fb * second(val));
+    C gphi[3];
+#pragma unroll
+    for (int k = 0; k < D; ++k) gphi[k] = first(g[k]);
+    R01 = R01 + fma_q(both<C>(K.isc), lane_v<C2, D>(pair(hs[0], hs[1]), rho2),
+                    pair(reflect(frho * gphi[0], sg[0]), reflect(frho * gphi[1], sg[1])));
+    if constexpr (D == 3) R2 = R2 + fma_q(K.isc, lane_v<C, D>(hs[2], rho), reflect(frho * gphi[2], sg[2]));
+  }
+  constexpr double cd = kVal * kVal;
+  const int ed = -2 * lev;
+  const C tsd = tau_s * div;
+  const C2 rd01 = times_const2(R01, cd, ed), su01 = both<C>(tau_m) * rd01;
+  const C rd2 = times_const(R2, cd, ed), su2 = tau_m * rd2;
+  {
+    C2 Phi[3];
+#pragma unroll
+    for (int j = 0; j < D; ++j) Phi[j] = fma_q(su01, both<C>(V[j]), g01[j]);
+    Phi[0] = pair(first(Phi[0]) + reflect(tsd, sg[0]), second(Phi[0]));
+    Phi[1] = pair(first(Phi[1]), second(Phi[1]) + reflect(tsd, sg[1]));
+    const C2 t = lane_test<C2, D>(rd01, Phi, rho2);
+    r[0] = first(t);
+    r[1] = second(t);
+  }
+  C Pq[3] = {reflect(first(su01), sg[0]), reflect(second(su01), sg[1]), reflect(su2, sg[2])};
+  if constexpr (D == 3) {
+    C2 Phi[3];
+#pragma unroll
+    for (int j = 0; j < D; ++j) Phi[j] = pair(fma_q(su2, V[j], first(g2p[j])), Pq[j]);
+    Phi[2] = pair(first(Phi[2]) + reflect(tsd, sg[2]), second(Phi[2]));
+    const C2 t = lane_test<C2, D>(pair(rd2, times_const(div, cd, ed)), Phi, rho2);
+    r[2] = first(t);
+    r[3] = second(t);
+  } else {
+    r[2] = C(0);
+    r[3] = lane_test<C, D>(times_const(div, cd, ed), Pq, rho);
+  }
+}
+constexpr double ns_weight_c(int D, int f) { return f < 3 ? ipow(kVal, 2 * D - 2) : ipow(kVal, 2 * D - 3); }
+__device__ __forceinline__ int ns_weight_e(int D, int lev, int f) { return (f < 3 ? 2 : 3) * lev - D * (lev + 1); }
+
+// adds r to the rows of a node: with MASK not to constrained rows (k_ns_init wrote them),
+// without it to all (k_ns_smooth and k_ns_restrict pass over them)
+template <bool MASK>
+__device__ __forceinline__ void add_rows(const NsBc& bc, const uint8_t* __restrict__ faces, double* out, int64_t id,
+                                         const double (&r)[4], double w) {
+  const uint8_t fm = MASK ? faces[id] : 0;
+#pragma unroll
+  for (int f = 0; f < 4; ++f)
+    if (!MASK || !ns_dir(bc, fm, id, f)) atomicAdd(out + 4 * id + f, w * r[f]);
+}
+template <bool MASK>
+__device__ __forceinline__ void add_rows(const NsBc& bc, const uint8_t* __restrict__ faces, float* out, int64_t id,
+                                         const float (&r)[4], float w) {
+  const uint8_t fm = MASK ? faces[id] : 0;
+  float x[4];
+#pragma unroll
+  for (int f = 0; f < 4; ++f) x[f] = MASK && ns_dir(bc, fm, id, f) ? 0.f : w * r[f];
+  atomicAdd(reinterpret_cast<float4*>(out) + id, make_float4(x[0], x[1], x[2], x[3]));
+}
+
+// One lane per (element, corner).  T: storage type of the vectors; C: arithmetic type (T, or
+// double-float for FP64 data: GB300 runs FP64 at 1/64 of the FP32 rate).  DATA adds the
+// history and body-force terms (the residual F = A X - b); without them the kernel applies
+// the matrix.  The double-float matrix action is bound by the FP32 pipe: 1.41 ms before,
+// 0.594 ms now per launch on the membrane-band octree (971,776 elements), by the scaled
+// operators, quick sums and integer conversions of lane_ops.cuh and df32.cuh.
+template <typename T>
+constexpr int ns_min_blocks() {  // FP32: 40 registers without spills
+  return sizeof(T) == 4 ? 6 : 2;
+}
+template <typename T, typename C, int D, bool DATA, bool MASK>
+__global__ void __launch_bounds__(256, ns_min_blocks<T>()) k_ns_lanes(NsArgs<T> A, NsBc bc, NsK<C> K) {
+  constexpr int NC = 1 << D;
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if ((t & ~int64_t(31)) / NC >= A.n_elem) return;  // shuffles need the whole warp
+  const int64_t e = t / NC;
+  const int c = (int)(t & (NC - 1));
+  const bool valid = e < A.n_elem;
+  const int32_t id = valid ? __ldg(A.conn + e * NC + c) : 0;
+  const int lev = valid ? A.level[e] : 0;
+  C xs[4], as[3], hs[3], body[2], rr[4];
+  {
+    T x[4], a[4];
+    load4(A.hang_par, A.hang_np, A.X, id, valid, x);
+    load4(A.hang_par, A.hang_np, A.adv, id, valid, a);
+#pragma unroll
+    for (int f = 0; f < 4; ++f) xs[f] = to_compute<C>(x[f]);
+#pragma unroll
+    for (int f = 0; f < 3; ++f) as[f] = to_compute<C>(a[f]);
+  }
+  if constexpr (DATA) {
+    double h4[4], u3[3] = {0.0, 0.0, 0.0};
+    load4(A.hang_par, A.hang_np, A.hv, id, valid, h4);
     if (valid) {
       if (id >= 0) {
 #pragma unroll
@@ -239,84 +320,60 @@ __global__ void __launch_bounds__(kNsThreads, ns_min_blocks<T>()) k_ns_lanes(NsA
         }
       }
     }
-    // f rho grad phi / a^D = (f a^(D-1) / h) rho~ s_i g~phi_i
-    C2 val, g[3];
-    lane_vg<C2, D, true>(pair(to_compute<C>(u3[2]), to_compute<C>(u3[0] - u3[1])), rho2, val, g);
-    const C frho = const_pow2(ipow(kVal, D - 1), lev, C(0)) * (K.fb * second(val));
-    C gphi[3];
 #pragma unroll
-    for (int k = 0; k < D; ++k) gphi[k] = first(g[k]);
-    R01 = R01 + fma_q(both<C>(K.isc), lane_v<C2, D>(pair(to_compute<C>(hs[0]), to_compute<C>(hs[1])), rho2),
-                    pair(reflect(frho * gphi[0], sg[0]), reflect(frho * gphi[1], sg[1])));
-    if constexpr (D == 3) R2 = R2 + fma_q(K.isc, lane_v<C, D>(to_compute<C>(hs[2]), rho), reflect(frho * gphi[2], sg[2]));
+    for (int f = 0; f < 3; ++f) hs[f] = to_compute<C>(h4[f]);
+    body[0] = to_compute<C>(u3[0] - u3[1]);
+    body[1] = to_compute<C>(u3[2]);
   }
-  constexpr double cW = ipow(kVal, 2 * D - 2), cWp = ipow(kVal, 2 * D - 3), cd = kVal * kVal;
-  const int eW = 2 * lev - D * (lev + 1), eWp = eW + lev, ed = -2 * lev;
-  const C tsd = tau_s * div;
-  T r[4];
-  const C2 rd01 = times_const2(R01, cd, ed), su01 = both<C>(tau_m) * rd01;
-  const C rd2 = times_const(R2, cd, ed), su2 = tau_m * rd2;
-  {
-    C2 Phi[3];
-#pragma unroll
-    for (int j = 0; j < D; ++j) Phi[j] = fma_q(su01, both<C>(V[j]), g01[j]);
-    Phi[0] = pair(first(Phi[0]) + reflect(tsd, sg[0]), second(Phi[0]));
-    Phi[1] = pair(first(Phi[1]), second(Phi[1]) + reflect(tsd, sg[1]));
-    const C2 t = lane_test<C2, D>(rd01, Phi, rho2);
-    r[0] = times_const(to_storage<T>(first(t)), cW, eW);
-    r[1] = times_const(to_storage<T>(second(t)), cW, eW);
-  }
-  C Pq[3] = {reflect(first(su01), sg[0]), reflect(second(su01), sg[1]), reflect(su2, sg[2])};
-  if constexpr (D == 3) {
-    C2 Phi[3];
-#pragma unroll
-    for (int j = 0; j < D; ++j) Phi[j] = pair(fma_q(su2, V[j], first(g2p[j])), Pq[j]);
-    Phi[2] = pair(first(Phi[2]) + reflect(tsd, sg[2]), second(Phi[2]));
-    const C2 t = lane_test<C2, D>(pair(rd2, times_const(div, cd, ed)), Phi, rho2);
-    r[2] = times_const(to_storage<T>(first(t)), cW, eW);
-    r[3] = times_const(to_storage<T>(second(t)), cWp, eWp);
-  } else {
-    r[2] = T(0);
-    r[3] = times_const(to_storage<T>(lane_test<C, D>(times_const(div, cd, ed), Pq, rho)), cWp, eWp);
-  }
+  lane_ns<C, D, DATA>(xs, as, hs, body, c, lev, K, rr);
   if (!valid) return;
-  scatter_rows(A, id, r);
+  T r[4];
+#pragma unroll
+  for (int f = 0; f < 4; ++f)
+    r[f] = times_const(to_storage<T>(rr[f]), f < 3 ? ns_weight_c(D, 0) : ns_weight_c(D, 3), ns_weight_e(D, lev, f));
+  if (id >= 0) {
+    add_rows<MASK>(bc, A.faces, A.out, id, r, T(1));
+  } else {
+    const int32_t h = -id - 1;
+    const int np = A.hang_np[h];
+    const T wgt = np == 2 ? T(0.5) : T(0.25);
+    for (int p = 0; p < np; ++p) add_rows<MASK>(bc, A.faces, A.out, A.hang_par[4 * h + p], r, wgt);
+  }
 }
 
-// Dirichlet / pin rows (mode 0: X - g, the residual; 1: X, the matrix) of free nodes.
+// The rows before the element kernel: zero on weak-form rows, X - g (mode 0, the residual)
+// or X (mode 1, the matrix) on Dirichlet, pin and inactive rows, the constraints X_h -
+// sum_p w_p X_p on hanging rows (threads past N).
 template <typename T>
-__global__ void k_ns_rows(int64_t N, const uint8_t* __restrict__ faces, NsBc bc, const T* __restrict__ X,
-                          T* __restrict__ out, int mode) {
+__global__ void k_ns_init(RowArgs R, NsBc bc, const T* __restrict__ X, T* __restrict__ out, int mode) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= N) return;
-  const uint8_t fm = faces[i];
-  if (fm & 0x80) return;
+  T o[4];
+  int64_t id = i;
+  if (i < R.n_nodes) {
+    const uint8_t fm = R.faces[i];
+    if (fm & 0x80) return;
 #pragma unroll
-  for (int f = 0; f < 4; ++f) {
-    const unsigned msk = fm & bc.dir[f] & 0x3F;
-    bool dir = msk != 0;
-    double g = dir ? bc.val[31 - __clz(msk)][f] : 0.0;
-    if (f == 2 && bc.dim == 2) { dir = true; g = 0.0; }
-    if (f == 3 && !dir && i == bc.pin) dir = true;  // g = 0
-    if (dir) out[4 * i + f] = mode == 0 ? T(double(X[4 * i + f]) - g) : X[4 * i + f];
-  }
-}
-
-// constraint rows of hanging nodes: out_h = X_h - sum_p w_p X_p
-template <typename T>
-__global__ void k_ns_hanging_rows(int64_t H, const int32_t* __restrict__ hnode, const int32_t* __restrict__ hpar,
-                                  const uint8_t* __restrict__ hnp, const T* __restrict__ X, T* __restrict__ out) {
-  const int64_t h = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (h >= H) return;
-  const int np = hnp[h];
-  const T wgt = np == 2 ? T(0.5) : T(0.25);
-  const int64_t id = hnode[h];
+    for (int f = 0; f < 4; ++f) {
+      o[f] = T(0);
+      if (!ns_dir(bc, fm, i, f)) continue;
+      const unsigned msk = fm & bc.dir[f] & 0x3F;
+      const double g = msk && !(f == 2 && bc.dim == 2) ? bc.val[31 - __clz(msk)][f] : 0.0;
+      o[f] = mode == 0 ? T(double(X[4 * i + f]) - g) : X[4 * i + f];
+    }
+  } else {
+    const int64_t h = i - R.n_nodes;
+    if (h >= R.n_hanging) return;
+    const int np = R.hnp[h];
+    const T wgt = np == 2 ? T(0.5) : T(0.25);
+    id = R.hnode[h];
 #pragma unroll
-  for (int f = 0; f < 4; ++f) {
-    T s = X[4 * id + f];
-    for (int p = 0; p < np; ++p) s -= wgt * X[4 * (int64_t)hpar[4 * h + p] + f];
-    out[4 * id + f] = s;
+    for (int f = 0; f < 4; ++f) {
+      o[f] = X[4 * id + f];
+      for (int p = 0; p < np; ++p) o[f] -= wgt * X[4 * (int64_t)R.hpar[4 * h + p] + f];
+    }
   }
+#pragma unroll
+  for (int f = 0; f < 4; ++f) out[4 * id + f] = o[f];
 }
 
 // 4x4 diagonal block of the lane's own node: sum over the element's Gauss points q of
@@ -644,75 +701,113 @@ __global__ void k_ns_velocity(int64_t N, const double* __restrict__ X, double* _
 }
 
 // ------------------------------------------------------------------ multigrid pieces
-// Dirichlet / pin / inactive row of slot f at a free node (hanging nodes: faces bit 7)
-__device__ __forceinline__ bool ns_dir(const NsBc& bc, uint8_t fm, int64_t i, int f) {
-  if (f == 2 && bc.dim == 2) return true;
-  const bool d = (fm & bc.dir[f] & 0x3F) != 0;
-  return d || (f == 3 && i == bc.pin);
+// One sweep xn = xo + omega D^-1 (b - A xo), 4x4 blocks; the first one xn = omega D^-1 b.
+// Ax holds the element sums of every row: the constrained rows of A xo are put in here (xo on
+// Dirichlet, pin and inactive rows; the constraint on hanging rows, by threads past N), and Ax
+// is left zero for the next application, so that a sweep is two launches.  Two buffers, as
+// hanging rows read their parents' xo.
+__device__ __forceinline__ float4 sub4(const float4& a, const float4& b) {
+  return make_float4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w);
 }
-
-// x = omega D^-1 b (first sweep) or x += omega D^-1 (b - Ax), 4x4 blocks
-__global__ void k_ns_smooth(int64_t N, const float* __restrict__ Dinv, const float4* __restrict__ b,
-                            const float4* __restrict__ Ax, float4* __restrict__ x, float om, int first) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= N) return;
-  float4 r = b[i];
-  if (!first) {
-    const float4 a = Ax[i];
-    r = make_float4(r.x - a.x, r.y - a.y, r.z - a.z, r.w - a.w);
-  }
+// node i (or hanging node i - N) of a sweep.  All of a node's loads come before its stores:
+// one after another they took three times as long.
+__device__ __forceinline__ void smooth_row(const RowArgs& R, const NsBc& bc, const float* __restrict__ Dinv,
+                                           const float4* b, float4* Ax, const float4* xo, float4* xn, float om,
+                                           bool first, int64_t i) {
+  const bool node = i < R.n_nodes;
+  const int64_t h = i - R.n_nodes;
+  if (!node && (first || h >= R.n_hanging)) return;
+  if (!node) i = R.hnode[h];
   const float4* M = reinterpret_cast<const float4*>(Dinv) + 4 * i;
-  const float4 m0 = M[0], m1 = M[1], m2 = M[2], m3 = M[3];
-  const float4 d = make_float4(om * (m0.x * r.x + m0.y * r.y + m0.z * r.z + m0.w * r.w),
-                               om * (m1.x * r.x + m1.y * r.y + m1.z * r.z + m1.w * r.w),
-                               om * (m2.x * r.x + m2.y * r.y + m2.z * r.z + m2.w * r.w),
-                               om * (m3.x * r.x + m3.y * r.y + m3.z * r.z + m3.w * r.w));
-  if (first) {
-    x[i] = d;
-  } else {
-    const float4 o = x[i];
-    x[i] = make_float4(o.x + d.x, o.y + d.y, o.z + d.z, o.w + d.w);
+  const float4 m0 = __ldg(M), m1 = __ldg(M + 1), m2 = __ldg(M + 2), m3 = __ldg(M + 3);
+  const uint8_t fm = R.faces[i];
+  float4 r = b[i];
+  float4 a = make_float4(0.f, 0.f, 0.f, 0.f), o = a;
+  if (!first) {
+    a = Ax[i];
+    o = xo[i];
+    if (node && (fm & 0x80)) return;  // a thread past N has it
   }
+  if (node) {
+    Ax[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (ns_dir(bc, fm, i, 0)) a.x = o.x;
+    if (ns_dir(bc, fm, i, 1)) a.y = o.y;
+    if (ns_dir(bc, fm, i, 2)) a.z = o.z;
+    if (ns_dir(bc, fm, i, 3)) a.w = o.w;
+  } else {
+    const int np = R.hnp[h];
+    const float w = np == 2 ? 0.5f : 0.25f;
+    a = o;
+    for (int p = 0; p < np; ++p) {
+      const float4 v = xo[R.hpar[4 * h + p]];
+      a.x -= w * v.x; a.y -= w * v.y; a.z -= w * v.z; a.w -= w * v.w;
+    }
+  }
+  r = sub4(r, a);
+  xn[i] = make_float4(o.x + om * (m0.x * r.x + m0.y * r.y + m0.z * r.z + m0.w * r.w),
+                      o.y + om * (m1.x * r.x + m1.y * r.y + m1.z * r.z + m1.w * r.w),
+                      o.z + om * (m2.x * r.x + m2.y * r.y + m2.z * r.z + m2.w * r.w),
+                      o.w + om * (m3.x * r.x + m3.y * r.y + m3.z * r.z + m3.w * r.w));
+}
+__global__ void k_ns_smooth(RowArgs R, NsBc bc, const float* __restrict__ Dinv, const float4* __restrict__ b,
+                            float4* __restrict__ Ax, const float4* __restrict__ xo, float4* __restrict__ xn, float om,
+                            bool first) {
+  smooth_row(R, bc, Dinv, b, Ax, xo, xn, om, first, blockIdx.x * (int64_t)blockDim.x + threadIdx.x);
 }
 
 // out[j] = sum_q w_q (b - Ax)[col_q] over the fine rows that are weak-form equations
 // (Dirichlet, pin, inactive and hanging rows carry no element contributions); coarse
-// constrained rows are zero
-__global__ void k_ns_restrict(int64_t Nc, const int64_t* __restrict__ ptr, const int32_t* __restrict__ col,
-                              const float* __restrict__ w, const float4* __restrict__ b, const float4* __restrict__ Ax,
-                              const uint8_t* __restrict__ faces_f, NsBc bcf, const uint8_t* __restrict__ faces_c,
-                              NsBc bcc, float4* __restrict__ out) {
-  const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (j >= Nc) return;
+// constrained rows are zero.  Eight lanes of a warp per coarse node (27 terms and more, each
+// behind an index: one thread per node took 14 us on the smallest levels, 54 us on the first).
+// The loads of Ax, faces and b are plain: k_ns_tail's block has written Ax and b itself.
+struct NsTransfer {
+  const int64_t* ptr;
+  const int32_t* col;
+  const float* w;
+};
+__device__ __forceinline__ void restrict_row(int64_t Nc, const NsTransfer& T, const float4* b, const float4* Ax,
+                                             const uint8_t* faces_f, const NsBc& bcf, const uint8_t* faces_c,
+                                             const NsBc& bcc, float4* out, int64_t t) {
+  const int64_t j = t >> 3;
   float s[4] = {0.f, 0.f, 0.f, 0.f};
-  for (int64_t q = ptr[j]; q < ptr[j + 1]; ++q) {
-    const int64_t i = col[q];
-    const uint8_t ff = faces_f[i];
-    if (ff & 0x80) continue;
-    const float wq = w[q];
-    const float4 bi = b[i], ai = Ax[i];
-    const float r[4] = {bi.x - ai.x, bi.y - ai.y, bi.z - ai.z, bi.w - ai.w};
+  if (j < Nc) {
+    for (int64_t q = T.ptr[j] + (t & 7); q < T.ptr[j + 1]; q += 8) {
+      const int64_t i = T.col[q];
+      const uint8_t ff = faces_f[i];
+      const float wq = T.w[q];
+      const float4 d = sub4(b[i], Ax[i]);
+      const float r[4] = {d.x, d.y, d.z, d.w};
+      if (ff & 0x80) continue;
 #pragma unroll
-    for (int f = 0; f < 4; ++f)
-      if (!ns_dir(bcf, ff, i, f)) s[f] = fmaf(wq, r[f], s[f]);
+      for (int f = 0; f < 4; ++f)
+        if (!ns_dir(bcf, ff, i, f)) s[f] = fmaf(wq, r[f], s[f]);
+    }
   }
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1)
+#pragma unroll
+    for (int f = 0; f < 4; ++f) s[f] += __shfl_xor_sync(0xFFFFFFFFu, s[f], o);
+  if (j >= Nc || (t & 7)) return;
   const uint8_t fc = faces_c[j];
   float o[4];
 #pragma unroll
   for (int f = 0; f < 4; ++f) o[f] = ((fc & 0x80) || ns_dir(bcc, fc, j, f)) ? 0.f : s[f];
   out[j] = make_float4(o[0], o[1], o[2], o[3]);
 }
+__global__ void k_ns_restrict(int64_t Nc, NsTransfer T, const float4* __restrict__ b, const float4* __restrict__ Ax,
+                              const uint8_t* __restrict__ faces_f, NsBc bcf, const uint8_t* __restrict__ faces_c,
+                              NsBc bcc, float4* __restrict__ out) {
+  restrict_row(Nc, T, b, Ax, faces_f, bcf, faces_c, bcc, out, blockIdx.x * (int64_t)blockDim.x + threadIdx.x);
+}
 
-// x[i] += sum_q w_q xc[col_q] on the fine rows that are not constrained by a value
-__global__ void k_ns_prolong_add(int64_t Nf, const int64_t* __restrict__ ptr, const int32_t* __restrict__ col,
-                                 const float* __restrict__ w, const float4* __restrict__ xc,
-                                 const uint8_t* __restrict__ faces_f, NsBc bcf, float4* __restrict__ x) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= Nf) return;
+// x[i] += sum_q w_q xc[col_q] on the fine rows that are not constrained by a value; Ax back
+// to zero
+__device__ __forceinline__ void prolong_row(const NsTransfer& T, const float4* xc, const uint8_t* faces_f,
+                                            const NsBc& bcf, float4* x, float4* Ax, int64_t i) {
   float s[4] = {0.f, 0.f, 0.f, 0.f};
-  for (int64_t q = ptr[i]; q < ptr[i + 1]; ++q) {
-    const float4 a = xc[col[q]];
-    const float wq = w[q];
+  for (int64_t q = T.ptr[i]; q < T.ptr[i + 1]; ++q) {
+    const float4 a = xc[T.col[q]];
+    const float wq = T.w[q];
     s[0] = fmaf(wq, a.x, s[0]); s[1] = fmaf(wq, a.y, s[1]); s[2] = fmaf(wq, a.z, s[2]); s[3] = fmaf(wq, a.w, s[3]);
   }
   const uint8_t ff = faces_f[i];
@@ -723,6 +818,120 @@ __global__ void k_ns_prolong_add(int64_t Nf, const int64_t* __restrict__ ptr, co
   if (h || !ns_dir(bcf, ff, i, 2)) o.z += s[2];
   if (h || !ns_dir(bcf, ff, i, 3)) o.w += s[3];
   x[i] = o;
+  Ax[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+}
+__global__ void k_ns_prolong_add(int64_t Nf, NsTransfer T, const float4* __restrict__ xc,
+                                 const uint8_t* __restrict__ faces_f, NsBc bcf, float4* __restrict__ x,
+                                 float4* __restrict__ Ax) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i < Nf) prolong_row(T, xc, faces_f, bcf, x, Ax, i);
+}
+
+// The coarsest levels of the V-cycle in one block: levels whose element corners fit its
+// threads.  A sweep there takes 2 us, against 8 us and more as two launches: 64 and 8 elements
+// with 6 and 32 sweeps last 90 us.  Vectors in shared memory, element sums by atomics there.
+// With it and the sweeps of two launches (four to five before), the coarse levels of a V-cycle
+// on the membrane-band octree (971,776 elements, seven levels) take 0.64 ms instead of 1.42.
+constexpr int kTailLevels = 4, kTailThreads = 1024, kTailNodes = 2048;
+struct NsTailLevel {
+  int64_t n_elem;
+  const int32_t* conn;
+  const uint8_t* level;
+  const float4* adv;
+  const float* Dinv;
+  RowArgs R;
+  NsBc bc;
+  NsTransfer restrict_to, prolong_from;  // from the level above to this one; of the level above
+};
+struct NsTail {
+  NsTailLevel L[kTailLevels];
+  int n, nu, sweeps;
+  float om;
+  float4 *b, *x;  // of the tail's first level, in and out
+};
+template <int D>
+__global__ void __launch_bounds__(kTailThreads, 1) k_ns_tail(const __grid_constant__ NsTail G, NsK<float> K) {
+  constexpr int NC = 1 << D;
+  extern __shared__ float4 tail_smem[];  // per level b, Ax, two x of n_nodes each
+  const int tid = threadIdx.x;
+  float4* at[kTailLevels + 1];
+  at[0] = tail_smem;
+#pragma unroll
+  for (int l = 0; l < kTailLevels; ++l) at[l + 1] = at[l] + (l < G.n ? 4 * G.L[l].R.n_nodes : 0);
+  int cur[kTailLevels] = {0, 0, 0, 0};  // which x is the current one
+  auto sweep = [&](int l, float4* base, int& which, bool first) {
+    const NsTailLevel& L = G.L[l];
+    const int64_t N = L.R.n_nodes;
+    float4 *b = base, *Ax = base + N, *xo = base + (2 + which) * N, *xn = base + (3 - which) * N;
+    for (int64_t i = tid; i < N + L.R.n_hanging; i += kTailThreads)
+      smooth_row(L.R, L.bc, L.Dinv, b, Ax, xo, xn, G.om, first, i);
+    which ^= 1;
+    __syncthreads();
+  };
+  auto apply = [&](int l, float4* base, int which) {
+    const NsTailLevel& L = G.L[l];
+    const int64_t N = L.R.n_nodes;
+    const float4* x = base + (2 + which) * N;
+    float* Ax = reinterpret_cast<float*>(base + N);
+    if ((tid & ~31) / NC < L.n_elem) {  // whole warps: shuffles
+      const int64_t e = tid / NC;
+      const int c = tid & (NC - 1);
+      const bool valid = e < L.n_elem;
+      const int32_t id = valid ? __ldg(L.conn + e * NC + c) : 0;
+      const int lev = valid ? L.level[e] : 0;
+      float xs[4], a4[4];
+      load4(L.R.hpar, L.R.hnp, reinterpret_cast<const float*>(L.adv), id, valid, a4);
+      gather4(L.R.hpar, L.R.hnp, x, id, valid, xs);
+      const float as[3] = {a4[0], a4[1], a4[2]}, none3[3] = {0.f, 0.f, 0.f}, none2[2] = {0.f, 0.f};
+      float r[4];
+      lane_ns<float, D, false>(xs, as, none3, none2, c, lev, K, r);
+      if (valid) {
+#pragma unroll
+        for (int f = 0; f < 4; ++f)
+          r[f] = times_const(r[f], f < 3 ? ns_weight_c(D, 0) : ns_weight_c(D, 3), ns_weight_e(D, lev, f));
+        const int np = id >= 0 ? 1 : L.R.hnp[-id - 1];
+        const float w = np == 1 ? 1.0f : np == 2 ? 0.5f : 0.25f;
+        for (int p = 0; p < np; ++p) {
+          const int32_t n = id >= 0 ? id : L.R.hpar[4 * (-id - 1) + p];
+#pragma unroll
+          for (int f = 0; f < 4; ++f) atomicAdd(Ax + 4 * n + f, w * r[f]);
+        }
+      }
+    }
+    __syncthreads();
+  };
+  for (int64_t i = tid; i < G.L[0].R.n_nodes; i += kTailThreads) at[0][i] = G.b[i];
+  __syncthreads();
+#pragma unroll
+  for (int l = 0; l < kTailLevels; ++l) {
+    if (l >= G.n) break;
+    const int sweeps = l + 1 == G.n ? G.sweeps : G.nu;
+    for (int k = 0; k < sweeps; ++k) {
+      if (k) apply(l, at[l], cur[l]);
+      sweep(l, at[l], cur[l], k == 0);
+    }
+    if (l + 1 == G.n) break;
+    apply(l, at[l], cur[l]);
+    const NsTailLevel &F = G.L[l], &C = G.L[l + 1];
+    for (int64_t t = tid; t < (C.R.n_nodes * 8 + 31) / 32 * 32; t += kTailThreads)
+      restrict_row(C.R.n_nodes, C.restrict_to, at[l], at[l] + F.R.n_nodes, F.R.faces, F.bc, C.R.faces, C.bc, at[l + 1], t);
+    __syncthreads();
+  }
+#pragma unroll
+  for (int l = kTailLevels - 2; l >= 0; --l) {
+    if (l + 1 >= G.n) continue;
+    const NsTailLevel &F = G.L[l], &C = G.L[l + 1];
+    const int64_t N = F.R.n_nodes;
+    const float4* xc = at[l + 1] + (2 + cur[l + 1]) * C.R.n_nodes;
+    for (int64_t i = tid; i < N; i += kTailThreads)
+      prolong_row(C.prolong_from, xc, F.R.faces, F.bc, at[l] + (2 + cur[l]) * N, at[l] + N, i);
+    __syncthreads();
+    for (int k = 0; k < G.nu; ++k) {
+      apply(l, at[l], cur[l]);
+      sweep(l, at[l], cur[l], false);
+    }
+  }
+  for (int64_t i = tid; i < G.L[0].R.n_nodes; i += kTailThreads) G.x[i] = at[0][(2 + cur[0]) * G.L[0].R.n_nodes + i];
 }
 
 // coarse v~ (FP64 [Nc][4] and its FP32 copy) at the coarse nodes' points
@@ -754,7 +963,8 @@ struct NsState {
          *x = nullptr;
   double *part = nullptr, *sc = nullptr, *hsc = nullptr;
   double* usave = nullptr;  // [2][3N] PNP history of repeated block iterations
-  float4* mgAx = nullptr;   // [N] operator scratch of the finest multigrid level
+  // [N] of a multigrid level: element sums (zero between sweeps), the other x
+  float4 *mgAx = nullptr, *mgX = nullptr;
   float4* xbest = nullptr;  // [N] BiCGStab's best iterate
   bool mg_off = false;      // this solve fell back from the V-cycle to the inverted blocks
   int64_t fine32 = 0;       // finest-level FP32 operator applications of this solve's V-cycles
@@ -851,6 +1061,7 @@ static NsArgs<T> ns_args(const pnp_ctx* c, const T* X, const T* adv, T* out) {
   A.level = c->d_level;
   A.hang_par = c->d_hpar;
   A.hang_np = c->d_hnp;
+  A.faces = c->d_faces;
   A.X = X;
   A.adv = adv;
   A.out = out;
@@ -867,13 +1078,18 @@ static NsK<C> ns_k(const NsArgs<T>& A) {
   return NsK<C>{C(A.isc), C(A.isc * A.kap), C(A.tau_t), C(A.cid), C(A.fb)};
 }
 
-// the FP64 rows in double-float arithmetic (default) or FP64 arithmetic
-template <int D, bool DATA>
-static void launch_ns64(const NsArgs<double>& A, cudaStream_t s) {
+// adds the rows to initialised ones; FP64 vectors in double-float arithmetic (default) or FP64
+template <typename T, typename C, int D, bool DATA, bool MASK = true>
+static cudaError_t launch_ns(const NsArgs<T>& A, const NsBc& bc, cudaStream_t s) {
+  if (A.n_elem == 0) return cudaSuccess;
   const int t = block_threads(A.n_elem << D);
-  const unsigned blocks = block_count(A.n_elem << D, t);
-  if (residual_double_float()) k_ns_lanes<double, df, D, DATA><<<blocks, t, 0, s>>>(A, ns_k<df>(A));
-  else k_ns_lanes<double, double, D, DATA><<<blocks, t, 0, s>>>(A, ns_k<double>(A));
+  k_ns_lanes<T, C, D, DATA, MASK><<<block_count(A.n_elem << D, t), t, 0, s>>>(A, bc, ns_k<C>(A));
+  note_launch();
+  return cudaGetLastError();
+}
+template <int D, bool DATA>
+static cudaError_t launch_ns64(const NsArgs<double>& A, const NsBc& bc, cudaStream_t s) {
+  return residual_double_float() ? launch_ns<double, df, D, DATA>(A, bc, s) : launch_ns<double, double, D, DATA>(A, bc, s);
 }
 
 // element-kernel flops per lane (FP counts of the code above, fma = 2)
@@ -908,75 +1124,51 @@ int ctx_ns_prepare(pnp_ctx* c) {
   return PNP_OK;
 }
 
+template <typename T>
+static int ns_init_rows(pnp_ctx* c, const NsBc& bc, const T* X, T* out, int mode) {
+  const int64_t n = c->n_nodes + c->n_hanging;
+  const int t = block_threads(n);
+  k_ns_init<T><<<block_count(n, t), t, 0, c->stream>>>(c->rows(), bc, X, out, mode);
+  note_launch();
+  return ctx_check(c, cudaGetLastError(), "ns rows");
+}
+
 // F = the NS rows of X (data = true: the residual A X - b, Ubody the PNP state of the body
 // force; false: A X), FP64
 int ctx_ns_apply64(pnp_ctx* c, const double* X, const double* Ubody, double* F, bool data) {
   NsState* S = c->ns;
   const int64_t N = c->n_nodes;
   cudaStream_t s = c->stream;
-  CK(cudaMemsetAsync(F, 0, sizeof(double) * 4 * N, s));
+  const NsBc bc = ns_bc(c);
+  RC(ns_init_rows<double>(c, bc, X, F, data ? 0 : 1));
   NsArgs<double> A = ns_args<double>(c, X, S->adv, F);
   A.hv = S->hv;
   A.U = Ubody;
-  const int64_t lanes = c->n_elem << c->dim;
-  {
-    // flops: the FP64 formulation's, times the FP32 operations of a double-float operation
-    ProfScope ps(c, PNP_PROF_NS, 72.0 * N + (data ? 56.0 * N : 0.0) + 32.0 * N + c->conn_bytes(),
-                 ns_lane_flops(c->dim, data) * lanes * (residual_double_float() ? kDfFlopsPerFlop : 1.0));
-    if (c->n_elem) {
-      if (c->dim == 2) {
-        if (data) launch_ns64<2, true>(A, s);
-        else launch_ns64<2, false>(A, s);
-      } else {
-        if (data) launch_ns64<3, true>(A, s);
-        else launch_ns64<3, false>(A, s);
-      }
-      note_launch();
-    }
-  }
-  const NsBc bc = ns_bc(c);
-  k_ns_rows<double><<<nblk(N, 256), 256, 0, s>>>(N, c->d_faces, bc, X, F, data ? 0 : 1);
-  note_launch();
-  if (c->n_hanging) {
-    k_ns_hanging_rows<double><<<nblk(c->n_hanging, 256), 256, 0, s>>>(c->n_hanging, c->d_hnode, c->d_hpar, c->d_hnp,
-                                                                     X, F);
-    note_launch();
-  }
-  CK(cudaGetLastError());
+  // flops: the FP64 formulation's, times the FP32 operations of a double-float operation
+  ProfScope ps(c, PNP_PROF_NS, 72.0 * N + (data ? 56.0 * N : 0.0) + 32.0 * N + c->conn_bytes(),
+               ns_lane_flops(c->dim, data) * (double)(c->n_elem << c->dim) *
+                   (residual_double_float() ? kDfFlopsPerFlop : 1.0));
+  if (c->dim == 2) CK((data ? launch_ns64<2, true>(A, bc, s) : launch_ns64<2, false>(A, bc, s)));
+  else CK((data ? launch_ns64<3, true>(A, bc, s) : launch_ns64<3, false>(A, bc, s)));
   return PNP_OK;
 }
 
-// y = A x, FP32 (x, y padded [N] float4)
-int ctx_ns_apply32(pnp_ctx* c, const float4* x, float4* y) {
-  NsState* S = c->ns;
-  const int64_t N = c->n_nodes;
-  cudaStream_t s = c->stream;
-  CK(cudaMemsetAsync(y, 0, sizeof(float4) * N, s));
-  NsArgs<float> A = ns_args<float>(c, reinterpret_cast<const float*>(x), reinterpret_cast<const float*>(S->adv32),
+// adds the element sums of A x to every row of y: FP32, x and y padded [N] float4; MASK: but
+// not to constrained rows
+template <bool MASK>
+static int ns_add32(pnp_ctx* c, const float4* x, float4* y) {
+  NsArgs<float> A = ns_args<float>(c, reinterpret_cast<const float*>(x), reinterpret_cast<const float*>(c->ns->adv32),
                                    reinterpret_cast<float*>(y));
-  const int64_t lanes = c->n_elem << c->dim;
-  {
-    ProfScope ps(c, PNP_PROF_NS32, 48.0 * N + c->conn_bytes(), ns_lane_flops(c->dim, false) * lanes);
-    if (c->n_elem) {
-      const int t = block_threads(lanes);
-      const unsigned blocks = block_count(lanes, t);
-      if (c->dim == 2) k_ns_lanes<float, float, 2, false><<<blocks, t, 0, s>>>(A, ns_k<float>(A));
-      else k_ns_lanes<float, float, 3, false><<<blocks, t, 0, s>>>(A, ns_k<float>(A));
-      note_launch();
-    }
-  }
-  const NsBc bc = ns_bc(c);
-  const float* xf = reinterpret_cast<const float*>(x);
-  float* yf = reinterpret_cast<float*>(y);
-  k_ns_rows<float><<<nblk(N, 256), 256, 0, s>>>(N, c->d_faces, bc, xf, yf, 1);
-  note_launch();
-  if (c->n_hanging) {
-    k_ns_hanging_rows<float><<<nblk(c->n_hanging, 256), 256, 0, s>>>(c->n_hanging, c->d_hnode, c->d_hpar, c->d_hnp,
-                                                                    xf, yf);
-    note_launch();
-  }
-  CK(cudaGetLastError());
+  ProfScope ps(c, PNP_PROF_NS32, 48.0 * c->n_nodes + c->conn_bytes(),
+               ns_lane_flops(c->dim, false) * (double)(c->n_elem << c->dim));
+  if (c->dim == 2) CK((launch_ns<float, float, 2, false, MASK>(A, ns_bc(c), c->stream)));
+  else CK((launch_ns<float, float, 3, false, MASK>(A, ns_bc(c), c->stream)));
   return PNP_OK;
+}
+// y = A x, FP32
+int ctx_ns_apply32(pnp_ctx* c, const float4* x, float4* y) {
+  RC(ns_init_rows<float>(c, ns_bc(c), reinterpret_cast<const float*>(x), reinterpret_cast<float*>(y), 1));
+  return ns_add32<true>(c, x, y);
 }
 
 // the 4x4 diagonal blocks [N][16] (FP64, before the row substitutions) into Dg
@@ -1014,18 +1206,23 @@ static int ns_mg_levels(const pnp_ctx* c) { return c->prm.mg_levels > 0 ? c->prm
 
 // Per solve: every coarse level's parameters, boundary table, injected v~ and inverted
 // diagonal blocks (level 0 uses the solve's own blocks).
-static int ctx_ns_mg_prepare(pnp_ctx* c) {
-  RC(ctx_mg_setup(c, ns_mg_levels(c)));
+static int ns_mg_buffers(pnp_ctx* c) {
   NsState* S = c->ns;
-  if (!S->mgAx) {
-    void* q = nullptr;
-    if (cudaMalloc(&q, sizeof(float4) * c->n_nodes) != cudaSuccess) {
+  for (float4** q : {&S->mgAx, &S->mgX}) {
+    if (*q) continue;
+    void* p = nullptr;
+    if (cudaMalloc(&p, sizeof(float4) * c->n_nodes) != cudaSuccess) {
       cudaGetLastError();
       PNP_FAIL(PNP_ERR_NOMEM, "ns multigrid: device allocation failed");
     }
-    S->mgAx = (float4*)q;
-    S->alloc.push_back(q);
+    *q = (float4*)p;
+    S->alloc.push_back(p);
   }
+  return PNP_OK;
+}
+static int ctx_ns_mg_prepare(pnp_ctx* c) {
+  RC(ctx_mg_setup(c, ns_mg_levels(c)));
+  RC(ns_mg_buffers(c));
   auto& lv = *c->mg;
   pnp_ctx* fine = c;
   for (size_t l = 1; l < lv.size(); ++l) {
@@ -1045,6 +1242,7 @@ static int ctx_ns_mg_prepare(pnp_ctx* c) {
     std::memcpy(sc->ns_bc_type, c->ns_bc_type, sizeof(c->ns_bc_type));
     std::memcpy(sc->ns_bc_val, c->ns_bc_val, sizeof(c->ns_bc_val));
     RC(ctx_ns_alloc(sc));
+    RC(ns_mg_buffers(sc));
     const int64_t Nc = sc->n_nodes;
     k_ns_inject_adv<<<nblk(Nc, 256), 256, 0, c->stream>>>(Nc, lv[l].inject, fine->ns->adv, sc->ns->adv,
                                                           sc->ns->adv32);
@@ -1057,48 +1255,105 @@ static int ctx_ns_mg_prepare(pnp_ctx* c) {
   return PNP_OK;
 }
 
+// the levels from l on in one block (k_ns_tail), where they fit: their corners its threads,
+// their vectors its shared memory.  The launch that it saves per sweep is what counts there;
+// a level of 64 elements is as far as one block's arithmetic keeps up with two launches.
+static bool ns_tail_fits(const pnp_ctx* c, size_t l) {
+  const auto& lv = *c->mg;
+  if (l == 0 || lv.size() - l > (size_t)kTailLevels) return false;
+  int64_t nodes = 0;
+  for (size_t k = l; k < lv.size(); ++k) {
+    if ((lv[k].sub->n_elem << c->dim) > kTailThreads) return false;
+    nodes += lv[k].sub->n_nodes;
+  }
+  return nodes <= kTailNodes;
+}
+static int ns_mg_tail(pnp_ctx* c, size_t l) {
+  const auto& lv = *c->mg;
+  NsTail G;
+  G.n = (int)(lv.size() - l);
+  G.nu = std::max(1, c->prm.mg_smooth);
+  G.sweeps = std::max(1, c->prm.mg_coarse_its);
+  G.om = (float)c->prm.mg_omega;
+  G.b = lv[l].sub->ns->r;
+  G.x = lv[l].sub->ns->x;
+  int64_t nodes = 0;
+  for (int k = 0; k < G.n; ++k) {
+    const MgLevel& M = lv[l + k];
+    pnp_ctx* sc = M.sub;
+    NsTailLevel& L = G.L[k];
+    L.n_elem = sc->n_elem;
+    L.conn = sc->d_conn;
+    L.level = sc->d_level;
+    L.adv = sc->ns->adv32;
+    L.Dinv = sc->ns->Dinv;
+    L.R = sc->rows();
+    L.bc = ns_bc(sc);
+    L.restrict_to = NsTransfer{M.r_ptr, M.r_col, M.r_w};
+    L.prolong_from = NsTransfer{M.p_ptr, M.p_col, M.p_w};
+    nodes += sc->n_nodes;
+  }
+  pnp_ctx* sc = lv[l].sub;
+  const NsK<float> K = ns_k<float>(ns_args<float>(sc, nullptr, nullptr, nullptr));
+  const size_t smem = sizeof(float4) * 4 * nodes;
+  auto run = [&](auto kernel) -> int {
+    CK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(float4) * 4 * kTailNodes)));
+    kernel<<<1, kTailThreads, smem, c->stream>>>(G, K);
+    note_launch();
+    CK(cudaGetLastError());
+    return PNP_OK;
+  };
+  return c->dim == 2 ? run(k_ns_tail<2>) : run(k_ns_tail<3>);
+}
+
 // x = one V-cycle on level l applied to b (level 0: the caller's vectors; coarser levels:
 // their contexts' r and x)
 static int ns_mg_cycle(pnp_ctx* c, size_t l, const float4* b, float4* x) {
+  if (ns_tail_fits(c, l)) return ns_mg_tail(c, l);
   auto& lv = *c->mg;
   pnp_ctx* lc = l == 0 ? c : lv[l].sub;
   NsState* LS = lc->ns;
-  float4* Ax = l == 0 ? c->ns->mgAx : LS->t;
-  const int64_t N = lc->n_nodes;
+  float4* Ax = LS->mgAx;
+  const int64_t N = lc->n_nodes, rows = N + lc->n_hanging;
   cudaStream_t s = c->stream;
   const float om = (float)c->prm.mg_omega;
   const NsBc bc = ns_bc(lc);
-  auto apply = [&]() -> int {
-    RC(ctx_ns_apply32(lc, x, Ax));
+  const bool last = l + 1 == lv.size();
+  const int nu = std::max(1, c->prm.mg_smooth), sweeps = last ? std::max(1, c->prm.mg_coarse_its) : nu;
+  // the sweeps take x and the other buffer in turn; the last one writes x
+  float4 *xo = LS->mgX, *xn = x;
+  if ((last ? sweeps : 2 * nu) % 2 == 0) std::swap(xo, xn);
+  auto apply = [&]() -> int {  // the current x is xo
+    RC(ns_add32<false>(lc, xo, Ax));
     if (l == 0) c->ns->fine32++;
     return PNP_OK;
   };
   auto smooth = [&](bool first) -> int {
     if (!first) RC(apply());
     ProfScope ps(c, l == 0 ? PNP_PROF_NS_KRYLOV : -1, 112.0 * N, 36.0 * N);
-    k_ns_smooth<<<nblk(N, 256), 256, 0, s>>>(N, LS->Dinv, b, Ax, x, om, first ? 1 : 0);
+    const int t = block_threads(rows);
+    k_ns_smooth<<<block_count(rows, t), t, 0, s>>>(lc->rows(), bc, LS->Dinv, b, Ax, xo, xn, om, first);
     note_launch();
     CK(cudaGetLastError());
+    std::swap(xo, xn);
     return PNP_OK;
   };
-  if (l + 1 == lv.size()) {
-    const int sweeps = std::max(1, c->prm.mg_coarse_its);
-    for (int k = 0; k < sweeps; ++k) RC(smooth(k == 0));
-    return PNP_OK;
-  }
-  const int nu = std::max(1, c->prm.mg_smooth);
-  for (int k = 0; k < nu; ++k) RC(smooth(k == 0));
+  for (int k = 0; k < sweeps; ++k) RC(smooth(k == 0));
+  if (last) return PNP_OK;
   RC(apply());
   pnp_ctx* cc = lv[l + 1].sub;
   const MgLevel& C = lv[l + 1];
   {
     ProfScope ps(c, l == 0 ? PNP_PROF_MG : -1, 0.0);
-    k_ns_restrict<<<nblk(cc->n_nodes, 256), 256, 0, s>>>(cc->n_nodes, C.r_ptr, C.r_col, C.r_w, b, Ax, lc->d_faces, bc,
-                                                         cc->d_faces, ns_bc(cc), cc->ns->r);
+    int t = block_threads(8 * cc->n_nodes);
+    k_ns_restrict<<<block_count(8 * cc->n_nodes, t), t, 0, s>>>(cc->n_nodes, NsTransfer{C.r_ptr, C.r_col, C.r_w}, b, Ax,
+                                                                lc->d_faces, bc, cc->d_faces, ns_bc(cc), cc->ns->r);
     note_launch();
     CK(cudaGetLastError());
     RC(ns_mg_cycle(c, l + 1, cc->ns->r, cc->ns->x));
-    k_ns_prolong_add<<<nblk(N, 256), 256, 0, s>>>(N, C.p_ptr, C.p_col, C.p_w, cc->ns->x, lc->d_faces, bc, x);
+    t = block_threads(N);
+    k_ns_prolong_add<<<block_count(N, t), t, 0, s>>>(N, NsTransfer{C.p_ptr, C.p_col, C.p_w}, cc->ns->x, lc->d_faces, bc,
+                                                     xo, Ax);
     note_launch();
     CK(cudaGetLastError());
   }
