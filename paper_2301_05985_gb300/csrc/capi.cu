@@ -323,7 +323,7 @@ int pnp_ctx_create(const pnp_mesh* m, const pnp_params* p, void* stream, pnp_ctx
   ALLOC(c->z, v3);
   ALLOC(c->r, v3);
   ALLOC(c->dflag, sizeof(int) * 8);
-  ALLOC(c->ticket, sizeof(unsigned));
+  ALLOC(c->ticket, 2 * sizeof(unsigned));
 #undef ALLOC
   if (cudaMallocHost((void**)&c->hflag, sizeof(int) * 4) != cudaSuccess) {
     cudaGetLastError();
@@ -342,7 +342,7 @@ int pnp_ctx_create(const pnp_mesh* m, const pnp_params* p, void* stream, pnp_ctx
     if (bytes && e == cudaSuccess) e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, s);
   };
   if (e == cudaSuccess) e = cudaMemsetAsync(c->dflag, 0, sizeof(int) * 8, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(c->ticket, 0, sizeof(unsigned), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(c->ticket, 0, 2 * sizeof(unsigned), s);
   up(c->d_conn, m->el_conn.data(), sizeof(int32_t) * m->el_conn.size());
   up(c->d_level, m->el_level.data(), m->el_level.size());
   up(c->d_faces, faces.data(), faces.size());
@@ -457,7 +457,7 @@ int ctx_alloc_inner(pnp_ctx* c, int m, int d) {
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->Qin, sizeof(float) * (size_t)(d + 1) * (size_t)c->ldq);
   if (e == cudaSuccess) e = cudaMemset(c->Qin, 0, sizeof(float) * (size_t)(d + 1) * (size_t)c->ldq);
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->Dinv32, sizeof(float) * 9 * (size_t)c->n_nodes);
-  if (e == cudaSuccess) e = cudaMalloc((void**)&c->isc, sizeof(double) * (inner_scalar_doubles(d) + 5 * (size_t)(d + 2)));
+  if (e == cudaSuccess) e = cudaMalloc((void**)&c->isc, sizeof(double) * (inner_scalar_doubles(d) + 5 * (size_t)(d + 2) + inner_sum_doubles()));
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->iinv, sizeof(float) * (size_t)(d + 2));
   if (e != cudaSuccess) {
     pnp_set_error("inner Krylov scratch allocation failed: %s", cudaGetErrorString(e));

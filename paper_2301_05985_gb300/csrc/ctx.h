@@ -71,7 +71,8 @@ struct pnp_ctx {
   // stored linearisation, [1] of pnp_jv; [2] the network inference.  wait_flag: [0], or on a multigrid level the owner's [0]
   int* hflag = nullptr;
   int* wait_flag = nullptr;
-  unsigned* ticket = nullptr;  // counter of the reductions' last block (this stream's launches)
+  // counters of this stream's launches: [0] the reductions' last block, [1] the grid barrier
+  unsigned* ticket = nullptr;
   int m_alloc = 0;
   cudaEvent_t step_done[2] = {nullptr, nullptr};  // GMRES iterations queued ahead of the host
   // flexible outer GMRES with an inner FP32 GMRES(d) preconditioner

@@ -13,6 +13,9 @@ namespace {
 
 inline int nblk(int64_t n, int t) { return (int)((n + t - 1) / t); }
 
+constexpr int kMaxInner = 64;
+constexpr int kGsSums = kMaxInner + 2;
+
 __device__ __forceinline__ float warp_sum4f(const float (&s)[4], int lane) {
   const bool hi4 = lane & 16, hi3 = lane & 8;
   const float a0 = (hi4 ? s[2] : s[0]) + __shfl_xor_sync(0xffffffffu, hi4 ? s[0] : s[2], 16);
@@ -39,70 +42,6 @@ __device__ __forceinline__ double block_sum_d(double v, double* sh) {
 // The inner basis has rows padded to a multiple of four floats (zeros beyond the
 // vector's length), so both Gram-Schmidt kernels move float4: four entries per load.
 
-// d_i = U_i . w (i < k) for FP32 vectors of n4 float4.  At most kInnerBlocks blocks (8 per
-// SM) stride over chunks of 256 x kRows float4; for every group of four basis vectors a
-// thread accumulates its rows of all chunks (w re-read from L2 per group), then one warp
-// reduce-scatter and a fixed-order block sum give the block's partials part[i][block].
-// Long vectors stream at HBM rate (89 %).  Short ones (a 163 k-node mesh: 240 chunks, the
-// basis in L2) are latency: there blockIdx.y takes a share of the groups, and the last block
-// adds the partials (`ticket` given) instead of a second launch.
-constexpr int kRows = 2;
-__device__ __forceinline__ float dot4(float4 a, float4 b, float s) {
-  return fmaf(a.x, b.x, fmaf(a.y, b.y, fmaf(a.z, b.z, fmaf(a.w, b.w, s))));
-}
-__global__ void __launch_bounds__(256, 8) k_multi_dot_f32(int64_t n4, int k, const float4* __restrict__ Ub,
-                                                          int64_t ld4, const float4* __restrict__ w, double* part,
-                                                          unsigned* ticket, double* __restrict__ d) {
-  __shared__ float sh[4][8];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int64_t chunk = 256 * kRows;
-  const int nb = gridDim.x;
-  const int per = ((k + 3) / 4 + gridDim.y - 1) / gridDim.y * 4;  // vectors of this block
-  const int je = min(k, ((int)blockIdx.y + 1) * per);
-  for (int j0 = blockIdx.y * per; j0 < je; j0 += 4) {
-    const int cnt = min(4, je - j0);
-    float s[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-    for (int64_t c0 = (int64_t)blockIdx.x * chunk; c0 < n4; c0 += (int64_t)gridDim.x * chunk) {
-      float4 wv[kRows];
-#pragma unroll
-      for (int r = 0; r < kRows; ++r) {
-        const int64_t t = c0 + threadIdx.x + r * 256;
-        wv[r] = t < n4 ? w[t] : make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        if (q < cnt) {
-          const float4* ui = Ub + (int64_t)(j0 + q) * ld4;
-#pragma unroll
-          for (int r = 0; r < kRows; ++r) {
-            const int64_t t = c0 + threadIdx.x + r * 256;
-            if (t < n4) s[q] = dot4(__ldg(ui + t), wv[r], s[q]);
-          }
-        }
-      }
-    }
-    const float tot = warp_sum4f(s, lane);
-    if ((lane & 7) == 0) sh[(lane >> 3) & 3][wid] = tot;
-    __syncthreads();
-    if (threadIdx.x < cnt) {
-      double t = 0.0;
-#pragma unroll
-      for (int v = 0; v < 8; ++v) t += (double)sh[threadIdx.x][v];
-      part[(int64_t)(j0 + threadIdx.x) * nb + blockIdx.x] = t;
-    }
-    __syncthreads();
-  }
-  if (!ticket || !last_block(ticket, gridDim.x * gridDim.y)) return;
-  for (int j = wid; j < k; j += 8) {
-    double t = 0.0;
-#pragma unroll 4
-    for (int b = lane; b < nb; b += 32) t += __ldcg(part + (int64_t)j * nb + b);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    if (lane == 0) d[j] = t;
-  }
-}
-
 // Arnoldi bookkeeping of the inner process.  Basis vectors u_i are kept unnormalised
 // with norms s_i (q_i = u_i / s_i).  The steps only store the Hessenberg columns
 // h_i = d_i / s_i, h_(j+1) = s_(j+1); the Givens rotations wait for the least-squares
@@ -112,37 +51,37 @@ __global__ void __launch_bounds__(256, 8) k_multi_dot_f32(int64_t n4, int k, con
 // Scalar layout: H [(d+1) x d] row-major.
 struct InnerStep {
   int j, d;            // column j of d; j < 0: the start vector
-  const double* dd;    // projections of the step
   double *sv, *dinv;   // norms s_i and 1 / s_i^2
   float* inv_s;        // 1 / s_i
   double* H;
+  double* sums;        // [2][kGsSums] projections and w . w, of even and of odd steps
+  unsigned* arrived;   // blocks at the step's barrier (zero between launches)
 };
+__device__ __forceinline__ float dot4(float4 a, float4 b, float s) {
+  return fmaf(a.x, b.x, fmaf(a.y, b.y, fmaf(a.z, b.z, fmaf(a.w, b.w, s))));
+}
+__device__ __forceinline__ void axpy4(float c, const float4& u, float4& a) {
+  a.x = fmaf(c, u.x, a.x);
+  a.y = fmaf(c, u.y, a.y);
+  a.z = fmaf(c, u.z, a.z);
+  a.w = fmaf(c, u.w, a.w);
+}
 
-// w -= sum_i (d_i dinv_i) U_i (i < k) in FP32 on n4 float4, and w . w: at most kUpdBlocks
-// blocks (6 per SM); the last one adds the partials and ends the Arnoldi step.
-constexpr int kUpdBlocks = 6 * 152;
-__global__ void __launch_bounds__(256, 6) k_multi_axpy_norm_f32(int64_t n4, int k, const float4* __restrict__ Ub,
-                                                             int64_t ld4, float4* __restrict__ w, double* part,
-                                                             unsigned* ticket, InnerStep S) {
-  extern __shared__ float cf[];
+__device__ __forceinline__ void finish_norm(const InnerStep& S, double ww) {
+  const double s = sqrt(ww);
+  S.sv[S.j + 1] = s;
+  S.dinv[S.j + 1] = s > 0 ? 1.0 / (s * s) : 0.0;
+  S.inv_s[S.j + 1] = s > 0 ? (float)(1.0 / s) : 0.0f;
+  if (S.j >= 0) S.H[(int64_t)(S.j + 1) * S.d + S.j] = s;
+}
+
+// The start vector's norm; clears the first step's sums
+__global__ void __launch_bounds__(256) k_inner_start(int64_t n4, const float4* __restrict__ u, double* part,
+                                                     unsigned* ticket, InnerStep S) {
   __shared__ double sh[256];
-  for (int i = threadIdx.x; i < k; i += blockDim.x) cf[i] = (float)(S.dd[i] * S.dinv[i]);
-  __syncthreads();
   float ss = 0.0f;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n4; t += (int64_t)gridDim.x * blockDim.x) {
-    float4 a = w[t];
-#pragma unroll 4
-    for (int i = 0; i < k; ++i) {
-      const float4 u = Ub[(int64_t)i * ld4 + t];
-      const float c = -cf[i];
-      a.x = fmaf(c, u.x, a.x);
-      a.y = fmaf(c, u.y, a.y);
-      a.z = fmaf(c, u.z, a.z);
-      a.w = fmaf(c, u.w, a.w);
-    }
-    if (k > 0) w[t] = a;
-    ss = fmaf(a.x, a.x, fmaf(a.y, a.y, fmaf(a.z, a.z, fmaf(a.w, a.w, ss))));
-  }
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n4; t += (int64_t)gridDim.x * blockDim.x)
+    ss = dot4(u[t], u[t], ss);
   double tot = block_sum_d((double)ss, sh);
   if (threadIdx.x == 0) part[blockIdx.x] = tot;
   if (!last_block(ticket, gridDim.x)) return;
@@ -150,15 +89,126 @@ __global__ void __launch_bounds__(256, 6) k_multi_axpy_norm_f32(int64_t n4, int 
 #pragma unroll 4
   for (int b = threadIdx.x; b < (int)gridDim.x; b += 256) tot += __ldcg(part + b);
   tot = block_sum_d(tot, sh);
-  const int i = threadIdx.x;
-  if (i == 0) {
-    const double s = sqrt(tot);
-    S.sv[S.j + 1] = s;
-    S.dinv[S.j + 1] = s > 0 ? 1.0 / (s * s) : 0.0;
-    S.inv_s[S.j + 1] = s > 0 ? (float)(1.0 / s) : 0.0f;
-    if (S.j >= 0) S.H[(int64_t)(S.j + 1) * S.d + S.j] = s;
+  if (threadIdx.x == 0) finish_norm(S, tot);
+  for (int i = threadIdx.x; i < kGsSums; i += 256) S.sums[i] = 0.0;
+}
+
+// One Gram-Schmidt step in one cooperative launch: d_i = U_i . w, a grid barrier, then
+// w -= sum_i (d_i / s_i^2) U_i and w . w, for k FP32 vectors of n4 float4.  Each block walks
+// its chunks of 256 float4 up for the sums and down for the update, so that the rows it ends
+// the sums with come from L1 and L2 again.  The sums of the blocks meet in FP64 atomics (one
+// per vector and block).  The barrier's wait is bounded: a block that gives up sets err (pinned
+// host memory) and skips the update, but arrives at the end as the others do, so the counters
+// are left as they were.
+// What bounds it, a step's mean over 24: 163,000 nodes (the basis in L2) latency, 16 us, 27 us as
+// a dot and an update kernel; 1,047,407 nodes memory, 57 us, 81 us as two (the basis read
+// twice: 51 us at HBM rate, 13 vectors each way).
+constexpr int kGsGroup = 24, kGsBatch = 8;
+constexpr int kGsPolls = 1 << 22;
+__global__ void __launch_bounds__(256, 3) k_inner_gs(int64_t n4, int k, const float4* __restrict__ Ub, int64_t ld4,
+                                                     float4* w, unsigned* ticket, int* err, InnerStep S) {
+  __shared__ float sh[kGsGroup][8];
+  __shared__ float cf[kMaxInner];
+  __shared__ bool passed;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int64_t chunks = (n4 + 255) / 256;
+  double *cur = S.sums + (S.j & 1) * kGsSums, *next = S.sums + (~S.j & 1) * kGsSums;
+  for (int g0 = 0; g0 < k; g0 += kGsGroup) {
+    float s[kGsGroup];
+#pragma unroll
+    for (int q = 0; q < kGsGroup; ++q) s[q] = 0.0f;
+    for (int64_t c = blockIdx.x; c < chunks; c += gridDim.x) {
+      const int64_t t = c * 256 + tid;
+      if (t >= n4) break;
+      const float4 wv = w[t];
+#pragma unroll
+      for (int b = 0; b < kGsGroup; b += kGsBatch) {
+        if (g0 + b >= k) break;
+        float4 u[kGsBatch];
+#pragma unroll
+        for (int q = 0; q < kGsBatch; ++q) u[q] = __ldg(Ub + (int64_t)min(g0 + b + q, k - 1) * ld4 + t);
+#pragma unroll
+        for (int q = 0; q < kGsBatch; ++q) s[b + q] = dot4(u[q], wv, s[b + q]);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < kGsGroup; q += 4) {
+      const float v[4] = {s[q], s[q + 1], s[q + 2], s[q + 3]};
+      const float tot = warp_sum4f(v, lane);
+      if ((lane & 7) == 0) sh[q + (lane >> 3)][wid] = tot;
+    }
+    __syncthreads();
+    if (tid < kGsGroup && g0 + tid < k) {
+      double t = 0.0;
+#pragma unroll
+      for (int v = 0; v < 8; ++v) t += (double)sh[tid][v];
+      atomicAdd(cur + g0 + tid, t);
+    }
+    __syncthreads();
   }
-  if (i <= S.j) S.H[(int64_t)i * S.d + S.j] = S.sv[i] > 0 ? S.dd[i] / S.sv[i] : 0.0;
+  // grid barrier
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) {
+    atomicAdd(S.arrived, 1u);
+    bool ok = false;
+    for (int i = 0; i < kGsPolls && !ok; ++i) {
+      unsigned n;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(n) : "l"(S.arrived) : "memory");
+      ok = n >= gridDim.x;
+    }
+    if (!ok) *reinterpret_cast<volatile int*>(err) = 1;
+    passed = ok;
+  }
+  __syncthreads();
+  float ss = 0.0f;
+  if (passed) {
+    if (tid < k) {
+      const double d = __ldcg(cur + tid);
+      cf[tid] = -(float)(d * S.dinv[tid]);
+      if (blockIdx.x == 0) S.H[(int64_t)tid * S.d + S.j] = S.sv[tid] > 0 ? d / S.sv[tid] : 0.0;
+    }
+    if (blockIdx.x == 0)
+      for (int i = tid; i < kGsSums; i += 256) next[i] = 0.0;
+    __syncthreads();
+    const int64_t mine = blockIdx.x < chunks ? (chunks - 1 - blockIdx.x) / gridDim.x : -1;
+    for (int64_t m = mine; m >= 0; --m) {
+      const int64_t t = (blockIdx.x + m * gridDim.x) * 256 + tid;
+      if (t >= n4) continue;
+      float4 a = w[t];
+      int i = 0;
+      for (; i + kGsBatch <= k; i += kGsBatch) {
+        float4 u[kGsBatch];
+#pragma unroll
+        for (int q = 0; q < kGsBatch; ++q) u[q] = __ldg(Ub + (int64_t)(i + q) * ld4 + t);
+#pragma unroll
+        for (int q = 0; q < kGsBatch; ++q) axpy4(cf[i + q], u[q], a);
+      }
+      if (i < k) {
+        float4 u[kGsBatch];
+#pragma unroll
+        for (int q = 0; q < kGsBatch; ++q) u[q] = __ldg(Ub + (int64_t)min(i + q, k - 1) * ld4 + t);
+#pragma unroll
+        for (int q = 0; q < kGsBatch; ++q)
+          if (i + q < k) axpy4(cf[i + q], u[q], a);
+      }
+      w[t] = a;
+      ss = dot4(a, a, ss);
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+  if (lane == 0) sh[0][wid] = ss;
+  __syncthreads();
+  if (tid == 0) {
+    double t = 0.0;
+#pragma unroll
+    for (int v = 0; v < 8; ++v) t += (double)sh[0][v];
+    atomicAdd(cur + kMaxInner, t);
+  }
+  if (!last_block(ticket, gridDim.x) || tid) return;
+  *S.arrived = 0;  // every block has passed the barrier
+  finish_norm(S, __ldcg(cur + kMaxInner));
 }
 
 // y_i = Dinv_i (inv_s[0] u_i) per node, FP32 3x3 blocks
@@ -178,7 +228,6 @@ __global__ void k_block_apply32(int64_t N, const float* __restrict__ Dinv, const
 // coef_i u_i.  Thread l holds column l: step j makes rotation j from column j and applies it
 // to the columns after it; then a column-oriented back-substitution over the columns before
 // the first breakdown (a zero rotated column).
-constexpr int kMaxInner = 64;
 __global__ void __launch_bounds__(kMaxInner) k_inner_lsq(int d, const double* __restrict__ sv,
                                                          const double* __restrict__ Hg, double* __restrict__ coef) {
   __shared__ double H[kMaxInner + 1][kMaxInner + 1], g[kMaxInner + 1], cs[kMaxInner], sn[kMaxInner], y[kMaxInner];
@@ -268,43 +317,39 @@ __global__ void k_to_f64_scaled(int64_t n, const float* __restrict__ x, double s
 
 }  // namespace
 
-int inner_dot_blocks(int64_t n) {
-  const int64_t chunk = 4 * 256 * kRows;
-  return (int)std::min<int64_t>(kInnerBlocks, std::max<int64_t>(1, (n + chunk - 1) / chunk));
-}
 int inner_max_depth() { return kMaxInner; }
+int inner_sum_doubles() { return 2 * kGsSums; }
 
-cudaError_t launch_multi_dot_f32(int64_t n, int k, const float* Ub, int64_t ld, const float* w, double* part,
-                                 unsigned* ticket, double* d, cudaStream_t s) {
-  if (k <= 0) return cudaSuccess;
-  if ((n | ld) & 3) return cudaErrorInvalidValue;  // rows padded to float4
-  const int nb = inner_dot_blocks(n), groups = (k + 3) / 4;
-  const int gy = std::min(groups, std::max(1, kInnerBlocks / nb));
-  // the last block adds up to 16 k partials; beyond that a block per vector does
-  const bool fused = (int64_t)nb * k <= 16384;
-  k_multi_dot_f32<<<dim3(nb, gy), 256, 0, s>>>(n / 4, k, (const float4*)Ub, ld / 4, (const float4*)w, part,
-                                               fused ? ticket : nullptr, d);
-  note_launch();
-  return fused ? cudaGetLastError() : launch_reduce_cols(nb, k, part, d, s);
-}
-
-static cudaError_t launch_update(int64_t n, int k, const float* Ub, int64_t ld, float* w, double* part,
-                                 unsigned* ticket, const InnerStep& S, cudaStream_t s) {
-  if ((n | ld) & 3) return cudaErrorInvalidValue;  // rows padded to float4
-  const int nb = (int)std::min<int64_t>(kUpdBlocks, std::max<int64_t>(1, (n / 4 + 255) / 256));
-  k_multi_axpy_norm_f32<<<nb, 256, (k > 0 ? k : 1) * sizeof(float), s>>>(n / 4, k, (const float4*)Ub, ld / 4, (float4*)w,
-                                                                        part, ticket, S);
+cudaError_t launch_inner_start(int64_t n, int d, const float* u0, double* part, unsigned* ticket, double* sv,
+                               double* dinv, float* inv_s, double* sums, cudaStream_t s) {
+  if (n & 3) return cudaErrorInvalidValue;  // rows padded to float4
+  const int nb = (int)std::min<int64_t>(kInnerBlocks, std::max<int64_t>(1, (n / 4 + 255) / 256));
+  k_inner_start<<<nb, 256, 0, s>>>(n / 4, (const float4*)u0, part, ticket,
+                                   InnerStep{-1, d, sv, dinv, inv_s, nullptr, sums, nullptr});
   note_launch();
   return cudaGetLastError();
 }
-cudaError_t launch_inner_start(int64_t n, int d, float* u0, double* part, unsigned* ticket, double* sv, double* dinv,
-                               float* inv_s, cudaStream_t s) {
-  return launch_update(n, 0, u0, n, u0, part, ticket, InnerStep{-1, d, nullptr, sv, dinv, inv_s, nullptr}, s);
-}
-cudaError_t launch_inner_update(int64_t n, int j, int d, const float* Ub, int64_t ld, const double* dd, float* w,
-                                double* part, unsigned* ticket, double* sv, double* dinv, float* inv_s, double* H,
-                                cudaStream_t s) {
-  return launch_update(n, j + 1, Ub, ld, w, part, ticket, InnerStep{j, d, dd, sv, dinv, inv_s, H}, s);
+cudaError_t launch_inner_gs(int64_t n, int j, int d, const float* Ub, int64_t ld, float* w, unsigned* ticket,
+                            double* sv, double* dinv, float* inv_s, double* H, double* sums, unsigned* arrived, int* err,
+                            cudaStream_t s) {
+  if ((n | ld) & 3 || j + 1 > kMaxInner) return cudaErrorInvalidValue;  // rows padded to float4
+  int dev = 0, n_sm = 0, per = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_inner_gs, 256, 0);
+  if (e != cudaSuccess) return e;
+  // chunks in equal shares of as many blocks as are resident together
+  const int64_t chunks = std::max<int64_t>(1, (n / 4 + 255) / 256), most = (int64_t)n_sm * std::max(1, per);
+  const int64_t share = (chunks + most - 1) / most, nb = (chunks + share - 1) / share;
+  int64_t n4 = n / 4, ld4 = ld / 4;
+  int k = j + 1;
+  const float4* U = (const float4*)Ub;
+  float4* w4 = (float4*)w;
+  InnerStep S{j, d, sv, dinv, inv_s, H, sums, arrived};
+  void* args[] = {&n4, &k, &U, &ld4, &w4, &ticket, &err, &S};
+  e = cudaLaunchCooperativeKernel(k_inner_gs, dim3((unsigned)nb), dim3(256), args, 0, s);
+  note_launch();
+  return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
 cudaError_t launch_block_apply32(int64_t N, const float* Dinv32, const float* u, const float* inv_s, float* y,

@@ -140,7 +140,7 @@ cudaError_t launch_diag_rows(const RowArgs& R, T* Dg, cudaStream_t s);
 constexpr int kRedBlocks = 608;  // 4 x 152 SMs
 // persistent grid of the inner FP32 Gram-Schmidt kernels: 8 blocks of 256 per SM, enough
 // loads in flight for a streaming kernel with few registers
-constexpr int kInnerBlocks = 8 * 152;
+constexpr int kInnerBlocks = 6 * 152;
 constexpr int kRedThreads = 256;
 
 // history h_s = (b1 c^k + b2 c^{k-1}) / dt, [N][2]
@@ -203,22 +203,20 @@ cudaError_t launch_reduce_cols(int nparts, int k, const double* part, double* ou
 
 // ---------------------------------------------- inner FP32 GMRES (inner_krylov.cu)
 // All on FP32 vectors of n entries, n and ld multiples of 4, 16-byte aligned (rows padded
-// with zeros); ticket: a zeroed counter of the stream; part: inner_dot_blocks(n) doubles per
-// vector, at least kInnerBlocks.
-int inner_dot_blocks(int64_t n);
+// with zeros); ticket, arrived: zeroed counters of the stream; part: kInnerBlocks doubles;
+// sums: inner_sum_doubles() doubles.
 int inner_max_depth();
-// d_i = U_i . w (i < k)
-cudaError_t launch_multi_dot_f32(int64_t n, int k, const float* Ub, int64_t ld, const float* w, double* part,
-                                 unsigned* ticket, double* d, cudaStream_t s);
+int inner_sum_doubles();
 // The Arnoldi bookkeeping stays on the device: norms s_i (sv), 1 / s_i^2 (dinv), 1 / s_i
-// (inv_s) and the Hessenberg matrix H [(d+1) x d].  start: s_0 = ||u0||; update: step j,
-// w -= sum_{i <= j} dd_i dinv_i U_i, s_(j+1) = ||w|| and column j of H; lsq: the least
-// squares, coef_i = y_i / s_i.
-cudaError_t launch_inner_start(int64_t n, int d, float* u0, double* part, unsigned* ticket, double* sv, double* dinv,
-                               float* inv_s, cudaStream_t s);
-cudaError_t launch_inner_update(int64_t n, int j, int d, const float* Ub, int64_t ld, const double* dd, float* w,
-                                double* part, unsigned* ticket, double* sv, double* dinv, float* inv_s, double* H,
-                                cudaStream_t s);
+// (inv_s) and the Hessenberg matrix H [(d+1) x d].  start: s_0 = ||u0||; gs: step j,
+// w -= sum_{i <= j} (U_i . w) dinv_i U_i, s_(j+1) = ||w|| and column j of H, in one cooperative
+// launch whose bounded wait sets err[0] = 1 (pinned host memory) when it gives up; lsq: the
+// least squares, coef_i = y_i / s_i.
+cudaError_t launch_inner_start(int64_t n, int d, const float* u0, double* part, unsigned* ticket, double* sv,
+                               double* dinv, float* inv_s, double* sums, cudaStream_t s);
+cudaError_t launch_inner_gs(int64_t n, int j, int d, const float* Ub, int64_t ld, float* w, unsigned* ticket,
+                            double* sv, double* dinv, float* inv_s, double* H, double* sums, unsigned* arrived, int* err,
+                            cudaStream_t s);
 inline size_t inner_scalar_doubles(int d) { return (size_t)(d + 1) * d; }
 cudaError_t launch_inner_lsq(int d, const double* sv, const double* H, double* coef, cudaStream_t s);
 // y = Dinv32 (inv_s[0] u) per node (inv_s may be null: scale 1)

@@ -337,7 +337,7 @@ static int apply_op(pnp_ctx* c, const double* U, const double* x, double* w, int
 // PNP_ERR_DEVICE_FLAG when a wait of the staged J V gave up (its copies never landed)
 int ctx_check_staged_waits(pnp_ctx* c) {
   CK(cudaStreamSynchronize(c->stream));
-  if (c->hflag[0]) PNP_FAIL(PNP_ERR_DEVICE_FLAG, "J V: a staged copy of the mesh tables did not complete");
+  if (c->hflag[0]) PNP_FAIL(PNP_ERR_DEVICE_FLAG, "J V or inner solve: a bounded wait on the device gave up");
   return PNP_OK;
 }
 
@@ -385,12 +385,12 @@ static int inner_gmres32_body(pnp_ctx* c) {
   double* H = c->isc;                            // Hessenberg matrix
   double* sv = H + inner_scalar_doubles(d);      // [d+1] norms s_i of the basis vectors
   double* dinv = sv + (d + 2);                   // [d+1] 1 / s_i^2
-  double* dd = dinv + (d + 2);                   // [d+1] projections
-  double* coef = dd + (d + 2);                   // [d] combination coefficients
+  double* coef = dinv + (d + 2);                 // [d] combination coefficients
+  double* sums = coef + (d + 2);                 // of the Gram-Schmidt steps
   float* inv_s = c->iinv;
   {
     ProfScope ps(c, PNP_PROF_INNER, 4.0 * n, 2.0 * n);
-    CK(launch_inner_start(ldq, d, Q, c->part, c->ticket, sv, dinv, inv_s, s));
+    CK(launch_inner_start(ldq, d, Q, c->part, c->ticket, sv, dinv, inv_s, sums, s));
   }
   const bool tiles = on_lanes(c);
   for (int j = 0; j < d; ++j) {
@@ -406,8 +406,7 @@ static int inner_gmres32_body(pnp_ctx* c) {
     {
       const double nj = (double)n * (j + 1);
       ProfScope ps(c, PNP_PROF_INNER, 4.0 * (nj + n) + 4.0 * (nj + 2.0 * n), 4.0 * nj + 2.0 * n);
-      CK(launch_multi_dot_f32(ldq, j + 1, Q, ldq, w, c->part, c->ticket, dd, s));
-      CK(launch_inner_update(ldq, j, d, Q, ldq, dd, w, c->part, c->ticket, sv, dinv, inv_s, H, s));
+      CK(launch_inner_gs(ldq, j, d, Q, ldq, w, c->ticket, sv, dinv, inv_s, H, sums, c->ticket + 1, c->hflag, s));
     }
   }
   CK(launch_inner_lsq(d, sv, H, coef, s));
