@@ -331,7 +331,7 @@ int pnp_ctx_create(const pnp_mesh* m, const pnp_params* p, void* stream, pnp_ctx
     pnp_set_error("pnp_ctx_create: out of pinned memory");
     return fail(PNP_ERR_NOMEM);
   }
-  c->hflag[0] = c->hflag[1] = c->hflag[2] = 0;
+  c->hflag[0] = c->hflag[1] = c->hflag[2] = c->hflag[3] = 0;
   c->wait_flag = c->hflag;
   std::vector<uint8_t> faces(m->node_faces);
   for (int64_t i = 0; i < N; ++i)
@@ -427,7 +427,8 @@ int ctx_alloc_krylov(pnp_ctx* c, int m) {
   cudaError_t e = cudaMalloc((void**)&c->basis, bb);
   const size_t part_rows =
       std::max<size_t>(std::max<size_t>((size_t)kRedBlocks, (size_t)kInnerBlocks), (size_t)multi_dot_blocks(c->n3()));
-  if (e == cudaSuccess) e = cudaMalloc((void**)&c->part, sizeof(double) * part_rows * (m + 2));
+  if (e == cudaSuccess)
+    e = cudaMalloc((void**)&c->part, sizeof(double) * std::max(part_rows * (m + 2), gs_step_part(c->n3(), m)));
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->dsc, sizeof(double) * (4 * (m + 2) + 16));
   if (e == cudaSuccess) e = cudaMallocHost((void**)&c->hpin, sizeof(double) * (6 * (m + 2) + 16));
   if (e != cudaSuccess) {

@@ -68,7 +68,7 @@ struct pnp_ctx {
   double* hpin = nullptr;  // pinned host mirror of dsc
   int* dflag = nullptr;
   // pinned, set by a kernel whose bounded wait gave up: the J V's [0] of solves and the
-  // stored linearisation, [1] of pnp_jv; [2] the network inference.  wait_flag: [0], or on a multigrid level the owner's [0]
+  // stored linearisation, [1] of pnp_jv; [2] the network inference; [3] a Gram-Schmidt step.  wait_flag: [0], or on a multigrid level the owner's [0]
   int* hflag = nullptr;
   int* wait_flag = nullptr;
   // counters of this stream's launches: [0] the reductions' last block, [1] the grid barrier

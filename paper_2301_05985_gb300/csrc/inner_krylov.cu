@@ -104,12 +104,10 @@ __global__ void __launch_bounds__(256) k_inner_start(int64_t n4, const float4* _
 // a dot and an update kernel; 1,047,407 nodes memory, 57 us, 81 us as two (the basis read
 // twice: 51 us at HBM rate, 13 vectors each way).
 constexpr int kGsGroup = 24, kGsBatch = 8;
-constexpr int kGsPolls = 1 << 22;
 __global__ void __launch_bounds__(256, 3) k_inner_gs(int64_t n4, int k, const float4* __restrict__ Ub, int64_t ld4,
                                                      float4* w, unsigned* ticket, int* err, InnerStep S) {
   __shared__ float sh[kGsGroup][8];
   __shared__ float cf[kMaxInner];
-  __shared__ bool passed;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int64_t chunks = (n4 + 255) / 256;
   double *cur = S.sums + (S.j & 1) * kGsSums, *next = S.sums + (~S.j & 1) * kGsSums;
@@ -146,21 +144,7 @@ __global__ void __launch_bounds__(256, 3) k_inner_gs(int64_t n4, int k, const fl
     }
     __syncthreads();
   }
-  // grid barrier
-  __threadfence();
-  __syncthreads();
-  if (tid == 0) {
-    atomicAdd(S.arrived, 1u);
-    bool ok = false;
-    for (int i = 0; i < kGsPolls && !ok; ++i) {
-      unsigned n;
-      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(n) : "l"(S.arrived) : "memory");
-      ok = n >= gridDim.x;
-    }
-    if (!ok) *reinterpret_cast<volatile int*>(err) = 1;
-    passed = ok;
-  }
-  __syncthreads();
+  const bool passed = grid_barrier(S.arrived, err, kBarrierPolls);
   float ss = 0.0f;
   if (passed) {
     if (tid < k) {

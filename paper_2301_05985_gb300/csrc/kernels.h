@@ -190,6 +190,13 @@ struct GsFinish {
 // w -= sum_i d[i] dinv[i] V_i (i < k), then what `f` says
 cudaError_t launch_multi_axpy_norm(int64_t n, int k, const double* Vb, int64_t ld, const double* d, const double* dinv,
                                    double* w, double* part, unsigned* ticket, const GsFinish& f, cudaStream_t s);
+// Both in one cooperative launch, for short vectors (gs_step_short): d_i = V_i . w first.
+// part: gs_step_part(n, m) doubles for k <= m + 1; ticket[0 .. 1] zeroed counters; err[0] = 1
+// (pinned host memory) when its bounded wait gave up.
+bool gs_step_short(int64_t n);
+size_t gs_step_part(int64_t n, int m);
+cudaError_t launch_gs_step(int64_t n, int k, const double* Vb, int64_t ld, double* d, const double* dinv, double* w,
+                           double* part, unsigned* ticket, int* err, const GsFinish& f, cudaStream_t s);
 // Dinv = inverse of the 3x3 blocks of D (Gauss-Jordan with partial pivoting, FP64);
 // flag[0] |= 1 on a singular or non-finite block.  D may alias Dinv when T = double.
 template <typename T>

@@ -17,3 +17,28 @@ __device__ __forceinline__ bool last_block(unsigned* ticket, unsigned total) {
   if (last) __threadfence();
   return last;
 }
+
+// Grid barrier of a cooperative launch: waits until every block has arrived; false in every
+// thread of a block whose wait gave up after `polls` polls (then *err = 1: device or mapped
+// host memory).  `arrived` is zero before the launch; a block that is the last to finish the
+// kernel (last_block after the barrier, in every block) sets it back.  Writes made before the
+// call by any block are visible after it (read them with __ldcg).
+__device__ __forceinline__ bool grid_barrier(unsigned* arrived, int* err, int polls) {
+  __shared__ bool passed;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    atomicAdd(arrived, 1u);
+    bool ok = false;
+    for (int i = 0; i < polls && !ok; ++i) {
+      unsigned n;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(n) : "l"(arrived) : "memory");
+      ok = n >= gridDim.x;
+    }
+    if (!ok) *reinterpret_cast<volatile int*>(err) = 1;
+    passed = ok;
+  }
+  __syncthreads();
+  return passed;
+}
+constexpr int kBarrierPolls = 1 << 22;

@@ -675,6 +675,8 @@ int ctx_gmres(pnp_ctx* c, const double* U, const double* b, double* x, double rt
   // discarded one per solve at most).  2^18 unknowns: there an FP64 iteration takes 1 ms and
   // the wait is 1 %.  3,267 unknowns: 47 us per iteration without, 36 us with it.
   const bool ahead = !flex && !flex64 && n <= (int64_t(1) << 18);
+  const bool one_launch = gs_step_short(n);
+  c->hflag[3] = 0;
   if (ahead)
     for (cudaEvent_t& e : c->step_done)
       if (!e) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
@@ -751,10 +753,6 @@ int ctx_gmres(pnp_ctx* c, const double* U, const double* b, double* x, double rt
       const double nj = (double)n * (j + 1);
       for (int pass = 0; pass < (two ? 2 : 1); ++pass) {
         double* dp = pass == 0 ? dd : dd2;
-        {
-          ProfScope ps(c, PNP_PROF_ORTHO, 8.0 * (nj + n), 2.0 * nj);
-          CK(launch_multi_dot(n, j + 1, V, n, w, c->part, c->ticket, dp, s));
-        }
         GsFinish f{dnrm};
         if (pass == (two ? 1 : 0)) {
           double* hj = hp[j & 1];
@@ -767,6 +765,15 @@ int ctx_gmres(pnp_ctx* c, const double* U, const double* b, double* x, double rt
             f.d1 = dd2;
             f.host1 = hp2[j & 1];
           }
+        }
+        if (one_launch) {
+          ProfScope ps(c, PNP_PROF_ORTHO_UPDATE, 8.0 * (2.0 * nj + 3.0 * n), 4.0 * nj + 2.0 * n);
+          CK(launch_gs_step(n, j + 1, V, n, dp, dinv, w, c->part, c->ticket, c->hflag + 3, f, s));
+          continue;
+        }
+        {
+          ProfScope ps(c, PNP_PROF_ORTHO, 8.0 * (nj + n), 2.0 * nj);
+          CK(launch_multi_dot(n, j + 1, V, n, w, c->part, c->ticket, dp, s));
         }
         ProfScope ps(c, PNP_PROF_ORTHO_UPDATE, 8.0 * (nj + 2.0 * n), 2.0 * (nj + n));
         CK(launch_multi_axpy_norm(n, j + 1, V, n, dp, dinv, w, c->part, c->ticket, f, s));
@@ -789,6 +796,7 @@ int ctx_gmres(pnp_ctx* c, const double* U, const double* b, double* x, double rt
       } else {
         CK(cudaStreamSynchronize(s));
       }
+      if (c->hflag[3]) PNP_FAIL(PNP_ERR_DEVICE_FLAG, "gmres: a bounded wait on the device gave up");
       const double *hj = hp[j & 1], *hj2 = hp2[j & 1];
       double w1sq;
       for (int i = 0; i <= j; ++i) h[i] = (two ? hj[i] + hj2[i] : hj[i]) / sv[i];

@@ -171,6 +171,19 @@ __global__ void __launch_bounds__(256, 4) k_multi_dot(int64_t n, int k, const do
   }
 }
 
+__device__ __forceinline__ void finish_step(const GsFinish& f, int k, double ss) {
+  if (threadIdx.x == 0) {
+    f.nrm2[0] = ss;
+    if (f.dinv_next) f.dinv_next[0] = ss > 0.0 ? 1.0 / ss : 0.0;
+    if (f.inv_s_next) f.inv_s_next[0] = ss > 0.0 ? 1.0 / sqrt(ss) : 0.0;
+    if (f.host_nrm2) f.host_nrm2[0] = ss;
+  }
+  if (f.host0)
+    for (int i = threadIdx.x; i < k; i += blockDim.x) f.host0[i] = __ldcg(f.d0 + i);
+  if (f.host1)
+    for (int i = threadIdx.x; i < k; i += blockDim.x) f.host1[i] = __ldcg(f.d1 + i);
+}
+
 // w -= sum_i (d_i * dinv_i) V_i and w . w of the updated w; the last block adds the partials
 // and finishes the Krylov step: w . w and its reciprocal for the next vector on the device,
 // and what the host needs of the step into mapped pinned memory (GsFinish)
@@ -204,16 +217,102 @@ __global__ void __launch_bounds__(kRedThreads) k_multi_axpy_norm(int64_t n, int 
   ss = 0.0;
   for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) ss += __ldcg(part + b);
   ss = block_sum(ss, sh);
-  if (threadIdx.x == 0) {
-    f.nrm2[0] = ss;
-    if (f.dinv_next) f.dinv_next[0] = ss > 0.0 ? 1.0 / ss : 0.0;
-    if (f.inv_s_next) f.inv_s_next[0] = ss > 0.0 ? 1.0 / sqrt(ss) : 0.0;
-    if (f.host_nrm2) f.host_nrm2[0] = ss;
+  finish_step(f, k, ss);
+}
+
+// One Gram-Schmidt step of short vectors in one cooperative launch: d_i = V_i . w, a grid
+// barrier, w -= sum_i (d_i dinv_i) V_i and w . w, and the step's end (GsFinish).  Sums: a block
+// per four vectors and chunk of rows (at most kGsChunks chunks), partials to
+// part[i][chunk], added in order by every block.  Update: a block per 32 rows, its warps
+// sharing the vectors.  The barrier's wait is bounded.  Latency, all of it.
+constexpr int kGsChunks = 64;
+constexpr int64_t kGsShort = int64_t(1) << 16;
+__global__ void __launch_bounds__(256) k_gs_step(int64_t n, int k, const double* __restrict__ Vb, int64_t ld,
+                                                 double* d, const double* __restrict__ dinv, double* w, double* part,
+                                                 unsigned* ticket, unsigned* arrived, int* err, GsFinish f) {
+  extern __shared__ double cf[];
+  __shared__ double sh[8][33];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int groups = (k + 3) / 4;
+  const int xb = (int)((n + 255) / 256 < kGsChunks ? (n + 255) / 256 : kGsChunks);
+  const int64_t rows = ((n + xb - 1) / xb + 255) / 256 * 256;
+  for (int task = blockIdx.x; task < xb * groups; task += gridDim.x) {
+    const int x = task % xb, j0 = task / xb * 4;
+    double s[4] = {0.0, 0.0, 0.0, 0.0};
+    const int64_t t1 = (x + 1) * rows < n ? (x + 1) * rows : n;
+#pragma unroll 2
+    for (int64_t t = x * rows + threadIdx.x; t < t1; t += 256) {
+      const double wv = w[t];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) s[q] = fma(__ldg(Vb + (int64_t)min(j0 + q, k - 1) * ld + t), wv, s[q]);
+    }
+    const double tot = warp_sum4(s, lane);
+    if ((lane & 7) == 0) sh[lane >> 3][wid] = tot;
+    __syncthreads();
+    if (threadIdx.x < 4 && j0 + (int)threadIdx.x < k) {
+      double t = 0.0;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) t += sh[threadIdx.x][q];
+      part[(int64_t)(j0 + threadIdx.x) * xb + x] = t;
+    }
+    __syncthreads();
   }
-  if (f.host0)
-    for (int i = threadIdx.x; i < k; i += blockDim.x) f.host0[i] = f.d0[i];
-  if (f.host1)
-    for (int i = threadIdx.x; i < k; i += blockDim.x) f.host1[i] = f.d1[i];
+  const bool passed = grid_barrier(arrived, err, kBarrierPolls);
+  double ss = 0.0;
+  if (passed) {
+    // four lanes per vector
+    for (int j0 = 0; j0 < k; j0 += 64) {
+      const int j = j0 + (threadIdx.x >> 2);
+      double t = 0.0;
+      if (j < k) {
+#pragma unroll 4
+        for (int b = threadIdx.x & 3; b < xb; b += 4) t += __ldcg(part + (int64_t)j * xb + b);
+      }
+      t += __shfl_xor_sync(0xffffffffu, t, 1);
+      t += __shfl_xor_sync(0xffffffffu, t, 2);
+      if (j < k && (threadIdx.x & 3) == 0) {
+        cf[j] = t * dinv[j];
+        if (blockIdx.x == 0) d[j] = t;
+      }
+    }
+    __syncthreads();
+    for (int64_t r0 = (int64_t)blockIdx.x * 32; r0 < n; r0 += (int64_t)gridDim.x * 32) {
+      const int64_t t = r0 + lane;
+      double v = 0.0;
+      if (t < n) {
+#pragma unroll 4
+        for (int i = wid; i < k; i += 8) v = fma(cf[i], __ldg(Vb + (int64_t)i * ld + t), v);
+      }
+      sh[wid][lane] = v;
+      __syncthreads();
+      if (wid == 0 && t < n) {
+        double a = w[t];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) a -= sh[q][lane];
+        w[t] = a;
+        ss = fma(a, a, ss);
+      }
+      __syncthreads();
+    }
+  }
+  if (wid == 0) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+    if (lane == 0) part[(int64_t)k * xb + blockIdx.x] = ss;
+  }
+  if (!last_block(ticket, gridDim.x)) return;
+  if (threadIdx.x == 0) *arrived = 0;  // every block has passed the barrier
+  ss = 0.0;
+  for (int b = threadIdx.x; b < (int)gridDim.x; b += 256) ss += __ldcg(part + (int64_t)k * xb + b);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+  __syncthreads();
+  if (lane == 0) sh[0][wid] = ss;
+  __syncthreads();
+  ss = 0.0;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) ss += sh[0][q];
+  finish_step(f, k, ss);
 }
 
 __global__ void __launch_bounds__(256) k_multi_axpy(int64_t n, int k, const double* __restrict__ Vb, int64_t ld,
@@ -430,6 +529,30 @@ cudaError_t launch_multi_axpy_norm(int64_t n, int k, const double* Vb, int64_t l
                                                                                            part, ticket, f);
   note_launch();
   return cudaGetLastError();
+}
+// Short vectors: one cooperative launch (k_gs_step).  GMRES(50) iterations with it and with the
+// two kernels, 2D: 867 unknowns 26.4 and 31.8 us, 3,267 27.4 and 32.5, 12,675 35.5 and 38.1,
+// 49,923 59.1 and 62.5, 198,147 137 and 131, 789,507 485 and 435 (the FP64 pipe; the barrier
+// and the sums in every block add to it).
+bool gs_step_short(int64_t n) { return n <= kGsShort; }
+size_t gs_step_part(int64_t n, int m) { return gs_step_short(n) ? (size_t)kGsChunks * (m + 2) + 2048 : 0; }
+cudaError_t launch_gs_step(int64_t n, int k, const double* Vb, int64_t ld, double* d, const double* dinv, double* w,
+                           double* part, unsigned* ticket, int* err, const GsFinish& f, cudaStream_t s) {
+  int dev = 0, n_sm = 0, per = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+  const size_t smem = sizeof(double) * (size_t)k;
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_gs_step, 256, smem);
+  if (e != cudaSuccess) return e;
+  const int64_t xb = std::min<int64_t>(kGsChunks, (n + 255) / 256);
+  const int64_t most = std::min<int64_t>((int64_t)n_sm * std::max(1, std::min(per, 4)), 2048);
+  const unsigned nb = (unsigned)std::min(most, std::max(xb * ((k + 3) / 4), (n + 31) / 32));
+  unsigned* arrived = ticket + 1;
+  GsFinish fin = f;
+  void* args[] = {&n, &k, &Vb, &ld, &d, &dinv, &w, &part, &ticket, &arrived, &err, &fin};
+  e = cudaLaunchCooperativeKernel(k_gs_step, dim3(nb), dim3(256), args, smem, s);
+  note_launch();
+  return e == cudaSuccess ? cudaGetLastError() : e;
 }
 cudaError_t launch_block_apply(int64_t N, const double* Dinv, const double* v, double scale, const double* scale_dev,
                                double* z, float* z32, cudaStream_t s) {
