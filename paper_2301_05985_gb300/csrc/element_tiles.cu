@@ -535,7 +535,7 @@ __global__ void k_block_apply_rows(RowArgs R, const T* __restrict__ Dinv, const 
   for (int f = 0; f < 3; ++f) out[3 * id + f] = v[f];
 }
 
-constexpr int kMaxSmem = 200 * 1024;  // a tile of 1,024 different nodes needs 84 KB
+constexpr int kMaxSmem = 200 * 1024;  // a tile of 512 different nodes needs 68 KB
 template <int D, bool ADV>
 cudaError_t plan_jv(TileTab& t) {
   const size_t smem = jv_smem_bytes(t, ADV);

@@ -190,7 +190,7 @@ static int ctx_tiles(pnp_ctx* c) {
   if (c->dim == 3 && t.threads > 128) t.threads = 128;
   t.corners = c->dim == 3 ? 4 * t.threads : t.threads;
   t.n = (c->n_elem * nc + t.corners - 1) / t.corners;
-  const TileMeshTables M{c->n_elem, c->n_nodes, c->n_hanging, c->d_conn, c->d_hpar, c->d_level, c->d_faces, c->d_hnp};
+  const TileMeshTables M{c->n_elem, c->d_conn, c->d_hpar, c->d_level, c->d_faces, c->d_hnp};
   CK(cudaMemsetAsync(c->dflag + 4, 0, 3 * sizeof(int), c->stream));
   CK(launch_build_tiles(c->dim, M, t.corners, 0, 0, nullptr, c->dflag + 4, c->stream));
   int most[3] = {0, 0, 0};

@@ -1,69 +1,71 @@
-// tiles.cu -- the node tables of the element tiles (tiles.h): one block per tile sorts its
-// (node, corner) pairs in shared memory.
+// tiles.cu -- the node tables of the element tiles (tiles.h): one block per tile, a thread per
+// corner.
 #include "kernels.h"
 #include "tiles.h"
 
 namespace {
 
-// Key: uint32_t while (nodes + hanging) x corners fits, else uint64_t.  The sort of 32-bit
-// keys takes a third of the instructions.
-template <typename Key>
-__global__ void __launch_bounds__(1024)
+// The nodes of a tile meet in a hash table in shared memory (twice as many places as corners);
+// entries are ranked by node id and an entry's corners by index, by counting the smaller ones,
+// so that a table does not depend on the order of the atomics.  (Ids in order: entries in the
+// order of their first corners made the J V 6 % slower on the uniform level-7 cube, its loads
+// and atomics touch more sectors.)  There, 32,768 tiles: 156 us to count, 412 us to build; sorting the
+// (node, corner) pairs took 475 and 539 us.
+constexpr int kMaxCorners = 512, kEmpty = INT32_MIN;
+__global__ void __launch_bounds__(kMaxCorners)
     k_build_tiles(TileMeshTables M, int nc, int cap, int hcap, uint8_t* __restrict__ rec, int* __restrict__ most) {
-  __shared__ Key key[1024];
-  __shared__ uint16_t slot_of[1024];
-  // per warp: heads (entries that start there), and heads of each class; then sums before it
-  __shared__ int heads[33], cls_heads[32][8];
+  __shared__ int node[2 * kMaxCorners], first[2 * kMaxCorners];
+  __shared__ uint16_t entry_of[2 * kMaxCorners], slot_of[kMaxCorners], list[kMaxCorners], rank_of[kMaxCorners];
+  __shared__ int count[kMaxCorners], start[kMaxCorners + 1];
+  // the record, written out as a whole (field by field its 2-byte stores took most of the time)
+  __shared__ uint4 image[(29 * kMaxCorners + 4 * kMaxCorners + kMaxCorners / 4 + 32) / 16];
+  __shared__ int heads[33][9];  // per warp, then before it: heads of each class, heads
+  __shared__ __align__(16) int head_id[kMaxCorners + 4];
   const int tl = blockDim.x, i = threadIdx.x, lane = i & 31, warp = i >> 5, n_warps = tl >> 5;
   const int64_t L = M.n_elem * nc, t0 = (int64_t)blockIdx.x * tl, t = t0 + i;
-  const int used = (int)(L - t0 < tl ? L - t0 : tl), bits = 31 - __clz(tl);
-  const int n_hanging = (int)M.n_hanging;
-  // ascending by signed id, then by corner; corners past the end last.  Bitonic, a pair's
-  // exchange within a warp by shuffles
-  Key mine = i < used ? (Key)((Key)(M.conn[t] + n_hanging) << bits | (Key)i) : ~Key(0);
-  for (int k = 2; k <= tl; k <<= 1)
-    for (int j = k >> 1; j > 0; j >>= 1) {
-      Key other;
-      if (j < 32) {
-        other = __shfl_xor_sync(0xFFFFFFFFu, mine, j);
-      } else {
-        __syncthreads();
-        key[i] = mine;
-        __syncthreads();
-        other = key[i ^ j];
-      }
-      const bool low = ((i & j) == 0) == ((i & k) == 0);  // keeps the smaller one
-      mine = low ? min(mine, other) : max(mine, other);
+  const int used = (int)(L - t0 < tl ? L - t0 : tl);
+  for (int h = i; h < 2 * tl; h += tl) {
+    node[h] = kEmpty;
+    first[h] = tl;
+  }
+  count[i] = 0;
+  __syncthreads();
+  const int32_t id = i < used ? M.conn[t] : 0;
+  int h = 0;
+  if (i < used) {
+    h = (int)((uint32_t)id * 2654435769u >> 12) & (2 * tl - 1);
+    for (;;) {
+      const int was = atomicCAS(node + h, kEmpty, id);
+      if (was == kEmpty || was == id) break;
+      h = (h + 1) & (2 * tl - 1);
     }
+    atomicMin(first + h, i);
+  }
   __syncthreads();
-  key[i] = mine;
-  __syncthreads();
-  const int corner = (int)(mine & (Key)(tl - 1)), cls = (corner / nc ^ corner) & (nc - 1);
-  const bool head = i < used && (i == 0 || (key[i - 1] >> bits) != (mine >> bits));
-  const unsigned before = (1u << lane) - 1, hm = __ballot_sync(0xFFFFFFFFu, head);
+  const bool head = i < used && first[h] == i;
+  const int cls = (i / nc ^ i) & (nc - 1);
+  const unsigned before = (1u << lane) - 1;
   int rank = 0;
   for (int c = 0; c < nc; ++c) {
     const unsigned m = __ballot_sync(0xFFFFFFFFu, head && cls == c);
     if (cls == c) rank = __popc(m & before);
-    if (lane == 0) cls_heads[warp][c] = __popc(m);
+    if (lane == 0) heads[warp][c] = __popc(m);
   }
-  if (lane == 0) heads[warp] = __popc(hm);
-  __syncthreads();
-  if (i <= nc) {  // sums over the warps: thread c < nc of class c, thread nc of all
+  const unsigned hm = __ballot_sync(0xFFFFFFFFu, head);
+  if (lane == 0) heads[warp][nc] = __popc(hm);
+  const int n_hang = __syncthreads_count(head && id < 0);
+  if (i <= nc) {
     int sum = 0;
     for (int w = 0; w < n_warps; ++w) {
-      int* p = i < nc ? &cls_heads[w][i] : &heads[w];
-      const int x = *p;
-      *p = sum;
+      const int x = heads[w][i];
+      heads[w][i] = sum;
       sum += x;
     }
-    if (i == nc) heads[n_warps] = sum;
-    else if (!rec) atomicMax(most + 1, sum * nc);
+    heads[32][i] = sum;
+    if (i < nc && !rec) atomicMax(most + 1, sum * nc);
   }
   __syncthreads();
-  const int cnt = heads[n_warps];
-  // hanging entries come first
-  const int n_hang = __syncthreads_count(head && (int64_t)(mine >> bits) < n_hanging);
+  const int cnt = heads[32][nc];
   if (!rec) {
     if (i == 0) {
       atomicMax(most, cnt);
@@ -71,29 +73,70 @@ __global__ void __launch_bounds__(1024)
     }
     return;
   }
-  const int u = heads[warp] + __popc(hm & (before | 1u << lane)) - 1;  // entry of this pair
-  const int sl = (cls_heads[warp][cls] + rank) * nc + cls;             // of a head
-  if (head) slot_of[u] = (uint16_t)sl;
+  const int sl = (heads[warp][cls] + rank) * nc + cls;  // of a head
+  const int packed = heads[warp][nc] + __popc(hm & before);  // of a head: ranked by packed threads
+  if (head) head_id[packed] = id;
+  if (i < 4) head_id[cnt + i] = INT32_MAX;
   __syncthreads();
-  uint8_t* r = rec + (int64_t)blockIdx.x * tile_bytes(tl, nc, cap, hcap);
-  int32_t* id = reinterpret_cast<int32_t*>(r);
+  if (i < cnt) {
+    const int mine = head_id[i];
+    int n = 0;
+    for (int k = 0; k < cnt; k += 4) {
+      const int4 o = *reinterpret_cast<const int4*>(head_id + k);
+      n += (o.x < mine) + (o.y < mine) + (o.z < mine) + (o.w < mine);
+    }
+    rank_of[i] = (uint16_t)n;
+  }
+  __syncthreads();
+  if (head) {
+    entry_of[h] = rank_of[packed];
+    slot_of[rank_of[packed]] = (uint16_t)sl;
+  }
+  __syncthreads();
+  const int u = i < used ? entry_of[h] : 0;
+  const int place = i < used ? atomicAdd(count + u, 1) : 0;
+  __syncthreads();
+  // start[u]: corners of the entries before u
+  {
+    const int c = count[i];
+    int x = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+      if (lane >= o) x += y;
+    }
+    if (lane == 31) heads[warp][0] = x;
+    __syncthreads();
+    int sum = 0;
+    for (int w = 0; w < warp; ++w) sum += heads[w][0];
+    start[i] = sum + x - c;
+    if (i == tl - 1) start[tl] = sum + x;
+  }
+  __syncthreads();
+  if (i < used) list[start[u] + place] = (uint16_t)i;
+  __syncthreads();
+  int at = i < used ? start[u] : 0;  // of corner i in its entry's list
+  if (i < used)
+    for (int k = start[u]; k < start[u + 1]; ++k) at += list[k] < i;
+  const int bytes = tile_bytes(tl, nc, cap, hcap);
+  uint8_t* r = reinterpret_cast<uint8_t*>(image);
+  int32_t* id_of = reinterpret_cast<int32_t*>(r);
   uint16_t *seg = reinterpret_cast<uint16_t*>(r + 4 * cap), *slot = seg + cap,
            *loc = reinterpret_cast<uint16_t*>(r + 9 * cap), *ord = loc + tl;
   uint8_t *face = r + 8 * cap, *lev = r + tile_level_at(tl, cap);
   int4* par = reinterpret_cast<int4*>(r + tile_par_at(tl, nc, cap));
   uchar4* pface = reinterpret_cast<uchar4*>(par + hcap);
   if (i < used) {
-    loc[corner] = slot_of[u];
-    ord[i] = (uint16_t)tile_share(corner, nc, tl);
+    loc[i] = slot_of[u];
+    ord[at] = (uint16_t)tile_share(i, nc, tl);
     if (head) {
-      const int32_t nid = (int32_t)(mine >> bits) - n_hanging;
-      id[u] = nid;
-      seg[u] = (uint16_t)i;
+      id_of[u] = id;
+      seg[u] = (uint16_t)start[u];
       slot[u] = (uint16_t)sl;
-      face[u] = nid >= 0 ? M.faces[nid] : 0;
-      if (nid < 0) {
-        const int32_t* p = M.hang_par + 4 * (int64_t)(-nid - 1);
-        const bool four = M.hang_np[-nid - 1] != 2;
+      face[u] = id >= 0 ? M.faces[id] : 0;
+      if (id < 0) {
+        const int32_t* p = M.hang_par + 4 * (int64_t)(-id - 1);
+        const bool four = M.hang_np[-id - 1] != 2;
         par[u] = make_int4(p[0], p[1], four ? p[2] : -1, four ? p[3] : -1);
         pface[u] = make_uchar4(M.faces[p[0]], M.faces[p[1]], four ? M.faces[p[2]] : 0, four ? M.faces[p[3]] : 0);
       }
@@ -102,12 +145,12 @@ __global__ void __launch_bounds__(1024)
     loc[i] = slot_of[0];  // corners past the end read entry 0
     ord[i] = 0;
   }
-  if (i < tl / nc) {
+  if (i < (tl / nc + 15) / 16 * 16) {
     const int64_t e = t0 / nc + i;
-    lev[i] = e < M.n_elem ? M.level[e] : 0;
+    lev[i] = i < tl / nc && e < M.n_elem ? M.level[e] : 0;
   }
   for (int w = cnt + i; w < cap; w += tl) {
-    id[w] = 0;
+    id_of[w] = 0;
     seg[w] = slot[w] = 0;
     face[w] = 0;
   }
@@ -119,7 +162,11 @@ __global__ void __launch_bounds__(1024)
     int32_t* tail = reinterpret_cast<int32_t*>(pface + hcap);
     tail[0] = cnt;
     tail[1] = used;
+    tail[2] = tail[3] = 0;
   }
+  __syncthreads();
+  uint4* out = reinterpret_cast<uint4*>(rec + (int64_t)blockIdx.x * bytes);
+  for (int k = i; k < bytes / 16; k += tl) out[k] = image[k];
 }
 
 }  // namespace
@@ -127,12 +174,9 @@ __global__ void __launch_bounds__(1024)
 cudaError_t launch_build_tiles(int dim, const TileMeshTables& M, int corners, int cap, int hcap, uint8_t* rec,
                                int* most, cudaStream_t s) {
   if (M.n_elem == 0) return cudaSuccess;
-  if (corners > 1024) return cudaErrorInvalidValue;
+  if (corners > kMaxCorners || cap > kMaxCorners || hcap > kMaxCorners) return cudaErrorInvalidValue;
   const unsigned n = (unsigned)(((M.n_elem << dim) + corners - 1) / corners);
-  if ((M.n_nodes + M.n_hanging) * corners < int64_t(0xFFFFFFFF))
-    k_build_tiles<uint32_t><<<n, corners, 0, s>>>(M, 1 << dim, cap, hcap, rec, most);
-  else
-    k_build_tiles<uint64_t><<<n, corners, 0, s>>>(M, 1 << dim, cap, hcap, rec, most);
+  k_build_tiles<<<n, corners, 0, s>>>(M, 1 << dim, cap, hcap, rec, most);
   note_launch();
   return cudaGetLastError();
 }

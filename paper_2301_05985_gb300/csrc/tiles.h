@@ -66,7 +66,7 @@ __host__ __device__ inline int tile_share(int corner, int nc, int corners) {
 // Counts (rec null: the largest counts of entries, slots and hanging entries into
 // most[0 .. 2], zeroed by the caller) or builds (rec) the records of a mesh (device tables conn [E][2^dim], level, faces).
 struct TileMeshTables {
-  int64_t n_elem, n_nodes, n_hanging;
+  int64_t n_elem;
   const int32_t *conn, *hang_par;
   const uint8_t *level, *faces, *hang_np;
 };
