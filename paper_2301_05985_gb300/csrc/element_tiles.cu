@@ -57,12 +57,12 @@ __device__ __forceinline__ void add_entry(const TileMesh& M, const TileView& v, 
 // shared-memory wavefronts 66 %: a third each the nodes' loads, the shuffles, the sums).  On
 // the uniform level-7 cube (2,097,152 elements) with advection 174 us a launch, 0.28 GB of
 // DRAM traffic; before, the state stored per Gauss point (64 bytes a lane, 1.1 GB a launch)
-// 262 us.  Membrane-band octree of 971,776 elements 95 us (115), of 143,872 elements 20 us
-// (24).  Steps on the way, level-7 cube: a lane per corner on such tiles 340 us; halves of
-// elements in tiles of 128 (two blocks per SM) 248; tiles of 64 (four blocks) and 16-byte
-// shares 187; nodes' values by asynchronous copies during the sums, slots by parity 174.
-// Hanging nodes' parents in the record: 104 to 95 us on the octree (their chain of loads held
-// the block's barrier).
+// 262 us.  Membrane-band octree of 971,776 elements 94 us (115), of 143,872 elements 19 us
+// (24), without advection 17 (five blocks fit an SM; 18 with four).  Steps on the way, level-7
+// cube: a lane per corner on such tiles 340 us; halves of elements in tiles of 128 (two blocks
+// per SM) 248; tiles of 64 (four blocks) and 16-byte shares 187; nodes' values by asynchronous
+// copies during the sums, slots by parity 174.  Hanging nodes' parents in the record: 104 to
+// 95 us on the octree (their chain of loads held the block's barrier).
 struct JvArgs {
   const float4* rec;
   const float* V;
@@ -341,7 +341,7 @@ __device__ __forceinline__ void fetch_entry(const TileMesh& M, const JvArgs& A, 
 // the Gauss points are evaluated, and its nodal values while the sums are made (the slots are
 // free then).
 template <int D, bool ADV>
-__global__ void __launch_bounds__(D == 3 ? 128 : 256, 4)
+__global__ void __launch_bounds__(D == 3 ? 128 : 256, D == 3 && !ADV ? 5 : 4)
     k_jv_tiles(TileMesh M, JvArgs A, LaneParams<float> K, int* err, int polls) {
   constexpr int NC = 1 << D;
   extern __shared__ __align__(128) uint8_t tile_smem[];
