@@ -127,6 +127,7 @@ __global__ void __launch_bounds__(256, sizeof(C) == 8 && !std::is_same<C, double
   const bool valid = e < A.n_elem;
   const int32_t id = valid ? __ldg(A.conn + e * NC + c) : 0;
   const int lev = valid ? A.level[e] : 0;
+  grid_dependency_wait();  // so far only the mesh's tables
   C un[3], vn[3], hn[2], dn[3];
   load_node_c<C, 3>(A, id, valid, A.U, 3, un);
   load_node_c<C, 3>(A, id, valid, A.adv, 3, vn);
@@ -377,10 +378,10 @@ static cudaError_t launch_lanes(int dim, const ElemArgs<double>& A, cudaStream_t
   const int t = block_threads(A.n_elem << dim);
   const unsigned blocks = block_count(A.n_elem << dim, t);
   const LaneParams<C> K = lane_params<C>(A.P, dim);
-  if (dim == 2) k_element_lanes<C, 2, JV><<<blocks, t, 0, s>>>(A, K);
-  else k_element_lanes<C, 3, JV><<<blocks, t, 0, s>>>(A, K);
+  const cudaError_t e = dim == 2 ? launch_kernel(true, k_element_lanes<C, 2, JV>, blocks, t, 0, s, A, K)
+                                 : launch_kernel(true, k_element_lanes<C, 3, JV>, blocks, t, 0, s, A, K);
   note_launch();
-  return cudaGetLastError();
+  return e == cudaSuccess ? cudaGetLastError() : e;
 }
 cudaError_t launch_residual_lanes(int dim, bool double_float, const ElemArgs<double>& A, cudaStream_t s) {
   return double_float ? launch_lanes<df, false>(dim, A, s) : launch_lanes<double, false>(dim, A, s);

@@ -375,10 +375,12 @@ __global__ void __launch_bounds__(D == 3 ? 128 : 256, D == 3 && !ADV ? 5 : 4)
   __syncthreads();
   if (tid == 0) issue(blockIdx.x, 0);
   if (__syncthreads_or(!mbar_wait(&bar[0], 0, polls))) {
+    grid_dependency_wait();
     give_up(0);
     return;
   }
   TileView v = tile_view(stage, M.tab);
+  grid_dependency_wait();  // so far only the mesh's tables
   fetch(v);
   for (int k = 0;; ++k) {
     const int64_t tile = blockIdx.x + k * G;
@@ -496,43 +498,66 @@ __global__ void k_init_rows(RowArgs R, const T* __restrict__ in, T* __restrict__
 // block-Jacobi apply y = Dinv (scale u), and the rows of the J V of y that follows (as
 // k_init_rows, mode 1; a hanging node's thread makes its parents' y again)
 template <typename T>
-__device__ __forceinline__ void apply3(const T* __restrict__ Dinv, const T* __restrict__ u, T sc, int64_t i, T (&y)[3]) {
-  const T* B = Dinv + 9 * i;
+__device__ __forceinline__ void apply3(const T (&B)[9], const T* u, T sc, int64_t i, T (&y)[3]) {
   const T a = sc * u[3 * i], b = sc * u[3 * i + 1], c = sc * u[3 * i + 2];
   y[0] = fma(B[0], a, fma(B[1], b, B[2] * c));
   y[1] = fma(B[3], a, fma(B[4], b, B[5] * c));
   y[2] = fma(B[6], a, fma(B[7], b, B[8] * c));
 }
 template <typename T>
-__global__ void k_block_apply_rows(RowArgs R, const T* __restrict__ Dinv, const T* __restrict__ u, T scale,
-                                   const T* __restrict__ scale_dev, T* __restrict__ y, T* __restrict__ out) {
+__device__ __forceinline__ void load_block(const T* __restrict__ Dinv, int64_t i, T (&B)[9]) {
+#pragma unroll
+  for (int q = 0; q < 9; ++q) B[q] = __ldg(Dinv + 9 * i + q);
+}
+// The blocks and the mesh's tables are older than the launch before; u and the scale are its
+// results.  FP64: a dependent launch, in the stream of small GMRES iterations (a 2D time step
+// with 3,267 unknowns 14.4 ms without any, 13.4 with the element kernel's, 12.4 with both).
+// FP32: not, nor the J V after it: between the nodes of the inner solve's graph dependent
+// launches cost more than they hide (17.3 ms a step on 143,872 elements, 17.8 with this one,
+// 18.0 with both).
+template <typename T>
+__global__ void k_block_apply_rows(RowArgs R, const T* __restrict__ Dinv, const T* u, T scale, const T* scale_dev,
+                                   T* __restrict__ y, T* __restrict__ out) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t h = i - R.n_nodes;
+  const bool node = i < R.n_nodes, hanging = !node && h < R.n_hanging;
+  T B[9], v[3];
+  uint8_t fm = 0;
+  int np = 0;
+  int64_t id = i;
+  if (node) {
+    load_block(Dinv, i, B);
+    fm = R.faces[i];
+  }
+  if (hanging) {
+    id = R.hnode[h];
+    np = R.hnp[h];
+    load_block(Dinv, id, B);
+  }
+  grid_dependency_wait();
+  grid_dependency_release();
   const T sc = scale_dev ? scale_dev[0] : scale;
-  T v[3];
-  if (i < R.n_nodes) {
-    apply3(Dinv, u, sc, i, v);
+  if (node) {
+    apply3(B, u, sc, i, v);
 #pragma unroll
     for (int f = 0; f < 3; ++f) y[3 * i + f] = v[f];
-    const uint8_t fm = R.faces[i];
     if (fm & 0x80) return;
 #pragma unroll
     for (int f = 0; f < 3; ++f) out[3 * i + f] = (fm & R.bc.dir_faces[f] & 0x3F) ? v[f] : T(0);
-    return;
-  }
-  const int64_t h = i - R.n_nodes;
-  if (h >= R.n_hanging) return;
-  const int np = R.hnp[h];
-  const T wgt = np == 2 ? T(0.5) : T(0.25);
-  const int64_t id = R.hnode[h];
-  apply3(Dinv, u, sc, id, v);
-  for (int p = 0; p < np; ++p) {
-    T w[3];
-    apply3(Dinv, u, sc, R.hpar[4 * h + p], w);
+  } else if (hanging) {
+    const T wgt = np == 2 ? T(0.5) : T(0.25);
+    apply3(B, u, sc, id, v);
+    for (int p = 0; p < np; ++p) {
+      T w[3];
+      const int64_t pid = R.hpar[4 * h + p];
+      load_block(Dinv, pid, B);
+      apply3(B, u, sc, pid, w);
 #pragma unroll
-    for (int f = 0; f < 3; ++f) v[f] -= wgt * w[f];
-  }
+      for (int f = 0; f < 3; ++f) v[f] -= wgt * w[f];
+    }
 #pragma unroll
-  for (int f = 0; f < 3; ++f) out[3 * id + f] = v[f];
+    for (int f = 0; f < 3; ++f) out[3 * id + f] = v[f];
+  }
 }
 
 constexpr int kMaxSmem = 200 * 1024;  // a tile of 512 different nodes needs 68 KB
@@ -551,11 +576,12 @@ cudaError_t plan_jv(TileTab& t) {
   return cudaSuccess;
 }
 template <int D, bool ADV>
-cudaError_t launch_jv(const TileMesh& M, const JvArgs& A, const LaneParams<float>& K, int* err, int polls,
-                      cudaStream_t s) {
-  k_jv_tiles<D, ADV><<<M.tab.blocks[ADV], M.tab.threads, jv_smem_bytes(M.tab, ADV), s>>>(M, A, K, err, polls);
+cudaError_t launch_jv(const TileMesh& M, const JvArgs& A, const LaneParams<float>& K, bool dependent, int* err,
+                      int polls, cudaStream_t s) {
+  const cudaError_t e = launch_kernel(dependent, k_jv_tiles<D, ADV>, (unsigned)M.tab.blocks[ADV], M.tab.threads,
+                                      jv_smem_bytes(M.tab, ADV), s, M, A, K, err, polls);
   note_launch();
-  return cudaGetLastError();
+  return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
 }  // namespace
@@ -567,14 +593,16 @@ cudaError_t plan_jv_tiles(int dim, TileTab& t) {
 }
 
 cudaError_t launch_jv_tiles(int dim, const TileMesh& M, const float4* rec, bool advection, const float* V,
-                            const PhysParams& P, float* out, int* err, int polls, cudaStream_t s) {
+                            const PhysParams& P, float* out, bool dependent, int* err, int polls, cudaStream_t s) {
   if (polls < 0) polls = kWaitPolls;
   if (M.tab.n == 0) return cudaSuccess;
   const JvArgs A{rec, V, out};
   const LaneParams<float> K = lane_params<float>(P, dim);
   if (dim == 2)
-    return advection ? launch_jv<2, true>(M, A, K, err, polls, s) : launch_jv<2, false>(M, A, K, err, polls, s);
-  return advection ? launch_jv<3, true>(M, A, K, err, polls, s) : launch_jv<3, false>(M, A, K, err, polls, s);
+    return advection ? launch_jv<2, true>(M, A, K, dependent, err, polls, s)
+                     : launch_jv<2, false>(M, A, K, dependent, err, polls, s);
+  return advection ? launch_jv<3, true>(M, A, K, dependent, err, polls, s)
+                   : launch_jv<3, false>(M, A, K, dependent, err, polls, s);
 }
 
 template <typename T>
@@ -607,8 +635,11 @@ cudaError_t launch_block_apply_rows(const RowArgs& R, const T* Dinv, const T* u,
   const int64_t n = R.n_nodes + R.n_hanging;
   if (n) {
     const int t = block_threads(n);
-    k_block_apply_rows<T><<<block_count(n, t), t, 0, s>>>(R, Dinv, u, scale, scale_dev, y, out);
+    const cudaError_t e =
+        launch_kernel(sizeof(T) == 8, k_block_apply_rows<T>, block_count(n, t), t, 0, s, R, Dinv, u, scale, scale_dev, y,
+                      out);
     note_launch();
+    if (e != cudaSuccess) return e;
   }
   return cudaGetLastError();
 }

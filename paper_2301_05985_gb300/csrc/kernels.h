@@ -45,6 +45,32 @@ struct RowArgs {
   BcTable bc;
 };
 
+// Launches a kernel; with `dependent` it may start while the one before it on the stream ends
+// (programmatic dependent launch): it calls grid_dependency_wait() before it touches anything that launch
+// makes or reads, and the other may call grid_dependency_release() when its blocks need no
+// more of the chip.
+template <typename... P, typename... A>
+inline cudaError_t launch_kernel(bool dependent, void (*kernel)(P...), unsigned blocks, int threads, size_t smem,
+                                 cudaStream_t s, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(blocks);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = dependent ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+#ifdef __CUDACC__
+__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_dependency_release() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+#endif
+
 // Counts every kernel the library launches (read by pnp_kernel_launches).
 void note_launch();
 // adds n launches (a replayed graph's kernels) and reads the counter
@@ -99,10 +125,10 @@ double element_kernel_flops(int dim, bool jv);
 // FP32 J V [N][3] on node tiles (element_tiles.cu) at the state of the node records
 // (launch_node_records); `advection` false when the advection field is zero.  err[0] = 1
 // (mapped pinned memory) when a wait on a staged table gave up after `polls` polls (< 0: the
-// default, about a second).  plan_jv_tiles: the grids for a table (t.blocks), once.
+// default, about a second).  dependent: as launch_kernel.  plan_jv_tiles: the grids for a table (t.blocks), once.
 cudaError_t plan_jv_tiles(int dim, TileTab& t);
 cudaError_t launch_jv_tiles(int dim, const TileMesh& M, const float4* rec, bool advection, const float* V,
-                            const PhysParams& P, float* out, int* err, int polls, cudaStream_t s);
+                            const PhysParams& P, float* out, bool dependent, int* err, int polls, cudaStream_t s);
 double jv_tiles_flops(int dim, bool advection);
 // out = 0 on weak-form rows, in - g (mode 0) or in (mode 1) on Dirichlet rows, the
 // constraint of in on hanging rows

@@ -231,10 +231,12 @@ int ctx_prepare_f32(pnp_ctx* c, const double* U, bool check_adv) {
 }
 
 // adds J V to the initialised rows of JV32, at the node records `rec`
-static int jv_tiles(pnp_ctx* c, const float4* rec, const PhysParams& P, bool adv, const float* V32, float* JV32) {
+static int jv_tiles(pnp_ctx* c, const float4* rec, const PhysParams& P, bool adv, const float* V32, float* JV32,
+                    bool dependent = true) {
   RC(ctx_tiles(c));
   ProfScope ps(c, PNP_PROF_JV32, 56.0 * c->n_nodes + c->conn_bytes(), jv_tiles_flops(c->dim, adv) * c->n_elem);
-  CK(launch_jv_tiles(c->dim, c->tile_mesh(), rec, adv, V32, P, JV32, c->wait_flag, c->wait_polls, c->stream));
+  CK(launch_jv_tiles(c->dim, c->tile_mesh(), rec, adv, V32, P, JV32, dependent, c->wait_flag, c->wait_polls,
+                     c->stream));
   c->jv_count++;
   return PNP_OK;
 }
@@ -401,7 +403,7 @@ static int inner_gmres32_body(pnp_ctx* c) {
         CK(launch_block_apply_rows<float>(c->rows(), c->Dinv32, Q + (size_t)j * ldq, 1.0f, inv_s + j, c->V32, w, s));
       else CK(launch_block_apply32(N, c->Dinv32, Q + (size_t)j * ldq, inv_s + j, c->V32, s));
     }
-    if (tiles) RC(jv_tiles(c, c->rec32, c->phys(), !c->adv_zero, c->V32, w));
+    if (tiles) RC(jv_tiles(c, c->rec32, c->phys(), !c->adv_zero, c->V32, w, false));
     else RC(ctx_jv32(c, c->V32, w));
     {
       const double nj = (double)n * (j + 1);

@@ -295,6 +295,7 @@ __global__ void __launch_bounds__(256) k_gs_step(int64_t n, int k, const double*
       __syncthreads();
     }
   }
+  grid_dependency_release();
   if (wid == 0) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
