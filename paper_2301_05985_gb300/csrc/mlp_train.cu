@@ -312,8 +312,16 @@ __global__ void __launch_bounds__(kFbThreads, 1) k_mlp_fwd_bwd(MlpGradArgs g) {
 // gives 17 tiles enough blocks: about 256 rows each, at most kSplits.
 constexpr int kSplits = 32, kWgThreads = 128, kWgRows = 32, kLdT = 72;
 constexpr int kWgTiles = 8 + 4 + 4 + 2;
+// more rows than this: the splits as one accumulation (1e-5 apart without at 8,192 rows)
+constexpr int64_t kThroughRows = 8192;
 
-__global__ void __launch_bounds__(kWgThreads) k_mlp_wgrad(MlpGradArgs g, float* __restrict__ part) {
+// base given: a split's accumulators start from the sum of the splits before it, and what it
+// adds to that is its partial.  The tensor core truncates its FP32 sums, so a sum over all
+// rows that runs through loses up to 1e-4 of itself at 65,536 rows against one in 32 short
+// pieces; with the base the gradient is that of one accumulation over the rows, whatever the
+// split, as it has been (1.1e-4 apart without, under 1e-6 with it).
+__global__ void __launch_bounds__(kWgThreads) k_mlp_wgrad(MlpGradArgs g, float* __restrict__ part,
+                                                          const float* __restrict__ base) {
   __shared__ __align__(16) bf16 At[2][kWgRows][kLdT], Bt[2][kWgRows][kLdT];
   int t = blockIdx.x;
   const bf16 *A, *B;
@@ -336,12 +344,20 @@ __global__ void __launch_bounds__(kWgThreads) k_mlp_wgrad(MlpGradArgs g, float* 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, gid = lane >> 2, tig = lane & 3;
   const int wm = (warp >> 1) * 32, wn = (warp & 1) * 32;
   float acc[2][4][4];
+  // entry of acc[i][j][q] in the split's parameters, -1 outside
+  auto entry = [&](int i, int j, int q) -> int64_t {
+    const int m = m0 + wm + 16 * i + gid + 8 * (q >> 1), n = n0 + wn + 8 * j + 2 * tig + (q & 1);
+    return m < m_end && n < n_end ? (int64_t)blockIdx.y * kParams + off + m * ldw + n : -1;
+  };
 #pragma unroll
   for (int i = 0; i < 2; ++i)
 #pragma unroll
     for (int j = 0; j < 4; ++j)
 #pragma unroll
-      for (int q = 0; q < 4; ++q) acc[i][j][q] = 0.f;
+      for (int q = 0; q < 4; ++q) {
+        const int64_t at = entry(i, j, q);
+        acc[i][j][q] = base && at >= 0 ? base[at] : 0.f;
+      }
   // 32 rows x 64 columns of each operand; what lies outside is filled with zeros
   auto stage = [&](int64_t k, int st) {
 #pragma unroll
@@ -380,16 +396,26 @@ __global__ void __launch_bounds__(kWgThreads) k_mlp_wgrad(MlpGradArgs g, float* 
     }
     __syncthreads();
   }
-  float* o = part + (int64_t)blockIdx.y * kParams + off;
 #pragma unroll
   for (int i = 0; i < 2; ++i)
 #pragma unroll
     for (int j = 0; j < 4; ++j)
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        const int m = m0 + wm + 16 * i + gid + 8 * (q >> 1), n = n0 + wn + 8 * j + 2 * tig + (q & 1);
-        if (m < m_end && n < n_end) o[m * ldw + n] = acc[i][j][q];
+        const int64_t at = entry(i, j, q);
+        if (at >= 0) part[at] = base ? acc[i][j][q] - base[at] : acc[i][j][q];
       }
+}
+// base of a split: the sum of the splits before it
+__global__ void __launch_bounds__(256) k_mlp_base(int splits, const float* __restrict__ part, float* __restrict__ base) {
+  const int64_t i = blockIdx.x * 256 + threadIdx.x;
+  if (i >= kParams) return;
+  float s = 0.f;
+#pragma unroll 8
+  for (int k = 0; k < splits; ++k) {
+    base[k * kParams + i] = s;
+    s += part[k * kParams + i];
+  }
 }
 
 // ---- the partials, summed in a fixed order: weights over the splits, biases and the loss
@@ -427,7 +453,7 @@ __global__ void __launch_bounds__(256) k_mlp_reduce(int64_t rows, int splits, in
 
 }  // namespace
 
-size_t mlp_grad_part_floats() { return (size_t)kFbCtas * kBias + (size_t)kSplits * kParams; }
+size_t mlp_grad_part_floats() { return (size_t)kFbCtas * kBias + 2 * (size_t)kSplits * kParams; }
 int mlp_grad_max_ctas() { return kFbCtas; }
 
 cudaError_t launch_mlp_grad(const MlpGradArgs& a, cudaStream_t s) {
@@ -451,7 +477,13 @@ cudaError_t launch_mlp_grad(const MlpGradArgs& a, cudaStream_t s) {
   const int splits = (int)std::min<int64_t>(kSplits, std::max<int64_t>(1, a.rows / 256));
   float* wpart = a.part + (size_t)kFbCtas * kBias;
   k_mlp_fwd_bwd<<<ctas, kFbThreads, kFbSmem, s>>>(a);
-  k_mlp_wgrad<<<dim3(kWgTiles, splits), kWgThreads, 0, s>>>(a, wpart);
+  k_mlp_wgrad<<<dim3(kWgTiles, splits), kWgThreads, 0, s>>>(a, wpart, nullptr);
+  if (a.rows > kThroughRows) {
+    float* base = wpart + (size_t)kSplits * kParams;
+    k_mlp_base<<<(unsigned)((kParams + 255) / 256), 256, 0, s>>>(splits, wpart, base);
+    k_mlp_wgrad<<<dim3(kWgTiles, splits), kWgThreads, 0, s>>>(a, wpart, base);
+    note_launches(2);
+  }
   k_mlp_reduce<<<(unsigned)((kParams + 255) / 256), 256, 0, s>>>(a.rows, splits, ctas, wpart, a.part, a.loss_part,
                                                                  a.grad, a.loss);
   note_launches(3);
