@@ -40,7 +40,7 @@ __device__ __forceinline__ double block_sum_d(double v, double* sh) {
 }
 
 // The inner basis has rows padded to a multiple of four floats (zeros beyond the
-// vector's length), so both Gram-Schmidt kernels move float4: four entries per load.
+// vector's length), so its kernels move float4: four entries per load.
 
 // Arnoldi bookkeeping of the inner process.  Basis vectors u_i are kept unnormalised
 // with norms s_i (q_i = u_i / s_i).  The steps only store the Hessenberg columns

@@ -315,11 +315,12 @@ constexpr int kWgTiles = 8 + 4 + 4 + 2;
 // more rows than this: the splits as one accumulation (1e-5 apart without at 8,192 rows)
 constexpr int64_t kThroughRows = 8192;
 
-// base given: a split's accumulators start from the sum of the splits before it, and what it
+// THROUGH: a split's accumulators start from the sum of the splits before it, and what it
 // adds to that is its partial.  The tensor core truncates its FP32 sums, so a sum over all
 // rows that runs through loses up to 1e-4 of itself at 65,536 rows against one in 32 short
 // pieces; with the base the gradient is that of one accumulation over the rows, whatever the
 // split, as it has been (1.1e-4 apart without, under 1e-6 with it).
+template <bool THROUGH>
 __global__ void __launch_bounds__(kWgThreads) k_mlp_wgrad(MlpGradArgs g, float* __restrict__ part,
                                                           const float* __restrict__ base) {
   __shared__ __align__(16) bf16 At[2][kWgRows][kLdT], Bt[2][kWgRows][kLdT];
@@ -355,8 +356,8 @@ __global__ void __launch_bounds__(kWgThreads) k_mlp_wgrad(MlpGradArgs g, float* 
     for (int j = 0; j < 4; ++j)
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        const int64_t at = entry(i, j, q);
-        acc[i][j][q] = base && at >= 0 ? base[at] : 0.f;
+        const int64_t at = THROUGH ? entry(i, j, q) : -1;
+        acc[i][j][q] = at >= 0 ? base[at] : 0.f;
       }
   // 32 rows x 64 columns of each operand; what lies outside is filled with zeros
   auto stage = [&](int64_t k, int st) {
@@ -403,7 +404,7 @@ __global__ void __launch_bounds__(kWgThreads) k_mlp_wgrad(MlpGradArgs g, float* 
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const int64_t at = entry(i, j, q);
-        if (at >= 0) part[at] = base ? acc[i][j][q] - base[at] : acc[i][j][q];
+        if (at >= 0) part[at] = THROUGH ? acc[i][j][q] - base[at] : acc[i][j][q];
       }
 }
 // base of a split: the sum of the splits before it
@@ -477,11 +478,11 @@ cudaError_t launch_mlp_grad(const MlpGradArgs& a, cudaStream_t s) {
   const int splits = (int)std::min<int64_t>(kSplits, std::max<int64_t>(1, a.rows / 256));
   float* wpart = a.part + (size_t)kFbCtas * kBias;
   k_mlp_fwd_bwd<<<ctas, kFbThreads, kFbSmem, s>>>(a);
-  k_mlp_wgrad<<<dim3(kWgTiles, splits), kWgThreads, 0, s>>>(a, wpart, nullptr);
+  k_mlp_wgrad<false><<<dim3(kWgTiles, splits), kWgThreads, 0, s>>>(a, wpart, nullptr);
   if (a.rows > kThroughRows) {
     float* base = wpart + (size_t)kSplits * kParams;
     k_mlp_base<<<(unsigned)((kParams + 255) / 256), 256, 0, s>>>(splits, wpart, base);
-    k_mlp_wgrad<<<dim3(kWgTiles, splits), kWgThreads, 0, s>>>(a, wpart, base);
+    k_mlp_wgrad<true><<<dim3(kWgTiles, splits), kWgThreads, 0, s>>>(a, wpart, base);
     note_launches(2);
   }
   k_mlp_reduce<<<(unsigned)((kParams + 255) / 256), 256, 0, s>>>(a.rows, splits, ctas, wpart, a.part, a.loss_part,

@@ -672,10 +672,11 @@ int ctx_gmres(pnp_ctx* c, const double* U, const double* b, double* x, double rt
   double* hco = c->hpin + 2 * (m + 2) + 2;  // [m+1]: the update coefficients
   double* hp2[2] = {c->hpin + 3 * (m + 2) + 2, c->hpin + 5 * (m + 2) + 16};
   const bool two = c->prm.gmres_cgs2 != 0;
-  // Small systems: an iteration is five launches of a few microseconds, as long as the host's
+  // Small systems: an iteration is a few launches of a few microseconds, as long as the host's
   // wait for it and the launches of the next.  The host then queues one iteration ahead (a
-  // discarded one per solve at most).  2^18 unknowns: there an FP64 iteration takes 1 ms and
-  // the wait is 1 %.  3,267 unknowns: 47 us per iteration without, 36 us with it.
+  // discarded one per solve at most).  2^18 unknowns: there an FP64 iteration takes 0.15 ms
+  // and more and the wait is some percent.  3,267 unknowns: 47 us per iteration without, 36 us
+  // with it (of five launches; 23 us now, of three).
   const bool ahead = !flex && !flex64 && n <= (int64_t(1) << 18);
   const bool one_launch = gs_step_short(n);
   c->hflag[3] = 0;

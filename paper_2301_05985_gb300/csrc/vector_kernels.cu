@@ -532,7 +532,7 @@ cudaError_t launch_multi_axpy_norm(int64_t n, int k, const double* Vb, int64_t l
   return cudaGetLastError();
 }
 // Short vectors: one cooperative launch (k_gs_step).  GMRES(50) iterations with it and with the
-// two kernels, 2D: 867 unknowns 26.4 and 31.8 us, 3,267 27.4 and 32.5, 12,675 35.5 and 38.1,
+// two kernels (none of an iteration's launches dependent), 2D: 867 unknowns 26.4 and 31.8 us, 3,267 27.4 and 32.5, 12,675 35.5 and 38.1,
 // 49,923 59.1 and 62.5, 198,147 137 and 131, 789,507 485 and 435 (the FP64 pipe; the barrier
 // and the sums in every block add to it).
 bool gs_step_short(int64_t n) { return n <= kGsShort; }
