@@ -465,7 +465,7 @@ struct HistoryArgs {
 };
 template <typename T>
 __global__ void k_init_rows(RowArgs R, const T* __restrict__ in, T* __restrict__ out, int mode, HistoryArgs H) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t i = row_last_first();
   if (i < R.n_nodes) {
     if (H.hs) {
       H.hs[2 * i + 0] = H.Uk ? (H.b1 * H.Uk[3 * i + 0] + H.b2 * H.Ukm1[3 * i + 0]) * H.inv_dt : 0.0;
@@ -518,7 +518,7 @@ __device__ __forceinline__ void load_block(const T* __restrict__ Dinv, int64_t i
 template <typename T>
 __global__ void k_block_apply_rows(RowArgs R, const T* __restrict__ Dinv, const T* u, T scale, const T* scale_dev,
                                    T* __restrict__ y, T* __restrict__ out) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t i = row_last_first();
   const int64_t h = i - R.n_nodes;
   const bool node = i < R.n_nodes, hanging = !node && h < R.n_hanging;
   T B[9], v[3];

@@ -347,7 +347,7 @@ __global__ void __launch_bounds__(256, ns_min_blocks<T>()) k_ns_lanes(NsArgs<T> 
 // sum_p w_p X_p on hanging rows (threads past N).
 template <typename T>
 __global__ void k_ns_init(RowArgs R, NsBc bc, const T* __restrict__ X, T* __restrict__ out, int mode) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t i = row_last_first();
   T o[4];
   int64_t id = i;
   if (i < R.n_nodes) {
@@ -756,7 +756,7 @@ __device__ __forceinline__ void smooth_row(const RowArgs& R, const NsBc& bc, con
 __global__ void k_ns_smooth(RowArgs R, NsBc bc, const float* __restrict__ Dinv, const float4* __restrict__ b,
                             float4* __restrict__ Ax, const float4* __restrict__ xo, float4* __restrict__ xn, float om,
                             bool first) {
-  smooth_row<true>(R, bc, Dinv, b, Ax, xo, xn, om, first, blockIdx.x * (int64_t)blockDim.x + threadIdx.x);
+  smooth_row<true>(R, bc, Dinv, b, Ax, xo, xn, om, first, row_last_first());
 }
 
 // out[j] = sum_q w_q (b - Ax)[col_q] over the fine rows that are weak-form equations
