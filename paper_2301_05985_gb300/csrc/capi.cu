@@ -406,6 +406,11 @@ int pnp_ctx_create(const pnp_mesh* m, const pnp_params* p, void* stream, pnp_ctx
       return fail(e == cudaErrorMemoryAllocation ? PNP_ERR_NOMEM : PNP_ERR_CUDA);
     }
   }
+  if (ctx_on_lanes(c)) {
+    // without room for the FP32 J V's tables the FP64 operators still work
+    const int rc = ctx_tiles(c);
+    if (rc && rc != PNP_ERR_NOMEM) return fail(rc);
+  }
   *out = c;
   return PNP_OK;
 }

@@ -131,7 +131,9 @@ double element_kernel_flops(int dim, bool jv);
 // FP32 J V [N][3] on node tiles (element_tiles.cu) at the state of the node records
 // (launch_node_records); `advection` false when the advection field is zero.  err[0] = 1
 // (mapped pinned memory) when a wait on a staged table gave up after `polls` polls (< 0: the
-// default, about a second).  dependent: as launch_kernel.  plan_jv_tiles: the grids for a table (t.blocks), once.
+// default, about a second).  dependent: as launch_kernel; the tables (tab.rec) must be older
+// than the launch before, as the kernel reads them before its wait.  plan_jv_tiles: the grids
+// for a table (t.blocks), once.
 cudaError_t plan_jv_tiles(int dim, TileTab& t);
 cudaError_t launch_jv_tiles(int dim, const TileMesh& M, const float4* rec, bool advection, const float* V,
                             const PhysParams& P, float* out, bool dependent, int* err, int polls, cudaStream_t s);

@@ -86,6 +86,7 @@ static int hanging_rows(pnp_ctx* c, const T* in, T* out) {
 // the operators add to initialised rows, unless an environment variable selects the patch
 // or the one-thread-per-element kernels
 static bool on_lanes(const pnp_ctx* c) { return !c->use_patches && element_kernel_is_lanes(); }
+bool ctx_on_lanes(const pnp_ctx* c) { return on_lanes(c); }
 static ElemArgs<double> lane_args(const pnp_ctx* c, const double* U, const double* V, double* out) {
   ElemArgs<double> A = elem_args<double>(c, U, V, c->hs, c->adv, out);
   A.faces = c->d_faces;
@@ -180,8 +181,11 @@ static int precond_jv64(pnp_ctx* c, const double* U, const double* u, double sca
 // The FP32 J V runs on node tiles and node records (on_lanes); the patch and the
 // one-thread-per-element kernels read FP32 copies of the fields.
 
-// the node tables of the tiles, built with their first use
-static int ctx_tiles(pnp_ctx* c) {
+// The node tables of the tiles: built with the context, or by the first call that reads them
+// when the device had no room for them then.  The host waits for the build: k_jv_tiles is a
+// dependent launch that reads them before it waits for the launch before it, so that launch
+// must not be the build.
+int ctx_tiles(pnp_ctx* c) {
   if (c->tab.rec || c->n_elem == 0) return PNP_OK;
   const int nc = 1 << c->dim;
   TileTab t;
@@ -203,11 +207,13 @@ static int ctx_tiles(pnp_ctx* c) {
   CK(plan_jv_tiles(c->dim, t));
   const cudaError_t e = cudaMalloc((void**)&c->d_tiles, (size_t)t.bytes * (size_t)t.n);
   if (e != cudaSuccess) {
+    cudaGetLastError();  // reported here, not by the next launch
     c->d_tiles = nullptr;
     PNP_FAIL(e == cudaErrorMemoryAllocation ? PNP_ERR_NOMEM : PNP_ERR_CUDA, "node tables: allocation failed: %s",
              cudaGetErrorString(e));
   }
   CK(launch_build_tiles(c->dim, M, t.corners, t.cap, t.hcap, c->d_tiles, nullptr, c->stream));
+  CK(cudaStreamSynchronize(c->stream));
   t.rec = c->d_tiles;
   c->tab = t;
   return PNP_OK;
@@ -350,6 +356,7 @@ int ctx_linearize(pnp_ctx* c, const double* U) {
   if (!c->rec_lin) {
     const cudaError_t e = cudaMalloc((void**)&c->rec_lin, sizeof(float4) * 2 * (size_t)c->n_nodes);
     if (e != cudaSuccess) {
+      cudaGetLastError();
       c->rec_lin = nullptr;
       PNP_FAIL(e == cudaErrorMemoryAllocation ? PNP_ERR_NOMEM : PNP_ERR_CUDA,
                "stored linearisation: allocation failed: %s", cudaGetErrorString(e));
