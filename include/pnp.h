@@ -317,9 +317,11 @@ int pnp_jv(pnp_ctx* c, const double* U, const void* V, void* JV, int precision);
  * pnp_linearize, or the start of the next flexible Krylov solve). */
 int pnp_linearize(pnp_ctx* c, const double* U);
 int pnp_jv_linearized(pnp_ctx* c, const float* V, float* JV);
-/* The poll limit of each bounded wait of the staged J V above (polls < 0: the default,
- * 2^22 polls, about a second; at most 2^30).  A limit of 0 makes every wait give up at
- * once while the copies still land: it exercises the failure path on a healthy GPU. */
+/* The poll limit of each bounded wait of the staged J V above and of the grid barrier in the
+ * solvers' Gram-Schmidt steps (polls < 0: the default, 2^22 polls, about a second; at most
+ * 2^30).  A limit of 0 makes every wait give up at once while the copies still land and the
+ * blocks still arrive: it exercises the failure path on a healthy GPU.  A solve in which a
+ * wait gave up returns PNP_ERR_DEVICE_FLAG. */
 int pnp_set_wait_limit(pnp_ctx* c, int64_t polls);
 /* 3x3 diagonal blocks of J(U): D device FP64 [n][3][3] (row-major per node), exact
  * for the assembled operator including hanging-node coupling.  Dirichlet rows are

@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(256) k_inner_start(int64_t n4, const float4* _
 // twice: 51 us at HBM rate, 13 vectors each way).
 constexpr int kGsGroup = 24, kGsBatch = 8;
 __global__ void __launch_bounds__(256, 3) k_inner_gs(int64_t n4, int k, const float4* __restrict__ Ub, int64_t ld4,
-                                                     float4* w, unsigned* ticket, int* err, InnerStep S) {
+                                                     float4* w, unsigned* ticket, int* err, int polls, InnerStep S) {
   __shared__ float sh[kGsGroup][8];
   __shared__ float cf[kMaxInner];
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(256, 3) k_inner_gs(int64_t n4, int k, const fl
     }
     __syncthreads();
   }
-  const bool passed = grid_barrier(S.arrived, err, kBarrierPolls);
+  const bool passed = grid_barrier(S.arrived, err, polls);
   float ss = 0.0f;
   if (passed) {
     if (tid < k) {
@@ -315,7 +315,7 @@ cudaError_t launch_inner_start(int64_t n, int d, const float* u0, double* part, 
 }
 cudaError_t launch_inner_gs(int64_t n, int j, int d, const float* Ub, int64_t ld, float* w, unsigned* ticket,
                             double* sv, double* dinv, float* inv_s, double* H, double* sums, unsigned* arrived, int* err,
-                            cudaStream_t s) {
+                            int polls, cudaStream_t s) {
   if ((n | ld) & 3 || j + 1 > kMaxInner) return cudaErrorInvalidValue;  // rows padded to float4
   int dev = 0, n_sm = 0, per = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -330,7 +330,7 @@ cudaError_t launch_inner_gs(int64_t n, int j, int d, const float* Ub, int64_t ld
   const float4* U = (const float4*)Ub;
   float4* w4 = (float4*)w;
   InnerStep S{j, d, sv, dinv, inv_s, H, sums, arrived};
-  void* args[] = {&n4, &k, &U, &ld4, &w4, &ticket, &err, &S};
+  void* args[] = {&n4, &k, &U, &ld4, &w4, &ticket, &err, &polls, &S};
   e = cudaLaunchCooperativeKernel(k_inner_gs, dim3((unsigned)nb), dim3(256), args, 0, s);
   note_launch();
   return e == cudaSuccess ? cudaGetLastError() : e;

@@ -226,11 +226,11 @@ cudaError_t launch_multi_axpy_norm(int64_t n, int k, const double* Vb, int64_t l
                                    double* w, double* part, unsigned* ticket, const GsFinish& f, cudaStream_t s);
 // Both in one cooperative launch, for short vectors (gs_step_short): d_i = V_i . w first.
 // part: gs_step_part(n, m) doubles for k <= m + 1; ticket[0 .. 1] zeroed counters; err[0] = 1
-// (pinned host memory) when its bounded wait gave up.
+// (pinned host memory) when its bounded wait gave up after `polls` polls (< 0: the default).
 bool gs_step_short(int64_t n);
 size_t gs_step_part(int64_t n, int m);
 cudaError_t launch_gs_step(int64_t n, int k, const double* Vb, int64_t ld, double* d, const double* dinv, double* w,
-                           double* part, unsigned* ticket, int* err, const GsFinish& f, cudaStream_t s);
+                           double* part, unsigned* ticket, int* err, int polls, const GsFinish& f, cudaStream_t s);
 // Dinv = inverse of the 3x3 blocks of D (Gauss-Jordan with partial pivoting, FP64);
 // flag[0] |= 1 on a singular or non-finite block.  D may alias Dinv when T = double.
 template <typename T>
@@ -251,13 +251,13 @@ int inner_sum_doubles();
 // The Arnoldi bookkeeping stays on the device: norms s_i (sv), 1 / s_i^2 (dinv), 1 / s_i
 // (inv_s) and the Hessenberg matrix H [(d+1) x d].  start: s_0 = ||u0||; gs: step j,
 // w -= sum_{i <= j} (U_i . w) dinv_i U_i, s_(j+1) = ||w|| and column j of H, in one cooperative
-// launch whose bounded wait sets err[0] = 1 (pinned host memory) when it gives up; lsq: the
-// least squares, coef_i = y_i / s_i.
+// launch whose bounded wait sets err[0] = 1 (pinned host memory) when it gives up after `polls`
+// polls (< 0: the default); lsq: the least squares, coef_i = y_i / s_i.
 cudaError_t launch_inner_start(int64_t n, int d, const float* u0, double* part, unsigned* ticket, double* sv,
                                double* dinv, float* inv_s, double* sums, cudaStream_t s);
 cudaError_t launch_inner_gs(int64_t n, int j, int d, const float* Ub, int64_t ld, float* w, unsigned* ticket,
                             double* sv, double* dinv, float* inv_s, double* H, double* sums, unsigned* arrived, int* err,
-                            cudaStream_t s);
+                            int polls, cudaStream_t s);
 inline size_t inner_scalar_doubles(int d) { return (size_t)(d + 1) * d; }
 cudaError_t launch_inner_lsq(int d, const double* sv, const double* H, double* coef, cudaStream_t s);
 // y = Dinv32 (inv_s[0] u) per node (inv_s may be null: scale 1)

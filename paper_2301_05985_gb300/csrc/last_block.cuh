@@ -19,12 +19,14 @@ __device__ __forceinline__ bool last_block(unsigned* ticket, unsigned total) {
 }
 
 // Grid barrier of a cooperative launch: waits until every block has arrived; false in every
-// thread of a block whose wait gave up after `polls` polls (then *err = 1: device or mapped
+// thread of a block whose wait gave up after `polls` polls (< 0: the default, about a second; then *err = 1: device or mapped
 // host memory).  `arrived` is zero before the launch; a block that is the last to finish the
 // kernel (last_block after the barrier, in every block) sets it back.  Writes made before the
 // call by any block are visible after it (read them with __ldcg).
+constexpr int kBarrierPolls = 1 << 22;
 __device__ __forceinline__ bool grid_barrier(unsigned* arrived, int* err, int polls) {
   __shared__ bool passed;
+  if (polls < 0) polls = kBarrierPolls;
   __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -41,4 +43,3 @@ __device__ __forceinline__ bool grid_barrier(unsigned* arrived, int* err, int po
   __syncthreads();
   return passed;
 }
-constexpr int kBarrierPolls = 1 << 22;

@@ -415,7 +415,8 @@ static int inner_gmres32_body(pnp_ctx* c) {
     {
       const double nj = (double)n * (j + 1);
       ProfScope ps(c, PNP_PROF_INNER, 4.0 * (nj + n) + 4.0 * (nj + 2.0 * n), 4.0 * nj + 2.0 * n);
-      CK(launch_inner_gs(ldq, j, d, Q, ldq, w, c->ticket, sv, dinv, inv_s, H, sums, c->ticket + 1, c->hflag, s));
+      CK(launch_inner_gs(ldq, j, d, Q, ldq, w, c->ticket, sv, dinv, inv_s, H, sums, c->ticket + 1, c->hflag,
+                         c->wait_polls, s));
     }
   }
   CK(launch_inner_lsq(d, sv, H, coef, s));
@@ -658,8 +659,11 @@ int ctx_gmres(pnp_ctx* c, const double* U, const double* b, double* x, double rt
   // the same flexible scheme entirely in FP64 (inner FP64 GMRES, FP64 J V)
   const bool flex64 = prec == PNP_F64 && c->prm.gmres_inner > 0;
   if (flex64) RC(ctx_alloc_inner64(c, m, c->prm.gmres_inner));
-  // the bounded waits of the tile J V raise a flag that is read at the end of the solve
-  const bool staged = prec == PNP_F32 && on_lanes(c);
+  // the bounded waits of the tile J V and of the inner solve's Gram-Schmidt steps (on every
+  // element path) raise a flag that is read at the end of the solve
+  const bool staged = prec == PNP_F32;
+  // before any other end of the solve is reported: what a wait that gave up left undone
+  auto gave_up = [&]() -> int { return staged ? ctx_check_staged_waits(c) : PNP_OK; };
   c->lin_user = false;  // a solve replaces any linearisation stored by pnp_linearize
   if (staged) {
     CK(cudaStreamSynchronize(s));
@@ -710,11 +714,15 @@ int ctx_gmres(pnp_ctx* c, const double* U, const double* b, double* x, double rt
   int total = 0;
   double beta_cycle = beta;  // true residual at the start of the current cycle
   while (true) {
-    if (!std::isfinite(beta)) PNP_FAIL(PNP_ERR_NAN, "gmres: residual norm is not finite");
+    if (!std::isfinite(beta)) {
+      RC(gave_up());
+      PNP_FAIL(PNP_ERR_NAN, "gmres: residual norm is not finite");
+    }
     if (beta <= tol) break;
     if (total >= max_it) {
       *its_out = total;
       *rel_out = beta / bn;
+      RC(gave_up());
       PNP_FAIL(PNP_ERR_KRYLOV_MAXIT, "gmres: %d iterations, relative residual %.3e > %.3e", total, beta / bn, rtol);
     }
     sv[0] = beta;
@@ -778,7 +786,7 @@ int ctx_gmres(pnp_ctx* c, const double* U, const double* b, double* x, double rt
         }
         if (one_launch) {
           ProfScope ps(c, PNP_PROF_ORTHO_UPDATE, 8.0 * (2.0 * nj + 3.0 * n), 4.0 * nj + 2.0 * n);
-          CK(launch_gs_step(n, j + 1, V, n, dp, dinv, w, c->part, c->ticket, c->hflag + 3, f, s));
+          CK(launch_gs_step(n, j + 1, V, n, dp, dinv, w, c->part, c->ticket, c->hflag + 3, c->wait_polls, f, s));
           continue;
         }
         {
@@ -812,7 +820,10 @@ int ctx_gmres(pnp_ctx* c, const double* U, const double* b, double* x, double rt
       for (int i = 0; i <= j; ++i) h[i] = (two ? hj[i] + hj2[i] : hj[i]) / sv[i];
       w1sq = hj[m + 1];
       const double nrm = std::sqrt(w1sq);
-      if (!std::isfinite(nrm)) PNP_FAIL(PNP_ERR_NAN, "gmres: Krylov vector norm is not finite");
+      if (!std::isfinite(nrm)) {
+        RC(gave_up());
+        PNP_FAIL(PNP_ERR_NAN, "gmres: Krylov vector norm is not finite");
+      }
       sv[j + 1] = nrm;
       for (int i = 0; i <= j; ++i) Hij(i, j) = h[i];
       Hij(j + 1, j) = nrm;
@@ -822,7 +833,10 @@ int ctx_gmres(pnp_ctx* c, const double* U, const double* b, double* x, double rt
         Hij(i, j) = t;
       }
       const double rr = std::hypot(Hij(j, j), Hij(j + 1, j));
-      if (rr == 0.0) PNP_FAIL(PNP_ERR_NAN, "gmres: singular Hessenberg matrix");
+      if (rr == 0.0) {
+        RC(gave_up());
+        PNP_FAIL(PNP_ERR_NAN, "gmres: singular Hessenberg matrix");
+      }
       cs[j] = Hij(j, j) / rr;
       sn[j] = Hij(j + 1, j) / rr;
       Hij(j, j) = rr;
@@ -890,7 +904,7 @@ int ctx_gmres(pnp_ctx* c, const double* U, const double* b, double* x, double rt
     }
     if (std::isfinite(beta) && beta > 0.95 * beta_cycle) {
       CK(cudaStreamSynchronize(s));
-      if (staged) RC(ctx_check_staged_waits(c));
+      RC(gave_up());
       *its_out = total;
       *rel_out = beta / bn;
       PNP_FAIL(PNP_ERR_KRYLOV_MAXIT, "gmres: stagnated after %d iterations at relative residual %.3e > %.3e", total,
@@ -901,8 +915,7 @@ int ctx_gmres(pnp_ctx* c, const double* U, const double* b, double* x, double rt
   CK(cudaStreamSynchronize(s));
   *its_out = total;
   *rel_out = beta / bn;
-  if (staged) RC(ctx_check_staged_waits(c));
-  return PNP_OK;
+  return gave_up();
 }
 
 int ctx_newton(pnp_ctx* c, pnp_solve_stats* st, const double* ref_state) {

@@ -229,7 +229,8 @@ constexpr int kGsChunks = 64;
 constexpr int64_t kGsShort = int64_t(1) << 16;
 __global__ void __launch_bounds__(256) k_gs_step(int64_t n, int k, const double* __restrict__ Vb, int64_t ld,
                                                  double* d, const double* __restrict__ dinv, double* w, double* part,
-                                                 unsigned* ticket, unsigned* arrived, int* err, GsFinish f) {
+                                                 unsigned* ticket, unsigned* arrived, int* err, int polls,
+                                                 GsFinish f) {
   extern __shared__ double cf[];
   __shared__ double sh[8][33];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -257,7 +258,7 @@ __global__ void __launch_bounds__(256) k_gs_step(int64_t n, int k, const double*
     }
     __syncthreads();
   }
-  const bool passed = grid_barrier(arrived, err, kBarrierPolls);
+  const bool passed = grid_barrier(arrived, err, polls);
   double ss = 0.0;
   if (passed) {
     // four lanes per vector
@@ -538,7 +539,7 @@ cudaError_t launch_multi_axpy_norm(int64_t n, int k, const double* Vb, int64_t l
 bool gs_step_short(int64_t n) { return n <= kGsShort; }
 size_t gs_step_part(int64_t n, int m) { return gs_step_short(n) ? (size_t)kGsChunks * (m + 2) + 2048 : 0; }
 cudaError_t launch_gs_step(int64_t n, int k, const double* Vb, int64_t ld, double* d, const double* dinv, double* w,
-                           double* part, unsigned* ticket, int* err, const GsFinish& f, cudaStream_t s) {
+                           double* part, unsigned* ticket, int* err, int polls, const GsFinish& f, cudaStream_t s) {
   int dev = 0, n_sm = 0, per = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
@@ -550,7 +551,7 @@ cudaError_t launch_gs_step(int64_t n, int k, const double* Vb, int64_t ld, doubl
   const unsigned nb = (unsigned)std::min(most, std::max(xb * ((k + 3) / 4), (n + 31) / 32));
   unsigned* arrived = ticket + 1;
   GsFinish fin = f;
-  void* args[] = {&n, &k, &Vb, &ld, &d, &dinv, &w, &part, &ticket, &arrived, &err, &fin};
+  void* args[] = {&n, &k, &Vb, &ld, &d, &dinv, &w, &part, &ticket, &arrived, &err, &polls, &fin};
   e = cudaLaunchCooperativeKernel(k_gs_step, dim3(nb), dim3(256), args, smem, s);
   note_launch();
   return e == cudaSuccess ? cudaGetLastError() : e;
