@@ -799,16 +799,30 @@ int ctx_gmres(pnp_ctx* c, const double* U, const double* b, double* x, double rt
       if (ahead) CK(cudaEventRecord(c->step_done[j & 1], s));
       return PNP_OK;
     };
-    bool queued = false;  // iteration j is already on the stream
+    // `next`: iteration j is already on the stream.  An iteration behind the one that ends the
+    // cycle is not part of the solve; when the end is an error return, it is waited for, as it
+    // reads the caller's U and writes the pinned numbers.
+    struct Queued {
+      pnp_ctx* c;
+      bool next;
+      void drop() {
+        if (next) c->jv_count--;
+        next = false;
+      }
+      ~Queued() {
+        if (next) cudaStreamSynchronize(c->stream);
+        drop();
+      }
+    } queued{c, false};
     for (int j = 0; j < m && total < max_it; ++j) {
-      if (!queued) RC(enqueue(j));
-      queued = false;
+      if (!queued.next) RC(enqueue(j));
+      queued.next = false;
       if (ahead) {
         // the next iteration follows without waiting for the host, unless this one may end
         // the solve (the last known residual near the tolerance)
         if (j + 1 < m && total + 1 < max_it && res > 4.0 * tol) {
+          queued.next = true;
           RC(enqueue(j + 1));
-          queued = true;
         }
         CK(cudaEventSynchronize(c->step_done[j & 1]));
       } else {
@@ -856,8 +870,7 @@ int ctx_gmres(pnp_ctx* c, const double* U, const double* b, double* x, double rt
         break;
       }
     }
-    // an iteration queued behind the one that ended the cycle is not part of the solve
-    if (queued) c->jv_count--;
+    queued.drop();
     // y = H^-1 g ; x += M^-1 (sum_i y_i u_i / s_i)
     for (int i = k - 1; i >= 0; --i) {
       double t = g[i];

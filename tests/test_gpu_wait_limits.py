@@ -42,3 +42,16 @@ def test_a_wait_that_gives_up_is_reported(path, precision, inner, monkeypatch):
     ctx.jv(U, x, r)
     # FP32 operator in the mixed solve: its rounding on top of the solver's tolerance
     assert float((b - r).norm() / b.norm()) <= (1e-5 if prec == pnp.PNP_F64 else 1e-3)
+
+
+def test_no_work_is_left_behind_an_error_return():
+    """The FP64 solve of a small system queues an iteration ahead of the host.  A solve that ends
+    in its first iteration (here by a wait that gives up) leaves nothing on the stream, where it
+    would read the caller's U after the call, and counts the initial residual's J V and its
+    own iteration's."""
+    pnp, torch, ctx, U, b, x = _system(gmres_restart=30, gmres_max_it=300)
+    ctx.set_wait_limit(0)
+    for _ in range(5):
+        st = ctx.gmres(U, b, x, 1e-6, pnp.PNP_F64, raise_on_error=False)
+        assert torch.cuda.current_stream().query()
+        assert st.status == pnp.PNP_ERR_DEVICE_FLAG and st.jv_evals == 2
