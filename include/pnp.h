@@ -440,7 +440,7 @@ int pnp_ns_block_diag(pnp_ctx* c, double* D);
  * correction around FP32 BiCGStab (App. A solves this block with BiCGStab) of at most
  * ns_inner_max_it iterations each (a step that raises ||F|| is undone, and with multigrid the
  * solve continues with the blocks).  PNP_ERR_KRYLOV_MAXIT after ns_max_it Krylov
- * iterations, 60 refinement steps, or when progress stops above 1e-9 ||F(X^0)|| (at or below
+ * iterations, 60 refinement steps (restart cycles not counted), or when progress stops above 1e-9 ||F(X^0)|| (at or below
  * it the solve ends as converged with st->floor_stop = 1); PNP_ERR_NAN on a non-finite
  * norm.  st->inner_its counts the Krylov iterations, st->refinements the FGMRES restart
  * cycles or refinement steps.  Uses the context's beta0..2. */

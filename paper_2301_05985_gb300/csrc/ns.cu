@@ -1647,7 +1647,7 @@ int ctx_ns_solve(pnp_ctx* c, const double* Ubody, pnp_ns_stats* st) {
   st->res0 = f;
   const double target = std::max(p.ns_rtol * f, p.ns_atol);
   S->mg_off = false;
-  int inner_total = 0, ref = 0, stalls = 0;
+  int inner_total = 0, ref = 0, stalls = 0, cycles = 0;  // cycles: of the FGMRES, counted in ref
   if (p.ns_fgmres > 0) {
     const int rc = f > target ? ns_fgmres(c, Ubody, target, f, st) : PNP_OK;
     if (rc >= 0) {
@@ -1661,7 +1661,7 @@ int ctx_ns_solve(pnp_ctx* c, const double* Ubody, pnp_ns_stats* st) {
     // steps add up in st->refinements, Krylov iterations in st->inner_its)
     st->krylov_fallbacks++;
     inner_total = st->inner_its;
-    ref = st->refinements;
+    ref = cycles = st->refinements;
     if (p.monitor) fprintf(stderr, "[pnp ns] FGMRES stagnated at ||F|| %.6e: BiCGStab refinement\n", f);
   }
   int rc = PNP_OK;
@@ -1672,7 +1672,7 @@ int ctx_ns_solve(pnp_ctx* c, const double* Ubody, pnp_ns_stats* st) {
   double* Fs = S->Dg + 4 * N;
   S->mg_off = false;
   while (f > target) {
-    if (ref >= kMaxRefine || inner_total >= p.ns_max_it) {
+    if (ref - cycles >= kMaxRefine || inner_total >= p.ns_max_it) {
       rc = PNP_ERR_KRYLOV_MAXIT;
       pnp_set_error("ns: %d refinements, %d BiCGStab iterations, ||F|| = %.3e > %.3e", ref, inner_total, f, target);
       break;
