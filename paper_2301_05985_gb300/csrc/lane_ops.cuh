@@ -224,7 +224,10 @@ __device__ __forceinline__ df2 flip(df2 a, int k) { return {flip(a.hi, k), flip(
 // 1.58e-14 both ways, 1.72e-14 with FP64-style interpolation in accurate operations; with
 // quick differences 1.70e-14).
 constexpr double kVal = 0.5 * (1.0 + kG);                 // a
-constexpr double kRho = (1.0 - kG) / (1.0 + kG);          // b' / a
+// b' / a = 2 - sqrt 3, rounded once: it acts on every axis of the interpolation and of the
+// tests the same way, so its error adds up (written as (1 - kG) / (1 + kG) it was one unit in
+// the last place off, and the FP64 J V 1.4 times as far from 64 bits)
+constexpr double kRho = 0.26794919243112270647255365849413;
 __host__ __device__ constexpr double ipow(double x, int n) { return n <= 0 ? 1.0 : x * ipow(x, n - 1); }
 
 template <typename T, int D>
