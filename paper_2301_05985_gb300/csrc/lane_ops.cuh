@@ -292,28 +292,33 @@ __device__ __forceinline__ double const_pow2(double c, int e, double) {
 }
 __device__ __forceinline__ df const_pow2(double c, int e, df) { return mul_pow2(df(c), pow2i(e, 0.0f)); }
 // x c 2^e.  In FP32 the constant is two floats (a rounded constant would be a factor on a
-// whole term: a^2 is 4e-8 off, as much as all other rounding of the FP32 kernels together)
+// whole term: a^2 is 4e-8 off, as much as all other rounding of the FP32 kernels together).
+// The low part's product goes into the fused operation of the high part, which then rounds
+// once; the other way round two roundings of the whole value meet.
+__host__ __device__ __forceinline__ float times_const_f(float x, double c, int e) {
+  const float h = (float)c, p = df_u2f((uint32_t)(127 + e) << 23);
+  return fmaf(x, h * p, x * ((float)(c - (double)h) * p));
+}
 template <typename C>
 __device__ __forceinline__ C times_const(C x, double c, int e) {
   return x * const_pow2(c, e, C(0));
 }
 template <>
 __device__ __forceinline__ float times_const(float x, double c, int e) {
-  const float h = (float)c, p = pow2i(e, 0.0f);
-  return fmaf(x, (float)(c - (double)h) * p, x * (h * p));
+  return times_const_f(x, c, e);
 }
 __device__ __forceinline__ d2 times_const2(d2 x, double c, int e) { return x * both<double>(const_pow2(c, e, 0.0)); }
 __device__ __forceinline__ df2 times_const2(df2 x, double c, int e) { return x * both<df>(const_pow2(c, e, df(0))); }
 __device__ __forceinline__ f2 times_const2(f2 x, double c, int e) {
   const float h = (float)c, p = pow2i(e, 0.0f);
-  return fma(x, both<float>((float)(c - (double)h) * p), x * both<float>(h * p));
+  return fma(x, both<float>(h * p), x * both<float>((float)(c - (double)h) * p));
 }
 // (c x, -c y)
 __device__ __forceinline__ d2 times_pm(d2 x, double c) { return x * pair(c, -c); }
 __device__ __forceinline__ df2 times_pm(df2 x, double c) { return x * pair(df(c), -df(c)); }
 __device__ __forceinline__ f2 times_pm(f2 x, double c) {
   const float h = (float)c, l = (float)(c - (double)h);
-  return fma(x, pair(l, -l), x * pair(h, -h));
+  return fma(x, pair(h, -h), x * pair(l, -l));
 }
 // x 2^e
 __device__ __forceinline__ float times_pow2(float x, int e) { return x * pow2i(e, 0.0f); }
