@@ -6,6 +6,7 @@
 #include <algorithm>
 #include <cstdint>
 
+#include "dot4.cuh"
 #include "kernels.h"
 #include "last_block.cuh"
 
@@ -57,9 +58,6 @@ struct InnerStep {
   double* sums;        // [2][kGsSums] projections and w . w, of even and of odd steps
   unsigned* arrived;   // blocks at the step's barrier (zero between launches)
 };
-__device__ __forceinline__ float dot4(float4 a, float4 b, float s) {
-  return fmaf(a.x, b.x, fmaf(a.y, b.y, fmaf(a.z, b.z, fmaf(a.w, b.w, s))));
-}
 __device__ __forceinline__ void axpy4(float c, const float4& u, float4& a) {
   a.x = fmaf(c, u.x, a.x);
   a.y = fmaf(c, u.y, a.y);
