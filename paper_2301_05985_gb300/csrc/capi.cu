@@ -276,6 +276,12 @@ int pnp_ctx_create(const pnp_mesh* m, const pnp_params* p, void* stream, pnp_ctx
   c->prm = *p;
   c->stream = (cudaStream_t)stream;
   cudaGetDevice(&c->device);
+  {
+    // "patch": deterministic shared-memory patch kernels; default: per-element kernels
+    // scattering with global atomics (faster on this hardware at present)
+    const char* ep = getenv("PNP_ELEMENT_PATH");
+    c->use_patches = ep && std::strcmp(ep, "patch") == 0;
+  }
   const int nc = 1 << m->dim;
   const int64_t N = m->n_nodes;
   auto fail = [&](int rc) {
@@ -306,9 +312,11 @@ int pnp_ctx_create(const pnp_mesh* m, const pnp_params* p, void* stream, pnp_ctx
   ALLOC(c->vel, v3);
   ALLOC(c->vel_prev, v3);
   ALLOC(c->hs, sizeof(double) * 2 * N);
-  ALLOC(c->U32, sizeof(float) * 3 * N);
-  ALLOC(c->adv32, sizeof(float) * 3 * N);
-  ALLOC(c->hs32, sizeof(float) * 2 * N);
+  if (!ctx_on_lanes(c)) {  // FP32 copies of the fields: the lane and tile kernels read node records
+    ALLOC(c->U32, sizeof(float) * 3 * N);
+    ALLOC(c->adv32, sizeof(float) * 3 * N);
+    ALLOC(c->hs32, sizeof(float) * 2 * N);
+  }
   ALLOC(c->rec32, sizeof(float4) * 2 * N);
   ALLOC(c->V32, sizeof(float) * 3 * N);
   ALLOC(c->JV32, sizeof(float) * (3 * N + 4));  // the inner solve writes whole float4
@@ -357,17 +365,17 @@ int pnp_ctx_create(const pnp_mesh* m, const pnp_params* p, void* stream, pnp_ctx
     return fail(PNP_ERR_CUDA);
   }
   if (int rc = ctx_alloc_krylov(c, p->gmres_restart)) return fail(rc);
+  if (ctx_on_lanes(c)) {
+    // built while the host copies the mesh; without room for the FP32 J V's tables the FP64
+    // operators still work
+    const int rc = ctx_build_tiles(c);
+    if (rc && rc != PNP_ERR_NOMEM) return fail(rc);
+  }
   try {
     c->host_mesh = *m;
   } catch (const std::bad_alloc&) {
     pnp_set_error("pnp_ctx_create: out of host memory");
     return fail(PNP_ERR_NOMEM);
-  }
-  {
-    // "patch": deterministic shared-memory patch kernels; default: per-element kernels
-    // scattering with global atomics (faster on this hardware at present)
-    const char* ep = getenv("PNP_ELEMENT_PATH");
-    c->use_patches = ep && std::strcmp(ep, "patch") == 0;
   }
   if (c->use_patches) {
     PatchData P;
@@ -406,10 +414,10 @@ int pnp_ctx_create(const pnp_mesh* m, const pnp_params* p, void* stream, pnp_ctx
       return fail(e == cudaErrorMemoryAllocation ? PNP_ERR_NOMEM : PNP_ERR_CUDA);
     }
   }
-  if (ctx_on_lanes(c)) {
-    // without room for the FP32 J V's tables the FP64 operators still work
-    const int rc = ctx_tiles(c);
-    if (rc && rc != PNP_ERR_NOMEM) return fail(rc);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  if (e != cudaSuccess) {
+    pnp_set_error("pnp_ctx_create: %s", cudaGetErrorString(e));
+    return fail(PNP_ERR_CUDA);
   }
   *out = c;
   return PNP_OK;

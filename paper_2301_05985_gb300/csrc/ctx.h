@@ -39,7 +39,7 @@ struct pnp_ctx {
   int32_t* d_hnode = nullptr;
   int32_t* d_hpar = nullptr;
   uint8_t* d_hnp = nullptr;
-  TileTab tab;              // node tables of the FP32 J V's tiles (ctx_tiles)
+  TileTab tab;              // node tables of the FP32 J V's tiles (ctx_build_tiles)
   uint8_t* d_tiles = nullptr;
 
   // Morton patches for the shared-memory element kernels (device), their partial buffers
@@ -220,7 +220,7 @@ struct ProfScope {
 int ctx_check(pnp_ctx* c, cudaError_t e, const char* what);
 int ctx_prepare_history(pnp_ctx* c);
 bool ctx_on_lanes(const pnp_ctx* c);
-int ctx_tiles(pnp_ctx* c);
+int ctx_build_tiles(pnp_ctx* c);
 int ctx_residual(pnp_ctx* c, const double* U, double* F);
 // the history (ctx_prepare_history) and the residual
 int ctx_history_residual(pnp_ctx* c, const double* U, double* F);

@@ -181,12 +181,11 @@ static int precond_jv64(pnp_ctx* c, const double* U, const double* u, double sca
 // The FP32 J V runs on node tiles and node records (on_lanes); the patch and the
 // one-thread-per-element kernels read FP32 copies of the fields.
 
-// The node tables of the tiles: built with the context, or by the first call that reads them
-// when the device had no room for them then.  The host waits for the build: k_jv_tiles is a
-// dependent launch that reads them before it waits for the launch before it, so that launch
-// must not be the build.
-int ctx_tiles(pnp_ctx* c) {
-  if (c->tab.rec || c->n_elem == 0) return PNP_OK;
+// The node tables of the tiles.  k_jv_tiles is a dependent launch that reads them before it
+// waits for the launch before it, which must not be the build: the host waits for the build
+// (pnp_ctx_create at its end, ctx_tiles here).
+int ctx_build_tiles(pnp_ctx* c) {
+  if (c->n_elem == 0) return PNP_OK;
   const int nc = 1 << c->dim;
   TileTab t;
   // two threads per hexahedron, four per quadrilateral
@@ -213,9 +212,15 @@ int ctx_tiles(pnp_ctx* c) {
              cudaGetErrorString(e));
   }
   CK(launch_build_tiles(c->dim, M, t.corners, t.cap, t.hcap, c->d_tiles, nullptr, c->stream));
-  CK(cudaStreamSynchronize(c->stream));
   t.rec = c->d_tiles;
   c->tab = t;
+  return PNP_OK;
+}
+// they come with the context; built now if the device had no room for them then
+static int ctx_tiles(pnp_ctx* c) {
+  if (c->tab.rec || c->n_elem == 0) return PNP_OK;
+  RC(ctx_build_tiles(c));
+  CK(cudaStreamSynchronize(c->stream));
   return PNP_OK;
 }
 
