@@ -170,10 +170,12 @@ template <typename T>
 cudaError_t launch_diag_rows(const RowArgs& R, T* Dg, cudaStream_t s);
 
 // ------------------------------------------------------------------ vector kernels
-// All reductions are deterministic: fixed grid, per-block partials, one final block.
+// FP64 reductions are deterministic: fixed grid, per-block partials, added in a fixed order.
+// The inner FP32 solve's are not: its Gram-Schmidt steps add the blocks' sums with FP64 atomics
+// as they arrive.  (A mixed-precision solve depends on the order of atomics on every element
+// path: the block diagonal is summed with them.)
 constexpr int kRedBlocks = 608;  // 4 x 152 SMs
-// persistent grid of the inner FP32 Gram-Schmidt kernels: 8 blocks of 256 per SM, enough
-// loads in flight for a streaming kernel with few registers
+// blocks at most of the inner FP32 solve's start norm (partials in `part`)
 constexpr int kInnerBlocks = 6 * 152;
 constexpr int kRedThreads = 256;
 

@@ -75,24 +75,6 @@ __device__ __forceinline__ T interp_v(T x, T nb) {
   return x;
 }
 
-// transpose: this lane's node contribution from the Gauss-point tests S, Phi
-template <typename T, int D>
-__device__ __forceinline__ T test_t(T S, T (&Phi)[3], T nb, const T (&sh)[3]) {
-  T A = S;
-#pragma unroll
-  for (int k = D - 1; k >= 0; --k) {
-    const T pA = flip(A, k);
-    const T pH = flip(Phi[k], k);
-    T pP[3];
-#pragma unroll
-    for (int j = 0; j < k; ++j) pP[j] = flip(Phi[j], k);
-    A = fma(nb, A - pA, fma(sh[k], Phi[k] + pH, A));
-#pragma unroll
-    for (int j = 0; j < k; ++j) Phi[j] = fma(nb, Phi[j] - pP[j], Phi[j]);
-  }
-  return A;
-}
-
 // ---- pairs -----------------------------------------------------------------------
 // Two scalars that go through the same operations (the two species, two velocity
 // components, two test rows) as one value.  For FP32 and double-float the pair's

@@ -691,8 +691,8 @@ int ctx_gmres(pnp_ctx* c, const double* U, const double* b, double* x, double rt
   // Small systems: an iteration is a few launches of a few microseconds, as long as the host's
   // wait for it and the launches of the next.  The host then queues one iteration ahead (a
   // discarded one per solve at most).  2^18 unknowns: there an FP64 iteration takes 0.15 ms
-  // and more and the wait is some percent.  3,267 unknowns: 47 us per iteration without, 36 us
-  // with it (of five launches; 23 us now, of three).
+  // and more and the wait is some percent.  3,267 unknowns: 36 us per iteration of five launches
+  // with it, 47 us without.
   const bool ahead = !flex && !flex64 && n <= (int64_t(1) << 18);
   const bool one_launch = gs_step_short(n);
   c->hflag[3] = 0;
