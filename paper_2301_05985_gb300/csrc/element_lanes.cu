@@ -108,13 +108,12 @@ __device__ __forceinline__ void load_node_c(const ElemArgs<double>& A, int32_t i
 // The operators on FP64 vectors, arithmetic C (double, or double-float).  They add to the
 // weak-form rows only (Dirichlet and hanging rows were written by the row initialisation).
 // What bounds it, on the membrane-band octree (971,776 elements) with advection:
-//   double-float residual: the FP32 pipe (480 M warp instructions, packed ones twice as
-//   long); 1.47 ms before, 0.595 ms now.  Before: accurate double-float operations only
-//   (FMA pipe 57 %), 41 conversions and FP64 additions per lane (FP64 pipe 45 %), 59 KB of
-//   straight code per warp.  (On node tiles as the FP32 J V: 0.591 ms, no gain: the barriers
+//   double-float residual: the FMA pipe (77 % of its cycles; 460 M warp instructions, packed
+//   ones two cycles each): 0.56 ms a launch, 1.47 ms with accurate operations throughout and
+//   conversions on the FP64 pipe.  (On node tiles as the FP32 J V: no gain, the barriers
 //   between its phases cost what the fewer loads and atomics save.)
-//   FP64 J V: the FP64 pipe (86 %); on the uniform level-6 cube 1.03 ms before, 0.76 ms now,
-//   by the operation count (318 to 230 FP64 instructions per lane).
+//   FP64 J V: the FP64 pipe (86 %); uniform level-6 cube 0.76 ms a launch, 1.03 ms with
+//   unscaled operators (318 instead of 230 FP64 instructions per lane).
 template <typename C, int D, bool JV>
 __global__ void __launch_bounds__(256, sizeof(C) == 8 && !std::is_same<C, double>::value ? 4 : 3)
     k_element_lanes(ElemArgs<double> A, LaneParams<C> K) {

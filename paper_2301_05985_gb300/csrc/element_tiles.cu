@@ -53,16 +53,13 @@ __device__ __forceinline__ void add_entry(const TileMesh& M, const TileView& v, 
 // tests take a shuffle per scalar and corner, the x and y factors run in registers; species,
 // (phi, dphi) and (v0, v1) as packed pairs.  Quadrilaterals: a lane per corner (pnp_lane.cuh).
 //
-// What bounds it: latency, with 16 warps of 118 registers on an SM (issue slots 58 % busy,
-// shared-memory wavefronts 66 %: a third each the nodes' loads, the shuffles, the sums).  On
-// the uniform level-7 cube (2,097,152 elements) with advection 174 us a launch, 0.28 GB of
-// DRAM traffic; before, the state stored per Gauss point (64 bytes a lane, 1.1 GB a launch)
-// 262 us.  Membrane-band octree of 971,776 elements 94 us (115), of 143,872 elements 19 us
-// (24), without advection 17 (five blocks fit an SM; 18 with four).  Steps on the way, level-7
-// cube: a lane per corner on such tiles 340 us; halves of elements in tiles of 128 (two blocks
-// per SM) 248; tiles of 64 (four blocks) and 16-byte shares 187; nodes' values by asynchronous
-// copies during the sums, slots by parity 174.  Hanging nodes' parents in the record: 104 to
-// 95 us on the octree (their chain of loads held the block's barrier).
+// What bounds it: latency, with 16 warps of 118 registers on an SM (IPC 2.3, shared memory
+// 66 %).  Uniform level-7 cube (2,097,152 elements) with advection 174 us a launch, 0.25 GB of
+// DRAM traffic; from a state stored per Gauss point (64 bytes a lane, 1.1 GB a launch) 262 us.
+// Membrane-band octree of 971,776 elements 94 us (115 stored), of 143,872 elements 19 us (24),
+// without advection 17 (five blocks fit an SM; 18 with four).  Other layouts, level-7 cube: a
+// lane per corner 340 us; tiles of 128 elements (two blocks per SM) 248; slots in the order of
+// the entries and nodes' values through registers 187.
 struct JvArgs {
   const float4* rec;
   const float* V;

@@ -117,7 +117,7 @@ __device__ __forceinline__ double warp_sum4(const double (&s)[4], int lane) {
 // one reduce-scatter over the warp, fixed order).  The partials go to part[i][block]; with
 // `ticket`, the last block adds them (a warp per vector).
 // Rows and split by size (multi_dot_shape): for long vectors the FP64 pipe bounds the kernel
-// (78 % of its peak) and R = 16 rows per thread keep the reduction adds small next to the
+// (84 % of its peak) and R = 16 rows per thread keep the reduction adds small next to the
 // FMAs; for short ones it is latency, and with R = 16 a 3,267-entry vector was one block
 // that swept the whole basis alone (28 us at up to 30 vectors).  Short vectors take one row
 // per thread and a block per four vectors.
