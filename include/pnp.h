@@ -276,7 +276,8 @@ int pnp_mesh_patch_stats(const pnp_mesh* m, int64_t* stats);
 
 /* ---------------------------------------------------------------- context -------- */
 /* Create a context on the current CUDA device: uploads the mesh (the mesh may be
- * destroyed afterwards), allocates fields and solver scratch.  stream: a cudaStream_t
+ * destroyed afterwards), allocates fields and solver scratch and builds the node tables of the
+ * FP32 J V (without room for these on the device, its first call builds them).  stream: a cudaStream_t
  * (NULL = legacy default stream) on which all of this context's work runs.  All
  * fields start at zero; all faces start with natural (zero-flux) conditions. */
 int pnp_ctx_create(const pnp_mesh* m, const pnp_params* p, void* stream, pnp_ctx** out);
@@ -311,9 +312,10 @@ int pnp_jv(pnp_ctx* c, const double* U, const void* V, void* JV, int precision);
  * pnp_jv(..., PNP_F32) at that U up to FP32 summation order.  A later solver call
  * (pnp_gmres, pnp_newton_solve, pnp_time_step) replaces the stored linearisation;
  * pnp_jv_linearized then returns PNP_ERR_STATE until pnp_linearize is called again.
- * The J V kernel streams its mesh tables through shared memory with bulk copies; if one of its bounded waits on them gives up, the block waits (with a longer bound) for
- * the copies it issued, exits, and the call raises PNP_ERR_DEVICE_FLAG (here, and from the
- * solver calls that use it).  The flag stays set until the next linearisation (a
+ * The J V kernel streams its mesh tables through shared memory with bulk copies; if one of its
+ * bounded waits on them gives up, the block waits (with a longer bound) for the copies it
+ * issued, exits, and the call raises PNP_ERR_DEVICE_FLAG (here, and from the solver calls that
+ * use it).  The flag stays set until the next linearisation (a
  * pnp_linearize, or the start of the next flexible Krylov solve). */
 int pnp_linearize(pnp_ctx* c, const double* U);
 int pnp_jv_linearized(pnp_ctx* c, const float* V, float* JV);
